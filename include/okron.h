@@ -167,17 +167,20 @@ typedef struct okr_summary {
     int64_t terms;              /* incremental engine, profile mode: (candidate, phase-node, scenario)
                                    items evaluated over the run, the initial evaluation, the merges'
                                    own evaluations and FP64 rescorings included (0 otherwise) */
-    /* incremental engine: the launch shape that ran (okr_inc_shape's meaning; 0 for the sweep) */
+    /* incremental engine: the launch shape that ran (okr_inc_shape's meaning; 0 for the sweep).  A
+     * feeder large enough is searched by a cluster of CTAs of that shape; inc_records is then the
+     * placement one CTA would have taken (the cluster keeps its records in shared memory). */
     int32_t inc_threads, inc_eval_warps, inc_shared_entries, inc_records;
     int64_t pruned;             /* prune_exact: candidates excluded by the certified bound over the run */
 } okr_summary;
 
-/* Launch shape of the incremental engine (one CTA runs one feeder's search).
- * Every shape gives the same results; only the time differs.  Set per
+/* Launch shape of the incremental engine: each CTA of a feeder's search (one,
+ * or the CTAs of a cluster; a forced record placement runs one).  Every shape gives the same results; only the time differs.  Set per
  * context (okr_set_inc_shape), used by the later okr_reduce* and
  * okr_reduce_batch calls on it.  A field of 0 takes its default. */
 typedef struct okr_inc_shape {
-    int32_t threads;            /* threads of the CTA: 256, 384 or 512 (0 = 384) */
+    int32_t threads;            /* threads of a CTA: 256, 384 or 512 (0 = 384 for one CTA, 256 for a
+                                   cluster's) */
     int32_t eval_warps;         /* warps that evaluate the merge's own new values while the others
                                    find the changed candidates: 1 .. threads/32 - 1 (0 = 2, or 4
                                    with 512 threads) */

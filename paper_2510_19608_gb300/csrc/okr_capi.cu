@@ -559,21 +559,17 @@ okr_status run_search_inc(okr_ctx *ctx, const okr_params *p) {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
-    const IncShape sh = inc_shape_resolve(ctx->inc_shape);
-    int rec_used = -1;
-    {
-        size_t bytes = 0;
-        if (!inc_smem(n, true, sh, &rec_used, &bytes))
-            return fail(ctx, OKR_EINVAL, "incremental search: the forced record placement does not fit shared memory "
-                                         "for %d buses", n);
-    }
-    ctx->last_shape = sh;
-    ctx->last_rec = rec_used;
+    IncPlan pl;
+    if (!inc_plan(n, p->precision, ctx->inc_shape, p->record_iters > 0, &pl))
+        return fail(ctx, OKR_EINVAL, "incremental search: the forced record placement does not fit shared memory "
+                                     "for %d buses", n);
+    ctx->last_shape = pl.sh;
+    ctx->last_rec = pl.rec;
     cudaEventRecord(e0, st);
     cudaError_t e = launch_search_inc(p->precision, ctx->fb.T, ctx->fb.S, X, ctx->fb.I, ctx->fb.C,
-                                      p->engine == OKR_ENGINE_VERIFY ? 1 : 0, sh, &rec_used, st);
+                                      p->engine == OKR_ENGINE_VERIFY ? 1 : 0, pl, st);
     cudaEventRecord(e1, st);
-    ctx->launches += 2;                     // the first evaluation on many CTAs, the search on one
+    ctx->launches += 2;                     // the first evaluation on many CTAs, the search
     okr_status s = OKR_OK;
     if (e != cudaSuccess) s = fail(ctx, OKR_ECUDA, "search launch: %s", cudaGetErrorString(e));
     if (s == OKR_OK) {

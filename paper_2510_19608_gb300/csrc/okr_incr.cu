@@ -143,6 +143,34 @@ __device__ __forceinline__ void sadd128(unsigned long long *lo, unsigned long lo
     atomicAdd(hi, vh + ((old + vl < old) ? 1ull : 0ull));
 }
 
+// ---------------------------------------------------------------- clusters
+// A search runs on one cluster of cs CTAs (1, 2, 4 or 8).  csync: every thread
+// of the cluster waits for every other's, and all memory written before it
+// (shared, remote shared, device) is seen after it.
+__device__ __forceinline__ void csync(int cs) {
+    if (cs == 1) {
+        __syncthreads();
+    } else {
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+}
+__device__ __forceinline__ int cluster_rank() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return (int)r;
+}
+// 32 bytes one warp publishes to another CTA's copy of the same shared array.
+struct __align__(16) Pub {
+    unsigned long long a, b, c, d;
+};
+__device__ __forceinline__ void publish(Pub *slot, int rank, const Pub &v) {
+    unsigned at;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((unsigned)__cvta_generic_to_shared(slot)), "r"(rank));
+    asm volatile("st.shared::cluster.v2.u64 [%0], {%1, %2};" ::"r"(at), "l"(v.a), "l"(v.b) : "memory");
+    asm volatile("st.shared::cluster.v2.u64 [%0], {%1, %2};" ::"r"(at + 16), "l"(v.c), "l"(v.d) : "memory");
+}
+
 // ---------------------------------------------------------------- block primitives
 // Every reduction: warps reduce with shuffles, warp 0 reduces the warps'
 // partials and publishes the result; two barriers.
@@ -843,7 +871,8 @@ __device__ __forceinline__ Cand entry_cand(const IncWork &w) {
 // phase masks in shared memory; further entries in global memory.
 constexpr int kSEMax = 256;
 struct Loc {
-    IncWork *wsm, *wgl;
+    IncWork *wsm, *wgl;         // (wgl: this CTA's part of the feeder's work buffer)
+    int *fpair, *rlist;         // this CTA's parts of Inc::fpair and Inc::rlist
     int se;                     // work entries in shared memory
     unsigned short *lst[2];
     const uint8_t *ph;
@@ -880,7 +909,10 @@ struct EvalSmem {
 //   tkey: the tie key (caller r, caller s), ~0u for an empty slot;
 //   maxm: per super-node, its largest MICE over the scenarios (0 when absorbed);
 //   span: per slot pair, what the changed-set scan tests first.
+// The slot pairs of a search are dealt out to its cluster's CTAs, pair w to
+// CTA w % cs; a CTA keeps its own pairs' records, pair w at index w / cs.
 struct Rec {
+    int lg;             // log2 of the cluster's size
     u128 *r0;
     ulonglong2 *r1;
     unsigned *tkey;
@@ -899,7 +931,10 @@ struct Rec {
     unsigned long long *bmx;    // [nb]
     unsigned char *dirty;       // [nb]
     int nb;
-    // (dirty is null in the first evaluation on many CTAs: the search marks every block)
+    // index of slot sl's record
+    __device__ __forceinline__ int at(int sl) const { return ((sl >> (lg + 1)) << 1) | (sl & 1); }
+    // (dirty is null where there are no summaries: the first evaluation on many
+    // CTAs, and a cluster of several CTAs, whose selection reads every record)
     __device__ __forceinline__ void touch(int sl) const { if (dirty) dirty[sl >> 5] = 1; }
     __device__ __forceinline__ void touch_sn(int k) const { if (dirty) dirty[k >> 4] = 1; }   // maxm of super-node k (slot 2k)
 };
@@ -928,8 +963,10 @@ __device__ __forceinline__ unsigned long long val_key(long long v) {
 
 __device__ __forceinline__ unsigned long long warp_max64(unsigned long long v) { return ~warp_min64(~v); }
 __device__ __forceinline__ u128 warp_min128(u128 v) {
-    for (int o = 16; o > 0; o >>= 1) v = umin(v, shfl_xor_u128(v, o));
-    return v;
+    // the smallest high word, then the smallest low word among the lanes that hold it
+    const unsigned long long hi = (unsigned long long)(v >> 64), mh = warp_min64(hi);
+    const unsigned long long ml = warp_min64(hi == mh ? (unsigned long long)v : ~0ull);
+    return ((u128)mh << 64) | ml;
 }
 
 // Pass B of the selection reads every record when they are in shared memory
@@ -972,8 +1009,9 @@ __device__ __forceinline__ void refresh_blocks(const Rec &R, int n) {
 template <int PREC>
 __device__ __forceinline__ void set_rec(const Rec &R, int sl, u128 d, u128 b, int viol, int vmay) {
     R.touch(sl);
+    const int at = R.at(sl);
     if (PREC == 0) {
-        R.r0[sl] = (viol == 0) ? okey(d) : kNone;
+        R.r0[at] = (viol == 0) ? okey(d) : kNone;
     } else {
         unsigned long long lo = kKeyNone, hi = kKeyNone;
         if (viol == 0) {
@@ -985,34 +1023,36 @@ __device__ __forceinline__ void set_rec(const Rec &R, int sl, u128 d, u128 b, in
                 if (!ok) hi = kKeyNone;
             }
         }
-        R.r1[sl] = make_ulonglong2(lo, hi);
+        R.r1[at] = make_ulonglong2(lo, hi);
     }
 }
 template <int PREC>
 __device__ __forceinline__ void kill_rec(const Rec &R, int sl) {
     R.touch(sl);
-    if (PREC == 0) R.r0[sl] = kNone;
-    else R.r1[sl] = make_ulonglong2(kKeyNone, kKeyNone);
-    R.tkey[sl] = ~0u;
+    const int at = R.at(sl);
+    if (PREC == 0) R.r0[at] = kNone;
+    else R.r1[at] = make_ulonglong2(kKeyNone, kKeyNone);
+    R.tkey[at] = ~0u;
 }
 
 // The merge's own evaluation (FP64, state before the merge): new voltage,
-// magnitude and MICE of each of its positions into the scratch.
+// magnitude and MICE of each of its positions into the scratch, the positions
+// spread over the cluster.
 struct Commit {
     const Win *h;
     Cand wc;
     const unsigned short *list;     // super-nodes before the merge
     const uint8_t *ph;
     Ovl O;                          // (not read: state 0)
-    unsigned short *map;            // the overlay map, filled here
 };
 
-// Run by warps [warp0, warp0 + nw) only.
+// Run by warps [warp0, warp0 + nw) of every CTA of the cluster (CTA cr of cs).
 __device__ __forceinline__ long long commit_groups(const Topo &T, const State &S, const Inc &I, int n, int L, int G,
-                                                   double margin, const Commit &cm, int warp0, int nw) {
+                                                   double margin, const Commit &cm, int warp0, int nw, int cr, int cs) {
     long long items = 0;
-    const int lw = ((int)threadIdx.x >> 5) - warp0, gpw = 32 / G, gl = threadIdx.x % G;
-    const int gi = lw * gpw + ((int)threadIdx.x & 31) / G, NG = nw * gpw;
+    // (positions go round the CTAs first, so that few positions meet few warps each)
+    const int lw = (((int)threadIdx.x >> 5) - warp0) * cs + cr, gpw = 32 / G, gl = threadIdx.x % G;
+    const int gi = lw * gpw + ((int)threadIdx.x & 31) / G, NG = nw * gpw * cs;
     const Win &h = *cm.h;
     const int n1 = h.q1hi - h.q1lo, n2 = h.q2hi - h.q2lo;
     for (int r0 = 0; r0 < h.npos; r0 += NG) {
@@ -1048,10 +1088,7 @@ __device__ __forceinline__ long long commit_groups(const Topo &T, const State &S
                 *cb_f4(cb, L, l, p) = make_float4(v32.x, v32.y, (float)(hh - mc), (float)(ll - mc));
             }
             if (l < L && p == 0) *cb_mice32(cb, L, l) = (float)cb[9 * L + l];
-            if (gl == 0) {
-                items += __popc(cm.ph[k]) * L;
-                cm.map[k] = (unsigned short)(q + 1);     // the terms after the merge read k's new values here
-            }
+            if (gl == 0) items += __popc(cm.ph[k]) * L;
         }
     }
     return items;
@@ -1223,8 +1260,8 @@ __device__ void rebuild_pair(const Topo &T, const State &S, const Search &X, con
                 hi = max(hi, max(max(c[d].s, c[d].r) + 1, max(c[d].js + c[d].ns, c[d].jr + c[d].nr)));
             }
             const bool any = c[0].s >= 0 || c[1].s >= 0;
-            R.span[w] = make_ushort4((unsigned short)(any ? lo : 0), (unsigned short)(any ? hi : 0),
-                                     (unsigned short)(x >= 0 ? x : 0xffff), (unsigned short)(any ? 1 : 0));
+            R.span[w >> R.lg] = make_ushort4((unsigned short)(any ? lo : 0), (unsigned short)(any ? hi : 0),
+                                             (unsigned short)(x >= 0 ? x : 0xffff), (unsigned short)(any ? 1 : 0));
         }
         for (int d = 0; d < 2; ++d) {
             const int sl = 2 * w + d;
@@ -1233,7 +1270,7 @@ __device__ void rebuild_pair(const Topo &T, const State &S, const Search &X, con
                 int2 seg[kIncMaxSeg];
                 const int ns = full_segments(c[d], Lc.rank, seg, V.r);
                 write_entry(Lc.ent(base + atomicAdd(cnt, 1)), sl, 1, ns, seg, c[d]);
-                R.tkey[sl] = (unsigned)c[d].key;
+                R.tkey[R.at(sl)] = (unsigned)c[d].key;
                 R.touch(sl);
             } else {
                 I.viol[sl] = kIncDead;
@@ -1260,12 +1297,15 @@ __device__ void rebuild_pairs(const Topo &T, const State &S, const Search &X, co
 // zeroes r*'s MICE.  `list`: the super-nodes before that merge.
 template <int NT>
 __device__ void write_back(const State &S, const Inc &I, const Win &hw, const unsigned short *list, const uint8_t *ph,
-                           unsigned short *map, int n, int L, int G) {
+                           unsigned short *map, int n, int L, int G, int cr, int cs) {
     // lanes from the last thread down (no shuffles here), beside the first
     // threads' updates of the entries' sums
     const int tid = threadIdx.x, rt = NT - 1 - tid, gl = rt % G, gi = rt / G, NG = NT / G, l = gl >> 2, p = gl & 3;
     const int n1 = hw.q1hi - hw.q1lo, n2 = hw.q2hi - hw.q2lo;
-    for (int j = gi; j < hw.npos; j += NG) {
+    // this CTA's own map
+    for (int j = rt; j < hw.npos; j += NT)
+        map[j < n1 ? list[hw.q1lo + j] : (j < n1 + n2 ? list[hw.q2lo + j - n1] : hw.s)] = 0;
+    for (int j = gi * cs + cr; j < hw.npos; j += NG * cs) {
         const int k = j < n1 ? list[hw.q1lo + j] : (j < n1 + n2 ? list[hw.q2lo + j - n1] : hw.s);
         if (k == hw.r) continue;
         const bool fx = j >= n1 + n2;
@@ -1290,23 +1330,23 @@ __device__ void write_back(const State &S, const Inc &I, const Win &hw, const un
             S.mice[(size_t)l * n + k] = cb[9 * L + l];
             S.mice32[(size_t)l * n + k] = *cb_mice32(cb, L, l);
         }
-        if (gl == 0) map[k] = 0;
     }
-    if (rt < L) {                           // r's cluster is gone
+    if (rt < L && cr == 0) {                // r's cluster is gone
         S.mice[(size_t)rt * n + hw.r] = 0.0;
         S.mice32[(size_t)rt * n + hw.r] = 0.0f;
     }
 }
 
 // ---------------------------------------------------------------- the search
-// Bytes of the selection records of an n-bus feeder.
+// Bytes of the selection records of n slot pairs.
 __host__ __device__ constexpr size_t rec_bytes(int n) { return (size_t)48 * n + 64; }
 // ... and with the per-super-node largest MICE after them (shared memory only).
 __host__ __device__ constexpr size_t rec_maxm_bytes(int n) { return rec_bytes(n) + (size_t)8 * n; }
 
-// Shared memory of one search: [work entries][two super-node lists][phase
-// masks][overlay map][super-node ranks][block summaries of the selection
-// records], then the selection records when they fit.
+// Shared memory of one CTA of a search: [work entries][two super-node lists]
+// [phase masks][overlay map][super-node ranks][a cluster of one: block
+// summaries of the selection records; of several: what they publish], then the records of the CTA's
+// slot pairs when they fit.
 __host__ __device__ constexpr size_t align16(size_t b) { return (b + 15) / 16 * 16; }
 // Blocks of 32 selection slots, and the bytes of their summaries.
 __host__ __device__ constexpr int sel_blocks(int n) { return (2 * n + 31) / 32; }
@@ -1314,20 +1354,30 @@ __host__ __device__ constexpr size_t sel_bytes(int n) {
     return align16((size_t)16 * sel_blocks(n)) + align16((size_t)4 * sel_blocks(n)) +
            align16((size_t)8 * sel_blocks(n)) + align16((size_t)sel_blocks(n));
 }
-// Every region is rounded up to 16 bytes: the block summaries and the
-// selection records are 16-byte keys.
-__host__ __device__ constexpr size_t base_bytes(int n, int se) {
+// What a cluster's warps publish to each other (at most 16 warps a CTA).
+constexpr int kMaxCluster = 8, kPubWarps = kMaxCluster * 16;
+__host__ __device__ constexpr size_t pub_bytes(int cs) {
+    return cs == 1 ? 0 : sizeof(Pub) * (2 * kPubWarps + 2 * kMaxCluster);
+}
+// Every region is rounded up to 16 bytes: the block summaries, the published
+// values and the selection records are 16-byte keys.
+__host__ __device__ constexpr size_t base_bytes(int n, int se, int cs) {
     return align16((size_t)se * sizeof(IncWork)) + align16((size_t)4 * n) + align16((size_t)n) + align16((size_t)2 * n) +
-           align16((size_t)4 * (n + 1)) + sel_bytes(n);
+           align16((size_t)4 * (n + 1)) + (cs == 1 ? sel_bytes(n) : pub_bytes(cs));
+}
+// Slot pairs of CTA cr of a cluster of cs, and how many the CTAs before it have.
+__host__ __device__ constexpr int own_pairs(int n, int cr, int cs) { return (n - cr + cs - 1) / cs; }
+__host__ __device__ constexpr int own_first(int n, int cr, int cs) {
+    return cr * (n / cs) + (cr < n % cs ? cr : n % cs);
 }
 
 template <int NT, int PREC>
 __device__ void inc_run(const Topo &T, const State &S, const Search &X, const Inc &I, Ctrl *C, bool verify,
-                        unsigned char *dyn, int rec_mode, int se, int cw, bool pre_init) {
+                        unsigned char *dyn, int rec_mode, int se, int cw, int cs) {
     static_assert(NT >= 128 && NT <= 1024 && NT % 32 == 0, "thread count");
     __shared__ __align__(16) EvalSmem<NT> E;
     __shared__ __align__(16) Red sred[33];
-    __shared__ __align__(16) Red64 s_sel[2];   // precision-1 selection accumulators: pass A, pass B
+    __shared__ __align__(16) Red64 s_sel;      // precision-1 selection accumulator of pass B, a cluster of one
     __shared__ int sscan[33];
     __shared__ unsigned long long s_sfx[2];     // SMICE of the committed state, fixed point
     __shared__ unsigned long long s_dsum[2];    // the last merge's change of it
@@ -1340,11 +1390,15 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
     const bool prof = C->profile != 0;
     const u128 tau_fx = to_fx(C->tau);
     if (C->done || C->t >= max_merges) return;
+    const int cr = cs == 1 ? 0 : cluster_rank(), lg = cs == 1 ? 0 : (cs == 2 ? 1 : (cs == 4 ? 2 : 3));
+    const int np = own_pairs(n, cr, cs), pfirst = own_first(n, cr, cs);     // this CTA's slot pairs: w = cr, cr + cs, ...
     // shared memory: entries, lists, phases; selection records: r0 or r1
-    // (2n x 16 B), tkey (2n x 4 B), span (n x 8 B)
+    // (16 B a slot), tkey (4 B a slot), span (8 B a pair)
     Loc Lc;
     Lc.wsm = reinterpret_cast<IncWork *>(dyn);
-    Lc.wgl = I.work;
+    Lc.wgl = I.work + 2 * (size_t)pfirst;
+    Lc.fpair = I.fpair + pfirst;
+    Lc.rlist = I.rlist + 2 * (size_t)pfirst;
     Lc.se = se;
     Lc.lst[0] = reinterpret_cast<unsigned short *>(dyn + align16((size_t)se * sizeof(IncWork)));
     Lc.lst[1] = Lc.lst[0] + n;
@@ -1359,14 +1413,25 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
     O.cbuf = I.cbuf;
     O.s = O.r = -1;
     O.nfree = 0;
-    unsigned char *recmem = rec_mode ? dyn + base_bytes(n, se) : I.recbuf;
+    unsigned char *recmem = rec_mode ? dyn + base_bytes(n, se, cs) : I.recbuf;      // (rec_mode 0: a cluster of one)
+    const int nrec = own_pairs(n, 0, cs);
+    // what each warp of each CTA publishes to every CTA: pass A, pass B; by CTA:
+    // the rescored candidates' minimum, their tie band (a cluster of one: unused)
+    Pub *s_pa = reinterpret_cast<Pub *>(dyn + base_bytes(n, se, cs) - pub_bytes(cs)), *s_pb = s_pa + kPubWarps,
+        *s_pc = s_pb + kPubWarps, *s_pd = s_pc + kMaxCluster;
     Rec R;
+    R.lg = lg;
     R.r0 = reinterpret_cast<u128 *>(recmem);
     R.r1 = reinterpret_cast<ulonglong2 *>(recmem);
-    R.tkey = reinterpret_cast<unsigned *>(recmem + (size_t)32 * n);
-    R.maxm = rec_mode == 2 ? reinterpret_cast<double *>(recmem + rec_bytes(n)) : I.maxm;
-    R.span = reinterpret_cast<ushort4 *>(recmem + (size_t)40 * n);
-    {
+    R.tkey = reinterpret_cast<unsigned *>(recmem + (size_t)32 * nrec);
+    R.span = reinterpret_cast<ushort4 *>(recmem + (size_t)40 * nrec);
+    R.maxm = rec_mode == 2 ? reinterpret_cast<double *>(recmem + rec_bytes(nrec)) : I.maxm;
+    R.bsum = nullptr;
+    R.bcnt = nullptr;
+    R.bmx = nullptr;
+    R.dirty = nullptr;
+    R.nb = 0;
+    if (cs == 1) {
         unsigned char *sm = reinterpret_cast<unsigned char *>(rank) + align16((size_t)4 * (n + 1));
         R.nb = sel_blocks(n);
         R.bsum = sm;
@@ -1381,21 +1446,18 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
     if (tid == 0) {
         s_sfx[0] = s_sfx[1] = 0ull;                 // every MICE starts at 0
         s_cnt[0] = s_cnt[1] = s_cnt[2] = s_cnt[3] = 0;
-        reset_sel(&s_sel[0]);
-        reset_sel(&s_sel[1]);
+        reset_sel(&s_sel);
     }
     unsigned long long tp = 0;
     auto stamp = [&](int i) {
-        if (prof && tid == 0) { const unsigned long long now = gtimer_inc(); C->phase_ns[i] += now - tp; tp = now; }
+        if (prof && tid == 0 && cr == 0) { const unsigned long long now = gtimer_inc(); C->phase_ns[i] += now - tp; tp = now; }
     };
     long long terms = 0, cands_run = 0;
     int rechecks = 0, recheck_cands = 0;
-    bool maxerr_done = true;                // dec_maxerr of the last merge written
 
-    // ---- every slot pair from the initial clusters (all singletons), every term
+    // ---- the initial clusters (all singletons); the first evaluation of every
+    // candidate ran on many CTAs (k_inc_init), its records in device memory
     for (int w = tid; w < n; w += NT) {
-        I.fpair[w] = w;
-        R.maxm[w] = 0.0;
         Lc.lst[0][w] = (unsigned short)w;
         phs[w] = __ldg(T.ph + w);
         ovl_map[w] = 0;
@@ -1403,76 +1465,121 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
     }
     if (tid == 0) rank[n] = S.sn_rank[n];
     for (int j = tid; j < R.nb; j += NT) R.dirty[j] = 1;
-    if (pre_init) {
-        // the first evaluation ran on many CTAs (k_inc_init): its records are in
-        // device memory in the same layout; bring them into shared memory
-        if (rec_mode) {
-            const uint4 *src = reinterpret_cast<const uint4 *>(I.recbuf);
-            uint4 *dst = reinterpret_cast<uint4 *>(recmem);
-            for (int i = tid; i < 3 * n; i += NT) dst[i] = src[i];       // 48 n bytes
+    {
+        const unsigned *tk = reinterpret_cast<const unsigned *>(I.recbuf + (size_t)32 * n);
+        const ushort4 *sp = reinterpret_cast<const ushort4 *>(I.recbuf + (size_t)40 * n);
+        for (int i = tid; i < np; i += NT) {
+            const int w = i * cs + cr;
+            R.maxm[i] = 0.0;
+            if (rec_mode) R.span[i] = sp[w];
+            for (int d = 0; d < 2; ++d) {
+                // the live candidates' keys from their carried sums (the first
+                // evaluation may have summed a candidate's terms on several CTAs)
+                const int sl = 2 * w + d, v = I.viol[sl];
+                if (rec_mode) R.tkey[2 * i + d] = tk[sl];
+                if (v == kIncDead) {
+                    if (rec_mode) kill_rec<PREC>(R, sl);
+                    continue;
+                }
+                set_rec<PREC>(R, sl, ld128(I.acc + 2 * (size_t)sl), PREC == 1 ? ld128(I.bnd + 2 * (size_t)sl) : (u128)0,
+                              v, PREC == 1 ? I.vmay[sl] : 0);
+            }
         }
-        __syncthreads();
-        // the live candidates' keys from their carried sums (the first evaluation
-        // may have summed a candidate's terms on several CTAs)
-        for (int sl = tid; sl < 2 * n; sl += NT) {
-            const int v = I.viol[sl];
-            if (v == kIncDead) continue;
-            set_rec<PREC>(R, sl, ld128(I.acc + 2 * (size_t)sl), PREC == 1 ? ld128(I.bnd + 2 * (size_t)sl) : (u128)0, v,
-                          PREC == 1 ? I.vmay[sl] : 0);
-        }
-        __syncthreads();
-    } else {
-        __syncthreads();
-        rebuild_pairs<NT, PREC>(T, S, X, I, n, I.fpair, n, &s_cnt[2], 0, R, Lc, no_view());
-        __syncthreads();
-        const int ne = s_cnt[2];
-        terms += run_entries<NT, PREC>(T, S, X, I, n, L, G, margin, mlo, mhi, 0, ne, kInit, Lc.lst[0], Lc.lst[0],
-                                       -1, O, E, sscan, R, Lc);
     }
+    csync(cs);                              // (every CTA runs before the first one publishes to another)
     if (prof && tid == 0) tp = gtimer_inc();
 
+    Win hw = {};                            // the last merge (a cluster of several CTAs writes it back in the next selection)
     for (;;) {
-        if (t >= max_merges) {
-            if (tid == 0) { C->done = 1; C->stop_reason = 0; }
-            break;
-        }
         const unsigned short *list_old = Lc.lst[t & 1];
         unsigned short *list_new = Lc.lst[(t + 1) & 1];
         // ============================================================ selection
-        // The blocks whose records changed are summarised again (one warp per
-        // block; the append counters are cleared before that barrier).
+        // pass A: precision 0: the minimum over feasible candidates; precision 1:
+        // the smallest lower end (m_lo) and the smallest upper end (m_hi); the
+        // largest MICE after the last merge; the candidates.
+        //   A cluster of one: the blocks whose records changed are summarised
+        // again (one warp per block, one barrier), then every warp reduces the
+        // summaries on its own.
+        //   A cluster of several: every warp reduces a strided share of its CTA's
+        // records (one or two a thread) and publishes the result to every CTA;
+        // one cluster barrier, then every warp of every CTA reduces what was
+        // published.
         if (tid == 0) s_cnt[0] = s_cnt[1] = s_cnt[2] = s_cnt[3] = 0;
-        refresh_blocks<NT, PREC>(R, n);
-        // pass A, by every warp on its own from the block summaries (no
-        // barrier): precision 0: the minimum over feasible candidates;
-        // precision 1: the smallest lower end (m_lo) and the smallest upper end
-        // (m_hi); the largest MICE after the last merge; the candidates.
         const int lane = tid & 31, wid = tid >> 5;
+        constexpr int NW = NT / 32;
         Red ra;
         ra.a = ra.b = ra.c = kNone;
         ra.i = 0;
         {
             unsigned long long mx = 0;
             unsigned cnt = 0;
-            if (PREC == 0) {
-                const u128 *bs = reinterpret_cast<const u128 *>(R.bsum);
-                u128 mn = kNone;
+            u128 mn = kNone;
+            unsigned long long lo = ~0ull, hi = ~0ull;
+            if (cs == 1) {
+                refresh_blocks<NT, PREC>(R, n);
                 for (int j = lane; j < R.nb; j += 32) {
-                    mn = umin(mn, bs[j]);
+                    if (PREC == 0) {
+                        mn = umin(mn, reinterpret_cast<const u128 *>(R.bsum)[j]);
+                    } else {
+                        const ulonglong2 b = reinterpret_cast<const ulonglong2 *>(R.bsum)[j];
+                        lo = b.x < lo ? b.x : lo;
+                        hi = b.y < hi ? b.y : hi;
+                    }
                     cnt += (unsigned)R.bcnt[j];
                     mx = R.bmx[j] > mx ? R.bmx[j] : mx;
                 }
+            } else {
+                for (int c = tid; c < 2 * np; c += NT) {
+                    if (PREC == 0) {
+                        mn = umin(mn, R.r0[c]);
+                    } else {
+                        const ulonglong2 q = R.r1[c];
+                        lo = q.x < lo ? q.x : lo;
+                        hi = q.y < hi ? q.y : hi;
+                    }
+                    cnt += R.tkey[c] != ~0u ? 1u : 0u;
+                    if ((c & 1) == 0) {
+                        const unsigned long long mb = (unsigned long long)__double_as_longlong(R.maxm[c >> 1]);
+                        mx = mb > mx ? mb : mx;
+                    }
+                }
+                {
+                    Pub v;
+                    if (PREC == 0) {
+                        mn = warp_min128(mn);
+                        v.a = (unsigned long long)mn;
+                        v.b = (unsigned long long)(mn >> 64);
+                    } else {
+                        v.a = warp_min64(lo);
+                        v.b = warp_min64(hi);
+                    }
+                    v.c = warp_max64(mx);
+                    v.d = __reduce_add_sync(0xffffffffu, cnt);
+                    if (lane < cs) publish(&s_pa[cr * NW + wid], lane, v);
+                }
+                csync(cs);
+                mn = kNone;
+                lo = hi = ~0ull;
+                mx = 0;
+                cnt = 0;
+                for (int j = lane; j < cs * NW; j += 32) {
+                    const Pub v = s_pa[j];
+                    if (PREC == 0) {
+                        mn = umin(mn, ((u128)v.b << 64) | (u128)v.a);
+                    } else {
+                        lo = v.a < lo ? v.a : lo;
+                        hi = v.b < hi ? v.b : hi;
+                    }
+                    mx = v.c > mx ? v.c : mx;
+                    cnt += (unsigned)v.d;
+                }
+                // the last merge's new values into the state (every CTA's terms
+                // have read the old ones; the barrier of pass B shows them)
+                if (t > 0 && !verify) write_back<NT>(S, I, hw, list_new, Lc.ph, ovl_map, n, L, G, cr, cs);
+            }
+            if (PREC == 0) {
                 ra.a = warp_min128(mn);
             } else {
-                const ulonglong2 *bs = reinterpret_cast<const ulonglong2 *>(R.bsum);
-                unsigned long long lo = ~0ull, hi = ~0ull;
-                for (int j = lane; j < R.nb; j += 32) {
-                    const ulonglong2 b = bs[j];
-                    lo = b.x < lo ? b.x : lo;
-                    hi = b.y < hi ? b.y : hi;
-                    cnt += (unsigned)R.bcnt[j];
-                    mx = R.bmx[j] > mx ? R.bmx[j] : mx;
-                }
                 lo = warp_min64(lo);
                 hi = warp_min64(hi);
                 ra.a = lo == kKeyNone ? kNone : (u128)lo;
@@ -1483,11 +1590,15 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
         }
         const int nvalid = ra.i;
         stamp(11);                                      // profile: block summaries and pass A
-        if (tid == 0) {
+        if (tid == 0 && cr == 0 && t > 0)
+            X.dec_maxerr[t - 1] = ra.c == kNone ? 0.0 : __longlong_as_double((long long)(unsigned long long)~ra.c);
+        if (t >= max_merges) {
+            if (tid == 0 && cr == 0) { C->done = 1; C->stop_reason = 0; }
+            break;
+        }
+        if (tid == 0 && cr == 0) {
             cands_run += nvalid;
             X.dec_ncand[t] = nvalid;
-            if (t > 0)
-                X.dec_maxerr[t - 1] = ra.c == kNone ? 0.0 : __longlong_as_double((long long)(unsigned long long)~ra.c);
         }
         if (t < X.rec_iters) {
             const double s_cur = fx_to_d(ld128(s_sfx));
@@ -1512,34 +1623,54 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
             if (tid == 0) X.rec_count[t] = nvalid;
         }
         if (ra.a == kNone) {                             // nothing (possibly) feasible
-            if (tid == 0) { C->done = 1; C->stop_reason = 1; }
-            maxerr_done = true;
+            if (tid == 0 && cr == 0) { C->done = 1; C->stop_reason = 1; }
             break;
         }
         // pass B: the smallest (tie key, slot) in the tie band and the smallest
         // key above it (precision 0); in precision 1, the smallest (tie key,
         // slot) surely in the band, the smallest tie key of a candidate the
         // screen cannot place, and the smallest lower end surely out of it.
-        // Records in shared memory, at most kFlatSelectMax buses: every record
-        // once, each thread a strided share of the slots, then one block
-        // reduction.  Otherwise only the blocks that may hold a candidate of the band are
+        // Records in shared memory, at most kFlatSelectMax buses (or a cluster of
+        // several CTAs): every record once, each thread a strided share of the
+        // slots, then one block reduction (the cluster: published by warp, as in
+        // pass A).  Otherwise only the blocks that may hold a candidate of the band are
         // read record by record (a block whose smallest key lies above the
         // band counts whole); with few such blocks every warp reads them all
         // and needs no barrier, with more they are spread over the warps.
         int ws = -1;
         double gap = INFINITY;
-        const bool flat_b = rec_mode != 0 && n <= kFlatSelectMax;
+        const bool flat_b = cs > 1 || (rec_mode != 0 && n <= kFlatSelectMax);
+        auto slot_of = [&](int c) { return ((((c >> 1) << lg) + cr) << 1) | (c & 1); };   // of the CTA's record c
         if (PREC == 0) {
             const u128 edge = (ra.a ^ kSignBit) + tau_fx, ek = okey(edge);
             u128 pa = kNone, pb = kNone;        // smallest (key, slot) in the band; smallest score above it
             if (flat_b) {
-                for (int c = tid; c < 2 * n; c += NT) {
+                for (int c = tid; c < 2 * np; c += NT) {
                     const u128 k = R.r0[c];
                     if (k == kNone) continue;
-                    if (k <= ek) pa = umin(pa, ((u128)R.tkey[c] << 32) | (u128)(unsigned)c);
+                    if (k <= ek) pa = umin(pa, ((u128)R.tkey[c] << 32) | (u128)(unsigned)slot_of(c));
                     else pb = umin(pb, k);
                 }
-                {
+                if (cs > 1) {
+                    // (a tie key with its slot fits 64 bits)
+                    Pub v;
+                    v.a = warp_min64((unsigned long long)pa);
+                    pb = warp_min128(pb);
+                    v.b = 0;
+                    v.c = (unsigned long long)pb;
+                    v.d = (unsigned long long)(pb >> 64);
+                    if (lane < cs) publish(&s_pb[cr * NW + wid], lane, v);
+                    csync(cs);
+                    unsigned long long qa = ~0ull;
+                    pb = kNone;
+                    for (int j = lane; j < cs * NW; j += 32) {
+                        const Pub u = s_pb[j];
+                        qa = u.a < qa ? u.a : qa;
+                        pb = umin(pb, ((u128)u.d << 64) | (u128)u.c);
+                    }
+                    pa = (u128)warp_min64(qa);
+                    pb = warp_min128(pb);
+                } else {
                     Red rb;
                     rb.a = pa;
                     rb.b = pb;
@@ -1606,13 +1737,13 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
             const unsigned long long eout = has_hi ? val_key(m_hi + tau_up) : kKeyNone;
             unsigned long long pa = ~0ull, pb = ~0ull, pc = ~0ull;
             if (flat_b) {
-                for (int c = tid; c < 2 * n; c += NT) {
+                for (int c = tid; c < 2 * np; c += NT) {
                     const ulonglong2 q = R.r1[c];
                     if (q.x == kKeyNone) continue;
                     const bool in_sure = q.y <= ein;
                     const bool out_sure = has_hi && q.x > eout;     // (never both: lo <= hi, m_lo <= m_hi)
                     if (in_sure) {
-                        const unsigned long long kc = ((unsigned long long)R.tkey[c] << 32) | (unsigned)c;
+                        const unsigned long long kc = ((unsigned long long)R.tkey[c] << 32) | (unsigned)slot_of(c);
                         pa = kc < pa ? kc : pa;
                     } else if (!out_sure) {
                         const unsigned long long key = R.tkey[c];
@@ -1621,13 +1752,31 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                         pc = q.x < pc ? q.x : pc;
                     }
                 }
-                {
+                if (cs > 1) {
+                    Pub v;
+                    v.a = warp_min64(pa);
+                    v.b = warp_min64(pb);
+                    v.c = warp_min64(pc);
+                    v.d = 0;
+                    if (lane < cs) publish(&s_pb[cr * NW + wid], lane, v);
+                    csync(cs);
+                    pa = pb = pc = ~0ull;
+                    for (int j = lane; j < cs * NW; j += 32) {
+                        const Pub u = s_pb[j];
+                        pa = u.a < pa ? u.a : pa;
+                        pb = u.b < pb ? u.b : pb;
+                        pc = u.c < pc ? u.c : pc;
+                    }
+                    pa = warp_min64(pa);
+                    pb = warp_min64(pb);
+                    pc = warp_min64(pc);
+                } else {
                     Red64 r6;
                     r6.a = pa;
                     r6.b = pb;
                     r6.c = pc;
                     r6.i = 0;
-                    r6 = block_sel64(r6, &s_sel[1]);
+                    r6 = block_sel64(r6, &s_sel);
                     pa = r6.a;
                     pb = r6.b;
                     pc = r6.c;
@@ -1686,7 +1835,7 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                     r6.b = pb;
                     r6.c = pc;
                     r6.i = 0;
-                    r6 = block_sel64(r6, &s_sel[1]);
+                    r6 = block_sel64(r6, &s_sel);
                     pa = r6.a;
                     pb = r6.b;
                     pc = r6.c;
@@ -1705,56 +1854,86 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                 // FP64 rescoring of R: the possible minimizers and the uncertain
                 // candidates with a key below the smallest surely-in key
                 const unsigned long long mh = has_hi ? (unsigned long long)ra.b : kKeyNone;
-                for (int c = tid; c < 2 * n; c += NT) {
+                for (int c = tid; c < 2 * np; c += NT) {
                     const ulonglong2 q = R.r1[c];
                     if (q.x == kKeyNone) continue;
                     const bool in_sure = q.y <= ein;
                     const bool out_sure = has_hi && q.x > eout;
                     const bool unc = !in_sure && !out_sure && (u128)R.tkey[c] < ks;
                     if (unc || q.x <= mh) {
-                        const int o = atomicAdd(&s_cnt[3], 1);
-                        I.rlist[o] = c;
+                        const int o = atomicAdd(&s_cnt[3], 1), sl = slot_of(c);
+                        Lc.rlist[o] = sl;
                         int2 seg[kIncMaxSeg];
-                        const int k = full_segments(X.slot[c], rank, seg);
-                        write_entry(Lc.ent(o), c, 1, k, seg, X.slot[c]);
+                        const int k = full_segments(X.slot[sl], rank, seg);
+                        write_entry(Lc.ent(o), sl, 1, k, seg, X.slot[sl]);
                     }
                 }
                 __syncthreads();
                 const int nR = s_cnt[3];
                 terms += run_entries<NT, PREC>(T, S, X, I, n, L, G, margin, mlo, mhi, 0, nR, kF64, list_old, list_old,
                                                -1, O, E, sscan, R, Lc);
-                // exact selection over R, with the surely-in candidate of key ks
+                // exact selection over every CTA's R, with the surely-in candidate of key ks
                 Red rc;
                 rc.a = rc.b = rc.c = kNone;
                 rc.i = 0;
                 for (int i = tid; i < nR; i += NT) {
-                    const int c = I.rlist[i];
+                    const int c = Lc.rlist[i];
                     if (I.vviol[c] == 0) rc.a = umin(rc.a, okey(ld128(I.vacc + 2 * (size_t)c)));
                 }
                 rc = block_red<NT>(rc, sred);
+                int nR_all = nR;
+                if (cs > 1) {
+                    Pub v;
+                    v.a = (unsigned long long)rc.a;
+                    v.b = (unsigned long long)(rc.a >> 64);
+                    v.c = (unsigned long long)nR;
+                    v.d = 0;
+                    if (tid < cs) publish(&s_pc[cr], tid, v);
+                    csync(cs);
+                    rc.a = kNone;
+                    nR_all = 0;
+                    for (int j = 0; j < cs; ++j) {
+                        rc.a = umin(rc.a, ((u128)s_pc[j].b << 64) | (u128)s_pc[j].a);
+                        nR_all += (int)s_pc[j].c;
+                    }
+                }
                 Red rd;
                 rd.a = rd.b = rd.c = kNone;
                 rd.i = 0;
                 if (rc.a != kNone) {
                     const u128 edge = (rc.a ^ kSignBit) + tau_fx, ek = okey(edge);
                     for (int i = tid; i < nR; i += NT) {
-                        const int c = I.rlist[i];
+                        const int c = Lc.rlist[i];
                         if (I.vviol[c] != 0) continue;
                         const u128 k = okey(ld128(I.vacc + 2 * (size_t)c));
-                        if (k <= ek) rd.a = umin(rd.a, ((u128)R.tkey[c] << 32) | (u128)(unsigned)c);
+                        if (k <= ek) rd.a = umin(rd.a, ((u128)R.tkey[R.at(c)] << 32) | (u128)(unsigned)c);
                         else rd.b = umin(rd.b, k);
                     }
                     rd = block_red<NT>(rd, sred);
+                    if (cs > 1) {
+                        Pub v;                      // (a tie key with its slot fits 64 bits; none: ~0)
+                        v.a = (unsigned long long)rd.a;
+                        v.b = (unsigned long long)rd.b;
+                        v.c = (unsigned long long)(rd.b >> 64);
+                        v.d = 0;
+                        if (tid < cs) publish(&s_pd[cr], tid, v);
+                        csync(cs);
+                        rd.a = rd.b = kNone;
+                        for (int j = 0; j < cs; ++j) {
+                            if (s_pd[j].a != ~0ull) rd.a = umin(rd.a, (u128)s_pd[j].a);
+                            rd.b = umin(rd.b, ((u128)s_pd[j].c << 64) | (u128)s_pd[j].b);
+                        }
+                    }
                     if (tid == 0 && rd.b != kNone) gap = fx_to_d((rd.b ^ kSignBit) - edge);
                 }
                 const u128 best = umin(rd.a, rb.a);
                 ws = best == kNone ? -1 : (int)(unsigned)(best & 0xffffffffu);
                 ++rechecks;
-                recheck_cands += nR;
+                recheck_cands += nR_all;
             }
         }
         if (ws < 0) {                                    // FP64 rescoring found nothing feasible
-            if (tid == 0) { C->done = 1; C->stop_reason = 1; }
+            if (tid == 0 && cr == 0) { C->done = 1; C->stop_reason = 1; }
             break;
         }
         stamp(0);
@@ -1763,12 +1942,11 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
         // thread knows ws; one broadcast load of its candidate), so no warp
         // waits for another's copy (r*'s subtree and the decision's bus ids
         // are looked up in the merge step).
-        constexpr int NW = NT / 32;
         const int CW = cw;                  // warps that evaluate the merge (1 .. NW - 1)
         const bool commit_warp = (tid >> 5) >= NW - CW;
-        const Win hw = make_win(X.slot[ws], ws, rank);
+        hw = make_win(X.slot[ws], ws, rank);
         if (tid == 0) {
-            X.dec_gap[t] = gap;
+            if (cr == 0) X.dec_gap[t] = gap;
             s_dsum[0] = 0ull;
             s_dsum[1] = 0ull;
         }
@@ -1778,8 +1956,8 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
         O.nfree = (hw.q1hi - hw.q1lo) + (hw.q2hi - hw.q2lo);
         // ---- which candidates change: rebuilt pairs (next to s* or r*) and
         // changed terms; entries are appended in any order (the sums are exact).
-        // The last warps evaluate the merge's own FP64 values meanwhile and
-        // map its positions for the overlay.
+        // Each CTA scans its own slot pairs.  The last warps evaluate the merge's
+        // own FP64 values meanwhile; the others map its positions for the overlay.
         {
             if (commit_warp) {
                 Commit cm;
@@ -1788,19 +1966,33 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                 cm.list = list_old;
                 cm.ph = Lc.ph;
                 cm.O = O;
-                cm.map = ovl_map;
-                terms += commit_groups(T, S, I, n, L, G, margin, cm, NW - CW, CW);
+                terms += commit_groups(T, S, I, n, L, G, margin, cm, NW - CW, CW, cr, cs);
             } else {
+                const int nsc = (NW - CW) * 32, n1 = hw.q1hi - hw.q1lo;
+                for (int q = tid; q < hw.npos; q += nsc) {      // the terms after the merge read k's new values here
+                    const int k = q < n1 ? list_old[hw.q1lo + q] : (q < O.nfree ? list_old[hw.q2lo + q - n1] : hw.s);
+                    if (k != hw.r) ovl_map[k] = (unsigned short)(q + 1);
+                }
+                // s takes r's injection (no term before the merge reads s's injection:
+                // every candidate with r = s* is rebuilt; the merge's own evaluation
+                // reads r's)
+                if (tid < 3 * L && cr == 0 && (Lc.ph[hw.r] >> (tid % 3) & 1u)) {
+                    const size_t is = sidx(tid / 3, tid % 3, hw.s, n), ir = sidx(tid / 3, tid % 3, hw.r, n);
+                    const double2 ni = cadd(S.icur[is], S.icur[ir]);
+                    S.icur[is] = ni;
+                    S.icur32[is] = make_float2((float)ni.x, (float)ni.y);
+                }
                 // the changed buses lie in [hl, hh): a candidate whose span misses it is unchanged
                 int hl = min(hw.s, hw.r), hh = max(hw.s, hw.r) + 1;
                 if (hw.w1lo < hw.w1hi) { hl = min(hl, hw.w1lo); hh = max(hh, hw.w1hi); }
                 if (hw.w2lo < hw.w2hi) { hl = min(hl, hw.w2lo); hh = max(hh, hw.w2hi); }
-                for (int w = tid; w < n; w += (NW - CW) * 32) {
-                    const ushort4 sp = R.span[w];
+                for (int i = tid; i < np; i += nsc) {
+                    const ushort4 sp = R.span[i];
+                    const int w = (i << lg) + cr;
                     if (sp.w == 0 || w == hw.r) continue;
                     const int qp = sp.z == 0xffff ? -1 : (int)sp.z;
                     if (w == hw.s || qp == hw.r || qp == hw.s) {
-                        I.fpair[atomicAdd(&s_cnt[0], 1)] = w;
+                        Lc.fpair[atomicAdd(&s_cnt[0], 1)] = w;
                         continue;
                     }
                     if ((int)sp.y <= hl || (int)sp.x >= hh) continue;
@@ -1814,12 +2006,9 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                 }
             }
         }
-        __syncthreads();
+        csync(cs);
         const int nf_tot = s_cnt[0], np_tot = s_cnt[1];   // (s_cnt[2] is 0: rebuilt entries follow these)
-        if (PREC == 1 && tid == 0) {                 // every thread has read both selection results
-            reset_sel(&s_sel[0]);
-            reset_sel(&s_sel[1]);
-        }
+        if (PREC == 1 && tid == 0) reset_sel(&s_sel);     // every thread has read the selection's result
         stamp(1);
         // ============================================================ the merge (score change, topology) and,
         // beside it, the rebuilt candidates
@@ -1854,8 +2043,8 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                     const unsigned long long y = __shfl_xor_sync(0xffffffffu, mb, o);
                     mb = y > mb ? y : mb;
                 }
-                if (valid && gl == 0) {
-                    R.maxm[k] = __longlong_as_double((long long)mb);
+                if (valid && gl == 0 && (k & (cs - 1)) == cr) {
+                    R.maxm[k >> lg] = __longlong_as_double((long long)mb);
                     R.touch_sn(k);
                 }
             }
@@ -1867,39 +2056,31 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
             constexpr int NB = NT - 32;
             if (tid < NB) {
                 const int rtop = S.top[hw.r], rtop_end = rtop + T.sz[rtop];
-                for (int b = rtop + tid; b < rtop_end; b += NB)
+                for (int b = rtop + tid * cs + cr; b < rtop_end; b += NB * cs)
                     if (S.label[b] == hw.r) S.label[b] = hw.s;
                 for (int j = tid; j < ns - 1; j += NB) list_new[j] = list_old[j + (j >= hw.jr ? 1 : 0)];
             }
-            // s takes r's injection (no term before the merge reads s's injection:
-            // every candidate with r = s* is rebuilt)
-            const unsigned phr = Lc.ph[hw.r];
-            if (tid < 3 * L) {
-                const int l = tid / 3, q = tid % 3;
-                if (phr >> q & 1u) {
-                    const size_t is = sidx(l, q, hw.s, n), ir = sidx(l, q, hw.r, n);
-                    const double2 ni = cadd(S.icur[is], S.icur[ir]);
-                    S.icur[is] = ni;
-                    S.icur32[is] = make_float2((float)ni.x, (float)ni.y);
-                }
-            }
-            if (tid == 0) {
+            if (tid == 0 && cr == 0) {
                 if (hw.dir == 1) {
                     S.top[hw.s] = S.top[hw.r];
                     S.ptop[hw.s] = S.ptop[hw.r];
                 }
                 I.qpar[hw.r] = -1;
-                R.maxm[hw.r] = 0.0;
-                R.touch_sn(hw.r);
                 X.dec_s[t] = T.orig[hw.s];
                 X.dec_r[t] = T.orig[hw.r];
             }
-            if (tid < 2) {
-                X.slot[2 * hw.r + tid].s = -1;
-                I.viol[2 * hw.r + tid] = kIncDead;
-                kill_rec<PREC>(R, 2 * hw.r + tid);
+            if ((hw.r & (cs - 1)) == cr) {
+                if (tid == 0) {
+                    R.maxm[hw.r >> lg] = 0.0;
+                    R.touch_sn(hw.r);
+                    R.span[hw.r >> lg] = make_ushort4(0, 0, 0xffff, 0);
+                }
+                if (tid < 2) {
+                    X.slot[2 * hw.r + tid].s = -1;
+                    I.viol[2 * hw.r + tid] = kIncDead;
+                    kill_rec<PREC>(R, 2 * hw.r + tid);
+                }
             }
-            if (tid == 0) R.span[hw.r] = make_ushort4(0, 0, 0xffff, 0);
         }
         // rebuilt pairs from the last thread down, reading the clusters through the
         // merge's view (the ranks change only after the terms below)
@@ -1908,7 +2089,7 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
             V.s = hw.s;
             V.r = hw.r;
             V.dir = hw.dir;
-            rebuild_pairs<NT, PREC>(T, S, X, I, n, I.fpair, nf_tot, &s_cnt[2], np_tot, R, Lc, V);
+            rebuild_pairs<NT, PREC>(T, S, X, I, n, Lc.fpair, nf_tot, &s_cnt[2], np_tot, R, Lc, V);
         }
         __syncthreads();
         ns -= 1;
@@ -1917,26 +2098,32 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
         if (tid == 0) {
             const u128 sfx = ld128(s_sfx) + ld128(s_dsum);
             st128(s_sfx, sfx);
-            X.dec_score[t] = fx_to_d(sfx);
+            if (cr == 0) X.dec_score[t] = fx_to_d(sfx);
         }
         // ============================================================ the terms that change
         terms += run_entries<NT, PREC>(T, S, X, I, n, L, G, margin, mlo, mhi, 0, ne_new, kMerge, list_old, list_new, hw.r,
-                                       O, E, sscan, R, Lc, prof ? C->phase_ns + 6 : nullptr, false);
+                                       O, E, sscan, R, Lc, prof && cr == 0 ? C->phase_ns + 6 : nullptr, false);
         // the new values into the state (no term reads the state before the
-        // merge any more; this overlaps the last tile's updates of the sums);
-        // ranks past r* drop by one
-        write_back<NT>(S, I, hw, list_old, Lc.ph, ovl_map, n, L, G);
+        // merge any more; this overlaps the last tile's updates of the sums), in
+        // a cluster of several CTAs once all of them are past their terms (in
+        // the next selection); ranks past r* drop by one
+        if (cs == 1) write_back<NT>(S, I, hw, list_old, Lc.ph, ovl_map, n, L, G, 0, 1);
         for (int b = hw.r + 1 + tid; b <= n; b += NT) rank[b] -= 1;
         __syncthreads();
         stamp(3);
         t += 1;
-        maxerr_done = false;
         if (verify) {
+            if (cs > 1) {
+                csync(cs);
+                write_back<NT>(S, I, hw, list_old, Lc.ph, ovl_map, n, L, G, cr, cs);
+                csync(cs);
+            }
             // every candidate again from scratch (after the merge, through the
             // overlay); the carried values must match bit for bit
             if (tid == 0) s_cnt[3] = 0;
             __syncthreads();
-            for (int c = tid; c < 2 * n; c += NT) {
+            for (int i = tid; i < 2 * np; i += NT) {
+                const int c = slot_of(i);
                 const Cand &cc = X.slot[c];
                 if (cc.s < 0) continue;
                 int2 seg[kIncMaxSeg];
@@ -1947,7 +2134,8 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
             run_entries<NT, PREC>(T, S, X, I, n, L, G, margin, mlo, mhi, 0, s_cnt[3], kFresh, list_new, list_new, -1,
                                   O, E, sscan, R, Lc);
             int bad = 0;
-            for (int c = tid; c < 2 * n; c += NT) {
+            for (int i = tid; i < 2 * np; i += NT) {
+                const int c = slot_of(i);
                 if (X.slot[c].s < 0) continue;
                 if (I.viol[c] != I.vviol[c] || ld128(I.acc + 2 * (size_t)c) != ld128(I.vacc + 2 * (size_t)c)) ++bad;
             }
@@ -1955,22 +2143,15 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
             rv.a = rv.b = rv.c = kNone;
             rv.i = bad;
             rv = block_red<NT>(rv, sred);
-            if (tid == 0 && rv.i) C->inc_mismatch += rv.i;
+            if (tid == 0 && rv.i) atomicAdd(&C->inc_mismatch, rv.i);
         }
-    }
-    if (!maxerr_done && t > 0) {
-        Red rm;
-        rm.a = rm.b = rm.c = kNone;
-        rm.i = 0;
-        for (int w = tid; w < n; w += NT) rm.a = umin(rm.a, ~(u128)(unsigned long long)__double_as_longlong(R.maxm[w]));
-        rm = block_red<NT>(rm, sred);
-        if (tid == 0) X.dec_maxerr[t - 1] = rm.a == kNone ? 0.0 : __longlong_as_double((long long)(unsigned long long)~rm.a);
     }
     if (prof) {                                     // (phase-node, scenario) items evaluated over the run
         unsigned long long tt = (unsigned long long)terms;
         for (int o = 16; o > 0; o >>= 1) tt += __shfl_xor_sync(0xffffffffu, tt, o);
         if ((tid & 31) == 0) atomicAdd(reinterpret_cast<unsigned long long *>(&C->sweep_ns), tt);
     }
+    if (cr != 0) return;
     for (int b = tid; b <= n; b += NT) S.sn_rank[b] = rank[b];
     if (tid == 0) {
         C->t = t;
@@ -1991,10 +2172,10 @@ namespace {
 // the merge beside the changed-set scan.
 template <int NT, int PREC>
 __global__ void __launch_bounds__(NT, 1) k_search_inc(Topo T, State S, Search X, Inc I, Ctrl *C, int verify,
-                                                      int rec_mode, int se, int cw, int pre_init) {
+                                                      int rec_mode, int se, int cw, int cs) {
     extern __shared__ __align__(16) unsigned char inc_dyn[];
     if (X.setup_err && *X.setup_err != 0) return;           // the setup failed: no result (C->done stays 0)
-    inc_run<NT, PREC>(T, S, X, I, C, verify != 0, inc_dyn, rec_mode, se, cw, pre_init != 0);
+    inc_run<NT, PREC>(T, S, X, I, C, verify != 0, inc_dyn, rec_mode, se, cw, cs);
 }
 
 // The first evaluation of every candidate (every slot pair from the initial
@@ -2035,11 +2216,13 @@ __device__ void inc_init_share(const Topo &T, const State &S, const Search &X, c
     Loc Lc;
     Lc.wsm = nullptr;
     Lc.wgl = I.work;
+    Lc.fpair = Lc.rlist = nullptr;
     Lc.se = 0;
     Lc.lst[0] = Lc.lst[1] = list;
     Lc.ph = T.ph;
     Lc.rank = S.sn_rank;
     Rec R;
+    R.lg = 0;
     R.r0 = reinterpret_cast<u128 *>(I.recbuf);
     R.r1 = reinterpret_cast<ulonglong2 *>(I.recbuf);
     R.tkey = reinterpret_cast<unsigned *>(I.recbuf + (size_t)32 * n);
@@ -2217,7 +2400,7 @@ __global__ void k_inc_zero_batch(const BatchFeeder *fd, const int *order, int nf
 // One CTA per feeder, feeders in the order given (largest first).
 template <int NT, int PREC>
 __global__ void __launch_bounds__(NT) k_search_inc_batch(const BatchFeeder *fd, const int *order, int nf,
-                                                         int rec_mode, int se, int cw, int pre_init) {
+                                                         int rec_mode, int se, int cw) {
     extern __shared__ __align__(16) unsigned char inc_dyn[];
     __shared__ Topo sT;
     __shared__ State sS;
@@ -2235,7 +2418,7 @@ __global__ void __launch_bounds__(NT) k_search_inc_batch(const BatchFeeder *fd, 
     __syncthreads();
     Ctrl *C = fd[f].C;
     const bool ok = *fd[f].setup_err == 0;
-    if (ok) inc_run<NT, PREC>(sT, sS, sX, sI, C, false, inc_dyn, rec_mode, se, cw, pre_init != 0);
+    if (ok) inc_run<NT, PREC>(sT, sS, sX, sI, C, false, inc_dyn, rec_mode, se, cw, 1);
     __syncthreads();
     for (int i = threadIdx.x; i < sT.n; i += NT) fd[f].super_out[i] = ok ? sT.orig[sS.label[sT.pre[i]]] : -1;
     if (threadIdx.x == 0) {
@@ -2246,6 +2429,7 @@ __global__ void __launch_bounds__(NT) k_search_inc_batch(const BatchFeeder *fd, 
 
 constexpr size_t kIncSmemMax = 200 * 1024;  // largest dynamic shared memory of one search
 constexpr int kInitThreads = 384;           // CTAs of the first evaluation
+constexpr int kClusterMin64 = 200, kClusterMin32 = 1500;    // buses from which a cluster searches (inc_plan)
 
 template <typename K>
 cudaError_t set_smem(K kern, size_t bytes) {
@@ -2269,7 +2453,7 @@ IncShape inc_shape_resolve(IncShape sh) {
 // false when a forced placement does not fit (or asks for the per-super-node
 // maximum where `maxm` is false).
 bool inc_smem(int n, bool maxm, const IncShape &sh, int *rec_mode, size_t *bytes) {
-    const size_t base = base_bytes(n, sh.se);
+    const size_t base = base_bytes(n, sh.se, 1);
     const bool fit2 = maxm && base + rec_maxm_bytes(n) <= kIncSmemMax;
     const bool fit1 = base + rec_bytes(n) <= kIncSmemMax;
     int m = sh.rec;
@@ -2280,13 +2464,39 @@ bool inc_smem(int n, bool maxm, const IncShape &sh, int *rec_mode, size_t *bytes
     return true;
 }
 
+// One CTA or a cluster of kMaxCluster.  A cluster shares out the scan over the
+// slot pairs, the FP64 evaluation of the merge, the changed terms and the
+// records (which then always fit shared memory), and pays three cluster
+// barriers a merge (about 0.5 us each with stores in flight) and L2 in place of
+// L1 latency.  Search ms, one CTA of 384 threads / eight of 256:
+//   FP64 terms:  40 buses 0.56 / 0.64, 333 buses (3 scenarios) 5.7 / 4.1, 1,000 9.8 / 8.2, 3,100 60.3 / 42.2
+//   FP32 terms: 333 buses 4.11 / 4.08, 1,000 7.14 / 7.40, 2,200 33.8 / 30.4, 3,100 46.2 / 37.4
+// (two and four CTAs lie between the two).  A forced record placement asks for
+// one CTA's memory, and recorded iterations are compacted by one CTA.
+bool inc_plan(int n, int precision, const IncShape &raw, bool records_iters, IncPlan *out) {
+    out->sh = inc_shape_resolve(raw);
+    out->cs = 1;
+    if (!inc_smem(n, true, out->sh, &out->rec, &out->bytes)) return false;
+    if (out->sh.rec >= 0 || records_iters || n < (precision == 0 ? kClusterMin64 : kClusterMin32)) return true;
+    const size_t b = base_bytes(n, out->sh.se, kMaxCluster) + rec_maxm_bytes(own_pairs(n, 0, kMaxCluster));
+    if (b > kIncSmemMax) return true;
+    out->cs = kMaxCluster;
+    out->bytes = b;
+    // fewer warps meet at the cluster's barriers (384 threads: 1,000 buses FP64 8.50 ms, 3,100 FP32 39.5)
+    if (raw.threads == 0) {
+        IncShape sh = raw;
+        sh.threads = 256;
+        out->sh = inc_shape_resolve(sh);
+    }
+    return true;
+}
+
 namespace {
 
 template <int NT, int PREC>
-cudaError_t launch_one(Topo T, State S, Search X, Inc I, Ctrl *C, int verify, int use, size_t smem, const IncShape &sh,
-                       cudaStream_t st) {
+cudaError_t launch_one(Topo T, State S, Search X, Inc I, Ctrl *C, int verify, const IncPlan &pl, cudaStream_t st) {
     // the first evaluation spread over the SMs (its sums start at zero), then
-    // the search on one CTA
+    // the search on one cluster
     static int sms = 0;
     if (sms == 0) {
         int dev = 0;
@@ -2301,9 +2511,21 @@ cudaError_t launch_one(Topo T, State S, Search X, Inc I, Ctrl *C, int verify, in
     if (e == cudaSuccess && ismem > 48 * 1024) e = set_smem(k_inc_init<kInitThreads, PREC>, ismem);
     if (e == cudaSuccess) k_inc_init<kInitThreads, PREC><<<ginit, kInitThreads, ismem, st>>>(T, S, X, I, C);
     if (e == cudaSuccess) e = cudaGetLastError();
-    if (e == cudaSuccess) e = set_smem(k_search_inc<NT, PREC>, smem);
-    if (e == cudaSuccess) k_search_inc<NT, PREC><<<1, NT, smem, st>>>(T, S, X, I, C, verify, use, sh.se, sh.cw, 1);
-    return e != cudaSuccess ? e : cudaGetLastError();
+    if (e == cudaSuccess) e = set_smem(k_search_inc<NT, PREC>, pl.bytes);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)pl.cs);
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = pl.bytes;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)pl.cs;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_search_inc<NT, PREC>, T, S, X, I, C, verify,
+                              pl.cs > 1 ? 2 : pl.rec, pl.sh.se, pl.sh.cw, pl.cs);
 }
 
 template <int NT>
@@ -2314,27 +2536,22 @@ cudaError_t set_batch_smem(int precision, size_t smem) {
 template <int NT>
 void launch_batch(int precision, const BatchFeeder *fd, const int *order, int nf, int use, size_t smem,
                   const IncShape &sh, cudaStream_t st) {
-    if (precision == 1) k_search_inc_batch<NT, 1><<<nf, NT, smem, st>>>(fd, order, nf, use, sh.se, sh.cw, 1);
-    else k_search_inc_batch<NT, 0><<<nf, NT, smem, st>>>(fd, order, nf, use, sh.se, sh.cw, 1);
+    if (precision == 1) k_search_inc_batch<NT, 1><<<nf, NT, smem, st>>>(fd, order, nf, use, sh.se, sh.cw);
+    else k_search_inc_batch<NT, 0><<<nf, NT, smem, st>>>(fd, order, nf, use, sh.se, sh.cw);
 }
 
 }  // namespace
 
-cudaError_t launch_search_inc(int precision, Topo T, State S, Search X, Inc I, Ctrl *C, int verify, IncShape sh,
-                              int *rec_used, cudaStream_t st) {
-    sh = inc_shape_resolve(sh);
-    int use = 0;
-    size_t smem = 0;
-    if (!inc_smem(T.n, true, sh, &use, &smem)) return cudaErrorInvalidValue;
-    if (rec_used) *rec_used = use;
-    if (sh.threads == 256)
-        return precision == 1 ? launch_one<256, 1>(T, S, X, I, C, verify, use, smem, sh, st)
-                              : launch_one<256, 0>(T, S, X, I, C, verify, use, smem, sh, st);
-    if (sh.threads == 384)
-        return precision == 1 ? launch_one<384, 1>(T, S, X, I, C, verify, use, smem, sh, st)
-                              : launch_one<384, 0>(T, S, X, I, C, verify, use, smem, sh, st);
-    return precision == 1 ? launch_one<512, 1>(T, S, X, I, C, verify, use, smem, sh, st)
-                          : launch_one<512, 0>(T, S, X, I, C, verify, use, smem, sh, st);
+cudaError_t launch_search_inc(int precision, Topo T, State S, Search X, Inc I, Ctrl *C, int verify, const IncPlan &pl,
+                              cudaStream_t st) {
+    if (pl.sh.threads == 256)
+        return precision == 1 ? launch_one<256, 1>(T, S, X, I, C, verify, pl, st)
+                              : launch_one<256, 0>(T, S, X, I, C, verify, pl, st);
+    if (pl.sh.threads == 384)
+        return precision == 1 ? launch_one<384, 1>(T, S, X, I, C, verify, pl, st)
+                              : launch_one<384, 0>(T, S, X, I, C, verify, pl, st);
+    return precision == 1 ? launch_one<512, 1>(T, S, X, I, C, verify, pl, st)
+                          : launch_one<512, 0>(T, S, X, I, C, verify, pl, st);
 }
 
 cudaError_t prepare_search_inc_batch(int precision, int max_n, IncShape sh) {

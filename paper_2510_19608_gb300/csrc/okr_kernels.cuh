@@ -145,8 +145,8 @@ cudaError_t launch_search(int precision, int grid, Topo T, State S, Search X, Ct
 int search_blocks_per_sm();     // CTAs of the search kernel that fit one SM (0 on error)
 __global__ void k_export(Topo T, State S, double *super_vred, int *super_of, double *vhat_out);
 
-// okr_incr.cu -- the search with scores carried across iterations: one CTA per
-// feeder (verify = 1: every merge also re-evaluates every candidate and counts
+// okr_incr.cu -- the search with scores carried across iterations: one CTA or
+// one cluster per feeder (verify = 1: every merge also re-evaluates every candidate and counts
 // mismatches of the carried scores in C->inc_mismatch).
 //
 // Launch shape of that CTA: threads (256, 384 or 512), warps that evaluate the
@@ -174,10 +174,19 @@ IncShape inc_shape_resolve(IncShape sh);
 // Dynamic shared memory and record placement of one search; false when a
 // forced placement does not fit.
 bool inc_smem(int n, bool maxm, const IncShape &sh, int *rec_mode, size_t *bytes);
-// cudaErrorInvalidValue when the shape's forced record placement does not fit;
-// *rec_used (may be NULL): the placement that ran.
-cudaError_t launch_search_inc(int precision, Topo T, State S, Search X, Inc I, Ctrl *C, int verify, IncShape sh,
-                              int *rec_used, cudaStream_t st);
+// How one feeder is searched: the shape of each CTA, the CTAs (one, or a
+// cluster that shares the feeder), the record placement of one CTA (a cluster
+// keeps its records in its CTAs' shared memory) and the dynamic shared memory.
+struct IncPlan {
+    IncShape sh;
+    int cs, rec;
+    size_t bytes;
+};
+// The plan of an n-bus search under the given (unresolved) shape; false when
+// the shape's forced record placement does not fit.
+bool inc_plan(int n, int precision, const IncShape &raw, bool records_iters, IncPlan *out);
+cudaError_t launch_search_inc(int precision, Topo T, State S, Search X, Inc I, Ctrl *C, int verify, const IncPlan &pl,
+                              cudaStream_t st);
 // Many feeders: one CTA each, in the order given (prepare_search_inc_batch with
 // the same precision, shape and at least the same largest feeder first: it
 // sets the kernel's shared-memory attribute, which a stream capture must not
