@@ -387,12 +387,86 @@ __device__ int slot_geometry(const Topo &T, const State &S, const View &V, int n
     return x;
 }
 
+// ---------------------------------------------------------------- sums of terms
+// The sums of one tile of kTile work entries, as kLimbs signed limbs of
+// kLimbBits bits in 32-bit words of shared memory (limb i counts units of
+// 2^(kLimbBits i - 100)): a term is added limb by limb by the four lanes of its
+// scenario, each with one 32-bit add that returns nothing, and the entry's
+// 128-bit sum is put together once, modulo 2^128 -- the same integer as adding
+// 128-bit terms, in any order.  An entry takes at most 2 states x 4 scenarios x
+// 13,900 positions, 111,200 adds below 2^14 in size, which 31 bits hold.  (The
+// 128-bit adds these replace, a 64-bit shared add that returns the old value,
+// then the carry's, cost about 500 cycles of each round's chain, and the
+// 128-bit shifts and shuffles before them as much.)
+constexpr int kLimbBits = 14, kLimbs = 10, kTile = 192;
+struct EvalSmem {
+    int d[kLimbs][kTile + 1], b[kLimbs][kTile + 1];     // (+ 1: the limbs of an entry in different banks)
+    int n1[kTile], n2[kTile];
+    int off[kTile + 1];
+};
+__device__ __forceinline__ u128 limb_sum(const int (*x)[kTile + 1], int i) {
+    u128 v = 0;
+#pragma unroll
+    for (int k = 0; k < kLimbs; ++k) v += (u128)(__int128)x[k][i] << (kLimbBits * k);
+    return v;
+}
+__device__ __forceinline__ void limb_add(int (*x)[kTile + 1], int i, int k, int piece) {
+    if (piece != 0 && k < kLimbs) atomicAdd(&x[k][i], piece);
+}
+// Adds sgn * to_fx32(f) to sum i: lane p of the scenario's four adds piece p
+// (a 24-bit mantissa at any shift lies in three limbs); p = 3 adds `extra` to
+// the lowest limb.
+__device__ __forceinline__ void add_fx32(int (*x)[kTile + 1], int i, float f, int sgn, int p, int extra) {
+    const unsigned b = __float_as_uint(f);
+    int e = (int)((b >> 23) & 0xff);
+    unsigned m = b & 0x7fffffu;
+    if (e == 0xff) m = 0;
+    else if (e == 0) e = 1;
+    else m |= 1u << 23;
+    int sh = e - 150 + kFxShift;
+    if (sh < 0) {
+        m = sh <= -32 ? 0u : m >> (-sh);
+        sh = 0;
+    }
+    const int k = sh / kLimbBits, r = sh - k * kLimbBits;
+    int piece = (int)((unsigned)(((unsigned long long)m << r) >> (kLimbBits * p)) & ((1u << kLimbBits) - 1));
+    if (b >> 31) piece = -piece;
+    if (p == 3) piece = extra;
+    limb_add(x, i, p == 3 ? 0 : k + p, sgn < 0 ? -piece : piece);
+}
+// Adds sgn * to_fx(v) to sum i: lane p adds piece p, lane 0 also piece 4 (a
+// 53-bit mantissa lies in five limbs).
+__device__ __forceinline__ void add_fx64(int (*x)[kTile + 1], int i, double v, int sgn, int p) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    int e = (int)((b >> 52) & 0x7ff);
+    unsigned long long m = b & 0xfffffffffffffull;
+    if (e == 0x7ff) m = 0;
+    else if (e == 0) e = 1;
+    else m |= 1ull << 52;
+    int sh = e - 1075 + kFxShift;
+    if (sh < 0) {
+        m = sh <= -64 ? 0ull : m >> (-sh);
+        sh = 0;
+    }
+    const int k = sh / kLimbBits, r = sh - k * kLimbBits;
+    const bool neg = ((b >> 63) != 0) != (sgn < 0);
+    const int mask = (1 << kLimbBits) - 1;
+    // bits [14 p, 14 p + 14) of m << r: m has 53 bits, r < 14
+    const int lo = kLimbBits * p - r;
+    const int piece = (int)(lo >= 0 ? m >> lo : m << -lo) & mask;
+    limb_add(x, i, k + p, neg ? -piece : piece);
+    if (p == 0) {
+        const int top = (int)(m >> (4 * kLimbBits - r)) & mask;
+        limb_add(x, i, k + 4, neg ? -top : top);
+    }
+}
+
 // ---------------------------------------------------------------- term groups
 // A term (candidate c, position k) is evaluated by a group of G = 4 Lp lanes
 // (Lp = scenarios rounded up to a power of two): lane gl takes scenario
 // l = gl / 4 and phase p = gl % 4 (p = 3 idles).  Every lane of the warp calls
-// the group function (it shuffles); the results are the group's sums over its
-// scenarios (every lane holds them).
+// the group function (it shuffles); the four lanes of a scenario add its term
+// to the sums of the group's work entry.
 //
 // A group evaluates its term on one or two states, e in [e_lo, e_hi) (the
 // same range for every group of a warp): e = 0, the state as stored; e = 1,
@@ -487,10 +561,10 @@ struct In64 {
     double h, lo, hr, lr, mo, mr;
 };
 struct Out64 {
-    u128 t;
+    double dd;
     int tv;
 };
-__device__ __forceinline__ Out64 term_arith64(In64 x, double2 dv, bool one, bool moves, bool is_s, bool lvp0,
+__device__ __forceinline__ Out64 term_arith64(In64 x, double2 dv, bool one, bool moves, bool is_s, bool lv,
                                               double margin, double *out, int l, int p, int L) {
     // every operation explicitly rounded (no contraction): each inlined copy
     // gives the same bits for the same inputs
@@ -513,26 +587,28 @@ __device__ __forceinline__ Out64 term_arith64(In64 x, double2 dv, bool one, bool
     }
     double m = fmax(em, __shfl_xor_sync(0xffffffffu, em, 1));
     m = fmax(m, __shfl_xor_sync(0xffffffffu, m, 2));
-    Out64 r;
-    r.t = 0;
+    Out64 r;                            // (the same in the scenario's four lanes)
+    r.dd = 0.0;
     r.tv = 0;
-    if (lvp0) {
-        if (out) out[9 * L + l] = m;
-        double dd = __dsub_rn(m, x.mo);
-        if (is_s) dd = __dsub_rn(dd, x.mr);
-        r.t = to_fx(dd);
-        r.tv = (m > margin) ? 1 : 0;
+    if (lv) {
+        if (out) {
+            if (p == 0) out[9 * L + l] = m;
+        } else {
+            r.dd = __dsub_rn(m, x.mo);
+            if (is_s) r.dd = __dsub_rn(r.dd, x.mr);
+            r.tv = (m > margin) ? 1 : 0;
+        }
     }
     return r;
 }
 
-// FP64 term.  d = sum over l of fixed(new MICE - MICE_k [- MICE_r]); nv = scenarios
-// whose new MICE exceeds the margin.  out != nullptr (state 0 only): the new
-// voltage and magnitude per (l, p) and the new MICE per l (the merge).
+// FP64 term, per l fixed(new MICE - MICE_k [- MICE_r]) and whether the new MICE
+// exceeds the margin, added to sum ei of E.  out != nullptr (state 0 only): the
+// new voltage and magnitude per (l, p) and the new MICE per l (the merge), and
+// nothing is added.
 __device__ __forceinline__ void group_term64(const Topo &T, const State &S, const uint8_t *ph, int n, int L, int G,
                                              const Cand &c, int k, int e_lo, int e_hi, bool v_old, bool v_new,
-                                             const Ovl &O, int gl, double margin, double *out, u128 *d_out,
-                                             int *nv_out) {
+                                             const Ovl &O, int gl, double margin, double *out, EvalSmem *E, int ei) {
     const bool valid = v_old || v_new;
     const int l = gl >> 2, p = gl & 3;
     const bool lv = valid && l < L;
@@ -555,7 +631,7 @@ __device__ __forceinline__ void group_term64(const Topo &T, const State &S, cons
             at64(S, O, e, k, li, pi, n, L, true, &x.v, &x.h, &x.lo);
             if (is_s) at64(S, O, e, c.r, li, pi, n, L, false, nullptr, &x.hr, &x.lr);
         }
-        if (lv && ve && p == 0) {
+        if (lv && ve && !out) {
             x.mo = mice64(S, O, e, k, l, n, L);
             if (is_s) x.mr = mice64(S, O, e, c.r, l, n, L);
         }
@@ -579,25 +655,20 @@ __device__ __forceinline__ void group_term64(const Topo &T, const State &S, cons
             dv = cadd(dv, cmul(g, iq[q]));
         }
     }
-    u128 d = 0;
-    int nv = 0;
 #pragma unroll 1
     for (int e = e_lo; e < e_hi; ++e) {
         const bool ve = e == 0 ? v_old : v_new;
         const bool one = on && ve;
         St nxt = cur;
         if (e + 1 < e_hi) fetch(e + 1, nxt);
-        const Out64 r = term_arith64(cur, dv, one, moves, is_s, lv && ve && p == 0, margin, out, l, p, L);
+        const Out64 r = term_arith64(cur, dv, one, moves, is_s, lv && ve, margin, out, l, p, L);
         cur = nxt;
-        if (e == 1 || e_hi - e_lo == 1) { d += r.t; nv += r.tv; }
-        else { d -= r.t; nv -= r.tv; }
+        if (lv && ve && !out) {
+            const int sgn = (e == 1 || e_hi - e_lo == 1) ? 1 : -1;
+            add_fx64(E->d, ei, r.dd, sgn, p);
+            if (p == 0 && r.tv) atomicAdd(&E->n1[ei], sgn);
+        }
     }
-    for (int o = 4; o < G; o <<= 1) {            // the group's sum over its scenarios
-        d += shfl_xor_u128(d, o);
-        nv += __shfl_xor_sync(0xffffffffu, nv, o);
-    }
-    *d_out = d;
-    *nv_out = nv;
 }
 
 // The arithmetic of one FP32 term with its bound on one state's inputs (every
@@ -609,11 +680,11 @@ struct In32 {
     double mck, mcr;
 };
 struct Out32 {
-    u128 td, tb;
+    float dd, bl;
     int ts, tm;
 };
 __device__ __forceinline__ Out32 term_arith32(In32 x, float2 dv, float sdv, bool one, bool moves, bool sterm,
-                                              bool lvp0, float margin_lo, float margin_hi) {
+                                              bool lv, float margin_lo, float margin_hi) {
     // every operation explicitly rounded (no contraction): each inlined copy
     // gives the same bits for the same inputs
     float em = 0.0f, b = 0.0f;
@@ -650,17 +721,15 @@ __device__ __forceinline__ Out32 term_arith32(In32 x, float2 dv, float sdv, bool
     m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
     float bm = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, 1));
     bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 2));
-    Out32 r;
-    r.td = r.tb = 0;
+    Out32 r;                            // (the same in the scenario's four lanes)
+    r.dd = r.bl = 0.0f;
     r.ts = r.tm = 0;
-    if (lvp0) {
-        const float dd = __fsub_rn(__fsub_rn(m, x.mo), x.mr);
+    if (lv) {
+        r.dd = __fsub_rn(__fsub_rn(m, x.mo), x.mr);
         // rounding of MICE_k, MICE_r to FP32 and of the two subtractions; the
         // factor 1.001 covers the rounding of the bound's own arithmetic
         const float am = __fadd_rn(__fadd_rn(fabsf(x.mo), fabsf(x.mr)), fabsf(m));
-        const float bl = __fmul_rn(1.001f, __fadd_rn(bm, __fmul_rn(3.0f * kU32, am)));
-        r.td = to_fx32(dd);
-        r.tb = to_fx32(bl) + 3;             // + the truncations of both terms to fixed point
+        r.bl = __fmul_rn(1.001f, __fadd_rn(bm, __fmul_rn(3.0f * kU32, am)));
         r.ts = (__fsub_rd(m, bm) > margin_hi) ? 1 : 0;
         r.tm = (__fadd_ru(m, bm) > margin_lo) ? 1 : 0;
     }
@@ -669,14 +738,14 @@ __device__ __forceinline__ Out32 term_arith32(In32 x, float2 dv, float sdv, bool
 
 // FP32 term with a rigorous bound (the screen of okr_persist.cu, per item
 // e = max(hr - delta, delta - lr) relative to the cluster's present magnitude).
-// d = sum over l of fixed(D32 term); b = sum over l of a fixed-point bound on
-// |fixed(D32 term) - fixed(D64 term)|; n_sure = scenarios whose new MICE is
-// surely above the margin; n_maybe = scenarios where it may be.  With two
-// states each is state 1's minus state 0's.
+// Added to sum ei of E, over l: d, fixed(D32 term); b, a fixed-point bound on
+// |fixed(D32 term) - fixed(D64 term)|; n1, scenarios whose new MICE is surely
+// above the margin; n2, scenarios where it may be.  With two states each is
+// state 1's minus state 0's.
 __device__ __forceinline__ void group_term32(const Topo &T, const State &S, const uint8_t *ph, int n, int L, int G,
                                              const Cand &c, int k, int e_lo, int e_hi, bool v_old, bool v_new,
-                                             const Ovl &O, int gl, float margin_lo, float margin_hi, u128 *d_out,
-                                             u128 *b_out, int *ns_out, int *nm_out) {
+                                             const Ovl &O, int gl, float margin_lo, float margin_hi, EvalSmem *E,
+                                             int ei) {
     const bool valid = v_old || v_new;
     const int l = gl >> 2, p = gl & 3;
     const bool lv = valid && l < L;
@@ -700,7 +769,7 @@ __device__ __forceinline__ void group_term32(const Topo &T, const State &S, cons
             float2 vr;
             at32(S, O, e, c.r, li, pi, n, L, false, true, &vr, &x.hrr, &x.lrr, &x.mcr);
         }
-        if (lv && ve && p == 0) {
+        if (lv && ve) {
             x.mo = mice32(S, O, e, k, l, n, L);
             if (is_s) x.mr = mice32(S, O, e, c.r, l, n, L);
         }
@@ -730,29 +799,22 @@ __device__ __forceinline__ void group_term32(const Topo &T, const State &S, cons
             sdv = fmaf(fabsf(gx) + fabsf(gy), fabsf(iq[q].x) + fabsf(iq[q].y), sdv);
         }
     }
-    u128 d = 0, bb = 0;
-    int ns = 0, nm = 0;
 #pragma unroll 1
     for (int e = e_lo; e < e_hi; ++e) {
         const bool ve = e == 0 ? v_old : v_new;
         const bool one = on && ve;
         St nxt = cur;
         if (e + 1 < e_hi) fetch(e + 1, nxt);
-        const Out32 r = term_arith32(cur, dv, sdv, one, moves, sterm, lv && ve && p == 0, margin_lo, margin_hi);
+        const Out32 r = term_arith32(cur, dv, sdv, one, moves, sterm, lv && ve, margin_lo, margin_hi);
         cur = nxt;
-        if (e == 1 || e_hi - e_lo == 1) { d += r.td; bb += r.tb; ns += r.ts; nm += r.tm; }
-        else { d -= r.td; bb -= r.tb; ns -= r.ts; nm -= r.tm; }
+        if (lv && ve) {
+            const int sgn = (e == 1 || e_hi - e_lo == 1) ? 1 : -1;
+            add_fx32(E->d, ei, r.dd, sgn, p, 0);
+            add_fx32(E->b, ei, r.bl, sgn, p, 3);        // (3: the truncations of both terms to fixed point)
+            if (p == 0 && r.ts) atomicAdd(&E->n1[ei], sgn);
+            if (p == 0 && r.tm) atomicAdd(&E->n2[ei], sgn);
+        }
     }
-    for (int o = 4; o < G; o <<= 1) {            // the group's sums over its scenarios
-        d += shfl_xor_u128(d, o);
-        bb += shfl_xor_u128(bb, o);
-        ns += __shfl_xor_sync(0xffffffffu, ns, o);
-        nm += __shfl_xor_sync(0xffffffffu, nm, o);
-    }
-    *d_out = d;
-    *b_out = bb;
-    *ns_out = ns;
-    *nm_out = nm;
 }
 
 // ---------------------------------------------------------------- the changed set of a merge
@@ -883,19 +945,10 @@ struct Loc {
 // ---------------------------------------------------------------- evaluation of work entries
 enum Pass {
     kMerge = 0,     // after a merge: mode 0 adds (term after - term before), mode 1 sets every term after
-    kInit = 1,      // the stored state, every term of the entries, set
     kFresh = 2,     // carried precision, every term after the merge in progress, into vacc / vviol
     kF64 = 3,       // FP64, every term on the stored state, into vacc / vviol
     kInitPart = 4   // the stored state, every term of the entries (parts of candidates): added to the carried
                     // sums with atomics, the records left to the search
-};
-
-// One tile of NT work entries (one per thread): their sums and offsets.
-template <int NT>
-struct EvalSmem {
-    unsigned long long dlo[NT], dhi[NT], blo[NT], bhi[NT];
-    int n1[NT], n2[NT];
-    int off[NT + 1];
 };
 
 // Per-slot selection records (shared memory when they fit, else global):
@@ -1051,8 +1104,10 @@ __device__ __forceinline__ long long commit_groups(const Topo &T, const State &S
                                                    double margin, const Commit &cm, int warp0, int nw, int cr, int cs) {
     long long items = 0;
     // (positions go round the CTAs first, so that few positions meet few warps each)
-    const int lw = (((int)threadIdx.x >> 5) - warp0) * cs + cr, gpw = 32 / G, gl = threadIdx.x % G;
-    const int gi = lw * gpw + ((int)threadIdx.x & 31) / G, NG = nw * gpw * cs;
+    // (G is a power of two: shifts, not divisions, on every thread's path)
+    const int lgG = __ffs(G) - 1, lane = threadIdx.x & 31;
+    const int lw = (((int)threadIdx.x >> 5) - warp0) * cs + cr, gpw = 32 >> lgG, gl = lane & (G - 1);
+    const int gi = lw * gpw + (lane >> lgG), NG = nw * gpw * cs;
     const Win &h = *cm.h;
     const int n1 = h.q1hi - h.q1lo, n2 = h.q2hi - h.q2lo;
     for (int r0 = 0; r0 < h.npos; r0 += NG) {
@@ -1064,10 +1119,8 @@ __device__ __forceinline__ long long commit_groups(const Topo &T, const State &S
             k = q < n1 ? cm.list[h.q1lo + q] : (q < n1 + n2 ? cm.list[h.q2lo + q - n1] : cm.wc.s);
             if (k == cm.wc.r) { valid = false; k = cm.wc.s; }
         }
-        u128 d;
-        int nv;
         group_term64(T, S, cm.ph, n, L, G, cm.wc, k, 0, 1, valid, false, cm.O, gl, margin,
-                     valid ? I.cbuf + (size_t)q * kIncCbStride * L : nullptr, &d, &nv);
+                     I.cbuf + (size_t)(valid ? q : 0) * kIncCbStride * L, nullptr, 0);
         if (valid) {
             // the FP32 copies of the new values (what the write-back will store),
             // from the FP64 values this lane has just written
@@ -1094,29 +1147,31 @@ __device__ __forceinline__ long long commit_groups(const Topo &T, const State &S
     return items;
 }
 
-// Evaluates the terms of work entries [e0, e1) (tiles of NT entries) and applies
+// Evaluates the terms of work entries [e0, e1) (tiles of kTile entries) and applies
 // them per the pass (without the barrier after the last tile's updates when
 // !last_barrier).  kMerge: mode-0 entries take positions from list_pre and
 // add, per term, its value after the merge (r* has none) minus its value before;
 // mode-1 entries take positions from list_post and set every term after the
-// merge.  kInit / kFresh / kF64: every term of the entries, positions from
+// merge.  kFresh / kF64 / kInitPart: every term of the entries, positions from
 // list_pre.  Returns the number of terms evaluated.
 template <int NT, int PREC>
 __device__ __forceinline__ long long run_entries(const Topo &T, const State &S, const Search &X, const Inc &I, int n, int L, int G,
                                  double margin, float mlo, float mhi, int e0, int e1, int pass,
                                  const unsigned short *list_pre, const unsigned short *list_post, int rstar,
-                                 const Ovl O, EvalSmem<NT> &E, int *sscan, const Rec &R, const Loc &Lc,
+                                 const Ovl O, EvalSmem &E, int *sscan, const Rec &R, const Loc &Lc,
                                  unsigned long long *prof = nullptr, bool last_barrier = true) {
     // the states every group evaluates (the same for the whole pass)
     const int st_lo = (pass == kFresh) ? 1 : 0, st_hi = (pass == kMerge || pass == kFresh) ? 2 : 1;
-    const int tid = threadIdx.x, gl = tid % G, gi = tid / G, NG = NT / G;
+    static_assert(NT >= kTile, "one thread per entry of a tile");
+    const int lgG = __ffs(G) - 1;
+    const int tid = threadIdx.x, gl = tid & (G - 1), gi = tid >> lgG, NG = NT >> lgG;
     long long terms = 0;
     unsigned long long tq = (prof && tid == 0) ? gtimer_inc() : 0;
     auto sub = [&](int i) {             // profile mode: time of the pass's steps (thread 0, after barriers)
         if (prof && tid == 0) { const unsigned long long now = gtimer_inc(); prof[i] += now - tq; tq = now; }
     };
-    for (int t0 = e0; t0 < e1; t0 += NT) {
-        const int ne = min(NT, e1 - t0);
+    for (int t0 = e0; t0 < e1; t0 += kTile) {
+        const int ne = min(kTile, e1 - t0);
         int cnt = 0;
         if (tid < ne) {
             const IncWork &w = *Lc.ent(t0 + tid);
@@ -1124,17 +1179,20 @@ __device__ __forceinline__ long long run_entries(const Topo &T, const State &S, 
         }
         int tot = 0;
         const int off = block_excl_scan<NT>(cnt, &tot, sscan);
-        E.off[tid] = off;
-        {
-            const int i = tid;
-            E.dlo[i] = E.dhi[i] = E.blo[i] = E.bhi[i] = 0ull;
-            E.n1[i] = E.n2[i] = 0;
+        if (tid < ne) {
+            E.off[tid] = off;
+#pragma unroll
+            for (int i = 0; i < kLimbs; ++i) {
+                E.d[i][tid] = 0;
+                if (PREC == 1) E.b[i][tid] = 0;
+            }
+            E.n1[tid] = E.n2[tid] = 0;
         }
         __syncthreads();
         sub(0);
         unsigned long long cq = (prof && tid == 0) ? clock64() : 0;
         for (int r0 = 0; r0 < tot; r0 += NG) {
-            if (r0 + (tid >> 5) * (32 / G) >= tot) break;     // this warp's groups are all past the end
+            if (r0 + ((tid >> 5) << (5 - lgG)) >= tot) break;     // this warp's groups are all past the end
             const int q = r0 + gi;
             bool valid = q < tot, v_old = false, v_new = false;
             int ei = 0, k = 0;
@@ -1175,25 +1233,10 @@ __device__ __forceinline__ long long run_entries(const Topo &T, const State &S, 
             }
             const unsigned long long c0 = (prof && tid == 0) ? clock64() : 0;
             if (prof && tid == 0) { prof[3] += c0 - cq; prof[7] += 1; }     // lookup cycles, rounds
-            if (PREC == 0 || pass == kF64) {
-                u128 d;
-                int nv;
-                group_term64(T, S, Lc.ph, n, L, G, c, k, st_lo, st_hi, v_old, v_new, O, gl, margin, nullptr, &d, &nv);
-                if (valid && gl == 0) {
-                    sadd128(&E.dlo[ei], &E.dhi[ei], d);
-                    if (nv) atomicAdd(&E.n1[ei], nv);
-                }
-            } else {
-                u128 d, b;
-                int ns, nm;
-                group_term32(T, S, Lc.ph, n, L, G, c, k, st_lo, st_hi, v_old, v_new, O, gl, mlo, mhi, &d, &b, &ns, &nm);
-                if (valid && gl == 0) {
-                    sadd128(&E.dlo[ei], &E.dhi[ei], d);
-                    sadd128(&E.blo[ei], &E.bhi[ei], b);
-                    if (ns) atomicAdd(&E.n1[ei], ns);
-                    if (nm) atomicAdd(&E.n2[ei], nm);
-                }
-            }
+            if (PREC == 0 || pass == kF64)
+                group_term64(T, S, Lc.ph, n, L, G, c, k, st_lo, st_hi, v_old, v_new, O, gl, margin, nullptr, &E, ei);
+            else
+                group_term32(T, S, Lc.ph, n, L, G, c, k, st_lo, st_hi, v_old, v_new, O, gl, mlo, mhi, &E, ei);
             if (prof && tid == 0) { cq = clock64(); prof[4] += cq - c0; }   // term cycles
         }
         __syncthreads();
@@ -1201,8 +1244,7 @@ __device__ __forceinline__ long long run_entries(const Topo &T, const State &S, 
         if (tid < ne) {
             const IncWork &w = *Lc.ent(t0 + tid);
             const int sl = w.slot;
-            const u128 d = ((u128)E.dhi[tid] << 64) | (u128)E.dlo[tid];
-            const u128 b = ((u128)E.bhi[tid] << 64) | (u128)E.blo[tid];
+            const u128 d = limb_sum(E.d, tid), b = PREC == 1 ? limb_sum(E.b, tid) : (u128)0;
             unsigned long long *a = I.acc + 2 * (size_t)sl, *bp = I.bnd + 2 * (size_t)sl;
             if (pass == kInitPart) {
                 sadd128(a, a + 1, d);
@@ -1211,7 +1253,7 @@ __device__ __forceinline__ long long run_entries(const Topo &T, const State &S, 
                     sadd128(bp, bp + 1, b);
                     if (E.n2[tid]) atomicAdd(I.vmay + sl, E.n2[tid]);
                 }
-            } else if (pass == kMerge || pass == kInit) {
+            } else if (pass == kMerge) {
                 u128 na, nb = 0;
                 int nv, nm = 0;
                 if (w.mode == 1) {
@@ -1235,7 +1277,7 @@ __device__ __forceinline__ long long run_entries(const Topo &T, const State &S, 
                 I.vviol[sl] = E.n1[tid];
             }
         }
-        if (last_barrier || t0 + NT < e1) __syncthreads();    // else the caller synchronises
+        if (last_barrier || t0 + kTile < e1) __syncthreads();    // else the caller synchronises
         sub(2);
     }
     return terms;
@@ -1300,7 +1342,9 @@ __device__ void write_back(const State &S, const Inc &I, const Win &hw, const un
                            unsigned short *map, int n, int L, int G, int cr, int cs) {
     // lanes from the last thread down (no shuffles here), beside the first
     // threads' updates of the entries' sums
-    const int tid = threadIdx.x, rt = NT - 1 - tid, gl = rt % G, gi = rt / G, NG = NT / G, l = gl >> 2, p = gl & 3;
+    const int lgG = __ffs(G) - 1;
+    const int tid = threadIdx.x, rt = NT - 1 - tid, gl = rt & (G - 1), gi = rt >> lgG, NG = NT >> lgG, l = gl >> 2,
+              p = gl & 3;
     const int n1 = hw.q1hi - hw.q1lo, n2 = hw.q2hi - hw.q2lo;
     // this CTA's own map
     for (int j = rt; j < hw.npos; j += NT)
@@ -1375,7 +1419,7 @@ template <int NT, int PREC>
 __device__ void inc_run(const Topo &T, const State &S, const Search &X, const Inc &I, Ctrl *C, bool verify,
                         unsigned char *dyn, int rec_mode, int se, int cw, int cs) {
     static_assert(NT >= 128 && NT <= 1024 && NT % 32 == 0, "thread count");
-    __shared__ __align__(16) EvalSmem<NT> E;
+    __shared__ __align__(16) EvalSmem E;
     __shared__ __align__(16) Red sred[33];
     __shared__ __align__(16) Red64 s_sel;      // precision-1 selection accumulator of pass B, a cluster of one
     __shared__ int sscan[33];
@@ -2017,11 +2061,12 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
         // until the terms before the merge have been evaluated)
         {
             const int n1 = hw.q1hi - hw.q1lo, n2 = hw.q2hi - hw.q2lo;
-            const int gl = tid % G, gi = tid / G, NG = NT / G, l = gl >> 2, p = gl & 3;
+            const int lgG = __ffs(G) - 1;
+            const int gl = tid & (G - 1), gi = tid >> lgG, NG = NT >> lgG, l = gl >> 2, p = gl & 3;
             u128 dsum = 0;
             // one lane per (position, scenario)
             for (int r0 = 0; r0 < hw.npos; r0 += NG) {
-                if (r0 + (tid >> 5) * (32 / G) >= hw.npos) break;
+                if (r0 + ((tid >> 5) << (5 - lgG)) >= hw.npos) break;
                 const int j = r0 + gi;
                 bool valid = j < hw.npos;
                 int k = hw.s;
@@ -2205,7 +2250,7 @@ constexpr int kInitCtasMax = kIncInitCtasMax;
 // 2n + 8n bytes, 16-byte aligned parts).
 template <int NT, int PREC>
 __device__ void inc_init_share(const Topo &T, const State &S, const Search &X, const Inc &I, Ctrl *C, int b, int B,
-                               unsigned char *dyn, EvalSmem<NT> &E, int *sscan, int &s_first, int &s_ne) {
+                               unsigned char *dyn, EvalSmem &E, int *sscan, int &s_first, int &s_ne) {
     const int n = T.n, L = T.L, tid = threadIdx.x;
     const int G = 4 * (L <= 1 ? 1 : (L <= 2 ? 2 : 4));
     const double margin = C->margin;
@@ -2337,7 +2382,7 @@ __device__ void inc_init_share(const Topo &T, const State &S, const Search &X, c
 template <int NT, int PREC>
 __global__ void __launch_bounds__(NT) k_inc_init(Topo T, State S, Search X, Inc I, Ctrl *C) {
     extern __shared__ __align__(16) unsigned char init_dyn[];
-    __shared__ __align__(16) EvalSmem<NT> E;
+    __shared__ __align__(16) EvalSmem E;
     __shared__ int sscan[33];
     __shared__ int s_first, s_ne;
     if (X.setup_err && *X.setup_err != 0) return;
@@ -2353,7 +2398,7 @@ template <int NT, int PREC>
 __global__ void __launch_bounds__(NT) k_inc_init_batch(const BatchFeeder *fd, const int *order, const int *cta_off,
                                                        int nf) {
     extern __shared__ __align__(16) unsigned char init_dyn[];
-    __shared__ __align__(16) EvalSmem<NT> E;
+    __shared__ __align__(16) EvalSmem E;
     __shared__ int sscan[33];
     __shared__ int s_first, s_ne;
     __shared__ Topo sT;
@@ -2469,8 +2514,8 @@ bool inc_smem(int n, bool maxm, const IncShape &sh, int *rec_mode, size_t *bytes
 // records (which then always fit shared memory), and pays three cluster
 // barriers a merge (about 0.5 us each with stores in flight) and L2 in place of
 // L1 latency.  Search ms, one CTA of 384 threads / eight of 256:
-//   FP64 terms:  40 buses 0.56 / 0.64, 333 buses (3 scenarios) 5.7 / 4.1, 1,000 9.8 / 8.2, 3,100 60.3 / 42.2
-//   FP32 terms: 333 buses 4.11 / 4.08, 1,000 7.14 / 7.40, 2,200 33.8 / 30.4, 3,100 46.2 / 37.4
+//   FP64 terms:  40 buses 0.56 / 0.64, 333 buses (3 scenarios) 5.7 / 4.1, 1,000 9.7 / 8.0, 3,100 59.7 / 41.0
+//   FP32 terms: 333 buses 4.11 / 4.08, 1,000 6.77 / 6.99, 2,200 32.0 / 29.0, 3,100 44.1 / 35.2
 // (two and four CTAs lie between the two).  A forced record placement asks for
 // one CTA's memory, and recorded iterations are compacted by one CTA.
 bool inc_plan(int n, int precision, const IncShape &raw, bool records_iters, IncPlan *out) {
@@ -2482,7 +2527,7 @@ bool inc_plan(int n, int precision, const IncShape &raw, bool records_iters, Inc
     if (b > kIncSmemMax) return true;
     out->cs = kMaxCluster;
     out->bytes = b;
-    // fewer warps meet at the cluster's barriers (384 threads: 1,000 buses FP64 8.50 ms, 3,100 FP32 39.5)
+    // fewer warps meet at the cluster's barriers (384 threads: 1,000 buses FP64 8.26 ms, 3,100 FP32 36.9)
     if (raw.threads == 0) {
         IncShape sh = raw;
         sh.threads = 256;
