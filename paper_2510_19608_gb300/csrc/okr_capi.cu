@@ -560,7 +560,7 @@ okr_status run_search_inc(okr_ctx *ctx, const okr_params *p) {
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     IncPlan pl;
-    if (!inc_plan(n, p->precision, ctx->inc_shape, p->record_iters > 0, &pl))
+    if (!inc_plan(n, ctx->inc_shape, p->record_iters > 0, &pl))
         return fail(ctx, OKR_EINVAL, "incremental search: the forced record placement does not fit shared memory "
                                      "for %d buses", n);
     ctx->last_shape = pl.sh;

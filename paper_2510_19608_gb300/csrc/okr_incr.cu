@@ -43,17 +43,24 @@
 // score it needs; those are evaluated in FP64 from scratch.  Merges are always
 // applied in FP64.
 //
-// Execution.  One CTA runs one feeder's whole search; its steps are separated
-// by __syncthreads only (no grid barrier, no device-side wait).  A term is
-// evaluated by a group of lanes, one per (scenario, phase).  A batch runs one
-// CTA per feeder.  Each merge takes four steps: selection; the changed set
-// (beside it, the merge's own FP64 evaluation into a scratch, and a map of its
-// positions); the merge's score change and topology, and beside it the
-// rebuilt candidates (which read the clusters through the merge's view); one
-// pass over the changed terms, which evaluates each term before the merge (the
-// state as stored) and after it (the stored state overlaid with the scratch's
-// new values) in the same lane group and adds the difference.  The new values
-// and ranks are written back to the state at the end of that pass.
+// Execution.  One CTA (a batch, a tiny feeder) or one cluster of eight runs a
+// feeder's whole search; its steps are separated by block or cluster barriers
+// only (no grid barrier, no device-side wait).  The chain of dependent merges
+// bounds it: neither a pipe nor memory is busy, so what counts is the number of
+// dependent steps per merge and the latency of each.  A term is evaluated by a
+// group of lanes, one per (scenario, phase).  Each merge takes three steps:
+//   1. selection over the records (in a cluster two exchanges of minima);
+//   2. the merge: its own FP64 evaluation into a scratch on the last warps and,
+//      beside it on the others, the previous merge's write-back, the changed
+//      candidates, the rebuilt ones (which read the clusters through the merge's
+//      view) and the bookkeeping of clusters and super-nodes;
+//   3. the terms that change, each before the merge (the state as stored) and
+//      after it (the stored state overlaid with the scratch's new values), and
+//      the merge's score.
+// The write-back waits for the next merge's step 2, whose evaluation reads the
+// not yet written values through the overlay, so no barrier is needed for it.
+// (Rebuilding in a step of its own, between barriers, with the write-back after
+// the terms took 14.0 us a merge on 1,000 buses, a cluster, FP32 terms; 9.9 now.)
 #include "okr_internal.cuh"
 #include "okr_kernels.cuh"
 
@@ -66,6 +73,7 @@ typedef unsigned __int128 u128;
 constexpr int kFxShift = 100;               // fixed point: value * 2^100
 constexpr u128 kSignBit = (u128)1 << 127;
 constexpr u128 kNone = ~(u128)0;
+constexpr int kMaxCluster = 8;              // CTAs of one search, at most
 constexpr float kU32 = 5.9604645e-08f;      // 2^-24
 
 __device__ __forceinline__ unsigned long long gtimer_inc() {
@@ -160,15 +168,18 @@ __device__ __forceinline__ int cluster_rank() {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return (int)r;
 }
-// 32 bytes one warp publishes to another CTA's copy of the same shared array.
+// What is published: written to another CTA's copy of the same shared array.
 struct __align__(16) Pub {
     unsigned long long a, b, c, d;
 };
-__device__ __forceinline__ void publish(Pub *slot, int rank, const Pub &v) {
+__device__ __forceinline__ void publish(void *slot, int rank, const void *v, int chunks) {     // chunks of 16 bytes
     unsigned at;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((unsigned)__cvta_generic_to_shared(slot)), "r"(rank));
-    asm volatile("st.shared::cluster.v2.u64 [%0], {%1, %2};" ::"r"(at), "l"(v.a), "l"(v.b) : "memory");
-    asm volatile("st.shared::cluster.v2.u64 [%0], {%1, %2};" ::"r"(at + 16), "l"(v.c), "l"(v.d) : "memory");
+#pragma unroll
+    for (int i = 0; i < chunks; ++i) {
+        const ulonglong2 q = static_cast<const ulonglong2 *>(v)[i];
+        asm volatile("st.shared::cluster.v2.u64 [%0], {%1, %2};" ::"r"(at + 16 * i), "l"(q.x), "l"(q.y) : "memory");
+    }
 }
 
 // ---------------------------------------------------------------- block primitives
@@ -402,7 +413,6 @@ constexpr int kLimbBits = 14, kLimbs = 10, kTile = 192;
 struct EvalSmem {
     int d[kLimbs][kTile + 1], b[kLimbs][kTile + 1];     // (+ 1: the limbs of an entry in different banks)
     int n1[kTile], n2[kTile];
-    int off[kTile + 1];
 };
 __device__ __forceinline__ u128 limb_sum(const int (*x)[kTile + 1], int i) {
     u128 v = 0;
@@ -468,8 +478,8 @@ __device__ __forceinline__ void add_fx64(int (*x)[kTile + 1], int i, double v, i
 // the group function (it shuffles); the four lanes of a scenario add its term
 // to the sums of the group's work entry.
 //
-// A group evaluates its term on one or two states, e in [e_lo, e_hi) (the
-// same range for every group of a warp): e = 0, the state as stored; e = 1,
+// A group evaluates its term on one or two states (as many in every group of a
+// warp): e = 0, the state as stored; e = 1,
 // the state after the merge in progress, whose new values (voltage,
 // magnitude, extremes, MICE of the merge's positions) are not yet written
 // back and are read through the overlay.  With both, the result is the term
@@ -480,11 +490,15 @@ __device__ __forceinline__ void add_fx64(int (*x)[kTile + 1], int i, double v, i
 // operation explicitly, so equal inputs give bit-equal results in every
 // inlined copy.
 
-// The merge in progress, as the terms after it see it: map[x] = 1 + the index
-// of super-node x among the merge's positions (0: unchanged), whose new values
-// the merge's own evaluation left in cbuf (per position: per (l, p) the new
-// voltage x, y and magnitude; per l the new MICE).  Positions from nfree on
-// are the fixed s (its voltage does not move).  s* takes r*'s extremes.
+// A merge whose new values are not in the state yet: map[x] = 1 + the index of
+// super-node x among the merge's positions (0: unchanged), whose new values the
+// merge's own evaluation left in cbuf (per position: per (l, p) the new voltage
+// x, y and magnitude; per l the new MICE).  Positions from nfree on are the
+// fixed s (its voltage does not move).  s* takes r*'s extremes.  A merge's
+// values are written back while the next merge is evaluated, which reads them
+// through the overlay, so there is one overlay (map and scratch) for the odd
+// merges and one for the even; the state under an overlay may be read before or
+// while it is written (s*'s extremes read the same either way).
 struct Ovl {
     const unsigned short *map;
     const double *cbuf;
@@ -498,6 +512,11 @@ __device__ __forceinline__ float4 *cb_f4(const double *cb_pos, int L, int l, int
 }
 __device__ __forceinline__ float *cb_mice32(const double *cb_pos, int L, int l) {
     return reinterpret_cast<float *>(const_cast<double *>(cb_pos) + 10 * L) + 12 * L + l;
+}
+
+// The super-node of a scratch position.
+__device__ __forceinline__ int *cb_bus(const double *cb_pos, int L) {
+    return reinterpret_cast<int *>(const_cast<double *>(cb_pos) + 10 * L) + 13 * L;
 }
 
 // FP64 state of super-node x, phase p, scenario l on state e (0 stored, 1 overlay).
@@ -563,12 +582,17 @@ struct In64 {
 struct Out64 {
     double dd;
     int tv;
+    double2 v;          // the merge's own evaluation: the new voltage, its magnitude, the cluster's extremes, its MICE
+    double mag, h, lo, m;
 };
 __device__ __forceinline__ Out64 term_arith64(In64 x, double2 dv, bool one, bool moves, bool is_s, bool lv,
-                                              double margin, double *out, int l, int p, int L) {
+                                              double margin) {
     // every operation explicitly rounded (no contraction): each inlined copy
     // gives the same bits for the same inputs
     double em = 0.0;
+    Out64 r;
+    r.v = make_double2(0.0, 0.0);
+    r.mag = r.h = r.lo = 0.0;
     if (one) {
         double2 v = x.v;
         if (moves) v = make_double2(__dadd_rn(v.x, dv.x), __dadd_rn(v.y, dv.y));
@@ -579,36 +603,33 @@ __device__ __forceinline__ Out64 term_arith64(In64 x, double2 dv, bool one, bool
             lo = fmin(lo, x.lr);
         }
         em = fmax(__dsub_rn(h, mag), __dsub_rn(mag, lo));
-        if (out) {
-            out[(l * 3 + p) * 3 + 0] = v.x;
-            out[(l * 3 + p) * 3 + 1] = v.y;
-            out[(l * 3 + p) * 3 + 2] = mag;
-        }
+        r.v = v;
+        r.mag = mag;
+        r.h = h;
+        r.lo = lo;
     }
     double m = fmax(em, __shfl_xor_sync(0xffffffffu, em, 1));
     m = fmax(m, __shfl_xor_sync(0xffffffffu, m, 2));
-    Out64 r;                            // (the same in the scenario's four lanes)
-    r.dd = 0.0;
+    r.dd = 0.0;                         // (dd, tv, m: the same in the scenario's four lanes)
     r.tv = 0;
+    r.m = m;
     if (lv) {
-        if (out) {
-            if (p == 0) out[9 * L + l] = m;
-        } else {
-            r.dd = __dsub_rn(m, x.mo);
-            if (is_s) r.dd = __dsub_rn(r.dd, x.mr);
-            r.tv = (m > margin) ? 1 : 0;
-        }
+        r.dd = __dsub_rn(m, x.mo);
+        if (is_s) r.dd = __dsub_rn(r.dd, x.mr);
+        r.tv = (m > margin) ? 1 : 0;
     }
     return r;
 }
 
 // FP64 term, per l fixed(new MICE - MICE_k [- MICE_r]) and whether the new MICE
-// exceeds the margin, added to sum ei of E.  out != nullptr (state 0 only): the
-// new voltage and magnitude per (l, p) and the new MICE per l (the merge), and
+// exceeds the margin, added to sum ei of E: ne states from e0 on (e0 may differ
+// between groups when ne = 1), state 1 with sign +, state 0 with sign sgn0.
+// COMMIT (one state): the merge's own evaluation; returns the new values, and
 // nothing is added.
-__device__ __forceinline__ void group_term64(const Topo &T, const State &S, const uint8_t *ph, int n, int L, int G,
-                                             const Cand &c, int k, int e_lo, int e_hi, bool v_old, bool v_new,
-                                             const Ovl &O, int gl, double margin, double *out, EvalSmem *E, int ei) {
+template <bool COMMIT>
+__device__ __forceinline__ Out64 group_term64(const Topo &T, const State &S, const uint8_t *ph, int n, int L, int G,
+                                              const Cand &c, int k, int e0, int ne, int sgn0, bool v_old, bool v_new,
+                                              const Ovl &O, int gl, double margin, EvalSmem *E, int ei) {
     const bool valid = v_old || v_new;
     const int l = gl >> 2, p = gl & 3;
     const bool lv = valid && l < L;
@@ -631,13 +652,13 @@ __device__ __forceinline__ void group_term64(const Topo &T, const State &S, cons
             at64(S, O, e, k, li, pi, n, L, true, &x.v, &x.h, &x.lo);
             if (is_s) at64(S, O, e, c.r, li, pi, n, L, false, nullptr, &x.hr, &x.lr);
         }
-        if (lv && ve && !out) {
+        if (lv && ve && !COMMIT) {
             x.mo = mice64(S, O, e, k, l, n, L);
             if (is_s) x.mr = mice64(S, O, e, c.r, l, n, L);
         }
     };
     St cur;
-    fetch(e_lo, cur);
+    fetch(e0, cur);
     // the voltage change at k (the same on both states)
     double2 dv = make_double2(0.0, 0.0);
     if (moves) {
@@ -655,20 +676,23 @@ __device__ __forceinline__ void group_term64(const Topo &T, const State &S, cons
             dv = cadd(dv, cmul(g, iq[q]));
         }
     }
+    Out64 r;
 #pragma unroll 1
-    for (int e = e_lo; e < e_hi; ++e) {
+    for (int i = 0; i < ne; ++i) {
+        const int e = e0 + i;
         const bool ve = e == 0 ? v_old : v_new;
         const bool one = on && ve;
         St nxt = cur;
-        if (e + 1 < e_hi) fetch(e + 1, nxt);
-        const Out64 r = term_arith64(cur, dv, one, moves, is_s, lv && ve, margin, out, l, p, L);
+        if (i + 1 < ne) fetch(e + 1, nxt);
+        r = term_arith64(cur, dv, one, moves, is_s, lv && ve, margin);
         cur = nxt;
-        if (lv && ve && !out) {
-            const int sgn = (e == 1 || e_hi - e_lo == 1) ? 1 : -1;
+        if (!COMMIT && lv && ve) {
+            const int sgn = e == 1 ? 1 : sgn0;
             add_fx64(E->d, ei, r.dd, sgn, p);
             if (p == 0 && r.tv) atomicAdd(&E->n1[ei], sgn);
         }
     }
+    return r;
 }
 
 // The arithmetic of one FP32 term with its bound on one state's inputs (every
@@ -740,10 +764,9 @@ __device__ __forceinline__ Out32 term_arith32(In32 x, float2 dv, float sdv, bool
 // e = max(hr - delta, delta - lr) relative to the cluster's present magnitude).
 // Added to sum ei of E, over l: d, fixed(D32 term); b, a fixed-point bound on
 // |fixed(D32 term) - fixed(D64 term)|; n1, scenarios whose new MICE is surely
-// above the margin; n2, scenarios where it may be.  With two states each is
-// state 1's minus state 0's.
+// above the margin; n2, scenarios where it may be.  States and signs as above.
 __device__ __forceinline__ void group_term32(const Topo &T, const State &S, const uint8_t *ph, int n, int L, int G,
-                                             const Cand &c, int k, int e_lo, int e_hi, bool v_old, bool v_new,
+                                             const Cand &c, int k, int e0, int ne, int sgn0, bool v_old, bool v_new,
                                              const Ovl &O, int gl, float margin_lo, float margin_hi, EvalSmem *E,
                                              int ei) {
     const bool valid = v_old || v_new;
@@ -775,7 +798,7 @@ __device__ __forceinline__ void group_term32(const Topo &T, const State &S, cons
         }
     };
     St cur;
-    fetch(e_lo, cur);
+    fetch(e0, cur);
     // the voltage change at k (the same on both states)
     float2 dv = make_float2(0.0f, 0.0f);
     float sdv = 0.0f;
@@ -800,15 +823,16 @@ __device__ __forceinline__ void group_term32(const Topo &T, const State &S, cons
         }
     }
 #pragma unroll 1
-    for (int e = e_lo; e < e_hi; ++e) {
+    for (int i = 0; i < ne; ++i) {
+        const int e = e0 + i;
         const bool ve = e == 0 ? v_old : v_new;
         const bool one = on && ve;
         St nxt = cur;
-        if (e + 1 < e_hi) fetch(e + 1, nxt);
+        if (i + 1 < ne) fetch(e + 1, nxt);
         const Out32 r = term_arith32(cur, dv, sdv, one, moves, sterm, lv && ve, margin_lo, margin_hi);
         cur = nxt;
         if (lv && ve) {
-            const int sgn = (e == 1 || e_hi - e_lo == 1) ? 1 : -1;
+            const int sgn = e == 1 ? 1 : sgn0;
             add_fx32(E->d, ei, r.dd, sgn, p, 0);
             add_fx32(E->b, ei, r.bl, sgn, p, 3);        // (3: the truncations of both terms to fixed point)
             if (p == 0 && r.ts) atomicAdd(&E->n1[ei], sgn);
@@ -829,7 +853,7 @@ struct Win {
 __device__ __forceinline__ bool in_range(int b, int lo, int hi) { return b >= lo && b < hi; }
 
 // The winner's record from its candidate (slot ws) and the super-node ranks.
-__device__ __forceinline__ Win make_win(const Cand &w, int ws, const int *rank) {
+__device__ __forceinline__ Win make_win(const Cand &w, int ws, const unsigned short *rank) {
     Win h;
     h.slot = ws; h.s = w.s; h.r = w.r; h.a = w.a; h.dir = w.dir; h.fixed = w.fixed;
     h.w1lo = w.js; h.w1hi = w.js + w.ns; h.w2lo = w.jr; h.w2hi = w.jr + w.nr;
@@ -861,7 +885,7 @@ __device__ __forceinline__ bool touched(const Cand &c, const Win &h) {
 
 // Rank ranges of the terms of candidate c that read an input the merge h
 // changes (c is not next to s* or r*).  Returns their number.
-__device__ int changed_segments(const Cand &c, const Win &h, const int *sn_rank, int2 *seg) {
+__device__ int changed_segments(const Cand &c, const Win &h, const unsigned short *sn_rank, int2 *seg) {
     int k = 0;
     const int clo[2] = {c.js, c.jr}, chi[2] = {c.js + c.ns, c.jr + c.nr};
     const int wlo[2] = {h.w1lo, h.w2lo}, whi[2] = {h.w1hi, h.w2hi};
@@ -894,7 +918,8 @@ __device__ int changed_segments(const Cand &c, const Win &h, const int *sn_rank,
 }
 
 // Every term of candidate c: its two ranges and the fixed s, as ranks.
-__device__ int full_segments(const Cand &c, const int *sn_rank, int2 *seg, int rdead = -1) {
+template <typename RK>
+__device__ int full_segments(const Cand &c, const RK *sn_rank, int2 *seg, int rdead = -1) {
     // rdead >= 0: ranks past bus rdead drop by one (the merge of r* = rdead)
     auto rk = [&](int b) { return sn_rank[b] - (rdead >= 0 && b > rdead ? 1 : 0); };
     int k = 0;
@@ -910,11 +935,19 @@ __device__ int full_segments(const Cand &c, const int *sn_rank, int2 *seg, int r
     return k;
 }
 
-__device__ __forceinline__ void write_entry(IncWork *w, int slot, int mode, int nseg, const int2 *seg, const Cand &c) {
+// The list of work entries: its length (low word) and the items of its entries
+// (high word), so that an entry learns its place and its first item at once.
+__device__ __forceinline__ unsigned long long append(unsigned long long *list, int nseg, const int2 *seg) {
+    int items = 0;
+    for (int i = 0; i < nseg; ++i) items += seg[i].y - seg[i].x;
+    return atomicAdd(list, ((unsigned long long)items << 32) | 1ull);
+}
+__device__ __forceinline__ void write_entry(IncWork *w, int slot, int mode, int off, int nseg, const int2 *seg,
+                                            const Cand &c) {
     w->slot = slot;
     w->mode = mode;
     w->nseg = nseg;
-    w->pad = 0;
+    w->off = off;
     for (int i = 0; i < nseg; ++i) w->seg[i] = seg[i];
     w->s = c.s; w->r = c.r; w->a = c.a;
     w->js = c.js; w->ns = c.ns; w->jr = c.jr; w->nr = c.nr; w->fixed = c.fixed;
@@ -934,11 +967,19 @@ __device__ __forceinline__ Cand entry_cand(const IncWork &w) {
 constexpr int kSEMax = 256;
 struct Loc {
     IncWork *wsm, *wgl;         // (wgl: this CTA's part of the feeder's work buffer)
-    int *fpair, *rlist;         // this CTA's parts of Inc::fpair and Inc::rlist
+    int *rlist;                 // this CTA's part of Inc::rlist
     int se;                     // work entries in shared memory
     unsigned short *lst[2];
     const uint8_t *ph;
-    int *rank;                  // [n + 1] rank of each bus's super-node among the super-nodes
+    unsigned short *rank;       // [n + 1] rank of each bus's super-node among the super-nodes
+    // the candidates and their carried sums and counts (as in Search::slot and
+    // Inc): in device memory by slot (lg < 0), or the CTA's own slots in shared
+    // memory, by record (lg: log2 of the cluster's size)
+    int lg;
+    Cand *slot;
+    unsigned long long *acc, *bnd;
+    int *viol, *vmay;
+    __device__ __forceinline__ int at(int sl) const { return lg < 0 ? sl : ((sl >> (lg + 1)) << 1) | (sl & 1); }
     __device__ __forceinline__ IncWork *ent(int i) const { return i < se ? wsm + i : wgl + (i - se); }
 };
 
@@ -1059,6 +1100,20 @@ __device__ __forceinline__ void refresh_blocks(const Rec &R, int n) {
     __syncthreads();
 }
 
+// The span record of a pair with candidates c (x: its quotient parent, -1: none).
+__device__ __forceinline__ ushort4 pair_span(int n, const Cand *c, int x) {
+    int lo = n, hi = 0;
+    for (int d = 0; d < 2; ++d) {
+        if (c[d].s < 0) continue;
+        lo = min(lo, min(min(c[d].s, c[d].r), c[d].ns > 0 ? c[d].js : n));
+        lo = min(lo, c[d].nr > 0 ? c[d].jr : n);
+        hi = max(hi, max(max(c[d].s, c[d].r) + 1, max(c[d].js + c[d].ns, c[d].jr + c[d].nr)));
+    }
+    const bool any = c[0].s >= 0 || c[1].s >= 0;
+    return make_ushort4((unsigned short)(any ? lo : 0), (unsigned short)(any ? hi : 0),
+                        (unsigned short)(x >= 0 ? x : 0xffff), (unsigned short)(any ? 1 : 0));
+}
+
 template <int PREC>
 __device__ __forceinline__ void set_rec(const Rec &R, int sl, u128 d, u128 b, int viol, int vmay) {
     R.touch(sl);
@@ -1096,15 +1151,16 @@ struct Commit {
     Cand wc;
     const unsigned short *list;     // super-nodes before the merge
     const uint8_t *ph;
-    Ovl O;                          // (not read: state 0)
+    Ovl O;                          // the merge before, still being written back
+    double *cbuf;                   // this merge's scratch
 };
 
 // Run by warps [warp0, warp0 + nw) of every CTA of the cluster (CTA cr of cs).
-__device__ __forceinline__ long long commit_groups(const Topo &T, const State &S, const Inc &I, int n, int L, int G,
-                                                   double margin, const Commit &cm, int warp0, int nw, int cr, int cs) {
+__device__ __forceinline__ long long commit_groups(const Topo &T, const State &S, int n, int L, int G, double margin,
+                                                   const Commit &cm, int warp0, int nw, int cr, int cs) {
     long long items = 0;
-    // (positions go round the CTAs first, so that few positions meet few warps each)
-    // (G is a power of two: shifts, not divisions, on every thread's path)
+    // (positions go round the CTAs first, so that few positions meet few warps each;
+    // G is a power of two: shifts, not divisions, on every thread's path)
     const int lgG = __ffs(G) - 1, lane = threadIdx.x & 31;
     const int lw = (((int)threadIdx.x >> 5) - warp0) * cs + cr, gpw = 32 >> lgG, gl = lane & (G - 1);
     const int gi = lw * gpw + (lane >> lgG), NG = nw * gpw * cs;
@@ -1117,51 +1173,46 @@ __device__ __forceinline__ long long commit_groups(const Topo &T, const State &S
         int k = cm.wc.s;
         if (valid) {
             k = q < n1 ? cm.list[h.q1lo + q] : (q < n1 + n2 ? cm.list[h.q2lo + q - n1] : cm.wc.s);
+            if (gl == 0) *cb_bus(cm.cbuf + (size_t)q * kIncCbStride * L, L) = k;
             if (k == cm.wc.r) { valid = false; k = cm.wc.s; }
         }
-        group_term64(T, S, cm.ph, n, L, G, cm.wc, k, 0, 1, valid, false, cm.O, gl, margin,
-                     I.cbuf + (size_t)(valid ? q : 0) * kIncCbStride * L, nullptr, 0);
+        const Out64 r = group_term64<true>(T, S, cm.ph, n, L, G, cm.wc, k, 1, 1, 1, false, valid, cm.O, gl, margin,
+                                           nullptr, 0);
         if (valid) {
-            // the FP32 copies of the new values (what the write-back will store),
-            // from the FP64 values this lane has just written
+            // the new values, and their FP32 copies (what the write-back will store)
             const int l = gl >> 2, p = gl & 3;
-            const double *cb = I.cbuf + (size_t)q * kIncCbStride * L;
-            const bool fx = q >= n1 + n2;
+            double *cb = cm.cbuf + (size_t)q * kIncCbStride * L;
             if (l < L && p < 3 && (cm.ph[k] >> p & 1u)) {
-                const size_t ik = sidx(l, p, k, n);
-                const double mc = fx ? S.mcur[ik] : cb[(l * 3 + p) * 3 + 2];
-                double hh = S.hi[ik], ll = S.lo[ik];
-                if (k == h.s) {
-                    const size_t ir = sidx(l, p, h.r, n);
-                    hh = fmax(hh, S.hi[ir]);
-                    ll = fmin(ll, S.lo[ir]);
-                }
-                const float2 v32 =
-                    fx ? S.v32[ik] : make_float2((float)cb[(l * 3 + p) * 3], (float)cb[(l * 3 + p) * 3 + 1]);
-                *cb_f4(cb, L, l, p) = make_float4(v32.x, v32.y, (float)(hh - mc), (float)(ll - mc));
+                double *o = cb + (l * 3 + p) * 3;
+                o[0] = r.v.x;
+                o[1] = r.v.y;
+                o[2] = r.mag;
+                *cb_f4(cb, L, l, p) = make_float4((float)r.v.x, (float)r.v.y, (float)(r.h - r.mag), (float)(r.lo - r.mag));
             }
-            if (l < L && p == 0) *cb_mice32(cb, L, l) = (float)cb[9 * L + l];
+            if (l < L && p == 0) {
+                cb[9 * L + l] = r.m;
+                *cb_mice32(cb, L, l) = (float)r.m;
+            }
             if (gl == 0) items += __popc(cm.ph[k]) * L;
         }
     }
     return items;
 }
 
-// Evaluates the terms of work entries [e0, e1) (tiles of kTile entries) and applies
-// them per the pass (without the barrier after the last tile's updates when
-// !last_barrier).  kMerge: mode-0 entries take positions from list_pre and
-// add, per term, its value after the merge (r* has none) minus its value before;
-// mode-1 entries take positions from list_post and set every term after the
-// merge.  kFresh / kF64 / kInitPart: every term of the entries, positions from
-// list_pre.  Returns the number of terms evaluated.
+// Evaluates the terms of work entries [0, ne_all), which hold `items` items (tiles
+// of kTile entries), and applies them per the pass; ends without a barrier after
+// the last tile's updates.  kMerge: mode-0 entries take positions from list_pre
+// and add, per term, its value after the merge (r* has none) minus its value
+// before; mode-1 entries take positions from list_post and set every term after
+// the merge.  kFresh / kF64 / kInitPart: every term of the entries, positions
+// from list_pre, on the state under the overlay (kInitPart: as stored).  The
+// sums E are zero before and after.  Returns the number of terms evaluated.
 template <int NT, int PREC>
-__device__ __forceinline__ long long run_entries(const Topo &T, const State &S, const Search &X, const Inc &I, int n, int L, int G,
-                                 double margin, float mlo, float mhi, int e0, int e1, int pass,
+__device__ __forceinline__ long long run_entries(const Topo &T, const State &S, const Inc &I, int n, int L, int G,
+                                 double margin, float mlo, float mhi, int ne_all, int items, int pass,
                                  const unsigned short *list_pre, const unsigned short *list_post, int rstar,
-                                 const Ovl O, EvalSmem &E, int *sscan, const Rec &R, const Loc &Lc,
-                                 unsigned long long *prof = nullptr, bool last_barrier = true) {
-    // the states every group evaluates (the same for the whole pass)
-    const int st_lo = (pass == kFresh) ? 1 : 0, st_hi = (pass == kMerge || pass == kFresh) ? 2 : 1;
+                                 const Ovl O, EvalSmem &E, const Rec &R, const Loc &Lc,
+                                 unsigned long long *prof = nullptr) {
     static_assert(NT >= kTile, "one thread per entry of a tile");
     const int lgG = __ffs(G) - 1;
     const int tid = threadIdx.x, gl = tid & (G - 1), gi = tid >> lgG, NG = NT >> lgG;
@@ -1170,73 +1221,61 @@ __device__ __forceinline__ long long run_entries(const Topo &T, const State &S, 
     auto sub = [&](int i) {             // profile mode: time of the pass's steps (thread 0, after barriers)
         if (prof && tid == 0) { const unsigned long long now = gtimer_inc(); prof[i] += now - tq; tq = now; }
     };
-    for (int t0 = e0; t0 < e1; t0 += kTile) {
-        const int ne = min(kTile, e1 - t0);
-        int cnt = 0;
-        if (tid < ne) {
-            const IncWork &w = *Lc.ent(t0 + tid);
-            for (int i = 0; i < w.nseg; ++i) cnt += w.seg[i].y - w.seg[i].x;
-        }
-        int tot = 0;
-        const int off = block_excl_scan<NT>(cnt, &tot, sscan);
-        if (tid < ne) {
-            E.off[tid] = off;
-#pragma unroll
-            for (int i = 0; i < kLimbs; ++i) {
-                E.d[i][tid] = 0;
-                if (PREC == 1) E.b[i][tid] = 0;
-            }
-            E.n1[tid] = E.n2[tid] = 0;
-        }
-        __syncthreads();
-        sub(0);
+    for (int t0 = 0; t0 < ne_all; t0 += kTile) {
+        const int ne = min(kTile, ne_all - t0);
+        const int q0 = t0 > 0 ? Lc.ent(t0)->off : 0, q1 = t0 + kTile < ne_all ? Lc.ent(t0 + kTile)->off : items;
+        // the states: after a merge two, one after the other in a group, or, when
+        // the CTA has groups enough for every item twice, one in each of two groups
+        const bool both = pass == kMerge, apart = both && 2 * (q1 - q0) <= NG;
+        const int tot = apart ? 2 * (q1 - q0) : q1 - q0;
         unsigned long long cq = (prof && tid == 0) ? clock64() : 0;
         for (int r0 = 0; r0 < tot; r0 += NG) {
             if (r0 + ((tid >> 5) << (5 - lgG)) >= tot) break;     // this warp's groups are all past the end
-            const int q = r0 + gi;
-            bool valid = q < tot, v_old = false, v_new = false;
+            const int u = r0 + gi, q = q0 + (apart ? u >> 1 : u);
+            const int st0 = apart ? u & 1 : (both || pass == kInitPart ? 0 : 1), nst = both && !apart ? 2 : 1;
+            bool valid = u < tot, v_old = false, v_new = false;
             int ei = 0, k = 0;
             Cand c;
             c.s = c.r = c.a = c.js = c.ns = c.jr = c.nr = c.fixed = 0;
             if (valid) {
-                // the entry holding item q: the last one whose offset is <= q
+                // the entry holding item q: the last one whose first item is <= q
                 {
                     int lo = 0, hi = ne - 1;
                     while (lo < hi) {
                         const int mid = (lo + hi + 1) >> 1;
-                        if (E.off[mid] <= q) lo = mid;
+                        if (Lc.ent(t0 + mid)->off <= q) lo = mid;
                         else hi = mid - 1;
                     }
                     ei = lo;
                 }
                 const IncWork &w = *Lc.ent(t0 + ei);
-                int rem = q - E.off[ei], j = 0;
+                int rem = q - w.off, j = 0;
                 for (int i = 0; i < w.nseg; ++i) {
                     const int len = w.seg[i].y - w.seg[i].x;
                     if (rem < len) { j = w.seg[i].x + rem; break; }
                     rem -= len;
                 }
-                k = ((pass == kMerge && w.mode == 1) ? list_post : list_pre)[j];
+                k = ((both && w.mode == 1) ? list_post : list_pre)[j];
                 c = entry_cand(w);
                 if (k == c.r) valid = false;
-                if (pass == kMerge) {
+                if (both) {
                     v_old = valid && w.mode == 0;
                     v_new = valid && !(w.mode == 0 && k == rstar);
                 } else {
                     v_old = v_new = valid;
                 }
-                valid = v_old || v_new;
             }
-            if (gl == 0) {                                            // (phase-node, scenario) items
-                const int it = (st_lo == 0 && v_old ? 1 : 0) + (st_hi == 2 && v_new ? 1 : 0);
-                if (it) terms += it * __popc(Lc.ph[k]) * L;
-            }
+            // (the state a group does not evaluate)
+            if (nst == 1 && st0 == 0) v_new = false;
+            if (nst == 1 && st0 == 1) v_old = false;
+            if (gl == 0 && (v_old || v_new))                          // (phase-node, scenario) items
+                terms += ((v_old ? 1 : 0) + (v_new ? 1 : 0)) * __popc(Lc.ph[k]) * L;
             const unsigned long long c0 = (prof && tid == 0) ? clock64() : 0;
             if (prof && tid == 0) { prof[3] += c0 - cq; prof[7] += 1; }     // lookup cycles, rounds
             if (PREC == 0 || pass == kF64)
-                group_term64(T, S, Lc.ph, n, L, G, c, k, st_lo, st_hi, v_old, v_new, O, gl, margin, nullptr, &E, ei);
+                group_term64<false>(T, S, Lc.ph, n, L, G, c, k, st0, nst, both ? -1 : 1, v_old, v_new, O, gl, margin, &E, ei);
             else
-                group_term32(T, S, Lc.ph, n, L, G, c, k, st_lo, st_hi, v_old, v_new, O, gl, mlo, mhi, &E, ei);
+                group_term32(T, S, Lc.ph, n, L, G, c, k, st0, nst, both ? -1 : 1, v_old, v_new, O, gl, mlo, mhi, &E, ei);
             if (prof && tid == 0) { cq = clock64(); prof[4] += cq - c0; }   // term cycles
         }
         __syncthreads();
@@ -1245,115 +1284,105 @@ __device__ __forceinline__ long long run_entries(const Topo &T, const State &S, 
             const IncWork &w = *Lc.ent(t0 + tid);
             const int sl = w.slot;
             const u128 d = limb_sum(E.d, tid), b = PREC == 1 ? limb_sum(E.b, tid) : (u128)0;
-            unsigned long long *a = I.acc + 2 * (size_t)sl, *bp = I.bnd + 2 * (size_t)sl;
+            const int n1 = E.n1[tid], n2 = E.n2[tid];
+#pragma unroll
+            for (int i = 0; i < kLimbs; ++i) {
+                E.d[i][tid] = 0;
+                if (PREC == 1) E.b[i][tid] = 0;
+            }
+            E.n1[tid] = E.n2[tid] = 0;
+            const int at = Lc.at(sl);
+            unsigned long long *a = Lc.acc + 2 * (size_t)at, *bp = Lc.bnd + 2 * (size_t)at;
             if (pass == kInitPart) {
                 sadd128(a, a + 1, d);
-                if (E.n1[tid]) atomicAdd(I.viol + sl, E.n1[tid]);
+                if (n1) atomicAdd(Lc.viol + at, n1);
                 if (PREC == 1) {
                     sadd128(bp, bp + 1, b);
-                    if (E.n2[tid]) atomicAdd(I.vmay + sl, E.n2[tid]);
+                    if (n2) atomicAdd(Lc.vmay + at, n2);
                 }
             } else if (pass == kMerge) {
                 u128 na, nb = 0;
                 int nv, nm = 0;
                 if (w.mode == 1) {
                     na = d;
-                    nv = E.n1[tid];
-                    if (PREC == 1) { nb = b; nm = E.n2[tid]; }
+                    nv = n1;
+                    if (PREC == 1) { nb = b; nm = n2; }
                 } else {
                     na = ld128(a) + d;
-                    nv = I.viol[sl] + E.n1[tid];
-                    if (PREC == 1) { nb = ld128(bp) + b; nm = I.vmay[sl] + E.n2[tid]; }
+                    nv = Lc.viol[at] + n1;
+                    if (PREC == 1) { nb = ld128(bp) + b; nm = Lc.vmay[at] + n2; }
                 }
                 st128(a, na);
-                I.viol[sl] = nv;
+                Lc.viol[at] = nv;
                 if (PREC == 1) {
                     st128(bp, nb);
-                    I.vmay[sl] = nm;
+                    Lc.vmay[at] = nm;
                 }
                 set_rec<PREC>(R, sl, na, nb, nv, nm);
             } else {
                 st128(I.vacc + 2 * (size_t)sl, d);
-                I.vviol[sl] = E.n1[tid];
+                I.vviol[sl] = n1;
             }
         }
-        if (last_barrier || t0 + kTile < e1) __syncthreads();    // else the caller synchronises
+        if (t0 + kTile < ne_all) __syncthreads();       // else the caller synchronises
         sub(2);
     }
     return terms;
 }
 
+// Clears the sums of a tile (the caller synchronises).
+template <int NT>
+__device__ __forceinline__ void clear_sums(EvalSmem &E) {
+    for (int i = threadIdx.x; i < kLimbs * (kTile + 1); i += NT) {
+        (&E.d[0][0])[i] = 0;
+        (&E.b[0][0])[i] = 0;
+    }
+    for (int i = threadIdx.x; i < kTile; i += NT) E.n1[i] = E.n2[i] = 0;
+}
+
 // Rebuilds slot pair w from the clusters as the view shows them and appends
-// a full work entry for each valid candidate at entry base + *cnt (*cnt: a
-// shared counter; the caller synchronises before reading it).
-template <int NT, int PREC>
-__device__ void rebuild_pair(const Topo &T, const State &S, const Search &X, const Inc &I, int n, int w, int *cnt,
-                             int base, const Rec &R, const Loc &Lc, const View &V) {
-    {
-        Cand c[2];
-        const int x = slot_geometry(T, S, V, n, w, c[0], c[1]);
-        I.qpar[w] = x;
-        {
-            int lo = n, hi = 0;
-            for (int d = 0; d < 2; ++d) {
-                if (c[d].s < 0) continue;
-                lo = min(lo, min(min(c[d].s, c[d].r), c[d].ns > 0 ? c[d].js : n));
-                lo = min(lo, c[d].nr > 0 ? c[d].jr : n);
-                hi = max(hi, max(max(c[d].s, c[d].r) + 1, max(c[d].js + c[d].ns, c[d].jr + c[d].nr)));
-            }
-            const bool any = c[0].s >= 0 || c[1].s >= 0;
-            R.span[w >> R.lg] = make_ushort4((unsigned short)(any ? lo : 0), (unsigned short)(any ? hi : 0),
-                                             (unsigned short)(x >= 0 ? x : 0xffff), (unsigned short)(any ? 1 : 0));
-        }
-        for (int d = 0; d < 2; ++d) {
-            const int sl = 2 * w + d;
-            X.slot[sl] = c[d];
-            if (c[d].s >= 0) {
-                int2 seg[kIncMaxSeg];
-                const int ns = full_segments(c[d], Lc.rank, seg, V.r);
-                write_entry(Lc.ent(base + atomicAdd(cnt, 1)), sl, 1, ns, seg, c[d]);
-                R.tkey[R.at(sl)] = (unsigned)c[d].key;
-                R.touch(sl);
-            } else {
-                I.viol[sl] = kIncDead;
-                st128(I.acc + 2 * (size_t)sl, 0);
-                kill_rec<PREC>(R, sl);
-            }
+// a full work entry for each valid candidate.
+template <int PREC>
+__device__ void rebuild_pair(const Topo &T, const State &S, int n, int w, unsigned long long *list, const Rec &R,
+                             const Loc &Lc, const View &V) {
+    Cand c[2];
+    const int x = slot_geometry(T, S, V, n, w, c[0], c[1]);
+    R.span[w >> R.lg] = pair_span(n, c, x);
+    for (int d = 0; d < 2; ++d) {
+        const int sl = 2 * w + d, at = Lc.at(sl);
+        Lc.slot[at] = c[d];
+        if (c[d].s >= 0) {
+            int2 seg[kIncMaxSeg];
+            const int ns = full_segments(c[d], Lc.rank, seg, V.r);
+            const unsigned long long o = append(list, ns, seg);
+            write_entry(Lc.ent((int)(unsigned)o), sl, 1, (int)(o >> 32), ns, seg, c[d]);
+            R.tkey[R.at(sl)] = (unsigned)c[d].key;
+            R.touch(sl);
+        } else {
+            Lc.viol[at] = kIncDead;
+            st128(Lc.acc + 2 * (size_t)at, 0);
+            kill_rec<PREC>(R, sl);
         }
     }
 }
 
-// The slot pairs listed in fp[0, nf), from the last thread down.
-template <int NT, int PREC>
-__device__ void rebuild_pairs(const Topo &T, const State &S, const Search &X, const Inc &I, int n, const int *fp, int nf,
-                              int *cnt, int base, const Rec &R, const Loc &Lc, const View &V) {
-    for (int i = NT - 1 - (int)threadIdx.x; i < nf; i += NT)
-        rebuild_pair<NT, PREC>(T, S, X, I, n, fp[i], cnt, base, R, Lc, V);
-}
-
 }  // namespace
 
-// Writes the merge hw's new values from its scratch into the state (the
-// values the overlay gave the terms after it: FP64 voltage, magnitude, MICE,
-// s*'s merged extremes, and their FP32 copies), clears its overlay map, and
-// zeroes r*'s MICE.  `list`: the super-nodes before that merge.
-template <int NT>
-__device__ void write_back(const State &S, const Inc &I, const Win &hw, const unsigned short *list, const uint8_t *ph,
-                           unsigned short *map, int n, int L, int G, int cr, int cs) {
-    // lanes from the last thread down (no shuffles here), beside the first
-    // threads' updates of the entries' sums
+// Writes the new values of the merge O (npos positions) from its scratch into
+// the state (the values the overlay gives: FP64 voltage, magnitude, MICE, s*'s
+// merged extremes, and their FP32 copies), and zeroes r*'s MICE.  By the first
+// nt threads of every CTA, from the last of them down.
+__device__ __forceinline__ void write_back(const State &S, const Ovl &O, int npos, const uint8_t *ph, int n, int L,
+                                           int G, int nt, int cr, int cs) {
     const int lgG = __ffs(G) - 1;
-    const int tid = threadIdx.x, rt = NT - 1 - tid, gl = rt & (G - 1), gi = rt >> lgG, NG = NT >> lgG, l = gl >> 2,
-              p = gl & 3;
-    const int n1 = hw.q1hi - hw.q1lo, n2 = hw.q2hi - hw.q2lo;
-    // this CTA's own map
-    for (int j = rt; j < hw.npos; j += NT)
-        map[j < n1 ? list[hw.q1lo + j] : (j < n1 + n2 ? list[hw.q2lo + j - n1] : hw.s)] = 0;
-    for (int j = gi * cs + cr; j < hw.npos; j += NG * cs) {
-        const int k = j < n1 ? list[hw.q1lo + j] : (j < n1 + n2 ? list[hw.q2lo + j - n1] : hw.s);
-        if (k == hw.r) continue;
-        const bool fx = j >= n1 + n2;
-        const double *cb = I.cbuf + (size_t)j * kIncCbStride * L;
+    const int rt = nt - 1 - (int)threadIdx.x;
+    if (rt < 0) return;
+    const int gl = rt & (G - 1), gi = rt >> lgG, NG = nt >> lgG, l = gl >> 2, p = gl & 3;
+    for (int j = gi * cs + cr; j < npos; j += NG * cs) {
+        const double *cb = O.cbuf + (size_t)j * kIncCbStride * L;
+        const int k = *cb_bus(cb, L);
+        if (k == O.r) continue;
+        const bool fx = j >= O.nfree;
         if (l < L && p < 3 && (ph[k] >> p & 1u)) {
             const size_t ik = sidx(l, p, k, n);
             const float4 f = *cb_f4(cb, L, l, p);
@@ -1362,8 +1391,8 @@ __device__ void write_back(const State &S, const Inc &I, const Win &hw, const un
                 S.mcur[ik] = cb[(l * 3 + p) * 3 + 2];
                 S.v32[ik] = make_float2(f.x, f.y);
             }
-            if (k == hw.s) {
-                const size_t ir = sidx(l, p, hw.r, n);
+            if (k == O.s) {
+                const size_t ir = sidx(l, p, O.r, n);
                 S.hi[ik] = fmax(S.hi[ik], S.hi[ir]);
                 S.lo[ik] = fmin(S.lo[ik], S.lo[ir]);
             }
@@ -1376,8 +1405,8 @@ __device__ void write_back(const State &S, const Inc &I, const Win &hw, const un
         }
     }
     if (rt < L && cr == 0) {                // r's cluster is gone
-        S.mice[(size_t)rt * n + hw.r] = 0.0;
-        S.mice32[(size_t)rt * n + hw.r] = 0.0f;
+        S.mice[(size_t)rt * n + O.r] = 0.0;
+        S.mice32[(size_t)rt * n + O.r] = 0.0f;
     }
 }
 
@@ -1387,10 +1416,23 @@ __host__ __device__ constexpr size_t rec_bytes(int n) { return (size_t)48 * n + 
 // ... and with the per-super-node largest MICE after them (shared memory only).
 __host__ __device__ constexpr size_t rec_maxm_bytes(int n) { return rec_bytes(n) + (size_t)8 * n; }
 
+// What a cluster's CTAs publish to each other: the minima of a pass of the
+// selection, and with them the candidate that holds the CTA's own.
+struct __align__(16) PubCand {
+    Pub v;
+    Cand c;
+};
+struct Pubs {
+    Pub w[16];                                          // by warp, within the CTA
+    Pub a[kMaxCluster], c[kMaxCluster];                 // by CTA: pass A, the rescored candidates' minimum
+    PubCand b[kMaxCluster], d[kMaxCluster];             // pass B, the rescored candidates' tie band
+};
+
 // Shared memory of one CTA of a search: [work entries][two super-node lists]
-// [phase masks][overlay map][super-node ranks][a cluster of one: block
-// summaries of the selection records; of several: what they publish], then the records of the CTA's
-// slot pairs when they fit.
+// [phase masks][two overlay maps][super-node ranks][a cluster of one: block
+// summaries of the selection records; of several: what its CTAs publish],
+// then the records of the CTA's slot pairs when they fit, then (a cluster of
+// several) their candidates and carried sums when they fit.
 __host__ __device__ constexpr size_t align16(size_t b) { return (b + 15) / 16 * 16; }
 // Blocks of 32 selection slots, and the bytes of their summaries.
 __host__ __device__ constexpr int sel_blocks(int n) { return (2 * n + 31) / 32; }
@@ -1398,34 +1440,33 @@ __host__ __device__ constexpr size_t sel_bytes(int n) {
     return align16((size_t)16 * sel_blocks(n)) + align16((size_t)4 * sel_blocks(n)) +
            align16((size_t)8 * sel_blocks(n)) + align16((size_t)sel_blocks(n));
 }
-// What a cluster's warps publish to each other (at most 16 warps a CTA).
-constexpr int kMaxCluster = 8, kPubWarps = kMaxCluster * 16;
-__host__ __device__ constexpr size_t pub_bytes(int cs) {
-    return cs == 1 ? 0 : sizeof(Pub) * (2 * kPubWarps + 2 * kMaxCluster);
-}
 // Every region is rounded up to 16 bytes: the block summaries, the published
 // values and the selection records are 16-byte keys.
 __host__ __device__ constexpr size_t base_bytes(int n, int se, int cs) {
-    return align16((size_t)se * sizeof(IncWork)) + align16((size_t)4 * n) + align16((size_t)n) + align16((size_t)2 * n) +
-           align16((size_t)4 * (n + 1)) + (cs == 1 ? sel_bytes(n) : pub_bytes(cs));
+    return align16((size_t)se * sizeof(IncWork)) + align16((size_t)4 * n) + align16((size_t)n) +
+           2 * align16((size_t)2 * n) + align16((size_t)2 * (n + 1)) + (cs == 1 ? sel_bytes(n) : sizeof(Pubs));
 }
+// The candidates (2 x 48 bytes a pair), sums (2 x 2 x 16) and counts (2 x 2 x 4) of n pairs.
+__host__ __device__ constexpr size_t sums_bytes(int n) { return (size_t)176 * n; }
 // Slot pairs of CTA cr of a cluster of cs, and how many the CTAs before it have.
 __host__ __device__ constexpr int own_pairs(int n, int cr, int cs) { return (n - cr + cs - 1) / cs; }
 __host__ __device__ constexpr int own_first(int n, int cr, int cs) {
     return cr * (n / cs) + (cr < n % cs ? cr : n % cs);
 }
 
+// rec_mode: where the selection records live (k_search_inc); + 4: the
+// candidates and carried sums in shared memory too.
 template <int NT, int PREC>
 __device__ void inc_run(const Topo &T, const State &S, const Search &X, const Inc &I, Ctrl *C, bool verify,
                         unsigned char *dyn, int rec_mode, int se, int cw, int cs) {
-    static_assert(NT >= 128 && NT <= 1024 && NT % 32 == 0, "thread count");
+    static_assert(NT >= 128 && NT <= 512 && NT % 32 == 0, "thread count");
     __shared__ __align__(16) EvalSmem E;
     __shared__ __align__(16) Red sred[33];
-    __shared__ __align__(16) Red64 s_sel;      // precision-1 selection accumulator of pass B, a cluster of one
+    __shared__ __align__(16) Red64 s_sel;       // precision-1 selection accumulator of pass B, a cluster of one
     __shared__ int sscan[33];
     __shared__ unsigned long long s_sfx[2];     // SMICE of the committed state, fixed point
     __shared__ unsigned long long s_dsum[2];    // the last merge's change of it
-    __shared__ int s_cnt[4];                    // append counters: rebuilt pairs, changed entries, entries, R
+    __shared__ unsigned long long s_app[2];     // work entries (append): the merge's; rescoring and verification
     const int n = T.n, L = T.L, tid = threadIdx.x;
     const int G = 4 * (L <= 1 ? 1 : (L <= 2 ? 2 : 4));
     const double margin = C->margin;
@@ -1436,33 +1477,28 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
     if (C->done || C->t >= max_merges) return;
     const int cr = cs == 1 ? 0 : cluster_rank(), lg = cs == 1 ? 0 : (cs == 2 ? 1 : (cs == 4 ? 2 : 3));
     const int np = own_pairs(n, cr, cs), pfirst = own_first(n, cr, cs);     // this CTA's slot pairs: w = cr, cr + cs, ...
+    const bool own = (rec_mode & 4) != 0;
+    rec_mode &= 3;
     // shared memory: entries, lists, phases; selection records: r0 or r1
     // (16 B a slot), tkey (4 B a slot), span (8 B a pair)
     Loc Lc;
     Lc.wsm = reinterpret_cast<IncWork *>(dyn);
     Lc.wgl = I.work + 2 * (size_t)pfirst;
-    Lc.fpair = I.fpair + pfirst;
     Lc.rlist = I.rlist + 2 * (size_t)pfirst;
     Lc.se = se;
     Lc.lst[0] = reinterpret_cast<unsigned short *>(dyn + align16((size_t)se * sizeof(IncWork)));
     Lc.lst[1] = Lc.lst[0] + n;
     uint8_t *phs = dyn + align16((size_t)se * sizeof(IncWork)) + align16((size_t)4 * n);
     Lc.ph = phs;
-    unsigned short *ovl_map = reinterpret_cast<unsigned short *>(phs + align16((size_t)n));
+    unsigned short *map0 = reinterpret_cast<unsigned short *>(phs + align16((size_t)n)),
+                   *map1 = map0 + align16((size_t)2 * n) / 2;
     // the super-node ranks live in shared memory during the search (copied back at the end)
-    int *rank = reinterpret_cast<int *>(reinterpret_cast<unsigned char *>(ovl_map) + align16((size_t)2 * n));
+    unsigned short *rank = map1 + align16((size_t)2 * n) / 2;
     Lc.rank = rank;
-    Ovl O;
-    O.map = ovl_map;
-    O.cbuf = I.cbuf;
-    O.s = O.r = -1;
-    O.nfree = 0;
+    unsigned char *aux = reinterpret_cast<unsigned char *>(rank) + align16((size_t)2 * (n + 1));
+    Pubs *pub = reinterpret_cast<Pubs *>(aux);                                      // (a cluster of several)
     unsigned char *recmem = rec_mode ? dyn + base_bytes(n, se, cs) : I.recbuf;      // (rec_mode 0: a cluster of one)
     const int nrec = own_pairs(n, 0, cs);
-    // what each warp of each CTA publishes to every CTA: pass A, pass B; by CTA:
-    // the rescored candidates' minimum, their tie band (a cluster of one: unused)
-    Pub *s_pa = reinterpret_cast<Pub *>(dyn + base_bytes(n, se, cs) - pub_bytes(cs)), *s_pb = s_pa + kPubWarps,
-        *s_pc = s_pb + kPubWarps, *s_pd = s_pc + kMaxCluster;
     Rec R;
     R.lg = lg;
     R.r0 = reinterpret_cast<u128 *>(recmem);
@@ -1476,7 +1512,7 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
     R.dirty = nullptr;
     R.nb = 0;
     if (cs == 1) {
-        unsigned char *sm = reinterpret_cast<unsigned char *>(rank) + align16((size_t)4 * (n + 1));
+        unsigned char *sm = aux;
         R.nb = sel_blocks(n);
         R.bsum = sm;
         sm += align16((size_t)16 * R.nb);
@@ -1486,10 +1522,31 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
         sm += align16((size_t)8 * R.nb);
         R.dirty = sm;
     }
+    Lc.lg = -1;
+    Lc.slot = X.slot;
+    Lc.acc = I.acc;
+    Lc.bnd = I.bnd;
+    Lc.viol = I.viol;
+    Lc.vmay = I.vmay;
+    if (own) {
+        unsigned char *sm = recmem + align16(rec_maxm_bytes(nrec));
+        Lc.lg = lg;
+        Lc.slot = reinterpret_cast<Cand *>(sm);
+        Lc.acc = reinterpret_cast<unsigned long long *>(sm + (size_t)96 * nrec);
+        Lc.bnd = Lc.acc + 4 * (size_t)nrec;
+        Lc.viol = reinterpret_cast<int *>(Lc.bnd + 4 * (size_t)nrec);
+        Lc.vmay = Lc.viol + 2 * (size_t)nrec;
+    }
+    Ovl O, P;                                   // the merge in progress; the one before it, until it is written back
+    O.s = O.r = -1;
+    O.nfree = 0;
+    O.map = map0;
+    O.cbuf = I.cbuf;
+    P = O;
+    int pnpos = 0;                              // positions of P
     int t = 0, ns = n;
     if (tid == 0) {
         s_sfx[0] = s_sfx[1] = 0ull;                 // every MICE starts at 0
-        s_cnt[0] = s_cnt[1] = s_cnt[2] = s_cnt[3] = 0;
         reset_sel(&s_sel);
     }
     unsigned long long tp = 0;
@@ -1504,10 +1561,11 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
     for (int w = tid; w < n; w += NT) {
         Lc.lst[0][w] = (unsigned short)w;
         phs[w] = __ldg(T.ph + w);
-        ovl_map[w] = 0;
-        rank[w] = S.sn_rank[w];
+        map0[w] = map1[w] = 0;
+        rank[w] = (unsigned short)S.sn_rank[w];
     }
-    if (tid == 0) rank[n] = S.sn_rank[n];
+    if (tid == 0) rank[n] = (unsigned short)S.sn_rank[n];
+    clear_sums<NT>(E);
     for (int j = tid; j < R.nb; j += NT) R.dirty[j] = 1;
     {
         const unsigned *tk = reinterpret_cast<const unsigned *>(I.recbuf + (size_t)32 * n);
@@ -1528,12 +1586,19 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                 set_rec<PREC>(R, sl, ld128(I.acc + 2 * (size_t)sl), PREC == 1 ? ld128(I.bnd + 2 * (size_t)sl) : (u128)0,
                               v, PREC == 1 ? I.vmay[sl] : 0);
             }
+            for (int d = 0; own && d < 2; ++d) {
+                const int sl = 2 * w + d, at = 2 * i + d;
+                Lc.slot[at] = X.slot[sl];
+                st128(Lc.acc + 2 * (size_t)at, ld128(I.acc + 2 * (size_t)sl));
+                st128(Lc.bnd + 2 * (size_t)at, ld128(I.bnd + 2 * (size_t)sl));
+                Lc.viol[at] = I.viol[sl];
+                Lc.vmay[at] = I.vmay[sl];
+            }
         }
     }
     csync(cs);                              // (every CTA runs before the first one publishes to another)
     if (prof && tid == 0) tp = gtimer_inc();
 
-    Win hw = {};                            // the last merge (a cluster of several CTAs writes it back in the next selection)
     for (;;) {
         const unsigned short *list_old = Lc.lst[t & 1];
         unsigned short *list_new = Lc.lst[(t + 1) & 1];
@@ -1544,11 +1609,10 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
         //   A cluster of one: the blocks whose records changed are summarised
         // again (one warp per block, one barrier), then every warp reduces the
         // summaries on its own.
-        //   A cluster of several: every warp reduces a strided share of its CTA's
-        // records (one or two a thread) and publishes the result to every CTA;
-        // one cluster barrier, then every warp of every CTA reduces what was
-        // published.
-        if (tid == 0) s_cnt[0] = s_cnt[1] = s_cnt[2] = s_cnt[3] = 0;
+        //   A cluster of several: every CTA reduces its own records (one or two a
+        // thread) and publishes the result to every CTA; one cluster barrier, then
+        // every warp of every CTA reduces what was published.
+        if (tid == 0) s_app[0] = s_app[1] = 0ull;
         const int lane = tid & 31, wid = tid >> 5;
         constexpr int NW = NT / 32;
         Red ra;
@@ -1587,7 +1651,8 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                         mx = mb > mx ? mb : mx;
                     }
                 }
-                {
+                // by warp, then by the first warp, then by every warp over the CTAs
+                auto fold = [&]() {
                     Pub v;
                     if (PREC == 0) {
                         mn = warp_min128(mn);
@@ -1599,27 +1664,32 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                     }
                     v.c = warp_max64(mx);
                     v.d = __reduce_add_sync(0xffffffffu, cnt);
-                    if (lane < cs) publish(&s_pa[cr * NW + wid], lane, v);
+                    return v;
+                };
+                auto take = [&](bool in, const Pub *src) {
+                    mn = kNone;
+                    lo = hi = ~0ull;
+                    mx = 0;
+                    cnt = 0;
+                    if (in) {
+                        const Pub v = *src;
+                        mn = ((u128)v.b << 64) | (u128)v.a;
+                        lo = v.a;
+                        hi = v.b;
+                        mx = v.c;
+                        cnt = (unsigned)v.d;
+                    }
+                };
+                const Pub v = fold();
+                if (lane == 0) pub->w[wid] = v;
+                __syncthreads();
+                if (wid == 0) {
+                    take(lane < NW, pub->w + lane);
+                    const Pub u = fold();
+                    if (lane < cs) publish(&pub->a[cr], lane, &u, 2);
                 }
                 csync(cs);
-                mn = kNone;
-                lo = hi = ~0ull;
-                mx = 0;
-                cnt = 0;
-                for (int j = lane; j < cs * NW; j += 32) {
-                    const Pub v = s_pa[j];
-                    if (PREC == 0) {
-                        mn = umin(mn, ((u128)v.b << 64) | (u128)v.a);
-                    } else {
-                        lo = v.a < lo ? v.a : lo;
-                        hi = v.b < hi ? v.b : hi;
-                    }
-                    mx = v.c > mx ? v.c : mx;
-                    cnt += (unsigned)v.d;
-                }
-                // the last merge's new values into the state (every CTA's terms
-                // have read the old ones; the barrier of pass B shows them)
-                if (t > 0 && !verify) write_back<NT>(S, I, hw, list_new, Lc.ph, ovl_map, n, L, G, cr, cs);
+                take(lane < cs, pub->a + lane);
             }
             if (PREC == 0) {
                 ra.a = warp_min128(mn);
@@ -1640,6 +1710,7 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
             if (tid == 0 && cr == 0) { C->done = 1; C->stop_reason = 0; }
             break;
         }
+        Cand wc;                                         // the winner
         if (tid == 0 && cr == 0) {
             cands_run += nvalid;
             X.dec_ncand[t] = nvalid;
@@ -1650,12 +1721,12 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
             int base = 0;
             for (int c0 = 0; c0 < 2 * n; c0 += NT) {
                 const int c = c0 + tid;
-                const int v = c < 2 * n ? I.viol[c] : kIncDead;
+                const int v = c < 2 * n ? Lc.viol[c] : kIncDead;      // (recording runs one CTA, sums in device memory)
                 const int f = v < kIncDead ? 1 : 0;
                 int tot = 0;
                 const int o = block_excl_scan<NT>(f, &tot, sscan) + base;
                 if (f) {
-                    const Cand &cc = X.slot[c];
+                    const Cand &cc = Lc.slot[c];
                     const size_t at = (size_t)t * 2 * n + o;
                     X.rec_s[at] = T.orig[cc.s];
                     X.rec_r[at] = T.orig[cc.r];
@@ -1697,23 +1768,41 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                 }
                 if (cs > 1) {
                     // (a tie key with its slot fits 64 bits)
-                    Pub v;
-                    v.a = warp_min64((unsigned long long)pa);
-                    pb = warp_min128(pb);
-                    v.b = 0;
-                    v.c = (unsigned long long)pb;
-                    v.d = (unsigned long long)(pb >> 64);
-                    if (lane < cs) publish(&s_pb[cr * NW + wid], lane, v);
-                    csync(cs);
-                    unsigned long long qa = ~0ull;
-                    pb = kNone;
-                    for (int j = lane; j < cs * NW; j += 32) {
-                        const Pub u = s_pb[j];
-                        qa = u.a < qa ? u.a : qa;
-                        pb = umin(pb, ((u128)u.d << 64) | (u128)u.c);
+                    unsigned long long qa = (unsigned long long)pa;
+                    auto fold = [&]() {
+                        Pub v;
+                        v.a = qa = warp_min64(qa);
+                        pb = warp_min128(pb);
+                        v.b = 0;
+                        v.c = (unsigned long long)pb;
+                        v.d = (unsigned long long)(pb >> 64);
+                        return v;
+                    };
+                    auto take = [&](bool in, const Pub *src) {
+                        qa = ~0ull;
+                        pb = kNone;
+                        if (in) {
+                            const Pub u = *src;
+                            qa = u.a;
+                            pb = ((u128)u.d << 64) | (u128)u.c;
+                        }
+                    };
+                    const Pub v = fold();
+                    if (lane == 0) pub->w[wid] = v;
+                    __syncthreads();
+                    if (wid == 0) {
+                        take(lane < NW, pub->w + lane);
+                        PubCand u;
+                        u.v = fold();
+                        u.c = Lc.slot[Lc.at(qa != ~0ull ? (int)(unsigned)qa : 2 * cr)];
+                        if (lane < cs) publish(&pub->b[cr], lane, &u, 5);
                     }
-                    pa = (u128)warp_min64(qa);
-                    pb = warp_min128(pb);
+                    csync(cs);
+                    take(lane < cs, &pub->b[lane < cs ? lane : 0].v);
+                    const unsigned long long q0 = qa;
+                    fold();
+                    pa = (u128)qa;
+                    wc = pub->b[__ffs(__ballot_sync(0xffffffffu, q0 == qa && lane < cs)) - 1].c;
                 } else {
                     Red rb;
                     rb.a = pa;
@@ -1797,23 +1886,38 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                     }
                 }
                 if (cs > 1) {
-                    Pub v;
-                    v.a = warp_min64(pa);
-                    v.b = warp_min64(pb);
-                    v.c = warp_min64(pc);
-                    v.d = 0;
-                    if (lane < cs) publish(&s_pb[cr * NW + wid], lane, v);
-                    csync(cs);
-                    pa = pb = pc = ~0ull;
-                    for (int j = lane; j < cs * NW; j += 32) {
-                        const Pub u = s_pb[j];
-                        pa = u.a < pa ? u.a : pa;
-                        pb = u.b < pb ? u.b : pb;
-                        pc = u.c < pc ? u.c : pc;
+                    auto fold = [&]() {
+                        Pub v;
+                        v.a = pa = warp_min64(pa);
+                        v.b = pb = warp_min64(pb);
+                        v.c = pc = warp_min64(pc);
+                        v.d = 0;
+                        return v;
+                    };
+                    auto take = [&](bool in, const Pub *src) {
+                        pa = pb = pc = ~0ull;
+                        if (in) {
+                            const Pub u = *src;
+                            pa = u.a;
+                            pb = u.b;
+                            pc = u.c;
+                        }
+                    };
+                    const Pub v = fold();
+                    if (lane == 0) pub->w[wid] = v;
+                    __syncthreads();
+                    if (wid == 0) {
+                        take(lane < NW, pub->w + lane);
+                        PubCand u;
+                        u.v = fold();
+                        u.c = Lc.slot[Lc.at(pa != ~0ull ? (int)(unsigned)pa : 2 * cr)];
+                        if (lane < cs) publish(&pub->b[cr], lane, &u, 5);
                     }
-                    pa = warp_min64(pa);
-                    pb = warp_min64(pb);
-                    pc = warp_min64(pc);
+                    csync(cs);
+                    take(lane < cs, &pub->b[lane < cs ? lane : 0].v);
+                    const unsigned long long p0 = pa;
+                    fold();
+                    wc = pub->b[__ffs(__ballot_sync(0xffffffffu, p0 == pa && lane < cs)) - 1].c;
                 } else {
                     Red64 r6;
                     r6.a = pa;
@@ -1905,17 +2009,20 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                     const bool out_sure = has_hi && q.x > eout;
                     const bool unc = !in_sure && !out_sure && (u128)R.tkey[c] < ks;
                     if (unc || q.x <= mh) {
-                        const int o = atomicAdd(&s_cnt[3], 1), sl = slot_of(c);
-                        Lc.rlist[o] = sl;
+                        const int sl = slot_of(c);
+                        const Cand cc = Lc.slot[Lc.at(sl)];
                         int2 seg[kIncMaxSeg];
-                        const int k = full_segments(X.slot[sl], rank, seg);
-                        write_entry(Lc.ent(o), sl, 1, k, seg, X.slot[sl]);
+                        const int k = full_segments(cc, rank, seg);
+                        const unsigned long long o = append(&s_app[1], k, seg);
+                        Lc.rlist[(int)(unsigned)o] = sl;
+                        write_entry(Lc.ent((int)(unsigned)o), sl, 1, (int)(o >> 32), k, seg, cc);
                     }
                 }
                 __syncthreads();
-                const int nR = s_cnt[3];
-                terms += run_entries<NT, PREC>(T, S, X, I, n, L, G, margin, mlo, mhi, 0, nR, kF64, list_old, list_old,
-                                               -1, O, E, sscan, R, Lc);
+                const int nR = (int)(unsigned)s_app[1];
+                terms += run_entries<NT, PREC>(T, S, I, n, L, G, margin, mlo, mhi, nR, (int)(s_app[1] >> 32), kF64,
+                                               list_old, list_old, -1, P, E, R, Lc);
+                __syncthreads();
                 // exact selection over every CTA's R, with the surely-in candidate of key ks
                 Red rc;
                 rc.a = rc.b = rc.c = kNone;
@@ -1932,13 +2039,13 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                     v.b = (unsigned long long)(rc.a >> 64);
                     v.c = (unsigned long long)nR;
                     v.d = 0;
-                    if (tid < cs) publish(&s_pc[cr], tid, v);
+                    if (tid < cs) publish(&pub->c[cr], tid, &v, 2);
                     csync(cs);
                     rc.a = kNone;
                     nR_all = 0;
                     for (int j = 0; j < cs; ++j) {
-                        rc.a = umin(rc.a, ((u128)s_pc[j].b << 64) | (u128)s_pc[j].a);
-                        nR_all += (int)s_pc[j].c;
+                        rc.a = umin(rc.a, ((u128)pub->c[j].b << 64) | (u128)pub->c[j].a);
+                        nR_all += (int)pub->c[j].c;
                     }
                 }
                 Red rd;
@@ -1955,17 +2062,22 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                     }
                     rd = block_red<NT>(rd, sred);
                     if (cs > 1) {
-                        Pub v;                      // (a tie key with its slot fits 64 bits; none: ~0)
-                        v.a = (unsigned long long)rd.a;
-                        v.b = (unsigned long long)rd.b;
-                        v.c = (unsigned long long)(rd.b >> 64);
-                        v.d = 0;
-                        if (tid < cs) publish(&s_pd[cr], tid, v);
+                        PubCand v;                  // (a tie key with its slot fits 64 bits; none: ~0)
+                        v.v.a = (unsigned long long)rd.a;
+                        v.v.b = (unsigned long long)rd.b;
+                        v.v.c = (unsigned long long)(rd.b >> 64);
+                        v.v.d = 0;
+                        v.c = Lc.slot[Lc.at(rd.a != kNone ? (int)(unsigned)rd.a : 2 * cr)];
+                        if (tid < cs) publish(&pub->d[cr], tid, &v, 5);
                         csync(cs);
                         rd.a = rd.b = kNone;
                         for (int j = 0; j < cs; ++j) {
-                            if (s_pd[j].a != ~0ull) rd.a = umin(rd.a, (u128)s_pd[j].a);
-                            rd.b = umin(rd.b, ((u128)s_pd[j].c << 64) | (u128)s_pd[j].b);
+                            const Pub u = pub->d[j].v;
+                            if (u.a != ~0ull && (u128)u.a < rd.a) {
+                                rd.a = (u128)u.a;
+                                if (rd.a < rb.a) wc = pub->d[j].c;
+                            }
+                            rd.b = umin(rd.b, ((u128)u.c << 64) | (u128)u.b);
                         }
                     }
                     if (tid == 0 && rd.b != kNone) gap = fx_to_d((rd.b ^ kSignBit) - edge);
@@ -1981,92 +2093,130 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
             break;
         }
         stamp(0);
-        // ============================================================ the merge's changed set
-        // The winner's record: every thread builds its own at once (every
-        // thread knows ws; one broadcast load of its candidate), so no warp
-        // waits for another's copy (r*'s subtree and the decision's bus ids
-        // are looked up in the merge step).
+        // ============================================================ the merge
+        // The winner's record: every thread builds its own at once, so no warp
+        // waits for another's copy.
         const int CW = cw;                  // warps that evaluate the merge (1 .. NW - 1)
-        const bool commit_warp = (tid >> 5) >= NW - CW;
-        hw = make_win(X.slot[ws], ws, rank);
+        const bool commit_warp = wid >= NW - CW;
+        if (cs == 1) {
+            wc = Lc.slot[Lc.at(ws)];
+            __syncthreads();                // (the rebuilt pairs below may write the winner's slot)
+        }
+        const Win hw = make_win(wc, ws, rank);
         if (tid == 0) {
             if (cr == 0) X.dec_gap[t] = gap;
             s_dsum[0] = 0ull;
             s_dsum[1] = 0ull;
         }
         stamp(12);                                      // profile: the winner's record
+        const int n1 = hw.q1hi - hw.q1lo, n2 = hw.q2hi - hw.q2lo;
+        O.map = t & 1 ? map1 : map0;
+        O.cbuf = I.cbuf + (t & 1 ? (size_t)n * kIncCbStride * L : 0);
         O.s = hw.s;
         O.r = hw.r;
-        O.nfree = (hw.q1hi - hw.q1lo) + (hw.q2hi - hw.q2lo);
-        // ---- which candidates change: rebuilt pairs (next to s* or r*) and
-        // changed terms; entries are appended in any order (the sums are exact).
-        // Each CTA scans its own slot pairs.  The last warps evaluate the merge's
-        // own FP64 values meanwhile; the others map its positions for the overlay.
-        {
-            if (commit_warp) {
-                Commit cm;
-                cm.h = &hw;
-                cm.wc = X.slot[ws];
-                cm.list = list_old;
-                cm.ph = Lc.ph;
-                cm.O = O;
-                terms += commit_groups(T, S, I, n, L, G, margin, cm, NW - CW, CW, cr, cs);
-            } else {
-                const int nsc = (NW - CW) * 32, n1 = hw.q1hi - hw.q1lo;
-                for (int q = tid; q < hw.npos; q += nsc) {      // the terms after the merge read k's new values here
-                    const int k = q < n1 ? list_old[hw.q1lo + q] : (q < O.nfree ? list_old[hw.q2lo + q - n1] : hw.s);
-                    if (k != hw.r) ovl_map[k] = (unsigned short)(q + 1);
-                }
-                // s takes r's injection (no term before the merge reads s's injection:
-                // every candidate with r = s* is rebuilt; the merge's own evaluation
-                // reads r's)
-                if (tid < 3 * L && cr == 0 && (Lc.ph[hw.r] >> (tid % 3) & 1u)) {
-                    const size_t is = sidx(tid / 3, tid % 3, hw.s, n), ir = sidx(tid / 3, tid % 3, hw.r, n);
-                    const double2 ni = cadd(S.icur[is], S.icur[ir]);
-                    S.icur[is] = ni;
-                    S.icur32[is] = make_float2((float)ni.x, (float)ni.y);
-                }
-                // the changed buses lie in [hl, hh): a candidate whose span misses it is unchanged
-                int hl = min(hw.s, hw.r), hh = max(hw.s, hw.r) + 1;
-                if (hw.w1lo < hw.w1hi) { hl = min(hl, hw.w1lo); hh = max(hh, hw.w1hi); }
-                if (hw.w2lo < hw.w2hi) { hl = min(hl, hw.w2lo); hh = max(hh, hw.w2hi); }
-                for (int i = tid; i < np; i += nsc) {
-                    const ushort4 sp = R.span[i];
-                    const int w = (i << lg) + cr;
-                    if (sp.w == 0 || w == hw.r) continue;
-                    const int qp = sp.z == 0xffff ? -1 : (int)sp.z;
-                    if (w == hw.s || qp == hw.r || qp == hw.s) {
-                        Lc.fpair[atomicAdd(&s_cnt[0], 1)] = w;
-                        continue;
-                    }
-                    if ((int)sp.y <= hl || (int)sp.x >= hh) continue;
+        O.nfree = n1 + n2;
+        // One step, nothing in it waiting for anything else in it:
+        //   - the last warps of every CTA evaluate the merge's own FP64 values
+        // into its scratch (the state under the overlay of the merge before, P);
+        //   - the others write P back, map the merge's positions, find the
+        // candidates that change among the CTA's own (their terms are listed in
+        // any order: the sums are exact), rebuild the pairs next to s* and r*
+        // through the merge's view of the clusters, and do the merge's
+        // bookkeeping (clusters, super-node list, s*'s injection).
+        if (commit_warp) {
+            Commit cm;
+            cm.h = &hw;
+            cm.wc = wc;
+            cm.list = list_old;
+            cm.ph = Lc.ph;
+            cm.O = P;
+            cm.cbuf = const_cast<double *>(O.cbuf);
+            terms += commit_groups(T, S, n, L, G, margin, cm, NW - CW, CW, cr, cs);
+        } else {
+            const int nsc = (NW - CW) * 32;
+            View V;
+            V.s = hw.s;
+            V.r = hw.r;
+            V.dir = hw.dir;
+            // the changed buses lie in [hl, hh): a candidate whose span misses it is unchanged
+            int hl = min(hw.s, hw.r), hh = max(hw.s, hw.r) + 1;
+            if (hw.w1lo < hw.w1hi) { hl = min(hl, hw.w1lo); hh = max(hh, hw.w1hi); }
+            if (hw.w2lo < hw.w2hi) { hl = min(hl, hw.w2lo); hh = max(hh, hw.w2hi); }
+            for (int i = tid; i < np; i += nsc) {
+                const ushort4 sp = R.span[i];
+                const int w = (i << lg) + cr;
+                if (w == hw.r) {                        // r's cluster is gone
+                    R.maxm[i] = 0.0;
+                    R.touch_sn(w);
+                    R.span[i] = make_ushort4(0, 0, 0xffff, 0);
                     for (int d = 0; d < 2; ++d) {
-                        const Cand &c = X.slot[2 * w + d];
-                        if (c.s < 0 || !touched(c, hw)) continue;
-                        int2 seg[kIncMaxSeg];
-                        const int k = changed_segments(c, hw, rank, seg);
-                        write_entry(Lc.ent(atomicAdd(&s_cnt[1], 1)), 2 * w + d, 0, k, seg, c);
+                        Lc.slot[Lc.at(2 * w + d)].s = -1;
+                        Lc.viol[Lc.at(2 * w + d)] = kIncDead;
+                        kill_rec<PREC>(R, 2 * w + d);
                     }
+                    continue;
                 }
+                if (sp.w == 0) continue;
+                const int qp = sp.z == 0xffff ? -1 : (int)sp.z;
+                if (w == hw.s || qp == hw.r || qp == hw.s) {
+                    rebuild_pair<PREC>(T, S, n, w, &s_app[0], R, Lc, V);
+                    continue;
+                }
+                if ((int)sp.y <= hl || (int)sp.x >= hh) continue;
+                for (int d = 0; d < 2; ++d) {
+                    const Cand c = Lc.slot[Lc.at(2 * w + d)];
+                    if (c.s < 0 || !touched(c, hw)) continue;
+                    int2 seg[kIncMaxSeg];
+                    const int k = changed_segments(c, hw, rank, seg);
+                    const unsigned long long o = append(&s_app[0], k, seg);
+                    write_entry(Lc.ent((int)(unsigned)o), 2 * w + d, 0, (int)(o >> 32), k, seg, c);
+                }
+            }
+            if (pnpos > 0) write_back(S, P, pnpos, Lc.ph, n, L, G, nsc, cr, cs);
+            unsigned short *map = t & 1 ? map1 : map0;
+            for (int q = tid; q < hw.npos; q += nsc) {      // the terms after the merge read k's new values here
+                const int k = q < n1 ? list_old[hw.q1lo + q] : (q < O.nfree ? list_old[hw.q2lo + q - n1] : hw.s);
+                if (k != hw.r) map[k] = (unsigned short)(q + 1);
+            }
+            // r's members join s (they lie in the subtree of r's top; a rebuilt pair
+            // reads either value the same); the new super-node list
+            const int rtop = S.top[hw.r], rtop_end = rtop + T.sz[rtop];
+            for (int b = rtop + tid * cs + cr; b < rtop_end; b += nsc * cs)
+                if (S.label[b] == hw.r) S.label[b] = hw.s;
+            for (int j = tid; j < ns - 1; j += nsc) list_new[j] = list_old[j + (j >= hw.jr ? 1 : 0)];
+            // s takes r's injection (no term before the merge reads s's injection:
+            // every candidate with r = s* is rebuilt; the merge's own evaluation
+            // reads r's)
+            if (tid < 3 * L && cr == 0 && (Lc.ph[hw.r] >> (tid % 3) & 1u)) {
+                const size_t is = sidx(tid / 3, tid % 3, hw.s, n), ir = sidx(tid / 3, tid % 3, hw.r, n);
+                const double2 ni = cadd(S.icur[is], S.icur[ir]);
+                S.icur[is] = ni;
+                S.icur32[is] = make_float2((float)ni.x, (float)ni.y);
+            }
+            if (tid == 0 && cr == 0) {
+                if (hw.dir == 1) {                      // (read through the view: r's)
+                    S.top[hw.s] = S.top[hw.r];
+                    S.ptop[hw.s] = S.ptop[hw.r];
+                }
+                X.dec_s[t] = T.orig[hw.s];
+                X.dec_r[t] = T.orig[hw.r];
             }
         }
         csync(cs);
-        const int nf_tot = s_cnt[0], np_tot = s_cnt[1];   // (s_cnt[2] is 0: rebuilt entries follow these)
+        ns -= 1;
+        const int ne = (int)(unsigned)s_app[0], items = (int)(s_app[0] >> 32);
         if (PREC == 1 && tid == 0) reset_sel(&s_sel);     // every thread has read the selection's result
         stamp(1);
-        // ============================================================ the merge (score change, topology) and,
-        // beside it, the rebuilt candidates
-        // (the new voltages, extremes and MICE stay in the scratch, with the
-        // FP32 copies the merge's evaluation derived, read through the overlay,
-        // until the terms before the merge have been evaluated)
+        // ============================================================ the terms that change, and the score
         {
-            const int n1 = hw.q1hi - hw.q1lo, n2 = hw.q2hi - hw.q2lo;
-            const int lgG = __ffs(G) - 1;
-            const int gl = tid & (G - 1), gi = tid >> lgG, NG = NT >> lgG, l = gl >> 2, p = gl & 3;
+            // the merge's exact score change (its FP64 terms in fixed point) and
+            // each position's largest MICE, one lane per (position, scenario), from
+            // the last thread down; P's map is cleared (its values are in the state)
+            const int lgG = __ffs(G) - 1, rt = NT - 1 - tid;
+            const int gl = rt & (G - 1), gi = rt >> lgG, NG = NT >> lgG, l = gl >> 2, p = gl & 3;
             u128 dsum = 0;
-            // one lane per (position, scenario)
             for (int r0 = 0; r0 < hw.npos; r0 += NG) {
-                if (r0 + ((tid >> 5) << (5 - lgG)) >= hw.npos) break;
+                if (r0 + ((rt >> 5) << (5 - lgG)) >= hw.npos) break;
                 const int j = r0 + gi;
                 bool valid = j < hw.npos;
                 int k = hw.s;
@@ -2074,115 +2224,71 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                     k = j < n1 ? list_old[hw.q1lo + j] : (j < n1 + n2 ? list_old[hw.q2lo + j - n1] : hw.s);
                     valid = k != hw.r;
                 }
-                const double *cb = I.cbuf + (size_t)j * kIncCbStride * L;
-                // the merge's exact score change: its FP64 terms in fixed point
+                const bool mine = valid && (k & (cs - 1)) == cr;
                 unsigned long long mb = 0;                  // MICE >= 0: bit patterns order like values
-                if (valid && l < L && p == 0) {
-                    const double m = cb[9 * L + l];
-                    double dd = m - S.mice[(size_t)l * n + k];
-                    if (k == hw.s) dd -= S.mice[(size_t)l * n + hw.r];
-                    dsum += to_fx(dd);
+                if (valid && l < L && p == 0 && (mine || cr == 0)) {
+                    const double m = O.cbuf[(size_t)j * kIncCbStride * L + 9 * L + l];
                     mb = (unsigned long long)__double_as_longlong(m);
+                    if (cr == 0) {
+                        double dd = m - S.mice[(size_t)l * n + k];
+                        if (k == hw.s) dd -= S.mice[(size_t)l * n + hw.r];
+                        dsum += to_fx(dd);
+                    }
                 }
                 for (int o = 4; o < G; o <<= 1) {
                     const unsigned long long y = __shfl_xor_sync(0xffffffffu, mb, o);
                     mb = y > mb ? y : mb;
                 }
-                if (valid && gl == 0 && (k & (cs - 1)) == cr) {
+                if (mine && gl == 0) {
                     R.maxm[k >> lg] = __longlong_as_double((long long)mb);
                     R.touch_sn(k);
                 }
             }
             if (dsum != 0) sadd128(&s_dsum[0], &s_dsum[1], dsum);
-            // r's members join s (they lie in the subtree of r's top); the new
-            // super-node list.  Not on the last warp, which goes straight to the
-            // rebuilt pairs below (their chain of dependent loads is this
-            // step's longest).
-            constexpr int NB = NT - 32;
-            if (tid < NB) {
-                const int rtop = S.top[hw.r], rtop_end = rtop + T.sz[rtop];
-                for (int b = rtop + tid * cs + cr; b < rtop_end; b += NB * cs)
-                    if (S.label[b] == hw.r) S.label[b] = hw.s;
-                for (int j = tid; j < ns - 1; j += NB) list_new[j] = list_old[j + (j >= hw.jr ? 1 : 0)];
-            }
-            if (tid == 0 && cr == 0) {
-                if (hw.dir == 1) {
-                    S.top[hw.s] = S.top[hw.r];
-                    S.ptop[hw.s] = S.ptop[hw.r];
-                }
-                I.qpar[hw.r] = -1;
-                X.dec_s[t] = T.orig[hw.s];
-                X.dec_r[t] = T.orig[hw.r];
-            }
-            if ((hw.r & (cs - 1)) == cr) {
-                if (tid == 0) {
-                    R.maxm[hw.r >> lg] = 0.0;
-                    R.touch_sn(hw.r);
-                    R.span[hw.r >> lg] = make_ushort4(0, 0, 0xffff, 0);
-                }
-                if (tid < 2) {
-                    X.slot[2 * hw.r + tid].s = -1;
-                    I.viol[2 * hw.r + tid] = kIncDead;
-                    kill_rec<PREC>(R, 2 * hw.r + tid);
-                }
-            }
+            unsigned short *pmap = t & 1 ? map0 : map1;
+            for (int j = rt; j < pnpos; j += NT) pmap[*cb_bus(P.cbuf + (size_t)j * kIncCbStride * L, L)] = 0;
         }
-        // rebuilt pairs from the last thread down, reading the clusters through the
-        // merge's view (the ranks change only after the terms below)
-        {
-            View V;
-            V.s = hw.s;
-            V.r = hw.r;
-            V.dir = hw.dir;
-            rebuild_pairs<NT, PREC>(T, S, X, I, n, Lc.fpair, nf_tot, &s_cnt[2], np_tot, R, Lc, V);
-        }
-        __syncthreads();
-        ns -= 1;
-        const int ne_new = np_tot + s_cnt[2];
-        stamp(2);
-        if (tid == 0) {
-            const u128 sfx = ld128(s_sfx) + ld128(s_dsum);
-            st128(s_sfx, sfx);
-            if (cr == 0) X.dec_score[t] = fx_to_d(sfx);
-        }
-        // ============================================================ the terms that change
-        terms += run_entries<NT, PREC>(T, S, X, I, n, L, G, margin, mlo, mhi, 0, ne_new, kMerge, list_old, list_new, hw.r,
-                                       O, E, sscan, R, Lc, prof && cr == 0 ? C->phase_ns + 6 : nullptr, false);
-        // the new values into the state (no term reads the state before the
-        // merge any more; this overlaps the last tile's updates of the sums), in
-        // a cluster of several CTAs once all of them are past their terms (in
-        // the next selection); ranks past r* drop by one
-        if (cs == 1) write_back<NT>(S, I, hw, list_old, Lc.ph, ovl_map, n, L, G, 0, 1);
-        for (int b = hw.r + 1 + tid; b <= n; b += NT) rank[b] -= 1;
+        terms += run_entries<NT, PREC>(T, S, I, n, L, G, margin, mlo, mhi, ne, items, kMerge, list_old, list_new, hw.r,
+                                       O, E, R, Lc, prof && cr == 0 ? C->phase_ns + 6 : nullptr);
+        for (int b = hw.r + 1 + tid; b <= n; b += NT) rank[b] -= 1;     // ranks past r* drop by one
         __syncthreads();
         stamp(3);
+        if (tid == 0 && cr == 0) {
+            const u128 sfx = ld128(s_sfx) + ld128(s_dsum);
+            st128(s_sfx, sfx);
+            X.dec_score[t] = fx_to_d(sfx);
+        }
+        P = O;
+        pnpos = hw.npos;
         t += 1;
         if (verify) {
-            if (cs > 1) {
-                csync(cs);
-                write_back<NT>(S, I, hw, list_old, Lc.ph, ovl_map, n, L, G, cr, cs);
-                csync(cs);
-            }
-            // every candidate again from scratch (after the merge, through the
-            // overlay); the carried values must match bit for bit
-            if (tid == 0) s_cnt[3] = 0;
-            __syncthreads();
+            // every candidate again from scratch, on the state with the merge
+            // written back; the carried values must match bit for bit
+            if (tid == 0) s_app[1] = 0ull;
+            csync(cs);
+            write_back(S, P, pnpos, Lc.ph, n, L, G, NT, cr, cs);
+            unsigned short *pmap = t & 1 ? map0 : map1;
+            for (int j = tid; j < pnpos; j += NT) pmap[*cb_bus(P.cbuf + (size_t)j * kIncCbStride * L, L)] = 0;
+            pnpos = 0;
+            csync(cs);
             for (int i = tid; i < 2 * np; i += NT) {
                 const int c = slot_of(i);
-                const Cand &cc = X.slot[c];
+                const Cand cc = Lc.slot[Lc.at(c)];
                 if (cc.s < 0) continue;
                 int2 seg[kIncMaxSeg];
                 const int k = full_segments(cc, rank, seg);
-                write_entry(Lc.ent(atomicAdd(&s_cnt[3], 1)), c, 1, k, seg, cc);
+                const unsigned long long o = append(&s_app[1], k, seg);
+                write_entry(Lc.ent((int)(unsigned)o), c, 1, (int)(o >> 32), k, seg, cc);
             }
             __syncthreads();
-            run_entries<NT, PREC>(T, S, X, I, n, L, G, margin, mlo, mhi, 0, s_cnt[3], kFresh, list_new, list_new, -1,
-                                  O, E, sscan, R, Lc);
+            run_entries<NT, PREC>(T, S, I, n, L, G, margin, mlo, mhi, (int)(unsigned)s_app[1], (int)(s_app[1] >> 32),
+                                  kFresh, list_new, list_new, -1, P, E, R, Lc);
+            __syncthreads();
             int bad = 0;
             for (int i = tid; i < 2 * np; i += NT) {
-                const int c = slot_of(i);
-                if (X.slot[c].s < 0) continue;
-                if (I.viol[c] != I.vviol[c] || ld128(I.acc + 2 * (size_t)c) != ld128(I.vacc + 2 * (size_t)c)) ++bad;
+                const int c = slot_of(i), at = Lc.at(c);
+                if (Lc.slot[at].s < 0) continue;
+                if (Lc.viol[at] != I.vviol[c] || ld128(Lc.acc + 2 * (size_t)at) != ld128(I.vacc + 2 * (size_t)c)) ++bad;
             }
             Red rv;
             rv.a = rv.b = rv.c = kNone;
@@ -2191,6 +2297,8 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
             if (tid == 0 && rv.i) atomicAdd(&C->inc_mismatch, rv.i);
         }
     }
+    // the last merge into the state (every CTA is past its terms: the selection's barrier)
+    if (pnpos > 0) write_back(S, P, pnpos, Lc.ph, n, L, G, NT, cr, cs);
     if (prof) {                                     // (phase-node, scenario) items evaluated over the run
         unsigned long long tt = (unsigned long long)terms;
         for (int o = 16; o > 0; o >>= 1) tt += __shfl_xor_sync(0xffffffffu, tt, o);
@@ -2250,7 +2358,7 @@ constexpr int kInitCtasMax = kIncInitCtasMax;
 // 2n + 8n bytes, 16-byte aligned parts).
 template <int NT, int PREC>
 __device__ void inc_init_share(const Topo &T, const State &S, const Search &X, const Inc &I, Ctrl *C, int b, int B,
-                               unsigned char *dyn, EvalSmem &E, int *sscan, int &s_first, int &s_ne) {
+                               unsigned char *dyn, EvalSmem &E, int *sscan, int &s_first, unsigned long long &s_app) {
     const int n = T.n, L = T.L, tid = threadIdx.x;
     const int G = 4 * (L <= 1 ? 1 : (L <= 2 ? 2 : 4));
     const double margin = C->margin;
@@ -2261,11 +2369,17 @@ __device__ void inc_init_share(const Topo &T, const State &S, const Search &X, c
     Loc Lc;
     Lc.wsm = nullptr;
     Lc.wgl = I.work;
-    Lc.fpair = Lc.rlist = nullptr;
+    Lc.rlist = nullptr;
     Lc.se = 0;
     Lc.lst[0] = Lc.lst[1] = list;
     Lc.ph = T.ph;
-    Lc.rank = S.sn_rank;
+    Lc.rank = nullptr;                          // (the ranks are read from S.sn_rank)
+    Lc.lg = -1;
+    Lc.slot = X.slot;
+    Lc.acc = I.acc;
+    Lc.bnd = I.bnd;
+    Lc.viol = I.viol;
+    Lc.vmay = I.vmay;
     Rec R;
     R.lg = 0;
     R.r0 = reinterpret_cast<u128 *>(I.recbuf);
@@ -2288,17 +2402,7 @@ __device__ void inc_init_share(const Topo &T, const State &S, const Search &X, c
     for (int w = b + B * tid; w < n; w += B * NT) {
         Cand c[2];
         const int x = slot_geometry(T, S, V, n, w, c[0], c[1]);
-        I.qpar[w] = x;
-        int lo = n, hi = 0;
-        for (int d = 0; d < 2; ++d) {
-            if (c[d].s < 0) continue;
-            lo = min(lo, min(min(c[d].s, c[d].r), c[d].ns > 0 ? c[d].js : n));
-            lo = min(lo, c[d].nr > 0 ? c[d].jr : n);
-            hi = max(hi, max(max(c[d].s, c[d].r) + 1, max(c[d].js + c[d].ns, c[d].jr + c[d].nr)));
-        }
-        const bool any = c[0].s >= 0 || c[1].s >= 0;
-        R.span[w] = make_ushort4((unsigned short)(any ? lo : 0), (unsigned short)(any ? hi : 0),
-                                 (unsigned short)(x >= 0 ? x : 0xffff), (unsigned short)(any ? 1 : 0));
+        R.span[w] = pair_span(n, c, x);
         for (int d = 0; d < 2; ++d) {
             const int sl = 2 * w + d;
             X.slot[sl] = c[d];
@@ -2320,14 +2424,15 @@ __device__ void inc_init_share(const Topo &T, const State &S, const Search &X, c
             int k = 0;
             if (c[d].s >= 0) {
                 int2 seg[kIncMaxSeg];
-                const int ns = full_segments(c[d], Lc.rank, seg);
+                const int ns = full_segments(c[d], S.sn_rank, seg);
                 for (int i = 0; i < ns; ++i) k += seg[i].y - seg[i].x;
             }
             pcnt[2 * w + d] = k;
             mine += k;
         }
     }
-    if (tid == 0) { s_first = 2 * n; s_ne = 0; }
+    if (tid == 0) { s_first = 2 * n; s_app = 0ull; }
+    clear_sums<NT>(E);
     int tot = 0;
     const int base = block_excl_scan<NT>(mine, &tot, sscan);
     // this CTA's share of the positions: [q0, q1)
@@ -2345,7 +2450,7 @@ __device__ void inc_init_share(const Topo &T, const State &S, const Search &X, c
     // the entries: one per candidate that meets the share, its segments cut to
     // the share, at [first slot + b, ...) (the CTAs' ranges do not overlap)
     {
-        const int e0 = s_first + b;
+        Lc.wgl = I.work + (s_first + b);
         int off = base;
         for (int sl = 2 * p0; sl < 2 * p1; ++sl) {
             const int k = pcnt[sl];
@@ -2354,7 +2459,7 @@ __device__ void inc_init_share(const Topo &T, const State &S, const Search &X, c
                 slot_geometry(T, S, V, n, sl >> 1, c[0], c[1]);
                 const Cand &cc = c[sl & 1];
                 int2 seg[kIncMaxSeg], cut[kIncMaxSeg];
-                const int ns = full_segments(cc, Lc.rank, seg);
+                const int ns = full_segments(cc, S.sn_rank, seg);
                 const int lo = max(q0 - off, 0), hi = min(q1 - off, k);    // the share, in the candidate's positions
                 int nc = 0, at = 0;
                 for (int i = 0; i < ns; ++i) {
@@ -2363,15 +2468,16 @@ __device__ void inc_init_share(const Topo &T, const State &S, const Search &X, c
                     if (a < z) cut[nc++] = make_int2(seg[i].x + (a - at), seg[i].x + (z - at));
                     at += len;
                 }
-                write_entry(Lc.ent(e0 + atomicAdd(&s_ne, 1)), sl, 1, nc, cut, cc);
+                const unsigned long long o = append(&s_app, nc, cut);
+                write_entry(Lc.ent((int)(unsigned)o), sl, 1, (int)(o >> 32), nc, cut, cc);
             }
             off += k;
         }
     }
     __syncthreads();
-    if (s_ne == 0) return;
-    const long long terms = run_entries<NT, PREC>(T, S, X, I, n, L, G, margin, mlo, mhi, s_first + b, s_first + b + s_ne,
-                                                  kInitPart, list, list, -1, O, E, sscan, R, Lc);
+    if (s_app == 0ull) return;
+    const long long terms = run_entries<NT, PREC>(T, S, I, n, L, G, margin, mlo, mhi, (int)(unsigned)s_app,
+                                                  (int)(s_app >> 32), kInitPart, list, list, -1, O, E, R, Lc);
     if (C->profile) {                           // (phase-node, scenario) items
         unsigned long long tt = (unsigned long long)terms;
         for (int o = 16; o > 0; o >>= 1) tt += __shfl_xor_sync(0xffffffffu, tt, o);
@@ -2384,9 +2490,10 @@ __global__ void __launch_bounds__(NT) k_inc_init(Topo T, State S, Search X, Inc 
     extern __shared__ __align__(16) unsigned char init_dyn[];
     __shared__ __align__(16) EvalSmem E;
     __shared__ int sscan[33];
-    __shared__ int s_first, s_ne;
+    __shared__ int s_first;
+    __shared__ unsigned long long s_app;
     if (X.setup_err && *X.setup_err != 0) return;
-    inc_init_share<NT, PREC>(T, S, X, I, C, blockIdx.x, gridDim.x, init_dyn, E, sscan, s_first, s_ne);
+    inc_init_share<NT, PREC>(T, S, X, I, C, blockIdx.x, gridDim.x, init_dyn, E, sscan, s_first, s_app);
 }
 
 // The same for many feeders: cta_off[i] = the first CTA of the i-th feeder of
@@ -2400,7 +2507,8 @@ __global__ void __launch_bounds__(NT) k_inc_init_batch(const BatchFeeder *fd, co
     extern __shared__ __align__(16) unsigned char init_dyn[];
     __shared__ __align__(16) EvalSmem E;
     __shared__ int sscan[33];
-    __shared__ int s_first, s_ne;
+    __shared__ int s_first;
+    __shared__ unsigned long long s_app;
     __shared__ Topo sT;
     __shared__ State sS;
     __shared__ Search sX;
@@ -2426,7 +2534,7 @@ __global__ void __launch_bounds__(NT) k_inc_init_batch(const BatchFeeder *fd, co
     __syncthreads();
     const int f = s_f;
     if (*fd[f].setup_err != 0 || s_b >= s_B) return;
-    inc_init_share<NT, PREC>(sT, sS, sX, sI, fd[f].C, s_b, s_B, init_dyn, E, sscan, s_first, s_ne);
+    inc_init_share<NT, PREC>(sT, sS, sX, sI, fd[f].C, s_b, s_B, init_dyn, E, sscan, s_first, s_app);
 }
 
 // The carried sums, violation counts and their bounds of every feeder of the
@@ -2474,7 +2582,7 @@ __global__ void __launch_bounds__(NT) k_search_inc_batch(const BatchFeeder *fd, 
 
 constexpr size_t kIncSmemMax = 200 * 1024;  // largest dynamic shared memory of one search
 constexpr int kInitThreads = 384;           // CTAs of the first evaluation
-constexpr int kClusterMin64 = 200, kClusterMin32 = 1500;    // buses from which a cluster searches (inc_plan)
+constexpr int kClusterMin = 32;             // buses from which a cluster searches (inc_plan)
 
 template <typename K>
 cudaError_t set_smem(K kern, size_t bytes) {
@@ -2511,23 +2619,27 @@ bool inc_smem(int n, bool maxm, const IncShape &sh, int *rec_mode, size_t *bytes
 
 // One CTA or a cluster of kMaxCluster.  A cluster shares out the scan over the
 // slot pairs, the FP64 evaluation of the merge, the changed terms and the
-// records (which then always fit shared memory), and pays three cluster
-// barriers a merge (about 0.5 us each with stores in flight) and L2 in place of
-// L1 latency.  Search ms, one CTA of 384 threads / eight of 256:
-//   FP64 terms:  40 buses 0.56 / 0.64, 333 buses (3 scenarios) 5.7 / 4.1, 1,000 9.7 / 8.0, 3,100 59.7 / 41.0
-//   FP32 terms: 333 buses 4.11 / 4.08, 1,000 6.77 / 6.99, 2,200 32.0 / 29.0, 3,100 44.1 / 35.2
-// (two and four CTAs lie between the two).  A forced record placement asks for
-// one CTA's memory, and recorded iterations are compacted by one CTA.
-bool inc_plan(int n, int precision, const IncShape &raw, bool records_iters, IncPlan *out) {
+// records (which then always fit shared memory, the carried sums and candidates
+// up to about 4,200 buses), and pays three cluster barriers a merge and L2 in
+// place of L1 latency.  Search ms, one CTA of 384 threads / eight of 256:
+//   FP64 terms:  40 buses 0.50 / 0.47, 101 1.21 / 1.12, 333 (3 scenarios) 5.4 / 3.2, 1,000 9.5 / 6.0, 3,100 59.2 / 33.0
+//   FP32 terms:  40 buses 0.54 / 0.54, 101 1.32 / 1.31, 333 (3 scenarios) 3.8 / 2.9, 1,000 6.7 / 4.9, 3,100 44.9 / 27.4
+// A forced record placement asks for one CTA's memory, and recorded iterations
+// are compacted by one CTA.
+bool inc_plan(int n, const IncShape &raw, bool records_iters, IncPlan *out) {
     out->sh = inc_shape_resolve(raw);
     out->cs = 1;
     if (!inc_smem(n, true, out->sh, &out->rec, &out->bytes)) return false;
-    if (out->sh.rec >= 0 || records_iters || n < (precision == 0 ? kClusterMin64 : kClusterMin32)) return true;
-    const size_t b = base_bytes(n, out->sh.se, kMaxCluster) + rec_maxm_bytes(own_pairs(n, 0, kMaxCluster));
+    out->mode = out->rec;
+    if (out->sh.rec >= 0 || records_iters || n < kClusterMin) return true;
+    const int np = own_pairs(n, 0, kMaxCluster);
+    const size_t b = base_bytes(n, out->sh.se, kMaxCluster) + align16(rec_maxm_bytes(np));
     if (b > kIncSmemMax) return true;
     out->cs = kMaxCluster;
-    out->bytes = b;
-    // fewer warps meet at the cluster's barriers (384 threads: 1,000 buses FP64 8.26 ms, 3,100 FP32 36.9)
+    const bool own = b + sums_bytes(np) <= kIncSmemMax;
+    out->mode = own ? 2 + 4 : 2;
+    out->bytes = own ? b + sums_bytes(np) : b;
+    // fewer warps meet at the cluster's barriers (384 threads: 1,000 buses 5.2 ms, 3,100 buses 26.6 ms)
     if (raw.threads == 0) {
         IncShape sh = raw;
         sh.threads = 256;
@@ -2570,7 +2682,7 @@ cudaError_t launch_one(Topo T, State S, Search X, Inc I, Ctrl *C, int verify, co
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k_search_inc<NT, PREC>, T, S, X, I, C, verify,
-                              pl.cs > 1 ? 2 : pl.rec, pl.sh.se, pl.sh.cw, pl.cs);
+                              pl.mode, pl.sh.se, pl.sh.cw, pl.cs);
 }
 
 template <int NT>

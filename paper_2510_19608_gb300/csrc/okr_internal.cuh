@@ -154,13 +154,14 @@ struct GridBar {
 constexpr int kIncMaxSeg = 7;
 // Doubles per scenario of one position's scratch in Inc::cbuf: 10 FP64 values
 // (voltage x, y and magnitude per phase, the MICE), then 8 doubles' room for
-// their FP32 copies (a 16-byte (v.x, v.y, hr, lr) per phase, the MICE).
+// their FP32 copies (a 16-byte (v.x, v.y, hr, lr) per phase, the MICE) and the
+// position's super-node.
 constexpr int kIncCbStride = 18;
 struct IncWork {
     int slot;           // candidate slot 2 w + d (w = the lower super-node of the quotient edge)
     int mode;           // 0: terms of changed clusters, ranks before the merge; 1: every term, ranks after
     int nseg;
-    int pad;
+    int off;            // items of the entries before it
     int2 seg[kIncMaxSeg];   // rank ranges [x, y)
     int s, r, a, js, ns, jr, nr, fixed;     // the candidate's geometry (as in Cand)
 };
@@ -172,10 +173,8 @@ struct Inc {
     int *viol;                  // [2n] precision 0: terms above the margin; precision 1: terms surely
                                 //      above it; kIncDead: no candidate in the slot
     int *vmay;                  // [2n] precision 1: terms not surely within the margin
-    int *qpar;                  // [n] super-node holding the parent of the cluster's top (-1: slack's cluster)
-    int *fpair;                 // [n] slot pairs whose candidates are rebuilt after the merge
     IncWork *work;              // [2n] work entries of one iteration
-    double *cbuf;               // [n * kIncCbStride L] the merge's new values per position (okr_incr.cu)
+    double *cbuf;               // [2][n * kIncCbStride L] a merge's new values per position (okr_incr.cu), by merge parity
     unsigned long long *vacc;   // [2n][2] FP64 rescoring (precision-1 recheck, verification)
     int *vviol;                 // [2n]
     int *rlist;                 // [2n] slots rescored in FP64 in one iteration

@@ -176,15 +176,16 @@ IncShape inc_shape_resolve(IncShape sh);
 bool inc_smem(int n, bool maxm, const IncShape &sh, int *rec_mode, size_t *bytes);
 // How one feeder is searched: the shape of each CTA, the CTAs (one, or a
 // cluster that shares the feeder), the record placement of one CTA (a cluster
-// keeps its records in its CTAs' shared memory) and the dynamic shared memory.
+// keeps its records in its CTAs' shared memory; mode: what the kernel is told)
+// and the dynamic shared memory.
 struct IncPlan {
     IncShape sh;
-    int cs, rec;
+    int cs, rec, mode;
     size_t bytes;
 };
 // The plan of an n-bus search under the given (unresolved) shape; false when
 // the shape's forced record placement does not fit.
-bool inc_plan(int n, int precision, const IncShape &raw, bool records_iters, IncPlan *out);
+bool inc_plan(int n, const IncShape &raw, bool records_iters, IncPlan *out);
 cudaError_t launch_search_inc(int precision, Topo T, State S, Search X, Inc I, Ctrl *C, int verify, const IncPlan &pl,
                               cudaStream_t st);
 // Many feeders: one CTA each, in the order given (prepare_search_inc_batch with

@@ -174,10 +174,8 @@ inline void layout_feeder(Carver &c, int n, int L, int rec, int grid, long long 
     c.take(I.rlist, 2 * N);
     c.take(I.recbuf, 48 * N + 64);
     c.take(I.maxm, N);
-    c.take(I.qpar, N);
-    c.take(I.fpair, N);
     c.take(I.work, 2 * N + kIncInitCtasMax);      // (+ the first evaluation's candidates cut between CTAs)
-    c.take(I.cbuf, N * (size_t)kIncCbStride * L);
+    c.take(I.cbuf, 2 * N * (size_t)kIncCbStride * L);
     c.take(I.vacc, 4 * N);
     c.take(I.vviol, 2 * N);
     if (chunks > 0) {

@@ -23,7 +23,7 @@ def ctx():
 
 
 @pytest.mark.parametrize("precision", [0, 1])
-@pytest.mark.parametrize("n,scen,target", [(9, 2, 1.0), (41, 1, 1.0), (199, 2, 0.9), (200, 3, 0.9), (257, 4, 0.8),
+@pytest.mark.parametrize("n,scen,target", [(9, 2, 1.0), (31, 1, 1.0), (32, 2, 1.0), (41, 1, 1.0), (199, 2, 0.9), (200, 3, 0.9), (257, 4, 0.8),
                                            (1025, 1, 0.3), (1499, 2, 0.1), (1500, 2, 0.2), (2100, 4, 0.04)])
 def test_cluster_and_one_cta_give_the_same_run(ctx, n, scen, target, precision):
     import paper_2510_19608_gb300 as K
