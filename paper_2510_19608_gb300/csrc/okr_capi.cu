@@ -78,10 +78,11 @@ struct okr_ctx {
     // learned scorer
     MlpBufs mb;
     MlpWork mw;
-    std::vector<void *> mlp_allocs, mlp_work_allocs, mlp_data_allocs;
+    std::vector<void *> mlp_allocs, mlp_work_allocs;
     float *mlp_x = nullptr, *mlp_t = nullptr;    // device copies of a data set
+    float *mlp_loss = nullptr;                   // squared errors by segment of an epoch's batches
     int *mlp_err = nullptr;                      // error flag of the tensor-core inference
-    long long mlp_data_cap = 0;
+    size_t mlp_x_cap = 0, mlp_t_cap = 0, mlp_loss_cap = 0;      // floats
     int mlp_step = 0;
 
     // device allocator (cudaMalloc / cudaFree unless the caller registered one)
@@ -173,11 +174,13 @@ void free_list(okr_ctx *ctx, std::vector<void *> &v) {
 void free_mlp(okr_ctx *ctx) {
     free_list(ctx, ctx->mlp_allocs);
     free_list(ctx, ctx->mlp_work_allocs);
-    free_list(ctx, ctx->mlp_data_allocs);
+    dev_free(ctx, ctx->mlp_x);
+    dev_free(ctx, ctx->mlp_t);
+    dev_free(ctx, ctx->mlp_loss);
     ctx->mb = MlpBufs{};
     ctx->mw = MlpWork{};
-    ctx->mlp_data_cap = 0;
-    ctx->mlp_x = ctx->mlp_t = nullptr;
+    ctx->mlp_x_cap = ctx->mlp_t_cap = ctx->mlp_loss_cap = 0;
+    ctx->mlp_x = ctx->mlp_t = ctx->mlp_loss = nullptr;
     dev_free(ctx, ctx->mlp_err);
     ctx->mlp_err = nullptr;
 }
@@ -2002,34 +2005,29 @@ okr_status mlp_ensure_work(okr_ctx *ctx, int N) {
     CK(grab(ctx, ctx->mlp_work_allocs, &w.d3, NH));
     CK(grab(ctx, ctx->mlp_work_allocs, &w.y, (size_t)N));
     CK(grab(ctx, ctx->mlp_work_allocs, &w.dy, (size_t)N));
-    CK(grab(ctx, ctx->mlp_work_allocs, &w.part, (size_t)mlp_segments(N) * (kMlpHidden + 1) * kMlpHidden));
+    CK(grab(ctx, ctx->mlp_work_allocs, &w.part, (size_t)mlp_segments(N) * mlp_param_count(kMlpMaxF)));
     w.cap = N;
+    return OKR_OK;
+}
+
+// A device buffer of at least `count` floats, kept with the context.
+okr_status mlp_buffer(okr_ctx *ctx, float **p, size_t *cap, size_t count) {
+    if (count <= *cap) return OKR_OK;
+    dev_free(ctx, *p);
+    *p = nullptr;
+    *cap = 0;
+    CK(dev_alloc(ctx, (void **)p, sizeof(float) * count));
+    *cap = count;
     return OKR_OK;
 }
 
 okr_status mlp_upload(okr_ctx *ctx, const float *x, const float *t, long long N) {
     const int F = ctx->mb.F;
-    if (N > ctx->mlp_data_cap) {
-        free_list(ctx, ctx->mlp_data_allocs);
-        ctx->mlp_data_cap = 0;
-        CK(grab(ctx, ctx->mlp_data_allocs, &ctx->mlp_x, (size_t)N * F));
-        CK(grab(ctx, ctx->mlp_data_allocs, &ctx->mlp_t, (size_t)N));
-        ctx->mlp_data_cap = N;
-    }
+    okr_status s = mlp_buffer(ctx, &ctx->mlp_x, &ctx->mlp_x_cap, (size_t)N * F);
+    if (s == OKR_OK) s = mlp_buffer(ctx, &ctx->mlp_t, &ctx->mlp_t_cap, (size_t)N);
+    if (s != OKR_OK) return s;
     CK(cudaMemcpyAsync(ctx->mlp_x, x, sizeof(float) * (size_t)N * F, cudaMemcpyHostToDevice, ctx->stream));
     if (t) CK(cudaMemcpyAsync(ctx->mlp_t, t, sizeof(float) * (size_t)N, cudaMemcpyHostToDevice, ctx->stream));
-    return OKR_OK;
-}
-
-okr_status mlp_batch_loss(okr_ctx *ctx, const float *y, const float *t, int N, double *sum) {
-    const int nseg = mlp_segments(N);
-    CK(mlp_sqerr(y, t, N, ctx->mw.part, ctx->stream));
-    std::vector<float> part(nseg);
-    CK(cudaMemcpyAsync(part.data(), ctx->mw.part, sizeof(float) * nseg, cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    double acc = 0.0;
-    for (float v : part) acc += v;
-    *sum = acc;
     return OKR_OK;
 }
 
@@ -2041,18 +2039,23 @@ okr_status okr_scorer_init(okr_ctx *ctx, int32_t n_features, const float *theta)
     if (!ctx) return OKR_EINVAL;
     if (n_features < 1 || n_features > kMlpMaxF) return fail(ctx, OKR_EINVAL, "n_features %d outside [1, %d]", n_features, kMlpMaxF);
     CK(cudaSetDevice(ctx->device));
-    free_mlp(ctx);
     MlpBufs &b = ctx->mb;
-    b.F = n_features;
     const int P = mlp_param_count(n_features);
-    CK(grab(ctx, ctx->mlp_allocs, &b.theta, (size_t)P));
-    CK(grab(ctx, ctx->mlp_allocs, &b.grad, (size_t)P));
-    CK(grab(ctx, ctx->mlp_allocs, &b.m, (size_t)P));
-    CK(grab(ctx, ctx->mlp_allocs, &b.v, (size_t)P));
-    CK(grab(ctx, ctx->mlp_allocs, &b.w1, (size_t)kMlpMaxF * kMlpHidden));
-    CK(grab(ctx, ctx->mlp_allocs, &b.w2, (size_t)kMlpHidden * kMlpHidden));
-    CK(grab(ctx, ctx->mlp_allocs, &b.w3, (size_t)kMlpHidden * kMlpHidden));
-    CK(grab(ctx, ctx->mlp_allocs, &b.w4, (size_t)kMlpHidden));
+    if (!b.theta) {                             // sized for the longest feature vector, kept with the context
+        const size_t Pm = mlp_param_count(kMlpMaxF);
+        free_list(ctx, ctx->mlp_allocs);        // (what a failed call left)
+        float *theta_d = nullptr;
+        CK(grab(ctx, ctx->mlp_allocs, &theta_d, Pm));
+        CK(grab(ctx, ctx->mlp_allocs, &b.grad, Pm));
+        CK(grab(ctx, ctx->mlp_allocs, &b.m, Pm));
+        CK(grab(ctx, ctx->mlp_allocs, &b.v, Pm));
+        CK(grab(ctx, ctx->mlp_allocs, &b.w1, (size_t)kMlpMaxF * kMlpHidden));
+        CK(grab(ctx, ctx->mlp_allocs, &b.w2, (size_t)kMlpHidden * kMlpHidden));
+        CK(grab(ctx, ctx->mlp_allocs, &b.w3, (size_t)kMlpHidden * kMlpHidden));
+        CK(grab(ctx, ctx->mlp_allocs, &b.w4, (size_t)kMlpHidden));
+        b.theta = theta_d;
+    }
+    b.F = n_features;
     cudaStream_t st = ctx->stream;
     if (theta) CK(cudaMemcpyAsync(b.theta, theta, sizeof(float) * P, cudaMemcpyHostToDevice, st));
     else CK(cudaMemsetAsync(b.theta, 0, sizeof(float) * P, st));
@@ -2080,11 +2083,14 @@ okr_status okr_scorer_gradient(okr_ctx *ctx, const float *x, const float *t, int
     CK(cudaSetDevice(ctx->device));
     okr_status s = mlp_ensure_work(ctx, n);
     if (s == OKR_OK) s = mlp_upload(ctx, x, t, n);
+    if (s == OKR_OK) s = mlp_buffer(ctx, &ctx->mlp_loss, &ctx->mlp_loss_cap, (size_t)mlp_segments(n));
     if (s != OKR_OK) return s;
-    CK(mlp_gradient(ctx->mb, ctx->mw, ctx->mlp_x, ctx->mlp_t, n, ctx->num_sms, ctx->stream));
+    CK(mlp_gradient(ctx->mb, ctx->mw, ctx->mlp_x, ctx->mlp_t, n, ctx->mlp_loss, 0.0f, 0, ctx->num_sms, ctx->stream));
+    std::vector<float> part(mlp_segments(n));
+    CK(cudaMemcpyAsync(part.data(), ctx->mlp_loss, sizeof(float) * part.size(), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
     double sum = 0.0;
-    s = mlp_batch_loss(ctx, ctx->mw.y, ctx->mlp_t, n, &sum);
-    if (s != OKR_OK) return s;
+    for (float v : part) sum += v;
     if (loss) *loss = sum / n;
     const int P = mlp_param_count(ctx->mb.F);
     if (grad) CK(cudaMemcpy(grad, ctx->mb.grad, sizeof(float) * P, cudaMemcpyDeviceToHost));
@@ -2099,20 +2105,32 @@ okr_status okr_scorer_train(okr_ctx *ctx, const float *x, const float *t, int64_
     const int B = (int)std::min<int64_t>(batch, n);
     okr_status s = mlp_ensure_work(ctx, B);
     if (s == OKR_OK) s = mlp_upload(ctx, x, t, n);
+    if (s == OKR_OK)
+        s = mlp_buffer(ctx, &ctx->mlp_loss, &ctx->mlp_loss_cap, (size_t)(n / B) * mlp_segments(B) + mlp_segments((int)(n % B)));
     if (s != OKR_OK) return s;
     const int F = ctx->mb.F;
+    // the host waits once an epoch, for the squared errors of all its batches
+    std::vector<float> part;
+    std::vector<int> segs;
     for (int e = 0; e < epochs; ++e) {
-        double sum = 0.0;
+        segs.clear();
+        size_t at = 0;
         for (int64_t b0 = 0; b0 < n; b0 += B) {
             const int nb = (int)std::min<int64_t>(B, n - b0);
-            const float *xb = ctx->mlp_x + (size_t)b0 * F;
-            const float *tb = ctx->mlp_t + b0;
-            CK(mlp_gradient(ctx->mb, ctx->mw, xb, tb, nb, ctx->num_sms, ctx->stream));
+            CK(mlp_gradient(ctx->mb, ctx->mw, ctx->mlp_x + (size_t)b0 * F, ctx->mlp_t + b0, nb, ctx->mlp_loss + at, lr,
+                            ++ctx->mlp_step, ctx->num_sms, ctx->stream));
+            segs.push_back(mlp_segments(nb));
+            at += segs.back();
+        }
+        part.resize(at);
+        CK(cudaMemcpyAsync(part.data(), ctx->mlp_loss, sizeof(float) * at, cudaMemcpyDeviceToHost, ctx->stream));
+        CK(cudaStreamSynchronize(ctx->stream));
+        double sum = 0.0;
+        at = 0;
+        for (int k : segs) {
             double bs = 0.0;
-            s = mlp_batch_loss(ctx, ctx->mw.y, tb, nb, &bs);
-            if (s != OKR_OK) return s;
+            for (int i = 0; i < k; ++i) bs += part[at++];
             sum += bs;
-            CK(mlp_adam(ctx->mb, lr, ++ctx->mlp_step, ctx->stream));
         }
         if (epoch_loss) epoch_loss[e] = sum / (double)n;
     }
@@ -2150,7 +2168,7 @@ okr_status okr_scorer_predict(okr_ctx *ctx, const float *x, int64_t n, float *y)
     okr_status s = mlp_upload(ctx, x, nullptr, n);
     if (s != OKR_OK) return s;
     float *yd = ctx->mlp_t;                     // the targets' buffer holds the predictions
-    CK(mlp_forward(ctx->mb, ctx->mlp_x, (int)n, nullptr, nullptr, nullptr, yd, ctx->num_sms, ctx->stream));
+    CK(mlp_forward(ctx->mb, ctx->mlp_x, (int)n, yd, ctx->num_sms, ctx->stream));
     CK(cudaMemcpyAsync(y, yd, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     return OKR_OK;

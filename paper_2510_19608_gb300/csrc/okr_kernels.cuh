@@ -101,17 +101,15 @@ struct MlpWork {
     int cap = 0;                    // samples the buffers hold
     float *h1 = nullptr, *h2 = nullptr, *h3 = nullptr, *d1 = nullptr, *d2 = nullptr, *d3 = nullptr;  // [cap][H]
     float *y = nullptr, *dy = nullptr;                                   // [cap]
-    float *part = nullptr;                                               // [segments][(H+1) x H]
+    float *part = nullptr;                                               // [segments][parameters]
 };
 int mlp_param_count(int F);
 int mlp_segments(int N);
 cudaError_t mlp_sync_bf16(const MlpBufs &b, cudaStream_t st);
-cudaError_t mlp_forward(const MlpBufs &b, const float *x, int N, float *h1, float *h2, float *h3, float *y, int num_sms,
-                        cudaStream_t st);
-cudaError_t mlp_gradient(const MlpBufs &b, const MlpWork &w, const float *x, const float *t, int N, int num_sms,
-                         cudaStream_t st);
-cudaError_t mlp_adam(const MlpBufs &b, float lr, int step, cudaStream_t st);
-cudaError_t mlp_sqerr(const float *y, const float *t, int N, float *part, cudaStream_t st);
+cudaError_t mlp_forward(const MlpBufs &b, const float *x, int N, float *y, int num_sms, cudaStream_t st);
+// Gradient and squared errors (loss[mlp_segments(N)]) of N samples; lr > 0: then Adam step `step`.
+cudaError_t mlp_gradient(const MlpBufs &b, const MlpWork &w, const float *x, const float *t, int N, float *loss, float lr,
+                         int step, int num_sms, cudaStream_t st);
 // okr_mlp_tc.cu: inference on the tensor cores (bfloat16 operands, FP32
 // accumulators in tensor memory); *err (device) is set to 1 when a wait gave up.
 cudaError_t mlp_forward_tc(const MlpBufs &b, const float *x, int N, float *y, int *err, int num_sms, cudaStream_t st);
