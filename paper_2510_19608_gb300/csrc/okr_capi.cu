@@ -44,10 +44,11 @@ struct okr_ctx {
     int cap_chunks = 0;
     int sum_sz = 0, max_depth = 0;      // of the current feeder
     Ctrl *C_host = nullptr;             // pinned
-    // the setup steps the load flow does not need (LCA table, path impedances)
-    // run on a second stream beside it; ev_side marks their end
+    // the setup steps the load flow does not need (line inverses, path
+    // impedances, LCA table) run on a second stream beside it; ev_inv and ev_side
+    // mark the end of the first and of all
     cudaStream_t side = nullptr;
-    cudaEvent_t ev_topo = nullptr, ev_lines = nullptr, ev_side = nullptr;
+    cudaEvent_t ev_topo = nullptr, ev_lines = nullptr, ev_inv = nullptr, ev_side = nullptr;
     bool side_pending = false;          // the stream has not waited for ev_side yet
 
     // counters of the last call
@@ -333,20 +334,22 @@ okr_status build_topology(okr_ctx *ctx, int n, int L, const double *vslack, bool
     // the later setup kernels index with the renumbering: stop here on an invalid tree
     okr_status s = read_setup_errors(ctx);
     if (s != OKR_OK) return s;
-    // the LCA table and the path impedances (on the side stream) are not read
-    // by the load flow: they run beside it, and the stream waits for them
-    // before the search (join_side)
+    // the line inverses, the path impedances and the LCA table (on the side
+    // stream) are not read by the load flow: they run beside it; the stream waits
+    // for the inverses before the injections, and for the rest before the search
+    // (join_side)
     cudaStream_t sd = ctx->side;
     CK(cudaEventRecord(ctx->ev_topo, st));
     CK(cudaStreamWaitEvent(sd, ctx->ev_topo, 0));
-    k_child_offsets<<<1, 1024, 0, st>>>(n, T, ctx->fb.coff_c, ctx->fb.child_c);
+    CK(launch_children_lines(n, T, ctx->fb.coff_c, ctx->fb.child_c, ctx->fb.z_in, ctx->num_sms, st));
+    CK(cudaEventRecord(ctx->ev_lines, st));
     const int LOG = log2_ceil(n) + 1;
     k_rmq_all<<<1, 1024, 0, sd>>>(n, LOG, T.depth, ctx->fb.rmq);
-    k_lca_fill<<<blocks_for((size_t)n * n, 256, ctx->num_sms * 8), 256, 0, sd>>>(n, T.parent, T.sz, T.depth, ctx->fb.rmq, T.lca);
-    CK(launch_line_inverses(n, T, ctx->fb.z_in, ctx->fb.err_dev, ctx->num_sms, st));
-    CK(cudaEventRecord(ctx->ev_lines, st));
     CK(cudaStreamWaitEvent(sd, ctx->ev_lines, 0));
+    CK(launch_line_inverses(n, T, ctx->fb.err_dev, ctx->num_sms, sd));
+    CK(cudaEventRecord(ctx->ev_inv, sd));
     CK(launch_path_impedance(n, T, sd));
+    k_lca_fill<<<blocks_for((size_t)n * n, 256, ctx->num_sms * 8), 256, 0, sd>>>(n, T.parent, T.sz, T.depth, ctx->fb.rmq, T.lca);
     CK(cudaEventRecord(ctx->ev_side, sd));
     ctx->side_pending = true;
     ctx->launches += 5;
@@ -384,15 +387,28 @@ okr_status setup_status(okr_ctx *ctx, int e) {
     return OKR_OK;
 }
 
+// The end of a setup built with check_lines = false: waits for all of it (the
+// side stream's part too) and reads its error flag and the load flow's sweeps.
+okr_status finish_setup(okr_ctx *ctx, int L) {
+    CK(join_side(ctx));
+    CK(cudaMemcpyAsync(host_pf_iters(ctx), ctx->fb.pf_iters, sizeof(int) * L, cudaMemcpyDeviceToHost, ctx->stream));
+    const okr_status s = read_setup_errors(ctx);
+    if (*host_err(ctx) == 2) ctx->have_topo = false;
+    return s;
+}
+
 // max_spins: polls per grid barrier of the load flow (params.max_spins; 0 = default).
 okr_status run_power_flow(okr_ctx *ctx, int n, int L, long long max_spins = 0) {
     cudaStream_t st = ctx->stream;
     Topo &T = ctx->fb.T;
-    // the load flow's work buffers alias T.ihat and T.amag, which the next two kernels fill
+    // the load flow's work buffers alias T.ihat and T.amag, which the next two
+    // kernels fill (a given limit on the barriers' polls asks for the barriers)
     CK(launch_power_flow(n, L, T, ctx->fb.s_in, kPfTol, kPfMaxIter, ctx->fb.J, T.ihat, T.amag, ctx->fb.pf_iters,
-                         ctx->fb.err_dev, ctx->num_sms, st, max_spins > 0 ? max_spins : kDefaultSpins));
-    k_line_currents<<<blocks_for((size_t)L * n, 256, ctx->num_sms * 8), 256, 0, st>>>(n, L, T, ctx->fb.J);
-    k_injections<<<blocks_for((size_t)L * n, 256, ctx->num_sms * 8), 256, 0, st>>>(n, L, T, ctx->fb.J);
+                         ctx->fb.err_dev, ctx->num_sms, st, max_spins > 0 ? max_spins : kDefaultSpins, max_spins <= 0));
+    CK(cudaStreamWaitEvent(st, ctx->ev_inv, 0));
+    const int blocks = blocks_for((size_t)3 * L * n, 64, ctx->num_sms * 16);
+    k_line_currents<<<blocks, 64, 0, st>>>(n, L, T, ctx->fb.J);
+    k_injections<<<blocks, 64, 0, st>>>(n, L, T, ctx->fb.J);
     ctx->launches += 3;
     CK(cudaGetLastError());
     return OKR_OK;
@@ -445,7 +461,7 @@ okr_status run_search(okr_ctx *ctx, const okr_params *p) {
         X.mlp_w3 = reinterpret_cast<const uint16_t *>(ctx->mb.w3);
         X.mlp_w4 = reinterpret_cast<const uint16_t *>(ctx->mb.w4);
     }
-    k_state_init<<<blocks_for((size_t)L * n, 256, ctx->num_sms * 8), 256, 0, st>>>(n, L, ctx->fb.T, ctx->fb.S);
+    k_state_init<<<blocks_for((size_t)3 * L * n, 64, ctx->num_sms * 16), 64, 0, st>>>(n, L, ctx->fb.T, ctx->fb.S);
     ctx->launches += 1;
     CK(cudaGetLastError());
     const int mm = merges_for(n, p);
@@ -537,7 +553,7 @@ okr_status run_search_inc(okr_ctx *ctx, const okr_params *p) {
     X.rec_iters = p->record_iters;
     X.topk = 0;
     X.prune_exact = 0;
-    k_state_init<<<blocks_for((size_t)L * n, 256, ctx->num_sms * 8), 256, 0, st>>>(n, L, ctx->fb.T, ctx->fb.S);
+    k_state_init<<<blocks_for((size_t)3 * L * n, 64, ctx->num_sms * 16), 64, 0, st>>>(n, L, ctx->fb.T, ctx->fb.S);
     ctx->launches += 1;
     CK(cudaGetLastError());
     const int mm = merges_for(n, p);
@@ -802,6 +818,7 @@ okr_status okr_create(okr_ctx **out, int device, void *stream) {
     if (cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->ev_topo, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->ev_lines, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->ev_inv, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->ev_side, cudaEventDisableTiming) != cudaSuccess) {
         okr_destroy(ctx);
         return OKR_ECUDA;
@@ -835,7 +852,7 @@ okr_status okr_destroy(okr_ctx *ctx) {
         cudaStreamSynchronize(ctx->side);
         cudaStreamDestroy(ctx->side);
     }
-    for (cudaEvent_t ev : {ctx->ev_topo, ctx->ev_lines, ctx->ev_side})
+    for (cudaEvent_t ev : {ctx->ev_topo, ctx->ev_lines, ctx->ev_inv, ctx->ev_side})
         if (ev) cudaEventDestroy(ev);
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
     delete ctx;
@@ -871,14 +888,14 @@ okr_status okr_power_flow(okr_ctx *ctx, const okr_feeder *f, double *vhat_out, d
     CK(cudaMemcpyAsync(ctx->fb.ph_in, f->phases, n, cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(ctx->fb.z_in, f->z_line, sizeof(double) * 18 * n, cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(ctx->fb.s_in, f->s_load, sizeof(double) * 6 * L * n, cudaMemcpyHostToDevice, st));
-    s = build_topology(ctx, n, L, &f->v_slack[0][0]);
+    s = build_topology(ctx, n, L, &f->v_slack[0][0], false);
     if (s != OKR_OK) return s;
     s = run_power_flow(ctx, n, L);
     if (s != OKR_OK) return s;
-    s = read_setup_errors(ctx);
+    s = finish_setup(ctx, L);
     if (s != OKR_OK) return s;
     // export: reuse k_export with the initial state (each bus its own super-node)
-    k_state_init<<<blocks_for((size_t)L * n, 256, ctx->num_sms * 8), 256, 0, st>>>(n, L, ctx->fb.T, ctx->fb.S);
+    k_state_init<<<blocks_for((size_t)3 * L * n, 64, ctx->num_sms * 16), 64, 0, st>>>(n, L, ctx->fb.T, ctx->fb.S);
     k_export<<<blocks_for((size_t)L * n, 256, ctx->num_sms * 8), 256, 0, st>>>(ctx->fb.T, ctx->fb.S, nullptr, nullptr,
                                                                                 ctx->fb.vhat_out);
     CK(cudaGetLastError());
@@ -893,10 +910,8 @@ okr_status okr_power_flow(okr_ctx *ctx, const okr_feeder *f, double *vhat_out, d
     }
     CK(cudaStreamSynchronize(st));
     if (sweeps) {
-        int it[kMaxScen];
-        CK(cudaMemcpy(it, ctx->fb.pf_iters, sizeof(int) * L, cudaMemcpyDeviceToHost));
         int w = 0;
-        for (int l = 0; l < L; ++l) w = it[l] > w ? it[l] : w;
+        for (int l = 0; l < L; ++l) w = host_pf_iters(ctx)[l] > w ? host_pf_iters(ctx)[l] : w;
         *sweeps = w;
     }
     return OKR_OK;
@@ -931,12 +946,6 @@ okr_status okr_evaluate(okr_ctx *ctx, const okr_feeder *f, const int32_t *super_
     CK(cudaMemcpyAsync(B.ph_in, f->phases, n, cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(B.z_in, f->z_line, sizeof(double) * 18 * n, cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(B.s_in, f->s_load, sizeof(double) * 6 * L * n, cudaMemcpyHostToDevice, st));
-    s = build_topology(ctx, n, L, &f->v_slack[0][0]);
-    if (s != OKR_OK) return s;
-    s = run_power_flow(ctx, n, L);
-    if (s != OKR_OK) return s;
-    s = read_setup_errors(ctx);
-    if (s != OKR_OK) return s;
     // the member lists go into buffers this call does not otherwise use
     // (super_out [n], base [2n+1], dec_s [n], score [2n >= 4])
     int *sup_d = B.super_out, *moff_d = B.X.base, *mem_d = B.X.dec_s;
@@ -944,8 +953,14 @@ okr_status okr_evaluate(okr_ctx *ctx, const okr_feeder *f, const int32_t *super_
     CK(cudaMemcpyAsync(moff_d, moff.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(mem_d, mem.data(), sizeof(int) * n, cudaMemcpyHostToDevice, st));
     double *err_d = B.X.score;
-    k_eval_reduced<<<L, 1024, 0, st>>>(B.T, sup_d, moff_d, mem_d, B.J, B.S.vcur, vred ? B.vred_out : nullptr, err_d);
-    CK(cudaGetLastError());
+    s = build_topology(ctx, n, L, &f->v_slack[0][0], false);
+    if (s != OKR_OK) return s;
+    s = run_power_flow(ctx, n, L);
+    if (s != OKR_OK) return s;
+    // (a failed load flow leaves valid indices: its outcome is read after the evaluation)
+    CK(launch_eval_reduced(B.T, sup_d, moff_d, mem_d, B.J, B.S.vcur, vred ? B.vred_out : nullptr, err_d, st));
+    s = finish_setup(ctx, L);
+    if (s != OKR_OK) return s;
     CK(cudaMemcpyAsync(max_error, err_d, sizeof(double) * L, cudaMemcpyDeviceToHost, st));
     if (vred) CK(cudaMemcpyAsync(vred, B.vred_out, sizeof(double) * 6 * L * n, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -1356,6 +1371,7 @@ static okr_status batch_fill(okr_ctx *ctx, BatchRun &R, const okr_feeder *feeder
     if (!R.ev_fork) CK(cudaEventCreateWithFlags(&R.ev_fork, cudaEventDisableTiming));
     if (!R.ev_join) CK(cudaEventCreateWithFlags(&R.ev_join, cudaEventDisableTiming));
     // attributes the launches need, set before any stream capture
+    CK(prepare_batch_setup());
     for (int g = 2; g < 4; ++g) {
         int max_n = 2;
         for (int f : R.ord[g]) max_n = std::max(max_n, R.nbus[f]);

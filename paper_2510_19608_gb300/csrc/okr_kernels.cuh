@@ -11,22 +11,24 @@ namespace okr {
 __global__ void __launch_bounds__(1024) k_topology(int n, const int *__restrict__ parent_in, const uint8_t *__restrict__ ph_in,
                            Topo T, int *dep, int *anc, int *anc2, int *d2, int *size, int *ccount,
                            int *coff_c, int *child_c, int *err);
-__global__ void __launch_bounds__(1024) k_child_offsets(int n, Topo T, const int *__restrict__ coff_c, const int *__restrict__ child_c);
 __global__ void k_rmq_level(int n, int j, const int *__restrict__ depth, uint16_t *st);
 __global__ void __launch_bounds__(1024) k_rmq_all(int n, int nlev, const int *__restrict__ depth, uint16_t *st);
 __global__ void k_lca_fill(int n, const int *__restrict__ parent, const int *__restrict__ sz,
                            const int *__restrict__ depth, const uint16_t *__restrict__ st, uint16_t *lca);
-// line inverses (grid) and path impedances (one CTA)
-cudaError_t launch_lines(int n, Topo T, const double *z_in, int *err, int num_sms, cudaStream_t st);
-cudaError_t launch_line_inverses(int n, Topo T, const double *z_in, int *err, int num_sms, cudaStream_t st);
+// children CSR and line impedances in preorder; line inverses (after them; a
+// singular line sets err = 2); path impedances (after the line impedances)
+cudaError_t launch_children_lines(int n, Topo T, const int *coff_c, const int *child_c, const double *z_in, int num_sms,
+                                  cudaStream_t st);
+cudaError_t launch_line_inverses(int n, Topo T, int *err, int num_sms, cudaStream_t st);
 cudaError_t launch_path_impedance(int n, Topo T, cudaStream_t st);
 // load flow of every scenario (cooperative launch).  J: [L*3n] line currents,
 // W: [L*3n] work (its contents are overwritten), red: [3L+1] doubles of
 // reduction slots and barrier counter (cleared by the launch), iters: [L].
-// Each grid barrier polls at most max_spins times (> 0), then sets err = 6.
+// Each grid barrier polls at most max_spins times (> 0), then sets err = 6;
+// one_cta allows one CTA per scenario, without grid barriers, on small feeders.
 cudaError_t launch_power_flow(int n, int L, Topo T, const double *s_in, double tol, int max_iter, double2 *J,
                               double2 *W, double *red, int *iters, int *err, int num_sms, cudaStream_t st,
-                              long long max_spins);
+                              long long max_spins, bool one_cta);
 __global__ void k_line_currents(int n, int L, Topo T, double2 *J);
 __global__ void k_injections(int n, int L, Topo T, const double2 *__restrict__ J);
 __global__ void k_import_ops(int n, int L, Topo T, const double *__restrict__ vh, const double *__restrict__ ih);
@@ -48,8 +50,11 @@ struct BatchSetup {
     double *dec_maxerr, *mrank, *bmax;
     int *arrive;
 };
-// Setup of many feeders in four launches (CTA per feeder, per feeder x scenario):
-// the LCA tables run on `side` (forked from st after the per-feeder prep by
+// prepare_batch_setup sets the load flow's shared-memory attribute (before any
+// stream capture).
+cudaError_t prepare_batch_setup();
+// Setup of many feeders in five launches (CTA per feeder, per feeder x scenario):
+// the line inverses, path impedances and LCA tables run on `side` (forked from st after the per-feeder prep by
 // ev_fork, joined back into st by ev_join before the call returns), the load
 // flows on st.
 cudaError_t launch_batch_setup(int nf, int max_L, long long max_nn, const BatchSetup *bs, double tol, int max_iter,
@@ -57,9 +62,8 @@ cudaError_t launch_batch_setup(int nf, int max_L, long long max_nn, const BatchS
                                cudaEvent_t ev_join);
 
 // The reduced network of a caller assignment (one CTA per scenario).
-__global__ void __launch_bounds__(1024) k_eval_reduced(Topo T, const int *__restrict__ sup, const int *__restrict__ moff,
-                                                      const int *__restrict__ mem, double2 *W, double2 *V, double *vred,
-                                                      double *err);
+cudaError_t launch_eval_reduced(Topo T, const int *sup, const int *moff, const int *mem, double2 *W, double2 *V,
+                                double *vred, double *err, cudaStream_t st);
 
 // okr_kron.cu
 constexpr int kKronShared = 64;     // groups up to this many phase-nodes are inverted in shared memory

@@ -10,39 +10,69 @@
 namespace okr {
 
 // ---------------------------------------------------------------- small dense helpers
+__device__ __forceinline__ double2 shfl8(double2 v, int src) {
+    return make_double2(__shfl_sync(0xffffffffu, v.x, src, 8), __shfl_sync(0xffffffffu, v.y, src, 8));
+}
+
 // Inverse of the sub-block of a 3x3 complex matrix on phase mask m (Gauss-Jordan
-// with partial pivoting); entries outside the sub-block are zero.  Returns false
-// if the sub-block is singular.
-__device__ bool inv3_sub(const double2 *a, unsigned m, double2 *out) {
-    int idx[3], k = 0;
-    for (int p = 0; p < 3; ++p)
-        if (m >> p & 1u) idx[k++] = p;
-    double2 w[3][6];
-    for (int i = 0; i < k; ++i)
-        for (int j = 0; j < 2 * k; ++j)
-            w[i][j] = (j < k) ? a[idx[i] * 3 + idx[j]] : make_double2(j - k == i ? 1.0 : 0.0, 0.0);
-    for (int c = 0; c < k; ++c) {
-        int piv = c;
-        double best = cmag(w[c][c]);
-        for (int i = c + 1; i < k; ++i) {
-            double v = cmag(w[i][c]);
-            if (v > best) { best = v; piv = i; }
-        }
-        if (best == 0.0) return false;
-        if (piv != c)
-            for (int j = 0; j < 2 * k; ++j) { double2 t = w[c][j]; w[c][j] = w[piv][j]; w[piv][j] = t; }
-        double2 d = w[c][c];
-        for (int j = 0; j < 2 * k; ++j) w[c][j] = cdiv(w[c][j], d);
-        for (int i = 0; i < k; ++i) {
-            if (i == c) continue;
-            double2 f = w[i][c];
-            for (int j = 0; j < 2 * k; ++j) w[i][j] = csub(w[i][j], cmul(f, w[c][j]));
+// with partial pivoting), by a group of eight lanes: lane j holds column j of the
+// augmented matrix [A | 1] (2 k columns), so that the divisions and the
+// elimination of a step, long chains of FP64 operations, run side by side (one
+// thread per line, with the rows in local memory: 37 us for 1,000 lines).  Every
+// lane of the warp calls it.  Returns false (in every lane of the group) if the
+// sub-block is singular; lane j in [k, 2 k) then holds nothing of use, otherwise
+// column j - k of the inverse in w, its rows the phases of m.
+__device__ bool inv3_lanes(const double2 *a, unsigned m, int j, double2 (&w)[3], int &k, int (&idx)[3]) {
+    k = 0;
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        if (m >> p & 1u) {
+            if (k == 0) idx[0] = p;
+            else if (k == 1) idx[1] = p;
+            else idx[2] = p;
+            ++k;
         }
     }
-    for (int q = 0; q < 9; ++q) out[q] = make_double2(0.0, 0.0);
-    for (int i = 0; i < k; ++i)
-        for (int j = 0; j < k; ++j) out[idx[i] * 3 + idx[j]] = w[i][k + j];
-    return true;
+    const int cj = j < k ? (j == 0 ? idx[0] : (j == 1 ? idx[1] : idx[2])) : 0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        w[i] = make_double2(j - k == i ? 1.0 : 0.0, 0.0);
+        if (i < k && j < k) w[i] = a[idx[i] * 3 + cj];
+    }
+    bool ok = true;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        double2 wc[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) wc[i] = shfl8(w[i], c);
+        if (c >= k) continue;
+        int piv = c;
+        double best = cmag(wc[c]);
+#pragma unroll
+        for (int i = c + 1; i < 3; ++i) {
+            if (i >= k) continue;
+            const double v = cmag(wc[i]);
+            if (v > best) { best = v; piv = i; }
+        }
+        if (best == 0.0) ok = false;
+#pragma unroll
+        for (int i = c + 1; i < 3; ++i) {
+            if (piv != i) continue;
+            double2 t = w[c];
+            w[c] = w[i];
+            w[i] = t;
+            t = wc[c];
+            wc[c] = wc[i];
+            wc[i] = t;
+        }
+        w[c] = cdiv(w[c], wc[c]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            if (i == c || i >= k) continue;
+            w[i] = csub(w[i], cmul(wc[i], w[c]));
+        }
+    }
+    return ok;
 }
 
 __device__ __forceinline__ void block_barrier() { __syncthreads(); }
@@ -255,10 +285,6 @@ __device__ void dev_child_offsets(int n, Topo T, const int *__restrict__ coff_c,
     }
 }
 
-__global__ void __launch_bounds__(1024) k_child_offsets(int n, Topo T, const int *__restrict__ coff_c, const int *__restrict__ child_c) {
-    dev_child_offsets(n, T, coff_c, child_c);
-}
-
 // Sparse table of the minimum-depth bus over preorder windows: st[j*n + v] is the
 // index of the shallowest bus in [v, v + 2^j).
 __global__ void k_rmq_level(int n, int j, const int *__restrict__ depth, uint16_t *st) {
@@ -334,78 +360,115 @@ __global__ void k_lca_fill(int n, const int *__restrict__ parent, const int *__r
     dev_lca_fill(n, parent, sz, depth, st, lca, (size_t)blockIdx.x * blockDim.x + threadIdx.x, (size_t)gridDim.x * blockDim.x);
 }
 
-// Line data in preorder: zl, yl (inverse on the bus phases); path impedance by
-// levels (parents first).  One CTA.
-// Line data: copies of the impedances and their inverses on the line's phases,
-// one thread per bus over the whole grid.
-__device__ void dev_line_inverses(int n, Topo T, const double *__restrict__ z_in, int *err, int first, int stride) {
-    for (int v = first; v < n; v += stride) {
-        const int i = T.orig[v];
-        double2 z[9];
-        for (int q = 0; q < 9; ++q) {
-            z[q] = (v == 0) ? make_double2(0.0, 0.0) : make_double2(z_in[((size_t)i * 9 + q) * 2], z_in[((size_t)i * 9 + q) * 2 + 1]);
-            T.zl[(size_t)v * 9 + q] = z[q];
-        }
-        double2 y[9];
-        if (v == 0) {
-            for (int q = 0; q < 9; ++q) y[q] = make_double2(0.0, 0.0);
-        } else if (!inv3_sub(z, T.ph[v], y)) {
-            atomicCAS(err, 0, 2);
-            for (int q = 0; q < 9; ++q) y[q] = make_double2(0.0, 0.0);
-        }
-        for (int q = 0; q < 9; ++q) T.yl[(size_t)v * 9 + q] = y[q];
+// Line impedances in preorder (a grid stride over the 9 n entries).
+__device__ void dev_line_copy(int n, Topo T, const double *__restrict__ z_in, int first, int stride) {
+    for (int e = first; e < 9 * n; e += stride) {
+        const int v = e / 9, q = e - 9 * v, i = T.orig[v];
+        const double2 *z = reinterpret_cast<const double2 *>(z_in) + (size_t)i * 9 + q;
+        T.zl[e] = v == 0 ? make_double2(0.0, 0.0) : *z;
     }
 }
 
-__global__ void k_line_inverses(int n, Topo T, const double *__restrict__ z_in, int *err) {
-    dev_line_inverses(n, T, z_in, err, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+// Their inverses on the lines' phases, eight lanes per line (whole warps call
+// it).  A singular line is reported whatever the load flow, which does not read
+// the inverses and may run beside them, reported before.
+__device__ void dev_line_inverses(int n, Topo T, int *err, int first, int stride) {
+    const int j = first & 7;
+    for (int w0 = (first & ~31) >> 3; w0 < n; w0 += stride >> 3) {
+        const int v = w0 + ((first & 31) >> 3);
+        const bool on = v > 0 && v < n;
+        const unsigned m = on ? T.ph[v] : 0u;
+        double2 w[3];
+        int k, idx[3] = {0, 0, 0};
+        const bool ok = inv3_lanes(T.zl + (size_t)(v < n ? v : 0) * 9, m, j, w, k, idx);
+        if (v >= n) continue;
+        if (!ok && j == 0) atomicExch(err, 2);
+        double2 *y = T.yl + (size_t)v * 9;
+        for (int q = j; q < 9; q += 8)
+            if (!ok || !(m >> (q / 3) & 1u) || !(m >> (q % 3) & 1u)) y[q] = make_double2(0.0, 0.0);
+        if (ok && j >= k && j < 2 * k) {
+            const int cj = j - k == 0 ? idx[0] : (j - k == 1 ? idx[1] : idx[2]);
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+                if (i < k) y[idx[i] * 3 + cj] = w[i];
+        }
+    }
 }
 
-// Path impedances root -> k level by level (one CTA), then their split into
-// two floats for the screening sweep.
-__device__ void dev_path_impedance(int n, Topo T) {
+__global__ void __launch_bounds__(32) k_line_inverses(int n, Topo T, int *err) {
+    dev_line_inverses(n, T, err, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
+
+// Children CSR (block 0) beside the line impedances (the other blocks).
+__global__ void __launch_bounds__(1024) k_children_lines(int n, Topo T, const int *__restrict__ coff_c,
+                                                         const int *__restrict__ child_c, const double *__restrict__ z_in) {
+    if (blockIdx.x == 0) dev_child_offsets(n, T, coff_c, child_c);
+    else dev_line_copy(n, T, z_in, (blockIdx.x - 1) * blockDim.x + threadIdx.x, (gridDim.x - 1) * blockDim.x);
+}
+
+// Path impedances root -> k, entry q of the 3x3 matrices, level by level, and
+// their split into two floats for the screening sweep (zc ~ zh + zlo).  z
+// (shared memory, n entries) or null: the chain in device memory.
+__device__ void dev_path_impedance(int n, Topo T, int q, double2 *z) {
     const int tid = threadIdx.x, nt = blockDim.x;
-    for (int q = tid; q < 9; q += nt) T.zc[q] = make_double2(0.0, 0.0);
+    const size_t st = z ? 1 : 9;
+    double2 *c = z ? z : T.zc + q;
+    if (tid == 0) c[0] = make_double2(0.0, 0.0);
+    if (z)
+        for (int v = tid; v < n; v += nt)
+            if (v > 0) z[v] = T.zl[(size_t)v * 9 + q];
     __syncthreads();
     const int maxd = T.maxd[0];
     for (int d = 1; d <= maxd; ++d) {
         for (int x = T.level_off[d] + tid; x < T.level_off[d + 1]; x += nt) {
-            int v = T.level_bus[x], p = T.parent[v];
-            for (int q = 0; q < 9; ++q) T.zc[(size_t)v * 9 + q] = cadd(T.zc[(size_t)p * 9 + q], T.zl[(size_t)v * 9 + q]);
+            const int v = T.level_bus[x], p = T.parent[v];
+            c[v * st] = cadd(c[p * st], z ? z[v] : T.zl[(size_t)v * 9 + q]);
         }
         __syncthreads();
     }
-    // single-precision split of the path impedances: zc ~ zh + zl
-    for (int e = tid; e < 9 * n; e += nt) {
-        const double2 z = T.zc[e];
-        const float2 h = make_float2((float)z.x, (float)z.y);
+    for (int v = tid; v < n; v += nt) {
+        const size_t e = (size_t)v * 9 + q;
+        const double2 x = c[v * st];
+        if (z) T.zc[e] = x;
+        const float2 h = make_float2((float)x.x, (float)x.y);
         T.zh[e] = h;
-        T.zlo[e] = make_float2((float)(z.x - (double)h.x), (float)(z.y - (double)h.y));
+        T.zlo[e] = make_float2((float)(x.x - (double)h.x), (float)(x.y - (double)h.y));
     }
 }
 
-__global__ void __launch_bounds__(1024) k_path_impedance(int n, Topo T) {
-    dev_path_impedance(n, T);
+// One CTA per entry of the matrices: the nine chains are independent (one CTA
+// for all of them, in device memory, took 73 us on 1,000 buses).
+constexpr int kPathShared = 8192;   // buses whose chain is kept in shared memory
+__global__ void __launch_bounds__(512) k_path_impedance(int n, Topo T) {
+    extern __shared__ double2 path_sm[];
+    dev_path_impedance(n, T, blockIdx.x, n <= kPathShared ? path_sm : nullptr);
 }
 
-cudaError_t launch_line_inverses(int n, Topo T, const double *z_in, int *err, int num_sms, cudaStream_t st) {
-    // one warp per CTA: each line's inverse is a chain of FP64 operations, and
-    // an SM's FP64 unit serves few warps at speed, so the lines go to as many
-    // SMs as possible
-    int blocks = (n + 31) / 32;
+cudaError_t launch_children_lines(int n, Topo T, const int *coff_c, const int *child_c, const double *z_in, int num_sms,
+                                  cudaStream_t st) {
+    int blocks = (9 * n + 1023) / 1024;
+    if (blocks > num_sms) blocks = num_sms;
+    k_children_lines<<<1 + blocks, 1024, 0, st>>>(n, T, coff_c, child_c, z_in);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_line_inverses(int n, Topo T, int *err, int num_sms, cudaStream_t st) {
+    // one warp per CTA: an SM's FP64 unit serves few warps at speed
+    int blocks = (n + 3) / 4;
     if (blocks > num_sms * 8) blocks = num_sms * 8;
-    k_line_inverses<<<blocks, 32, 0, st>>>(n, T, z_in, err);
+    k_line_inverses<<<blocks, 32, 0, st>>>(n, T, err);
     return cudaGetLastError();
 }
 
 cudaError_t launch_path_impedance(int n, Topo T, cudaStream_t st) {
-    k_path_impedance<<<1, 1024, 0, st>>>(n, T);
+    const size_t smem = n <= kPathShared ? sizeof(double2) * (size_t)n : 0;
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(k_path_impedance, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)(sizeof(double2) * kPathShared));
+        if (e != cudaSuccess) return e;
+    }
+    k_path_impedance<<<9, 512, smem, st>>>(n, T);
     return cudaGetLastError();
-}
-
-cudaError_t launch_lines(int n, Topo T, const double *z_in, int *err, int num_sms, cudaStream_t st) {
-    const cudaError_t e = launch_line_inverses(n, T, z_in, err, num_sms, st);
-    return e != cudaSuccess ? e : launch_path_impedance(n, T, st);
 }
 
 // ---------------------------------------------------------------- load flow
@@ -430,7 +493,32 @@ cudaError_t launch_lines(int n, Topo T, const double *z_in, int *err, int num_sm
 // (D overwrites I1, Vn overwrites D in place, I1 overwrites Vn).  The
 // arithmetic is the same, operation for operation, as a one-thread-per-bus
 // sweep.
-constexpr int kPfShared = 2048;     // buses whose (l, p) slice is staged in shared memory
+constexpr int kPfShared = 2048;     // buses whose (l, p) slice and tree are staged in shared memory
+
+// The tree of a feeder in shared memory, 16-bit (at most 32,768 buses): the
+// level loops chase level -> bus -> children or parent, and each of these was a
+// trip to L2 per level.
+struct TreeSm {
+    uint16_t *lb, *lo, *co, *ch, *par;      // level buses, level offsets, child offsets, children, parents
+};
+__host__ __device__ constexpr size_t tree_bytes(int n) { return ((size_t)2 * (5 * (size_t)n + 4) + 15) / 16 * 16; }
+__device__ __forceinline__ TreeSm load_tree(const Topo &T, int n, int maxd, void *mem) {
+    TreeSm t;
+    t.lb = static_cast<uint16_t *>(mem);
+    t.lo = t.lb + n;                        // maxd + 2 <= n + 1
+    t.co = t.lo + n + 1;
+    t.ch = t.co + n + 1;
+    t.par = t.ch + n;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        t.lb[i] = (uint16_t)T.level_bus[i];
+        t.co[i] = (uint16_t)T.child_off[i];
+        t.ch[i] = (uint16_t)(i < n - 1 ? T.child[i] : 0);
+        t.par[i] = (uint16_t)(i > 0 ? T.parent[i] : 0);
+    }
+    for (int i = threadIdx.x; i < maxd + 2; i += blockDim.x) t.lo[i] = (uint16_t)T.level_off[i];
+    if (threadIdx.x == 0) t.co[n] = (uint16_t)T.child_off[n];
+    return t;                               // (the caller synchronises)
+}
 
 __device__ __forceinline__ unsigned pf_ld_acquire(const unsigned *p) {
     unsigned v;
@@ -478,14 +566,24 @@ __global__ void __launch_bounds__(256) k_power_flow(int n, int L, Topo T, const 
     const double tol2 = tol * tol;                  // the test is max |dV|^2 < tol^2
     unsigned epoch = 0;
     for (size_t e = gt; e < tot; e += gs) {
-        const int v = (int)(e % n), p = (int)((e / n) % 3);
+        const unsigned q = (unsigned)e / (unsigned)n;
+        const int v = (int)((unsigned)e - q * (unsigned)n), p = (int)(q % 3u);
         T.vhat[e] = (T.ph[v] >> p & 1u) ? T.vslack[p] : make_double2(0.0, 0.0);
     }
     if (tid < kMaxScen) s_live[tid] = tid < L;
     const bool line_cta = blockIdx.x < (unsigned)(3 * L);
     const int ll = blockIdx.x / 3, lp = blockIdx.x % 3;      // (scenario, phase) of a level CTA
     double2 *const loc = n <= kPfShared ? pf_sm : nullptr;
+    TreeSm tr = {};
+    if (loc && line_cta) tr = load_tree(T, n, maxd, pf_sm + n);
     bool conv_all = false;
+    // element e of the [L][3][n] arrays (fewer than 2^31)
+    auto split = [&](size_t e, int &l, int &p, int &v) {
+        const unsigned q = (unsigned)e / (unsigned)n;
+        v = (int)((unsigned)e - q * (unsigned)n);
+        l = (int)(q / 3u);
+        p = (int)(q - 3u * (unsigned)l);
+    };
     // the load current of element e on voltage vv (S1)
     auto set_load_current = [&](size_t e, int l, int p, int v, double2 vv) {
         double2 j = make_double2(0.0, 0.0);
@@ -499,7 +597,8 @@ __global__ void __launch_bounds__(256) k_power_flow(int n, int L, Topo T, const 
     __syncthreads();                                         // (s_live)
     // S1 of the first sweep (each element on the thread that set its voltage)
     for (size_t e = gt; e < tot; e += gs) {
-        const int l = (int)(e / N3), p = (int)((e / n) % 3), v = (int)(e % n);
+        int l, p, v;
+        split(e, l, p, v);
         set_load_current(e, l, p, v, T.vhat[e]);
     }
     if (!pf_grid_sync(bar, err, G, epoch, max_spins)) return;
@@ -516,7 +615,16 @@ __global__ void __launch_bounds__(256) k_power_flow(int n, int L, Topo T, const 
                 for (int v = tid; v < n; v += nt) Jx[v] = W[off + v];
             }
             __syncthreads();
-            for (int d = maxd; d >= 1; --d) {
+            for (int d = maxd; loc && d >= 1; --d) {
+                for (int x = tr.lo[d] + tid; x < tr.lo[d + 1]; x += nt) {
+                    const int v = tr.lb[x];
+                    double2 j = loc[v];
+                    for (int c = tr.co[v]; c < tr.co[v + 1]; ++c) j = cadd(j, loc[tr.ch[c]]);
+                    loc[v] = j;
+                }
+                __syncthreads();
+            }
+            for (int d = maxd; !loc && d >= 1; --d) {
                 for (int x = T.level_off[d] + tid; x < T.level_off[d + 1]; x += nt) {
                     const int v = T.level_bus[x];
                     double2 j = Jx[v];
@@ -531,7 +639,8 @@ __global__ void __launch_bounds__(256) k_power_flow(int n, int L, Topo T, const 
         if (!pf_grid_sync(bar, err, G, epoch, max_spins)) return;
         // S3: drops z J on the phases of each line (root excluded)
         for (size_t e = gt; e < tot; e += gs) {
-            const int l = (int)(e / N3), p = (int)((e / n) % 3), v = (int)(e % n);
+            int l, p, v;
+            split(e, l, p, v);
             if (!s_live[l]) continue;
             const unsigned ph = T.ph[v];
             double2 drop = make_double2(0.0, 0.0);
@@ -551,7 +660,14 @@ __global__ void __launch_bounds__(256) k_power_flow(int n, int L, Topo T, const 
             __syncthreads();
             if (tid == 0) Vx[0] = T.vhat[off];
             __syncthreads();
-            for (int d = 1; d <= maxd; ++d) {
+            for (int d = 1; loc && d <= maxd; ++d) {
+                for (int x = tr.lo[d] + tid; x < tr.lo[d + 1]; x += nt) {
+                    const int v = tr.lb[x];
+                    loc[v] = csub(loc[tr.par[v]], loc[v]);
+                }
+                __syncthreads();
+            }
+            for (int d = 1; !loc && d <= maxd; ++d) {
                 for (int x = T.level_off[d] + tid; x < T.level_off[d + 1]; x += nt) {
                     const int v = T.level_bus[x];
                     Vx[v] = csub(Vx[T.parent[v]], Vx[v]);
@@ -565,7 +681,8 @@ __global__ void __launch_bounds__(256) k_power_flow(int n, int L, Topo T, const 
         // S5: change of the voltages, per-scenario maximum; then S1 of the next sweep
         double mx[kMaxScen] = {0.0, 0.0, 0.0, 0.0};
         for (size_t e = gt; e < tot; e += gs) {
-            const int l = (int)(e / N3), p = (int)((e / n) % 3), v = (int)(e % n);
+            int l, p, v;
+            split(e, l, p, v);
             if (!s_live[l]) continue;
             double2 vv = T.vhat[e];
             if (v != 0 && (T.ph[v] >> p & 1u)) {
@@ -608,17 +725,135 @@ __global__ void __launch_bounds__(256) k_power_flow(int n, int L, Topo T, const 
     }
 }
 
-// Blocks of the cooperative load flow: enough for the grid-wide stages, at
-// least one per (scenario, phase), at most one per SM.
+// The load flow of one scenario by one CTA with everything it touches in a sweep
+// but the loads and the line impedances in shared memory (voltages, currents and
+// the tree): the same sweep, operation for operation, as k_power_flow, with block
+// barriers in place of grid barriers.  For small feeders, whose grid barriers and
+// trips to L2 were the time (40 buses: 145 us), and for batches, whose many CTAs
+// spread the FP64 work.
+constexpr int kPfCta = 1920;        // buses whose load flow fits one CTA's shared memory
+constexpr int kPfSmall = 256;       // buses up to which a single feeder takes one CTA per scenario
+constexpr int kPfThreads = 512;
+__host__ __device__ constexpr size_t pf_cta_bytes(int n) { return sizeof(double2) * 6 * (size_t)n + tree_bytes(n); }
+__device__ void dev_power_flow_smem(int n, int l, const Topo &T, const double *__restrict__ s_in, double tol,
+                                    int max_iter, int *iters, int *err, double2 *sm) {
+    __shared__ double s_mx[32];
+    __shared__ int s_ok;
+    const int tid = threadIdx.x, nt = blockDim.x, maxd = T.maxd[0];
+    double2 *V = sm, *W = sm + 3 * (size_t)n;
+    const TreeSm tr = load_tree(T, n, maxd, sm + 6 * (size_t)n);
+    for (int e = tid; e < 3 * n; e += nt) {
+        const int p = e / n, v = e - p * n;
+        V[e] = (T.ph[v] >> p & 1u) ? T.vslack[p] : make_double2(0.0, 0.0);
+    }
+    __syncthreads();
+    const double tol2 = tol * tol;                  // the test is max |dV|^2 < tol^2
+    int it;
+    bool conv = false;
+    for (it = 1; it <= max_iter; ++it) {
+        for (int e = tid; e < 3 * n; e += nt) {     // load currents
+            const int p = e / n, v = e - p * n;
+            double2 j = make_double2(0.0, 0.0);
+            if (T.ph[v] >> p & 1u) {
+                const size_t o = (((size_t)l * n + T.orig[v]) * 3 + p) * 2;
+                j = load_current(make_double2(__ldg(s_in + o), __ldg(s_in + o + 1)), V[e]);
+            }
+            W[e] = j;
+        }
+        __syncthreads();
+        for (int d = maxd; d >= 1; --d) {           // line currents, deepest level first
+            const int x0 = tr.lo[d], k = 3 * (tr.lo[d + 1] - x0);
+            for (int i = tid; i < k; i += nt) {
+                const int v = tr.lb[x0 + i / 3];
+                double2 *Jp = W + (size_t)(i % 3) * n;
+                double2 j = Jp[v];
+                for (int c = tr.co[v]; c < tr.co[v + 1]; ++c) j = cadd(j, Jp[tr.ch[c]]);
+                Jp[v] = j;
+            }
+            __syncthreads();
+        }
+        for (int v = tid; v < n; v += nt) {         // drops z J, in place
+            const unsigned ph = T.ph[v];
+            double2 J[3], D[3];
+#pragma unroll
+            for (int p = 0; p < 3; ++p) J[p] = W[(size_t)p * n + v];
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+                double2 drop = make_double2(0.0, 0.0);
+                if (v > 0 && (ph >> p & 1u))
+#pragma unroll
+                    for (int q = 0; q < 3; ++q)
+                        if (ph >> q & 1u) drop = cadd(drop, cmul(T.zl[(size_t)v * 9 + p * 3 + q], J[q]));
+                D[p] = drop;
+            }
+#pragma unroll
+            for (int p = 0; p < 3; ++p) W[(size_t)p * n + v] = v > 0 ? D[p] : V[(size_t)p * n];
+        }
+        __syncthreads();
+        for (int d = 1; d <= maxd; ++d) {           // new voltages, top down (over the drops)
+            const int x0 = tr.lo[d], k = 3 * (tr.lo[d + 1] - x0);
+            for (int i = tid; i < k; i += nt) {
+                const int v = tr.lb[x0 + i / 3];
+                double2 *Vp = W + (size_t)(i % 3) * n;
+                Vp[v] = csub(Vp[tr.par[v]], Vp[v]);
+            }
+            __syncthreads();
+        }
+        double mx = 0.0;
+        for (int e = tid; e < 3 * n; e += nt) {
+            const int p = e / n, v = e - p * n;
+            if (v == 0 || !(T.ph[v] >> p & 1u)) continue;
+            const double2 vn = W[e];
+            double dd = cmag2(csub(vn, V[e]));      // squared change
+            if (!isfinite(dd)) dd = INFINITY;       // a diverging sweep never converges
+            mx = fmax(mx, dd);
+            V[e] = vn;
+        }
+        for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if ((tid & 31) == 0) s_mx[tid >> 5] = mx;
+        __syncthreads();
+        if (tid < 32) {
+            double m = tid < nt / 32 ? s_mx[tid] : 0.0;
+            for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if (tid == 0) s_ok = m < tol2;
+        }
+        __syncthreads();
+        if (s_ok) { conv = true; break; }
+    }
+    for (int e = tid; e < 3 * n; e += nt) T.vhat[(size_t)l * 3 * n + e] = V[e];
+    if (tid == 0) {
+        iters[l] = conv ? it : -1;
+        if (!conv) atomicCAS(err, 0, 3);
+    }
+}
+
+__global__ void __launch_bounds__(kPfThreads) k_power_flow_cta(int n, Topo T, const double *__restrict__ s_in, double tol,
+                                                               int max_iter, int *iters, int *err) {
+    extern __shared__ double2 pfc_sm[];
+    // an earlier setup step failed
+    if (*reinterpret_cast<volatile const int *>(err) != 0) return;
+    dev_power_flow_smem(n, blockIdx.x, T, s_in, tol, max_iter, iters, err, pfc_sm);
+}
+
+// One CTA per scenario on small feeders; otherwise the cooperative load flow
+// (blocks enough for the grid-wide stages, at least one per (scenario, phase),
+// at most one per SM).  A limit on the polls of a barrier asks for the barriers.
 cudaError_t launch_power_flow(int n, int L, Topo T, const double *s_in, double tol, int max_iter, double2 *J,
                               double2 *W, double *red, int *iters, int *err, int num_sms, cudaStream_t st,
-                              long long max_spins) {
+                              long long max_spins, bool one_cta) {
+    if (one_cta && n <= kPfSmall) {
+        k_power_flow_cta<<<L, kPfThreads, pf_cta_bytes(n), st>>>(n, T, s_in, tol, max_iter, iters, err);
+        return cudaGetLastError();
+    }
     int G = (int)(((size_t)3 * L * n + 127) / 128);
     if (G < 3 * L) G = 3 * L;
     if (G > num_sms) G = num_sms;
-    const size_t smem = n <= kPfShared ? sizeof(double2) * (size_t)n : 0;
+    const size_t smem = n <= kPfShared ? sizeof(double2) * (size_t)n + tree_bytes(n) : 0;
     unsigned *bar = reinterpret_cast<unsigned *>(red + 3 * L);
     cudaError_t e = cudaMemsetAsync(red, 0, sizeof(double) * (3 * L + 1), st);
+    if (e == cudaSuccess && smem > 48 * 1024)
+        e = cudaFuncSetAttribute(k_power_flow, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(sizeof(double2) * kPfShared + tree_bytes(kPfShared)));
     if (e != cudaSuccess) return e;
     void *args[] = {&n, &L, &T, &s_in, &tol, &max_iter, &J, &W, &red, &bar, &iters, &err, &max_spins};
     return cudaLaunchCooperativeKernel((const void *)k_power_flow, dim3(G), dim3(256), args, smem, st);
@@ -626,22 +861,29 @@ cudaError_t launch_power_flow(int n, int L, Topo T, const double *s_in, double t
 
 // Ihat = Y Vhat line by line: line current J_k = y_k (V_parent - V_k) on the
 // phases of k; injection I_k = sum of children's J - J_k.  Also |Vhat|.
+// One thread per (scenario, phase, bus) in all three: FP64 chains, so the more
+// SMs share them the better (one thread per (scenario, bus): 11 us on 1,000).
+__device__ __forceinline__ void lpv(size_t e, int n, int &l, int &p, int &v) {
+    const unsigned q = (unsigned)e / (unsigned)n;
+    v = (int)((unsigned)e - q * (unsigned)n);
+    l = (int)(q / 3u);
+    p = (int)(q - 3u * (unsigned)l);
+}
 __device__ void dev_line_currents(int n, int L, Topo T, double2 *J, size_t first, size_t stride) {
-    size_t tot = (size_t)L * n;
+    const size_t tot = (size_t)3 * L * n;
     for (size_t e = first; e < tot; e += stride) {
-        int l = (int)(e / n), v = (int)(e % n);
-        for (int p = 0; p < 3; ++p) {
-            double2 j = make_double2(0.0, 0.0);
-            if (v > 0 && (T.ph[v] >> p & 1u)) {
-                int par = T.parent[v];
-                for (int q = 0; q < 3; ++q)
-                    if (T.ph[v] >> q & 1u)
-                        j = cadd(j, cmul(T.yl[(size_t)v * 9 + p * 3 + q], csub(T.vhat[sidx(l, q, par, n)], T.vhat[sidx(l, q, v, n)])));
-            }
-            J[sidx(l, p, v, n)] = j;
-            double2 vv = T.vhat[sidx(l, p, v, n)];
-            T.amag[sidx(l, p, v, n)] = (T.ph[v] >> p & 1u) ? cmag(vv) : 0.0;
+        int l, p, v;
+        lpv(e, n, l, p, v);
+        const unsigned ph = T.ph[v];
+        double2 j = make_double2(0.0, 0.0);
+        if (v > 0 && (ph >> p & 1u)) {
+            const int par = T.parent[v];
+            for (int q = 0; q < 3; ++q)
+                if (ph >> q & 1u)
+                    j = cadd(j, cmul(T.yl[(size_t)v * 9 + p * 3 + q], csub(T.vhat[sidx(l, q, par, n)], T.vhat[sidx(l, q, v, n)])));
         }
+        J[e] = j;
+        T.amag[e] = (ph >> p & 1u) ? cmag(T.vhat[e]) : 0.0;
     }
 }
 
@@ -650,14 +892,13 @@ __global__ void k_line_currents(int n, int L, Topo T, double2 *J) {
 }
 
 __device__ void dev_injections(int n, int L, Topo T, const double2 *__restrict__ J, size_t first, size_t stride) {
-    size_t tot = (size_t)L * n;
+    const size_t tot = (size_t)3 * L * n;
     for (size_t e = first; e < tot; e += stride) {
-        int l = (int)(e / n), v = (int)(e % n);
-        for (int p = 0; p < 3; ++p) {
-            double2 s = make_double2(0.0, 0.0);
-            for (int c = T.child_off[v]; c < T.child_off[v + 1]; ++c) s = cadd(s, J[sidx(l, p, T.child[c], n)]);
-            T.ihat[sidx(l, p, v, n)] = csub(s, J[sidx(l, p, v, n)]);
-        }
+        int l, p, v;
+        lpv(e, n, l, p, v);
+        double2 s = make_double2(0.0, 0.0);
+        for (int c = T.child_off[v]; c < T.child_off[v + 1]; ++c) s = cadd(s, J[sidx(l, p, T.child[c], n)]);
+        T.ihat[e] = csub(s, J[e]);
     }
 }
 
@@ -685,10 +926,11 @@ __global__ void k_import_ops(int n, int L, Topo T, const double *__restrict__ vh
 // Initial state of Algorithm 1: every bus is its own super-node, I = Ihat,
 // V = Vhat, cluster extremes = |Vhat|, MICE = 0.
 __device__ void dev_state_init(int n, int L, Topo T, State S, size_t first, size_t stride) {
-    size_t tot = (size_t)L * n;
+    const size_t tot = (size_t)3 * L * n;
     for (size_t e = first; e < tot; e += stride) {
-        int l = (int)(e / n), v = (int)(e % n);
-        if (l == 0) {
+        int l, p, v;
+        lpv(e, n, l, p, v);
+        if (l == 0 && p == 0) {
             S.label[v] = v;
             S.top[v] = v;
             S.ptop[v] = T.parent[v];
@@ -696,21 +938,22 @@ __device__ void dev_state_init(int n, int L, Topo T, State S, size_t first, size
             S.sn_rank[v] = v;
             if (v == n - 1) S.sn_rank[n] = n;
         }
-        S.mice[(size_t)l * n + v] = 0.0;
-        S.mice32[(size_t)l * n + v] = 0.0f;
-        for (int p = 0; p < 3; ++p) {
-            size_t q = sidx(l, p, v, n);
-            bool on = T.ph[v] >> p & 1u;
-            S.vcur[q] = T.vhat[q];
-            S.icur[q] = T.ihat[q];
-            S.hi[q] = on ? T.amag[q] : -INFINITY;
-            S.lo[q] = on ? T.amag[q] : INFINITY;
-            S.mcur[q] = T.amag[q];
-            S.v32[q] = make_float2((float)T.vhat[q].x, (float)T.vhat[q].y);
-            S.hr32[q] = 0.0f;
-            S.lr32[q] = 0.0f;
-            S.icur32[q] = make_float2((float)T.ihat[q].x, (float)T.ihat[q].y);
+        if (p == 0) {
+            S.mice[(size_t)l * n + v] = 0.0;
+            S.mice32[(size_t)l * n + v] = 0.0f;
         }
+        const bool on = T.ph[v] >> p & 1u;
+        const double2 vh = T.vhat[e], ih = T.ihat[e];
+        const double am = T.amag[e];
+        S.vcur[e] = vh;
+        S.icur[e] = ih;
+        S.hi[e] = on ? am : -INFINITY;
+        S.lo[e] = on ? am : INFINITY;
+        S.mcur[e] = am;
+        S.v32[e] = make_float2((float)vh.x, (float)vh.y);
+        S.hr32[e] = 0.0f;
+        S.lr32[e] = 0.0f;
+        S.icur32[e] = make_float2((float)ih.x, (float)ih.y);
     }
 }
 
@@ -723,9 +966,8 @@ __global__ void k_state_init(int n, int L, Topo T, State S) {
 namespace okr {
 
 // ---------------------------------------------------------------- many feeders
-// Load flow of one scenario by one CTA (the batch runs many such CTAs side by
-// side, which spreads the FP64 arithmetic over the SMs): the same sweep,
-// operation for operation, as k_power_flow.
+// Load flow of one scenario of a feeder too large for one CTA's shared memory:
+// the same sweep, operation for operation, as k_power_flow.
 __device__ void dev_power_flow_cta(int n, int l, const Topo &T, const double *__restrict__ s_in, double tol,
                                    int max_iter, double2 *J, int *iters, int *err) {
     const int tid = threadIdx.x, nt = blockDim.x;
@@ -805,9 +1047,16 @@ __global__ void __launch_bounds__(1024) k_batch_prep(const BatchSetup *bs) {
     dev_child_offsets(b.n, b.T, b.coff_c, b.child_c);
     __syncthreads();
     dev_rmq_all(b.n, b.nlev, b.T.depth, b.rmq);
-    dev_line_inverses(b.n, b.T, b.z_in, b.err, threadIdx.x, blockDim.x);
-    __syncthreads();
-    dev_path_impedance(b.n, b.T);
+    dev_line_copy(b.n, b.T, b.z_in, threadIdx.x, blockDim.x);
+}
+
+// Line inverses (blockIdx.x = 9) and path impedances, entry blockIdx.x of the
+// matrices; blockIdx.y = feeder.  Beside the load flows, which read neither.
+__global__ void __launch_bounds__(256) k_batch_lines(const BatchSetup *bs) {
+    const BatchSetup &b = bs[blockIdx.y];
+    if (*(volatile int *)b.err == 1) return;
+    if (blockIdx.x >= 9) dev_line_inverses(b.n, b.T, b.err, (blockIdx.x - 9) * blockDim.x + threadIdx.x, (gridDim.x - 9) * blockDim.x);
+    else dev_path_impedance(b.n, b.T, blockIdx.x, nullptr);
 }
 
 // LCA tables: blockIdx.y = feeder.
@@ -819,12 +1068,14 @@ __global__ void k_batch_lca(const BatchSetup *bs) {
 }
 
 // Load flow: blockIdx.y = feeder, blockIdx.x = scenario.
-__global__ void __launch_bounds__(256) k_batch_pf(const BatchSetup *bs, double tol, int max_iter) {
+__global__ void __launch_bounds__(kPfThreads) k_batch_pf(const BatchSetup *bs, double tol, int max_iter) {
+    extern __shared__ double2 pfb_sm[];
     __shared__ BatchSetup b;
     if (threadIdx.x == 0) b = bs[blockIdx.y];
     __syncthreads();
     if ((int)blockIdx.x >= b.L || *(volatile int *)b.err == 1) return;
-    dev_power_flow_cta(b.n, blockIdx.x, b.T, b.s_in, tol, max_iter, b.J, b.pf_iters, b.err);
+    if (b.n <= kPfCta) dev_power_flow_smem(b.n, blockIdx.x, b.T, b.s_in, tol, max_iter, b.pf_iters, b.err, pfb_sm);
+    else dev_power_flow_cta(b.n, blockIdx.x, b.T, b.s_in, tol, max_iter, b.J, b.pf_iters, b.err);
 }
 
 // Per feeder, one CTA: Ihat = Y Vhat, |Vhat|, the initial search state and the
@@ -849,29 +1100,39 @@ __global__ void __launch_bounds__(1024) k_batch_finish(const BatchSetup *bs) {
     for (int i = threadIdx.x; i < b.n / 32 + 2; i += blockDim.x) b.bmax[i] = 0.0;
 }
 
+// Dynamic shared memory of a batch's load flows (its largest feeder; larger than
+// kPfCta run in device memory).
+static size_t batch_pf_smem(long long max_nn) {
+    int n = 1;
+    while (n < kPfCta && (long long)n * n < max_nn) ++n;
+    return pf_cta_bytes(n);
+}
+cudaError_t prepare_batch_setup() {
+    return cudaFuncSetAttribute(k_batch_pf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pf_cta_bytes(kPfCta));
+}
+
 cudaError_t launch_batch_setup(int nf, int max_L, long long max_nn, const BatchSetup *bs, double tol, int max_iter,
                                int num_sms, cudaStream_t st, cudaStream_t side, cudaEvent_t ev_fork,
                                cudaEvent_t ev_join) {
     if (nf <= 0) return cudaSuccess;
     k_batch_prep<<<nf, 1024, 0, st>>>(bs);
-    // the LCA tables (integer work, read only by the searches) on the side
-    // stream beside the load flows (FP64 work)
+    // what the load flows do not read -- line inverses, path impedances, LCA
+    // tables -- on the side stream beside them
     cudaError_t e = cudaEventRecord(ev_fork, st);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(side, ev_fork, 0);
     if (e != cudaSuccess) return e;
     long long bx = (max_nn + 255) / 256;
     if (bx > num_sms * 2) bx = num_sms * 2;
     if (bx < 1) bx = 1;
+    k_batch_lines<<<dim3(9 + 8, nf), 256, 0, side>>>(bs);
     k_batch_lca<<<dim3((unsigned)bx, nf), 256, 0, side>>>(bs);
     e = cudaEventRecord(ev_join, side);
     if (e != cudaSuccess) return e;
-    // 256 threads: every (feeder, scenario) CTA resident at once, so that the
-    // SMs interleave many CTAs' level-by-level chains (1,024-thread CTAs ran
-    // in waves: 4.0 -> 3.2 ms for 256 feeders)
-    k_batch_pf<<<dim3(max_L, nf), 256, 0, st>>>(bs, tol, max_iter);
+    k_batch_pf<<<dim3(max_L, nf), kPfThreads, batch_pf_smem(max_nn), st>>>(bs, tol, max_iter);
+    e = cudaStreamWaitEvent(st, ev_join, 0);            // (the injections read the line inverses)
+    if (e != cudaSuccess) return e;
     k_batch_finish<<<nf, 1024, 0, st>>>(bs);
-    e = cudaStreamWaitEvent(st, ev_join, 0);
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return cudaGetLastError();
 }
 
 }  // namespace okr
@@ -891,8 +1152,14 @@ namespace okr {
 __global__ void __launch_bounds__(1024) k_eval_reduced(Topo T, const int *__restrict__ sup, const int *__restrict__ moff,
                                                       const int *__restrict__ mem, double2 *W, double2 *V, double *vred,
                                                       double *err) {
+    extern __shared__ double2 eval_sm[];
     const int n = T.n, l = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
-    double2 *Wl = W + (size_t)l * 3 * n, *Vl = V + (size_t)l * 3 * n;
+    // currents, voltages and the tree in shared memory when they fit
+    const bool in_sm = n <= kPfCta;
+    double2 *Wl = in_sm ? eval_sm : W + (size_t)l * 3 * n, *Vl = in_sm ? eval_sm + 3 * (size_t)n : V + (size_t)l * 3 * n;
+    const int maxd = T.maxd[0];
+    TreeSm tr = {};
+    if (in_sm) tr = load_tree(T, n, maxd, eval_sm + 6 * (size_t)n);
     __shared__ double s_red[32];
     // aggregated injections at the super-nodes (preorder), zero elsewhere
     for (int e = tid; e < 3 * n; e += nt) {
@@ -906,8 +1173,18 @@ __global__ void __launch_bounds__(1024) k_eval_reduced(Topo T, const int *__rest
     }
     __syncthreads();
     // line currents J_v = -I_v + sum of the children's J, deepest level first
-    const int maxd = T.maxd[0];
-    for (int d = maxd; d >= 1; --d) {
+    for (int d = maxd; in_sm && d >= 1; --d) {
+        const int x0 = tr.lo[d], k = 3 * (tr.lo[d + 1] - x0);
+        for (int i = tid; i < k; i += nt) {
+            const int v = tr.lb[x0 + i / 3];
+            double2 *Jp = Wl + (size_t)(i % 3) * n;
+            double2 j = make_double2(-Jp[v].x, -Jp[v].y);
+            for (int c = tr.co[v]; c < tr.co[v + 1]; ++c) j = cadd(j, Jp[tr.ch[c]]);
+            Jp[v] = j;
+        }
+        __syncthreads();
+    }
+    for (int d = maxd; !in_sm && d >= 1; --d) {
         for (int x = T.level_off[d] + tid; x < T.level_off[d + 1]; x += nt) {
             const int v = T.level_bus[x];
             for (int p = 0; p < 3; ++p) {
@@ -921,7 +1198,28 @@ __global__ void __launch_bounds__(1024) k_eval_reduced(Topo T, const int *__rest
     // voltages, top down: V_v = V_parent - z_v J_v on the phases of v
     for (int e = tid; e < 3; e += nt) Vl[(size_t)e * n] = (T.ph[0] >> e & 1u) ? T.vslack[e] : make_double2(0.0, 0.0);
     __syncthreads();
-    for (int d = 1; d <= maxd; ++d) {
+    // (in shared memory the drops first, every line at once, into V)
+    for (int v = tid; in_sm && v < n; v += nt) {
+        if (v == 0) continue;
+        for (int p = 0; p < 3; ++p) {
+            double2 drop = make_double2(0.0, 0.0);
+            if (T.ph[v] >> p & 1u)
+                for (int q = 0; q < 3; ++q)
+                    if (T.ph[v] >> q & 1u) drop = cadd(drop, cmul(T.zl[(size_t)v * 9 + p * 3 + q], Wl[(size_t)q * n + v]));
+            Vl[(size_t)p * n + v] = drop;
+        }
+    }
+    __syncthreads();
+    for (int d = 1; in_sm && d <= maxd; ++d) {
+        const int x0 = tr.lo[d], k = 3 * (tr.lo[d + 1] - x0);
+        for (int i = tid; i < k; i += nt) {
+            const int v = tr.lb[x0 + i / 3], p = i % 3;
+            double2 *Vp = Vl + (size_t)p * n;
+            Vp[v] = (T.ph[v] >> p & 1u) ? csub(Vp[tr.par[v]], Vp[v]) : make_double2(0.0, 0.0);
+        }
+        __syncthreads();
+    }
+    for (int d = 1; !in_sm && d <= maxd; ++d) {
         for (int x = T.level_off[d] + tid; x < T.level_off[d + 1]; x += nt) {
             const int v = T.level_bus[x], par = T.parent[v];
             for (int p = 0; p < 3; ++p) {
@@ -959,6 +1257,18 @@ __global__ void __launch_bounds__(1024) k_eval_reduced(Topo T, const int *__rest
         for (int w = 0; w < (nt + 31) / 32; ++w) r = fmax(r, s_red[w]);
         err[l] = r;
     }
+}
+
+cudaError_t launch_eval_reduced(Topo T, const int *sup, const int *moff, const int *mem, double2 *W, double2 *V,
+                                double *vred, double *err, cudaStream_t st) {
+    const size_t smem = T.n <= kPfCta ? pf_cta_bytes(T.n) : 0;
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(k_eval_reduced, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)pf_cta_bytes(kPfCta));
+        if (e != cudaSuccess) return e;
+    }
+    k_eval_reduced<<<T.L, 1024, smem, st>>>(T, sup, moff, mem, W, V, vred, err);
+    return cudaGetLastError();
 }
 
 }  // namespace okr

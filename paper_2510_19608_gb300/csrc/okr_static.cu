@@ -221,8 +221,8 @@ extern "C" okr_status okr_power_flow_static(const okr_feeder *f, double *vhat_ou
     // the next kernels index with the renumbering: stop on an invalid tree
     s = read_err(w.err, st);
     if (s != OKR_OK) return s;
-    k_child_offsets<<<1, 1024, 0, st>>>(n, T, w.coff_c, w.child_c);
-    if (launch_lines(n, T, f->z_line, w.err, slot.num_sms, st) != cudaSuccess) return OKR_ECUDA;
+    if (launch_children_lines(n, T, w.coff_c, w.child_c, f->z_line, slot.num_sms, st) != cudaSuccess) return OKR_ECUDA;
+    if (launch_line_inverses(n, T, w.err, slot.num_sms, st) != cudaSuccess) return OKR_ECUDA;
     // a singular line block (err = 2) stops here, as okr_power_flow does: the
     // load flow would run on undefined admittances and its own outcome would
     // overwrite the flag
@@ -230,10 +230,10 @@ extern "C" okr_status okr_power_flow_static(const okr_feeder *f, double *vhat_ou
     if (s != OKR_OK) return s;
     // the load flow's work buffers alias T.ihat and T.amag, which the next two kernels fill
     if (launch_power_flow(n, L, T, f->s_load, kPfTol, kPfMaxIter, w.J, T.ihat, T.amag, w.sweeps, w.err,
-                          slot.num_sms, st, kPfSpins) != cudaSuccess)
+                          slot.num_sms, st, kPfSpins, true) != cudaSuccess)
         return OKR_ECUDA;
-    k_line_currents<<<grid_for((size_t)L * n, slot.num_sms), 256, 0, st>>>(n, L, T, w.J);
-    k_injections<<<grid_for((size_t)L * n, slot.num_sms), 256, 0, st>>>(n, L, T, w.J);
+    k_line_currents<<<grid_for((size_t)3 * L * n, slot.num_sms), 256, 0, st>>>(n, L, T, w.J);
+    k_injections<<<grid_for((size_t)3 * L * n, slot.num_sms), 256, 0, st>>>(n, L, T, w.J);
     k_export_static<<<grid_for((size_t)L * n, slot.num_sms), 256, 0, st>>>(T, vhat_out, ihat_out);
     if (cudaGetLastError() != cudaSuccess) return OKR_ECUDA;
     s = read_err(w.err, st);
