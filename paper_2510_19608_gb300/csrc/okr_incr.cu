@@ -64,6 +64,8 @@
 #include "okr_internal.cuh"
 #include "okr_kernels.cuh"
 
+#include <climits>
+
 namespace okr {
 
 namespace {
@@ -226,76 +228,13 @@ __device__ __forceinline__ Red block_red(Red v, Red *sm) {
     return sm[32];
 }
 
-// The same with 64-bit minima (precision 1: every key fits 64 bits).
-struct Red64 {
-    unsigned long long a, b, c;
-    int i;
-};
-
-template <int NT>
-__device__ __forceinline__ Red64 block_red64(Red64 v, Red64 *sm) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    auto op = [](Red64 x, Red64 y) {
-        Red64 r;
-        r.a = x.a < y.a ? x.a : y.a;
-        r.b = x.b < y.b ? x.b : y.b;
-        r.c = x.c < y.c ? x.c : y.c;
-        r.i = x.i + y.i;
-        return r;
-    };
-    auto shfl = [](Red64 x, int o) {
-        Red64 r;
-        r.a = __shfl_xor_sync(0xffffffffu, x.a, o);
-        r.b = __shfl_xor_sync(0xffffffffu, x.b, o);
-        r.c = __shfl_xor_sync(0xffffffffu, x.c, o);
-        r.i = __shfl_xor_sync(0xffffffffu, x.i, o);
-        return r;
-    };
-    for (int o = 16; o > 0; o >>= 1) v = op(v, shfl(v, o));
-    if (lane == 0) sm[wid] = v;
-    __syncthreads();
-    if (wid == 0) {
-        Red64 x;
-        x.a = x.b = x.c = ~0ull;
-        x.i = 0;
-        if (lane < NT / 32) x = sm[lane];
-        for (int o = 16; o > 0; o >>= 1) x = op(x, shfl(x, o));
-        if (lane == 0) sm[32] = x;
-    }
-    __syncthreads();
-    return sm[32];
-}
-
-// Selection reductions of precision 1 in one barrier: each warp reduces with
-// redux.sync (a 64-bit minimum as the minimum of the high words, then of the
-// low words among the lanes that hold it), lane 0 folds the warp's result
-// into the shared accumulator with atomics, one barrier, every thread reads
-// it.  The accumulator must hold the identity (reset_sel) before the first
-// atomic; the caller resets it only after a later barrier.
+// A 64-bit minimum over the warp by redux.sync: the minimum of the high words,
+// then of the low words among the lanes that hold it.
 __device__ __forceinline__ unsigned long long warp_min64(unsigned long long v) {
     const unsigned hi = (unsigned)(v >> 32);
     const unsigned mh = __reduce_min_sync(0xffffffffu, hi);
     const unsigned ml = __reduce_min_sync(0xffffffffu, hi == mh ? (unsigned)v : 0xffffffffu);
     return ((unsigned long long)mh << 32) | ml;
-}
-__device__ __forceinline__ void reset_sel(Red64 *acc) {
-    acc->a = acc->b = acc->c = ~0ull;
-    acc->i = 0;
-}
-__device__ __forceinline__ Red64 block_sel64(Red64 v, Red64 *acc) {
-    Red64 w;
-    w.a = warp_min64(v.a);
-    w.b = warp_min64(v.b);
-    w.c = warp_min64(v.c);
-    w.i = (int)__reduce_add_sync(0xffffffffu, (unsigned)v.i);
-    if ((threadIdx.x & 31) == 0) {
-        if (w.a != ~0ull) atomicMin(&acc->a, w.a);
-        if (w.b != ~0ull) atomicMin(&acc->b, w.b);
-        if (w.c != ~0ull) atomicMin(&acc->c, w.c);
-        if (w.i) atomicAdd(&acc->i, w.i);
-    }
-    __syncthreads();
-    return *acc;
 }
 
 // Exclusive prefix sum of one int per thread; *total = the block's sum.
@@ -582,8 +521,8 @@ struct In64 {
 struct Out64 {
     double dd;
     int tv;
-    double2 v;          // the merge's own evaluation: the new voltage, its magnitude, the cluster's extremes, its MICE
-    double mag, h, lo, m;
+    double2 v;          // the merge's own evaluation: the new voltage, its magnitude, the distances of the
+    double mag, up, dn, m;      // cluster's extremes above and below it, its MICE
 };
 __device__ __forceinline__ Out64 term_arith64(In64 x, double2 dv, bool one, bool moves, bool is_s, bool lv,
                                               double margin) {
@@ -592,7 +531,7 @@ __device__ __forceinline__ Out64 term_arith64(In64 x, double2 dv, bool one, bool
     double em = 0.0;
     Out64 r;
     r.v = make_double2(0.0, 0.0);
-    r.mag = r.h = r.lo = 0.0;
+    r.mag = r.up = r.dn = 0.0;
     if (one) {
         double2 v = x.v;
         if (moves) v = make_double2(__dadd_rn(v.x, dv.x), __dadd_rn(v.y, dv.y));
@@ -602,11 +541,11 @@ __device__ __forceinline__ Out64 term_arith64(In64 x, double2 dv, bool one, bool
             h = fmax(h, x.hr);
             lo = fmin(lo, x.lr);
         }
-        em = fmax(__dsub_rn(h, mag), __dsub_rn(mag, lo));
+        r.up = __dsub_rn(h, mag);
+        r.dn = __dsub_rn(mag, lo);
+        em = fmax(r.up, r.dn);
         r.v = v;
         r.mag = mag;
-        r.h = h;
-        r.lo = lo;
     }
     double m = fmax(em, __shfl_xor_sync(0xffffffffu, em, 1));
     m = fmax(m, __shfl_xor_sync(0xffffffffu, m, 2));
@@ -668,11 +607,13 @@ __device__ __forceinline__ Out64 group_term64(const Topo &T, const State &S, con
             iq[q] = (phr >> q & 1u) ? S.icur[sidx(li, q, c.r, n)] : make_double2(0.0, 0.0);
             za[q] = __ldg(T.zc + (size_t)c.a * 9 + pi * 3 + q);
         }
-        const double2 *zy = T.zc + (size_t)y * 9 + pi * 3;
+        // (every entry is loaded whatever the phases: one trip to L2, not three)
+        const double2 *zp = T.zc + (size_t)y * 9 + pi * 3;
+        const double2 zy[3] = {__ldg(zp), __ldg(zp + 1), __ldg(zp + 2)};
+#pragma unroll
         for (int q = 0; q < 3; ++q) {
             if (!(phr >> q & 1u)) continue;
-            const double2 zyq = __ldg(zy + q);
-            const double2 g = sside ? csub(zyq, za[q]) : csub(za[q], zyq);
+            const double2 g = sside ? csub(zy[q], za[q]) : csub(za[q], zy[q]);
             dv = cadd(dv, cmul(g, iq[q]));
         }
     }
@@ -810,10 +751,14 @@ __device__ __forceinline__ void group_term32(const Topo &T, const State &S, cons
             ha[q] = __ldg(T.zh + (size_t)c.a * 9 + pi * 3 + q);
             la[q] = __ldg(T.zlo + (size_t)c.a * 9 + pi * 3 + q);
         }
-        const float2 *zhy = T.zh + (size_t)y * 9 + pi * 3, *zly = T.zlo + (size_t)y * 9 + pi * 3;
+        // (every entry is loaded whatever the phases: one trip to L2, not three)
+        const float2 *zhp = T.zh + (size_t)y * 9 + pi * 3, *zlp = T.zlo + (size_t)y * 9 + pi * 3;
+        const float2 zhy[3] = {__ldg(zhp), __ldg(zhp + 1), __ldg(zhp + 2)};
+        const float2 zly[3] = {__ldg(zlp), __ldg(zlp + 1), __ldg(zlp + 2)};
+#pragma unroll
         for (int q = 0; q < 3; ++q) {
             if (!(phr >> q & 1u)) continue;
-            const float2 hy = __ldg(zhy + q), ly = __ldg(zly + q);
+            const float2 hy = zhy[q], ly = zly[q];
             float gx = (hy.x - ha[q].x) + (ly.x - la[q].x);
             float gy = (hy.y - ha[q].y) + (ly.y - la[q].y);
             if (!sside) { gx = -gx; gy = -gy; }
@@ -1187,7 +1132,7 @@ __device__ __forceinline__ long long commit_groups(const Topo &T, const State &S
                 o[0] = r.v.x;
                 o[1] = r.v.y;
                 o[2] = r.mag;
-                *cb_f4(cb, L, l, p) = make_float4((float)r.v.x, (float)r.v.y, (float)(r.h - r.mag), (float)(r.lo - r.mag));
+                *cb_f4(cb, L, l, p) = make_float4((float)r.v.x, (float)r.v.y, (float)r.up, 0.0f - (float)r.dn);
             }
             if (l < L && p == 0) {
                 cb[9 * L + l] = r.m;
@@ -1229,6 +1174,11 @@ __device__ __forceinline__ long long run_entries(const Topo &T, const State &S, 
         const bool both = pass == kMerge, apart = both && 2 * (q1 - q0) <= NG;
         const int tot = apart ? 2 * (q1 - q0) : q1 - q0;
         unsigned long long cq = (prof && tid == 0) ? clock64() : 0;
+        // the first items of the tile's entries, two a lane, when 64 hold them all
+        const bool near = ne <= 64;
+        int of0 = INT_MAX, of1 = INT_MAX;
+        if (near && (tid & 31) < ne) of0 = Lc.ent(t0 + (tid & 31))->off;
+        if (near && (tid & 31) + 32 < ne) of1 = Lc.ent(t0 + (tid & 31) + 32)->off;
         for (int r0 = 0; r0 < tot; r0 += NG) {
             if (r0 + ((tid >> 5) << (5 - lgG)) >= tot) break;     // this warp's groups are all past the end
             const int u = r0 + gi, q = q0 + (apart ? u >> 1 : u);
@@ -1237,9 +1187,17 @@ __device__ __forceinline__ long long run_entries(const Topo &T, const State &S, 
             int ei = 0, k = 0;
             Cand c;
             c.s = c.r = c.a = c.js = c.ns = c.jr = c.nr = c.fixed = 0;
+            // the entry holding item q: the last one whose first item is <= q
+            if (near) {
+                const int g0 = r0 + ((tid >> 5) << (5 - lgG));      // the warp's first group
+                for (int g = 0; g < (32 >> lgG); ++g) {
+                    const int qg = q0 + (apart ? (g0 + g) >> 1 : g0 + g);
+                    const int k2 = __popc(__ballot_sync(0xffffffffu, of0 <= qg)) + __popc(__ballot_sync(0xffffffffu, of1 <= qg));
+                    if (g0 + g == u) ei = k2 - 1;
+                }
+            }
             if (valid) {
-                // the entry holding item q: the last one whose first item is <= q
-                {
+                if (!near) {
                     int lo = 0, hi = ne - 1;
                     while (lo < hi) {
                         const int mid = (lo + hi + 1) >> 1;
@@ -1423,7 +1381,6 @@ struct __align__(16) PubCand {
     Cand c;
 };
 struct Pubs {
-    Pub w[16];                                          // by warp, within the CTA
     Pub a[kMaxCluster], c[kMaxCluster];                 // by CTA: pass A, the rescored candidates' minimum
     PubCand b[kMaxCluster], d[kMaxCluster];             // pass B, the rescored candidates' tie band
 };
@@ -1462,7 +1419,7 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
     static_assert(NT >= 128 && NT <= 512 && NT % 32 == 0, "thread count");
     __shared__ __align__(16) EvalSmem E;
     __shared__ __align__(16) Red sred[33];
-    __shared__ __align__(16) Red64 s_sel;       // precision-1 selection accumulator of pass B, a cluster of one
+    __shared__ Pub wpub[NT / 32];               // the warps' minima of a selection pass
     __shared__ int sscan[33];
     __shared__ unsigned long long s_sfx[2];     // SMICE of the committed state, fixed point
     __shared__ unsigned long long s_dsum[2];    // the last merge's change of it
@@ -1474,6 +1431,12 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
     const int max_merges = C->max_merges;
     const bool prof = C->profile != 0;
     const u128 tau_fx = to_fx(C->tau);
+    long long tau_dn, tau_up;                   // in key units, rounded down and up
+    {
+        bool ok;
+        tau_dn = key_val(key_floor(tau_fx, &ok));
+        tau_up = key_val(key_ceil(tau_fx, &ok));
+    }
     if (C->done || C->t >= max_merges) return;
     const int cr = cs == 1 ? 0 : cluster_rank(), lg = cs == 1 ? 0 : (cs == 2 ? 1 : (cs == 4 ? 2 : 3));
     const int np = own_pairs(n, cr, cs), pfirst = own_first(n, cr, cs);     // this CTA's slot pairs: w = cr, cr + cs, ...
@@ -1547,7 +1510,6 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
     int t = 0, ns = n;
     if (tid == 0) {
         s_sfx[0] = s_sfx[1] = 0ull;                 // every MICE starts at 0
-        reset_sel(&s_sel);
     }
     unsigned long long tp = 0;
     auto stamp = [&](int i) {
@@ -1681,10 +1643,10 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                     }
                 };
                 const Pub v = fold();
-                if (lane == 0) pub->w[wid] = v;
+                if (lane == 0) wpub[wid] = v;
                 __syncthreads();
                 if (wid == 0) {
-                    take(lane < NW, pub->w + lane);
+                    take(lane < NW, wpub + lane);
                     const Pub u = fold();
                     if (lane < cs) publish(&pub->a[cr], lane, &u, 2);
                 }
@@ -1766,7 +1728,7 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                     if (k <= ek) pa = umin(pa, ((u128)R.tkey[c] << 32) | (u128)(unsigned)slot_of(c));
                     else pb = umin(pb, k);
                 }
-                if (cs > 1) {
+                {
                     // (a tie key with its slot fits 64 bits)
                     unsigned long long qa = (unsigned long long)pa;
                     auto fold = [&]() {
@@ -1788,30 +1750,26 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                         }
                     };
                     const Pub v = fold();
-                    if (lane == 0) pub->w[wid] = v;
+                    if (lane == 0) wpub[wid] = v;
                     __syncthreads();
-                    if (wid == 0) {
-                        take(lane < NW, pub->w + lane);
-                        PubCand u;
-                        u.v = fold();
-                        u.c = Lc.slot[Lc.at(qa != ~0ull ? (int)(unsigned)qa : 2 * cr)];
-                        if (lane < cs) publish(&pub->b[cr], lane, &u, 5);
+                    if (cs > 1) {
+                        if (wid == 0) {
+                            take(lane < NW, wpub + lane);
+                            PubCand u;
+                            u.v = fold();
+                            u.c = Lc.slot[Lc.at(qa != ~0ull ? (int)(unsigned)qa : 2 * cr)];
+                            if (lane < cs) publish(&pub->b[cr], lane, &u, 5);
+                        }
+                        csync(cs);
+                        take(lane < cs, &pub->b[lane < cs ? lane : 0].v);
+                        const unsigned long long q0 = qa;
+                        fold();
+                        wc = pub->b[__ffs(__ballot_sync(0xffffffffu, q0 == qa && lane < cs)) - 1].c;
+                    } else {
+                        take(lane < NW, wpub + lane);
+                        fold();
                     }
-                    csync(cs);
-                    take(lane < cs, &pub->b[lane < cs ? lane : 0].v);
-                    const unsigned long long q0 = qa;
-                    fold();
-                    pa = (u128)qa;
-                    wc = pub->b[__ffs(__ballot_sync(0xffffffffu, q0 == qa && lane < cs)) - 1].c;
-                } else {
-                    Red rb;
-                    rb.a = pa;
-                    rb.b = pb;
-                    rb.c = kNone;
-                    rb.i = 0;
-                    rb = block_red<NT>(rb, sred);
-                    pa = rb.a;
-                    pb = rb.b;
+                    pa = qa == ~0ull ? kNone : (u128)qa;
                 }
             } else {
                 const u128 *bs = reinterpret_cast<const u128 *>(R.bsum);
@@ -1862,8 +1820,6 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
             if (tid == 0 && pb != kNone) gap = fx_to_d((pb ^ kSignBit) - edge);
         } else {
             const bool has_hi = ra.b != kNone;
-            bool ok;
-            const long long tau_dn = key_val(key_floor(tau_fx, &ok)), tau_up = key_val(key_ceil(tau_fx, &ok));
             const long long m_lo = key_val((unsigned long long)ra.a);
             const long long m_hi = has_hi ? key_val((unsigned long long)ra.b) : 0;
             const unsigned long long ein = val_key(m_lo + tau_dn);
@@ -1885,7 +1841,7 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                         pc = q.x < pc ? q.x : pc;
                     }
                 }
-                if (cs > 1) {
+                {
                     auto fold = [&]() {
                         Pub v;
                         v.a = pa = warp_min64(pa);
@@ -1904,30 +1860,25 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                         }
                     };
                     const Pub v = fold();
-                    if (lane == 0) pub->w[wid] = v;
+                    if (lane == 0) wpub[wid] = v;
                     __syncthreads();
-                    if (wid == 0) {
-                        take(lane < NW, pub->w + lane);
-                        PubCand u;
-                        u.v = fold();
-                        u.c = Lc.slot[Lc.at(pa != ~0ull ? (int)(unsigned)pa : 2 * cr)];
-                        if (lane < cs) publish(&pub->b[cr], lane, &u, 5);
+                    if (cs > 1) {
+                        if (wid == 0) {
+                            take(lane < NW, wpub + lane);
+                            PubCand u;
+                            u.v = fold();
+                            u.c = Lc.slot[Lc.at(pa != ~0ull ? (int)(unsigned)pa : 2 * cr)];
+                            if (lane < cs) publish(&pub->b[cr], lane, &u, 5);
+                        }
+                        csync(cs);
+                        take(lane < cs, &pub->b[lane < cs ? lane : 0].v);
+                        const unsigned long long p0 = pa;
+                        fold();
+                        wc = pub->b[__ffs(__ballot_sync(0xffffffffu, p0 == pa && lane < cs)) - 1].c;
+                    } else {
+                        take(lane < NW, wpub + lane);
+                        fold();
                     }
-                    csync(cs);
-                    take(lane < cs, &pub->b[lane < cs ? lane : 0].v);
-                    const unsigned long long p0 = pa;
-                    fold();
-                    wc = pub->b[__ffs(__ballot_sync(0xffffffffu, p0 == pa && lane < cs)) - 1].c;
-                } else {
-                    Red64 r6;
-                    r6.a = pa;
-                    r6.b = pb;
-                    r6.c = pc;
-                    r6.i = 0;
-                    r6 = block_sel64(r6, &s_sel);
-                    pa = r6.a;
-                    pb = r6.b;
-                    pc = r6.c;
                 }
             } else {
                 const ulonglong2 *bs = reinterpret_cast<const ulonglong2 *>(R.bsum);
@@ -1973,20 +1924,23 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
                         ++kq;
                     }
                 }
-                if (few) {
-                    pa = warp_min64(pa);
-                    pb = warp_min64(pb);
-                    pc = warp_min64(pc);
-                } else {
-                    Red64 r6;
-                    r6.a = pa;
-                    r6.b = pb;
-                    r6.c = pc;
-                    r6.i = 0;
-                    r6 = block_sel64(r6, &s_sel);
-                    pa = r6.a;
-                    pb = r6.b;
-                    pc = r6.c;
+                pa = warp_min64(pa);
+                pb = warp_min64(pb);
+                pc = warp_min64(pc);
+                if (!few) {
+                    if (lane == 0) {
+                        Pub v;
+                        v.a = pa;
+                        v.b = pb;
+                        v.c = pc;
+                        v.d = 0;
+                        wpub[wid] = v;
+                    }
+                    __syncthreads();
+                    const Pub u = wpub[lane < NW ? lane : 0];
+                    pa = warp_min64(u.a);
+                    pb = warp_min64(u.b);
+                    pc = warp_min64(u.c);
                 }
             }
             Red rb;
@@ -2205,7 +2159,6 @@ __device__ void inc_run(const Topo &T, const State &S, const Search &X, const In
         csync(cs);
         ns -= 1;
         const int ne = (int)(unsigned)s_app[0], items = (int)(s_app[0] >> 32);
-        if (PREC == 1 && tid == 0) reset_sel(&s_sel);     // every thread has read the selection's result
         stamp(1);
         // ============================================================ the terms that change, and the score
         {
