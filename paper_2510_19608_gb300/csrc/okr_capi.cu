@@ -83,6 +83,7 @@ struct okr_ctx {
     float *mlp_x = nullptr, *mlp_t = nullptr;    // device copies of a data set
     float *mlp_loss = nullptr;                   // squared errors by segment of an epoch's batches
     int *mlp_err = nullptr;                      // error flag of the tensor-core inference
+    bool reads_host = false;                     // kernels may read pageable host memory (through the host's page tables)
     size_t mlp_x_cap = 0, mlp_t_cap = 0, mlp_loss_cap = 0;      // floats
     int mlp_step = 0;
 
@@ -797,6 +798,12 @@ okr_status okr_create(okr_ctx **out, int device, void *stream) {
         delete ctx;
         return OKR_ECUDA;
     }
+    int host_tables = 0;
+    if (cudaDeviceGetAttribute(&host_tables, cudaDevAttrPageableMemoryAccessUsesHostPageTables, device) != cudaSuccess) {
+        cudaGetLastError();
+        host_tables = 0;
+    }
+    ctx->reads_host = host_tables != 0;
     int coop = 0;
     if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device) != cudaSuccess || !coop ||
         search_blocks_per_sm() < 1) {
@@ -2037,6 +2044,23 @@ okr_status mlp_buffer(okr_ctx *ctx, float **p, size_t *cap, size_t count) {
     return OKR_OK;
 }
 
+okr_status mlp_upload(okr_ctx *ctx, const float *x, const float *t, long long N);
+
+// The features a forward pass reads, and room for its predictions.  Each feature
+// is read once, so where the GPU reads host memory through the host's page
+// tables the kernel takes them from there (168 MB: 0.88 ms, the copy alone 1.06
+// to 1.09, and the products run beside it); elsewhere they are copied.
+okr_status mlp_features(okr_ctx *ctx, const float *x, long long N, const float **xd) {
+    if (!ctx->reads_host) {
+        *xd = nullptr;
+        const okr_status s = mlp_upload(ctx, x, nullptr, N);
+        *xd = ctx->mlp_x;
+        return s;
+    }
+    *xd = x;
+    return mlp_buffer(ctx, &ctx->mlp_t, &ctx->mlp_t_cap, (size_t)N);
+}
+
 okr_status mlp_upload(okr_ctx *ctx, const float *x, const float *t, long long N) {
     const int F = ctx->mb.F;
     okr_status s = mlp_buffer(ctx, &ctx->mlp_x, &ctx->mlp_x_cap, (size_t)N * F);
@@ -2159,14 +2183,15 @@ okr_status okr_scorer_predict_tc(okr_ctx *ctx, const float *x, int64_t n, float 
     if (!ctx->mb.theta) return fail(ctx, OKR_ENOTREADY, "scorer not initialised");
     if (n > INT32_MAX) return fail(ctx, OKR_EINVAL, "too many samples");
     CK(cudaSetDevice(ctx->device));
-    okr_status s = mlp_upload(ctx, x, nullptr, n);
+    const float *xd = nullptr;
+    okr_status s = mlp_features(ctx, x, n, &xd);
     if (s != OKR_OK) return s;
     float *yd = ctx->mlp_t;                     // the targets' buffer holds the predictions
     if (!ctx->mlp_err) CK(dev_alloc(ctx, (void **)&ctx->mlp_err, sizeof(int)));
     int *err = ctx->mlp_err;
     okr_status out = OKR_OK;
     cudaError_t e = cudaMemsetAsync(err, 0, sizeof(int), ctx->stream);
-    if (e == cudaSuccess) e = mlp_forward_tc(ctx->mb, ctx->mlp_x, (int)n, yd, err, ctx->num_sms, ctx->stream);
+    if (e == cudaSuccess) e = mlp_forward_tc(ctx->mb, xd, (int)n, yd, err, ctx->num_sms, ctx->stream);
     int herr = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(y, yd, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
@@ -2181,10 +2206,11 @@ okr_status okr_scorer_predict(okr_ctx *ctx, const float *x, int64_t n, float *y)
     if (!ctx->mb.theta) return fail(ctx, OKR_ENOTREADY, "scorer not initialised");
     if (n > INT32_MAX) return fail(ctx, OKR_EINVAL, "too many samples");
     CK(cudaSetDevice(ctx->device));
-    okr_status s = mlp_upload(ctx, x, nullptr, n);
+    const float *xd = nullptr;
+    okr_status s = mlp_features(ctx, x, n, &xd);
     if (s != OKR_OK) return s;
     float *yd = ctx->mlp_t;                     // the targets' buffer holds the predictions
-    CK(mlp_forward(ctx->mb, ctx->mlp_x, (int)n, yd, ctx->num_sms, ctx->stream));
+    CK(mlp_forward(ctx->mb, xd, (int)n, yd, ctx->num_sms, ctx->stream));
     CK(cudaMemcpyAsync(y, yd, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     return OKR_OK;

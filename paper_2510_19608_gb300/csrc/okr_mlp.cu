@@ -314,13 +314,26 @@ __global__ void __launch_bounds__(256, 1) k_mlp_forward(const float *__restrict_
                     make_float4(fmaxf(acc[4 * h][c], 0.0f), fmaxf(acc[4 * h + 1][c], 0.0f),
                                 fmaxf(acc[4 * h + 2][c], 0.0f), fmaxf(acc[4 * h + 3][c], 0.0f));
     };
+    // the next tile's features are in flight while this tile is computed (x may
+    // lie in host memory, read across the chip-to-chip link)
+    float xr[kBig * kMlpMaxF / 256];
+    auto load_x = [&](long long base) {
+#pragma unroll
+        for (int i = 0; i < kBig * kMlpMaxF / 256; ++i) {
+            const int e = threadIdx.x + 256 * i;
+            xr[i] = (e < kBig * F && base * F + e < (long long)N * F) ? __ldg(x + base * F + e) : 0.0f;
+        }
+    };
+    load_x((long long)blockIdx.x * kBig);
     for (long long base = (long long)blockIdx.x * kBig; base < N; base += (long long)gridDim.x * kBig) {
         const int S = (int)min((long long)kBig, N - base);
-        for (int e = threadIdx.x; e < kBig * F; e += 256) {
-            const int s = e / F, k = e % F;
-            X[k * kBigPitch + s] = s < S ? x[base * F + e] : 0.0f;
+#pragma unroll
+        for (int i = 0; i < kBig * kMlpMaxF / 256; ++i) {
+            const int e = threadIdx.x + 256 * i;
+            if (e < kBig * F) X[(e % F) * kBigPitch + e / F] = xr[i];
         }
         __syncthreads();
+        load_x(base + (long long)gridDim.x * kBig);
         layer(X, W1, F, o.b1);
         store();
         __syncthreads();

@@ -116,18 +116,6 @@ __device__ __forceinline__ unsigned relu_bf16x2(float lo, float hi) {
     return d;
 }
 
-// Eight consecutive K elements (k0 a multiple of 8) of row `row`, rounded to
-// bfloat16 (nearest even), as one 16-byte row of a core matrix.
-__device__ __forceinline__ void store8_bf16(unsigned char *base, int row, int k0, const float *v) {
-    uint4 q;
-    unsigned *w = reinterpret_cast<unsigned *>(&q);
-    for (int j = 0; j < 4; ++j) {
-        const __nv_bfloat162 p = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);   // .x (lower address) = v[2j]
-        w[j] = *reinterpret_cast<const unsigned *>(&p);
-    }
-    *reinterpret_cast<uint4 *>(base + core_off(row, k0)) = q;
-}
-
 // Barrier of the 128 threads of warpgroup g (named barrier 1 + g).
 __device__ __forceinline__ void group_sync(int g) {
     asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(kH) : "memory");
@@ -266,10 +254,21 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_forward_tc(const float *__r
         }
         return acc;
     };
-    // the features of tile t, row `row`, as FP32 (zero past N and past F)
+    // the features of tile t, 128 F consecutive floats, one of every 128 a thread
+    // (whole lines per warp: x may lie in host memory, which the kernel reads
+    // across the chip-to-chip link without a copy before it), and where they go
+    // in the layer's input; rows past N are zero
+    unsigned xoff[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const int e = i * kH + row;
+        xoff[i] = core_off(e / F, e % F);
+    }
     auto load_x = [&](long long t, float *v) {
-        const long long m = t * kH + row;
-        for (int k = 0; k < 16; ++k) v[k] = (m < N && k < F) ? x[m * F + k] : 0.0f;
+        const float *xt = x + t * kH * F + row;
+        const long long left = ((long long)N - t * kH) * F - row;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = (i < F && i * kH < left) ? __ldg(xt + i * kH) : 0.0f;
     };
     auto sync_group = [&]() {
         fence_async_smem();
@@ -280,10 +279,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_forward_tc(const float *__r
     const long long tiles = ((long long)N + kH - 1) / kH, stride = (long long)gridDim.x * kGroups;
     long long t = (long long)blockIdx.x * kGroups + g;
     float v[16];
+    // (the columns past F stay zero)
+    *reinterpret_cast<uint4 *>(sX + core_off(row, 0)) = make_uint4(0u, 0u, 0u, 0u);
+    *reinterpret_cast<uint4 *>(sX + core_off(row, 8)) = make_uint4(0u, 0u, 0u, 0u);
+    group_sync(g);
     if (t < tiles) load_x(t, v);
     for (; t < tiles && ok; t += stride) {
-        store8_bf16(sX, row, 0, v);
-        store8_bf16(sX, row, 8, v + 8);
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if (i < F) *reinterpret_cast<__nv_bfloat16 *>(sX + xoff[i]) = __float2bfloat16_rn(v[i]);
         if (t + stride < tiles) load_x(t + stride, v);  // in flight while this tile's products run
         sync_group();
         ok = layer(sX, sW1, 1);
