@@ -1109,6 +1109,8 @@ okr_status batch_status_of_setup(int e) {
 struct BatchRun {
     int nf = 0, config = 0, team = 1, max_teams = 1, maxL = 1, ctas = 0;
     IncShape shape{0, 0, 0, -1};                    // incremental engine: launch shape (resolved)
+    int clusters[2] = {0, 0};                       // ... by precision: feeders searched by clusters, and the
+    IncPlan plan[2][2]{};                           // launches' plans (clusters, one CTA each)
     long long max_nn = 1, tot_n = 0;
     int per_sm[2] = {0, 0};
     std::vector<int> merges, nbus, nscen, ord[4];
@@ -1206,7 +1208,7 @@ static okr_status batch_measure(okr_ctx *ctx, int32_t nf, const okr_feeder *feed
         for (int f : R.ord[g]) max_n = std::max(max_n, R.nbus[f]);
         int rec = 0;
         size_t bytes = 0;
-        if (!inc_smem(max_n, false, R.shape, &rec, &bytes))
+        if (!inc_smem(max_n, false, R.shape, &rec, &bytes))     // (one CTA's placement decides, also for a cluster)
             return fail(ctx, OKR_EINVAL, "batch: the incremental shape's record placement does not fit (%d buses; "
                                          "the largest MICE per super-node is single-feeder only)", max_n);
     }
@@ -1383,7 +1385,20 @@ static okr_status batch_fill(okr_ctx *ctx, BatchRun &R, const okr_feeder *feeder
         int max_n = 2;
         for (int f : R.ord[g]) max_n = std::max(max_n, R.nbus[f]);
         if (!R.ord[g].empty()) {
-            CK(prepare_search_inc_batch(g - 2, max_n, R.shape));
+            // the largest by clusters, the others by one CTA each beside them
+            std::vector<int> nb, mg;
+            for (int f : R.ord[g]) {
+                nb.push_back(R.nbus[f]);
+                mg.push_back(R.merges[f]);
+            }
+            int k = 0, cs = 1;
+            inc_batch_clusters(g - 2, (int)nb.size(), nb.data(), mg.data(), ctx->num_sms, ctx->inc_shape, &k, &cs);
+            R.clusters[g - 2] = k;
+            if ((k > 0 && !inc_batch_plan(*std::max_element(nb.begin(), nb.begin() + k), cs, ctx->inc_shape, &R.plan[g - 2][0])) ||
+                (k < (int)nb.size() && !inc_batch_plan(*std::max_element(nb.begin() + k, nb.end()), 1, ctx->inc_shape, &R.plan[g - 2][1])))
+                return fail(ctx, OKR_EINTERNAL, "batch: no launch plan");
+            if (k > 0) CK(prepare_search_inc_batch(g - 2, R.plan[g - 2][0]));
+            if (k < (int)nb.size()) CK(prepare_search_inc_batch(g - 2, R.plan[g - 2][1]));
             CK(prepare_inc_init_batch(g - 2, max_n));
         }
     }
@@ -1405,13 +1420,29 @@ static okr_status batch_enqueue(okr_ctx *ctx, BatchRun &R, cudaStream_t st, bool
     for (int g = 0, first = 0; g < 4; first += (int)R.ord[g].size(), ++g) {
         const int cnt = (int)R.ord[g].size();
         if (cnt == 0) continue;
-        if (g >= 2) {                           // one CTA per feeder
-            R.ctas = std::max(R.ctas, cnt);
+        if (g >= 2) {
             int max_n = 2;
             for (int f : R.ord[g]) max_n = std::max(max_n, R.nbus[f]);
-            CK(launch_inc_init_batch(g - 2, max_n, R.bf_d, R.order_d + first, R.ictas_d + first, cnt,
-                                     R.init_ctas[g - 2], st));
-            CK(launch_search_inc_batch(g - 2, max_n, R.bf_d, R.order_d + first, cnt, R.shape, st));
+            const int k = R.clusters[g - 2];
+            const IncPlan *pl = R.plan[g - 2];
+            // the clusters' feeders first, on the side stream: they hold their SMs
+            // before the others' first evaluations are done and take the rest
+            int c0 = 0;
+            for (int i = 0; i < k; ++i) c0 += inc_init_batch_ctas(R.nbus[R.ord[g][i]]);
+            if (k > 0) {
+                CK(launch_inc_init_batch(g - 2, max_n, R.bf_d, R.order_d + first, R.ictas_d + first, k, 0, c0, st));
+                CK(cudaEventRecord(R.ev_fork, st));
+                CK(cudaStreamWaitEvent(ctx->side, R.ev_fork, 0));
+                CK(launch_search_inc_batch(g - 2, R.bf_d, R.order_d + first, k, pl[0], ctx->side));
+                CK(cudaEventRecord(R.ev_join, ctx->side));
+            }
+            if (k < cnt) {
+                CK(launch_inc_init_batch(g - 2, max_n, R.bf_d, R.order_d + first + k, R.ictas_d + first + k, cnt - k, c0,
+                                         R.init_ctas[g - 2] - c0, st));
+                CK(launch_search_inc_batch(g - 2, R.bf_d, R.order_d + first + k, cnt - k, pl[1], st));
+            }
+            if (k > 0) CK(cudaStreamWaitEvent(st, R.ev_join, 0));
+            R.ctas = std::max(R.ctas, (k > 0 ? k * pl[0].cs : 0) + cnt - k);
             continue;
         }
         const int nteams = std::min(cnt, ctx->num_sms * R.per_sm[g] / R.team);

@@ -43,8 +43,8 @@
 // score it needs; those are evaluated in FP64 from scratch.  Merges are always
 // applied in FP64.
 //
-// Execution.  One CTA (a batch, a tiny feeder) or one cluster of eight runs a
-// feeder's whole search; its steps are separated by block or cluster barriers
+// Execution.  One cluster of eight CTAs (inc_plan; in a batch one CTA, or a
+// cluster for the longest searches, inc_batch_clusters) runs a feeder's whole search; its steps are separated by block or cluster barriers
 // only (no grid barrier, no device-side wait).  The chain of dependent merges
 // bounds it: neither a pipe nor memory is busy, so what counts is the number of
 // dependent steps per merge and the latency of each.  A term is evaluated by a
@@ -65,6 +65,7 @@
 #include "okr_kernels.cuh"
 
 #include <climits>
+#include <type_traits>
 
 namespace okr {
 
@@ -1412,10 +1413,14 @@ __host__ __device__ constexpr int own_first(int n, int cr, int cs) {
 }
 
 // rec_mode: where the selection records live (k_search_inc); + 4: the
-// candidates and carried sums in shared memory too.
-template <int NT, int PREC>
+// candidates and carried sums in shared memory too.  CS: CTAs of the search, a
+// constant: one kernel for both kinds holds the code of both selections, and
+// the instructions of a merge, executed once each, miss the instruction cache
+// (16 % of the stalls): a batch's search was 3 to 7 % slower with CS a variable.
+template <int NT, int PREC, int CS>
 __device__ void inc_run(const Topo &T, const State &S, const Search &X, const Inc &I, Ctrl *C, bool verify,
-                        unsigned char *dyn, int rec_mode, int se, int cw, int cs) {
+                        unsigned char *dyn, int rec_mode, int se, int cw) {
+    constexpr int cs = CS;
     static_assert(NT >= 128 && NT <= 512 && NT % 32 == 0, "thread count");
     __shared__ __align__(16) EvalSmem E;
     __shared__ __align__(16) Red sred[33];
@@ -2276,20 +2281,20 @@ namespace {
 // in I.recbuf; 1: in shared memory; 2: in shared memory, with the largest MICE
 // per super-node.  se: work entries in shared memory; cw: warps that evaluate
 // the merge beside the changed-set scan.
-template <int NT, int PREC>
+template <int NT, int PREC, int CS>
 __global__ void __launch_bounds__(NT, 1) k_search_inc(Topo T, State S, Search X, Inc I, Ctrl *C, int verify,
-                                                      int rec_mode, int se, int cw, int cs) {
+                                                      int rec_mode, int se, int cw) {
     extern __shared__ __align__(16) unsigned char inc_dyn[];
     if (X.setup_err && *X.setup_err != 0) return;           // the setup failed: no result (C->done stays 0)
-    inc_run<NT, PREC>(T, S, X, I, C, verify != 0, inc_dyn, rec_mode, se, cw, cs);
+    inc_run<NT, PREC, CS>(T, S, X, I, C, verify != 0, inc_dyn, rec_mode, se, cw);
 }
 
 // The first evaluation of every candidate (every slot pair from the initial
 // clusters, all singletons, every term), which needs no merge before it: its
-// work is spread over many CTAs instead of the one CTA of the search.  The
+// work is spread over many CTAs instead of the search's one to eight.  The
 // CTAs write the candidates, carried sums and tie keys to device memory, in
-// the layout the search reads (k_search_inc with pre_init copies the records
-// into shared memory and derives the selection keys from the sums).  The
+// the layout the search reads (it copies its records into shared memory and
+// derives the selection keys from the sums).  The
 // terms are evaluated by the same code as in the search, so the carried sums
 // are the ones the search's own first evaluation gives.
 constexpr int kInitPairs = kIncInitPairs;
@@ -2456,7 +2461,7 @@ __global__ void __launch_bounds__(NT) k_inc_init(Topo T, State S, Search X, Inc 
 // every feeder start at zero (k_inc_zero_batch).
 template <int NT, int PREC>
 __global__ void __launch_bounds__(NT) k_inc_init_batch(const BatchFeeder *fd, const int *order, const int *cta_off,
-                                                       int nf) {
+                                                       int nf, int cta0) {
     extern __shared__ __align__(16) unsigned char init_dyn[];
     __shared__ __align__(16) EvalSmem E;
     __shared__ int sscan[33];
@@ -2467,7 +2472,7 @@ __global__ void __launch_bounds__(NT) k_inc_init_batch(const BatchFeeder *fd, co
     __shared__ Search sX;
     __shared__ Inc sI;
     __shared__ int s_f, s_b, s_B;
-    const int b = blockIdx.x;
+    const int b = blockIdx.x + cta0;             // (cta0: the first CTA of the launch's first feeder)
     if (threadIdx.x == 0) {
         int lo = 0, hi = nf - 1;                 // the last feeder whose first CTA is <= b
         while (lo < hi) {
@@ -2478,7 +2483,7 @@ __global__ void __launch_bounds__(NT) k_inc_init_batch(const BatchFeeder *fd, co
         const int f = order[lo];
         s_f = f;
         s_b = b - cta_off[lo];
-        s_B = (lo + 1 < nf ? cta_off[lo + 1] : (int)gridDim.x) - cta_off[lo];
+        s_B = (lo + 1 < nf ? cta_off[lo + 1] : (int)gridDim.x + cta0) - cta_off[lo];
         sT = fd[f].T;
         sS = fd[f].S;
         sX = fd[f].X;
@@ -2493,7 +2498,7 @@ __global__ void __launch_bounds__(NT) k_inc_init_batch(const BatchFeeder *fd, co
 // The carried sums, violation counts and their bounds of every feeder of the
 // order set to zero before its first evaluation adds to them (one CTA per
 // feeder).
-__global__ void k_inc_zero_batch(const BatchFeeder *fd, const int *order, int nf) {
+static __global__ void k_inc_zero_batch(const BatchFeeder *fd, const int *order, int nf) {
     const int q = blockIdx.x;
     if (q >= nf) return;
     const Inc &I = fd[order[q]].I;
@@ -2503,16 +2508,17 @@ __global__ void k_inc_zero_batch(const BatchFeeder *fd, const int *order, int nf
     for (size_t i = threadIdx.x; i < bytes / 4; i += blockDim.x) reinterpret_cast<unsigned *>(p0)[i] = 0u;
 }
 
-// One CTA per feeder, feeders in the order given (largest first).
-template <int NT, int PREC>
+// One CTA or cluster (of CS CTAs) per feeder, feeders in the order given (largest first).
+template <int NT, int PREC, int CS>
 __global__ void __launch_bounds__(NT) k_search_inc_batch(const BatchFeeder *fd, const int *order, int nf,
                                                          int rec_mode, int se, int cw) {
+    constexpr int cs = CS;
     extern __shared__ __align__(16) unsigned char inc_dyn[];
     __shared__ Topo sT;
     __shared__ State sS;
     __shared__ Search sX;
     __shared__ Inc sI;
-    const int q = blockIdx.x;
+    const int q = blockIdx.x / cs;
     if (q >= nf) return;
     const int f = order[q];
     if (threadIdx.x == 0) {
@@ -2524,8 +2530,9 @@ __global__ void __launch_bounds__(NT) k_search_inc_batch(const BatchFeeder *fd, 
     __syncthreads();
     Ctrl *C = fd[f].C;
     const bool ok = *fd[f].setup_err == 0;
-    if (ok) inc_run<NT, PREC>(sT, sS, sX, sI, C, false, inc_dyn, rec_mode, se, cw, 1);
-    __syncthreads();
+    if (ok) inc_run<NT, PREC, CS>(sT, sS, sX, sI, C, false, inc_dyn, rec_mode, se, cw);
+    csync(cs);                              // (every CTA's labels)
+    if (cs > 1 && cluster_rank() != 0) return;
     for (int i = threadIdx.x; i < sT.n; i += NT) fd[f].super_out[i] = ok ? sT.orig[sS.label[sT.pre[i]]] : -1;
     if (threadIdx.x == 0) {
         const int t = ok ? C->t : 0;
@@ -2536,6 +2543,7 @@ __global__ void __launch_bounds__(NT) k_search_inc_batch(const BatchFeeder *fd, 
 constexpr size_t kIncSmemMax = 200 * 1024;  // largest dynamic shared memory of one search
 constexpr int kInitThreads = 384;           // CTAs of the first evaluation
 constexpr int kClusterMin = 32;             // buses from which a cluster searches (inc_plan)
+constexpr int kBatchCluster = 500;          // ... one of a batch's feeders (inc_batch_clusters)
 
 template <typename K>
 cudaError_t set_smem(K kern, size_t bytes) {
@@ -2543,6 +2551,19 @@ cudaError_t set_smem(K kern, size_t bytes) {
 }
 
 }  // namespace
+
+// The launches of one precision: its kernels are compiled in a translation unit
+// of their own (okr_incr64.cu includes this file for the FP64 terms), so that
+// the two compile side by side.
+template <int PREC> cudaError_t launch_one_prec(Topo T, State S, Search X, Inc I, Ctrl *C, int verify, const IncPlan &pl, cudaStream_t st);
+template <int PREC> cudaError_t prepare_batch_prec(const IncPlan &pl);
+template <int PREC> cudaError_t launch_batch_prec(const BatchFeeder *fd, const int *order, int nf, const IncPlan &pl, cudaStream_t st);
+template <int PREC> int batch_clusters_prec(const IncPlan &pl);          // clusters of the plan resident at once
+template <int PREC> cudaError_t prepare_init_prec(size_t ismem);
+template <int PREC> void launch_init_prec(const BatchFeeder *fd, const int *order, const int *cta_off, int nf, int cta0, int ctas,
+                                          size_t ismem, cudaStream_t st);
+
+#ifndef OKR_INCR_FP64
 
 IncShape inc_shape_resolve(IncShape sh) {
     if (sh.threads != 256 && sh.threads != 384 && sh.threads != 512) sh.threads = kIncDefaultThreads;
@@ -2601,7 +2622,32 @@ bool inc_plan(int n, const IncShape &raw, bool records_iters, IncPlan *out) {
     return true;
 }
 
+#endif
+
 namespace {
+
+cudaLaunchConfig_t search_config(int ctas, int threads, int cs, size_t bytes, cudaStream_t st, cudaLaunchAttribute *at) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ctas);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = bytes;
+    cfg.stream = st;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = (unsigned)cs;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = cs > 1 ? 1 : 0;
+    return cfg;
+}
+
+template <int NT, int PREC, int CS>
+cudaError_t launch_cs(Topo T, State S, Search X, Inc I, Ctrl *C, int verify, const IncPlan &pl, cudaStream_t st) {
+    const cudaError_t e = set_smem(k_search_inc<NT, PREC, CS>, pl.bytes);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at[1];
+    const cudaLaunchConfig_t cfg = search_config(CS, NT, CS, pl.bytes, st, at);
+    return cudaLaunchKernelEx(&cfg, k_search_inc<NT, PREC, CS>, T, S, X, I, C, verify, pl.mode, pl.sh.se, pl.sh.cw);
+}
 
 template <int NT, int PREC>
 cudaError_t launch_one(Topo T, State S, Search X, Inc I, Ctrl *C, int verify, const IncPlan &pl, cudaStream_t st) {
@@ -2621,86 +2667,171 @@ cudaError_t launch_one(Topo T, State S, Search X, Inc I, Ctrl *C, int verify, co
     if (e == cudaSuccess && ismem > 48 * 1024) e = set_smem(k_inc_init<kInitThreads, PREC>, ismem);
     if (e == cudaSuccess) k_inc_init<kInitThreads, PREC><<<ginit, kInitThreads, ismem, st>>>(T, S, X, I, C);
     if (e == cudaSuccess) e = cudaGetLastError();
-    if (e == cudaSuccess) e = set_smem(k_search_inc<NT, PREC>, pl.bytes);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)pl.cs);
-    cfg.blockDim = dim3(NT);
-    cfg.dynamicSmemBytes = pl.bytes;
-    cfg.stream = st;
+    if (pl.cs == 1) return launch_cs<NT, PREC, 1>(T, S, X, I, C, verify, pl, st);
+    return launch_cs<NT, PREC, kMaxCluster>(T, S, X, I, C, verify, pl, st);
+}
+
+template <int NT, int PREC, int CS>
+cudaError_t launch_batch(const BatchFeeder *fd, const int *order, int nf, const IncPlan &pl, cudaStream_t st) {
     cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)pl.cs;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_search_inc<NT, PREC>, T, S, X, I, C, verify,
-                              pl.mode, pl.sh.se, pl.sh.cw, pl.cs);
+    const cudaLaunchConfig_t cfg = search_config(nf * CS, NT, CS, pl.bytes, st, at);
+    return cudaLaunchKernelEx(&cfg, k_search_inc_batch<NT, PREC, CS>, fd, order, nf, pl.mode, pl.sh.se, pl.sh.cw);
 }
 
-template <int NT>
-cudaError_t set_batch_smem(int precision, size_t smem) {
-    return precision == 1 ? set_smem(k_search_inc_batch<NT, 1>, smem) : set_smem(k_search_inc_batch<NT, 0>, smem);
+// The batch kernels: one CTA of 256, 384 or 512 threads, clusters of two of 384
+// and of eight of 256 (inc_batch_plan).
+template <int PREC, typename F>
+cudaError_t batch_kernels(int cs, int threads, F f) {
+    if (cs == kMaxCluster) return f(std::integral_constant<int, 256>(), std::integral_constant<int, kMaxCluster>());
+    if (cs == 2) return f(std::integral_constant<int, 384>(), std::integral_constant<int, 2>());
+    if (threads == 256) return f(std::integral_constant<int, 256>(), std::integral_constant<int, 1>());
+    if (threads == 384) return f(std::integral_constant<int, 384>(), std::integral_constant<int, 1>());
+    return f(std::integral_constant<int, 512>(), std::integral_constant<int, 1>());
 }
-
-template <int NT>
-void launch_batch(int precision, const BatchFeeder *fd, const int *order, int nf, int use, size_t smem,
-                  const IncShape &sh, cudaStream_t st) {
-    if (precision == 1) k_search_inc_batch<NT, 1><<<nf, NT, smem, st>>>(fd, order, nf, use, sh.se, sh.cw);
-    else k_search_inc_batch<NT, 0><<<nf, NT, smem, st>>>(fd, order, nf, use, sh.se, sh.cw);
-}
-
 }  // namespace
+
+template <int PREC>
+cudaError_t launch_one_prec(Topo T, State S, Search X, Inc I, Ctrl *C, int verify, const IncPlan &pl, cudaStream_t st) {
+    if (pl.sh.threads == 256) return launch_one<256, PREC>(T, S, X, I, C, verify, pl, st);
+    if (pl.sh.threads == 384) return launch_one<384, PREC>(T, S, X, I, C, verify, pl, st);
+    return launch_one<512, PREC>(T, S, X, I, C, verify, pl, st);
+}
+template <int PREC>
+cudaError_t prepare_batch_prec(const IncPlan &pl) {
+    return batch_kernels<PREC>(pl.cs, pl.sh.threads, [&](auto nt, auto c) {
+        return set_smem(k_search_inc_batch<decltype(nt)::value, PREC, decltype(c)::value>, pl.bytes);
+    });
+}
+template <int PREC>
+cudaError_t launch_batch_prec(const BatchFeeder *fd, const int *order, int nf, const IncPlan &pl, cudaStream_t st) {
+    return batch_kernels<PREC>(pl.cs, pl.sh.threads, [&](auto nt, auto c) {
+        return launch_batch<decltype(nt)::value, PREC, decltype(c)::value>(fd, order, nf, pl, st);
+    });
+}
+template <int PREC>
+int batch_clusters_prec(const IncPlan &pl) {
+    int count = 0;
+    const cudaError_t e = batch_kernels<PREC>(pl.cs, pl.sh.threads, [&](auto nt, auto c) {
+        constexpr int cs = decltype(c)::value;
+        const auto kern = k_search_inc_batch<decltype(nt)::value, PREC, cs>;
+        cudaLaunchAttribute at[1];
+        const cudaLaunchConfig_t cfg = search_config(cs, decltype(nt)::value, cs, pl.bytes, nullptr, at);
+        const cudaError_t e1 = set_smem(kern, pl.bytes);
+        return e1 != cudaSuccess ? e1 : cudaOccupancyMaxActiveClusters(&count, kern, &cfg);
+    });
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess ? count : 0;
+}
+template <int PREC>
+cudaError_t prepare_init_prec(size_t ismem) {
+    return set_smem(k_inc_init_batch<kInitThreads, PREC>, ismem);
+}
+template <int PREC>
+void launch_init_prec(const BatchFeeder *fd, const int *order, const int *cta_off, int nf, int cta0, int ctas, size_t ismem,
+                      cudaStream_t st) {
+    k_inc_init_batch<kInitThreads, PREC><<<ctas, kInitThreads, ismem, st>>>(fd, order, cta_off, nf, cta0);
+}
+
+#ifdef OKR_INCR_FP64
+
+template cudaError_t launch_one_prec<0>(Topo, State, Search, Inc, Ctrl *, int, const IncPlan &, cudaStream_t);
+template cudaError_t prepare_batch_prec<0>(const IncPlan &);
+template cudaError_t launch_batch_prec<0>(const BatchFeeder *, const int *, int, const IncPlan &, cudaStream_t);
+template int batch_clusters_prec<0>(const IncPlan &);
+template cudaError_t prepare_init_prec<0>(size_t);
+template void launch_init_prec<0>(const BatchFeeder *, const int *, const int *, int, int, int, size_t, cudaStream_t);
+
+#else
+
+extern template cudaError_t launch_one_prec<0>(Topo, State, Search, Inc, Ctrl *, int, const IncPlan &, cudaStream_t);
+extern template cudaError_t prepare_batch_prec<0>(const IncPlan &);
+extern template cudaError_t launch_batch_prec<0>(const BatchFeeder *, const int *, int, const IncPlan &, cudaStream_t);
+extern template int batch_clusters_prec<0>(const IncPlan &);
+extern template cudaError_t prepare_init_prec<0>(size_t);
+extern template void launch_init_prec<0>(const BatchFeeder *, const int *, const int *, int, int, int, size_t, cudaStream_t);
 
 cudaError_t launch_search_inc(int precision, Topo T, State S, Search X, Inc I, Ctrl *C, int verify, const IncPlan &pl,
                               cudaStream_t st) {
-    if (pl.sh.threads == 256)
-        return precision == 1 ? launch_one<256, 1>(T, S, X, I, C, verify, pl, st)
-                              : launch_one<256, 0>(T, S, X, I, C, verify, pl, st);
-    if (pl.sh.threads == 384)
-        return precision == 1 ? launch_one<384, 1>(T, S, X, I, C, verify, pl, st)
-                              : launch_one<384, 0>(T, S, X, I, C, verify, pl, st);
-    return precision == 1 ? launch_one<512, 1>(T, S, X, I, C, verify, pl, st)
-                          : launch_one<512, 0>(T, S, X, I, C, verify, pl, st);
+    return precision == 1 ? launch_one_prec<1>(T, S, X, I, C, verify, pl, st) : launch_one_prec<0>(T, S, X, I, C, verify, pl, st);
 }
 
-cudaError_t prepare_search_inc_batch(int precision, int max_n, IncShape sh) {
-    sh = inc_shape_resolve(sh);
-    int use = 0;
-    size_t smem = 0;
-    if (!inc_smem(max_n, false, sh, &use, &smem)) return cudaErrorInvalidValue;
-    if (sh.threads == 384) return set_batch_smem<384>(precision, smem);
-    return sh.threads == 256 ? set_batch_smem<256>(precision, smem) : set_batch_smem<512>(precision, smem);
+bool inc_batch_plan(int max_n, int cs, const IncShape &raw, IncPlan *out) {
+    IncShape sh = raw;
+    if (sh.threads == 0 && cs == kMaxCluster) sh.threads = 256;
+    out->sh = inc_shape_resolve(sh);
+    out->cs = cs;
+    if (cs == 1) {
+        if (!inc_smem(max_n, false, out->sh, &out->rec, &out->bytes)) return false;
+        out->mode = out->rec;
+        return true;
+    }
+    const int np = own_pairs(max_n, 0, cs);
+    const size_t b = base_bytes(max_n, out->sh.se, cs) + align16(rec_maxm_bytes(np));
+    if (b > kIncSmemMax) return false;
+    const bool own = b + sums_bytes(np) <= kIncSmemMax;
+    out->rec = 2;
+    out->mode = own ? 2 + 4 : 2;
+    out->bytes = own ? b + sums_bytes(np) : b;
+    return true;
 }
 
-cudaError_t launch_search_inc_batch(int precision, int max_n, const BatchFeeder *fd, const int *order, int nf,
-                                    IncShape sh, cudaStream_t st) {
+// How many of the first feeders (largest first) are searched by clusters, and of
+// how many CTAs (none under a forced record placement or another thread count).
+// With SMs for eight CTAs a feeder, all that gain take eight, as far as those
+// clusters are resident at once (a merge on one CTA / eight, FP32 terms, one
+// scenario: 600 buses 12.2 / 9.8 us, 1,500 13.8 / 9.8).  Otherwise the feeders
+// whose chain alone outlasts an even share of the work by a quarter take two (a
+// merge on two CTAs costs 1.7 of the SM time of one, on four 2.7: more would take
+// from the others what the longest chains gain).  256 feeders of 60 .. 1,600
+// buses, FP32: 30.1 ms of search, 32.8 with one CTA each; 48 feeders of 60 .. 400
+// with eight for the 14 largest 4.8 ms, with one CTA each 4.6.
+void inc_batch_clusters(int precision, int nf, const int *n, const int *merges, int num_sms, const IncShape &raw, int *count,
+                        int *cs) {
+    *count = 0;
+    *cs = 1;
+    const bool spare = (long long)nf * kMaxCluster <= num_sms;
+    if (raw.rec >= 0 || (raw.threads != 0 && raw.threads != (spare ? 256 : 384)) || nf < 1) return;
+    auto chain = [&](int i) { return merges[i] * (11.0 + 0.002 * n[i]); };     // us on one CTA
+    double sum = 0.0;
+    for (int i = 0; i < nf; ++i) sum += chain(i);
+    int k = 0, max_n = 2;
+    while (k < nf && n[k] >= kBatchCluster && (spare || (chain(k) > 1.25 * sum / num_sms && 4 * (k + 1) <= num_sms)))
+        max_n = std::max(max_n, n[k++]);
+    IncPlan pl;
+    if (k == 0 || !inc_batch_plan(max_n, spare ? kMaxCluster : 2, raw, &pl)) return;
+    k = std::min(k, precision == 1 ? batch_clusters_prec<1>(pl) : batch_clusters_prec<0>(pl));
+    if (k < 1) return;
+    *count = k;
+    *cs = pl.cs;
+}
+
+cudaError_t prepare_search_inc_batch(int precision, const IncPlan &pl) {
+    return precision == 1 ? prepare_batch_prec<1>(pl) : prepare_batch_prec<0>(pl);
+}
+
+cudaError_t launch_search_inc_batch(int precision, const BatchFeeder *fd, const int *order, int nf, const IncPlan &pl,
+                                    cudaStream_t st) {
     if (nf <= 0) return cudaSuccess;
-    sh = inc_shape_resolve(sh);
-    int use = 0;
-    size_t smem = 0;
-    if (!inc_smem(max_n, false, sh, &use, &smem)) return cudaErrorInvalidValue;
-    if (sh.threads == 256) launch_batch<256>(precision, fd, order, nf, use, smem, sh, st);
-    else if (sh.threads == 384) launch_batch<384>(precision, fd, order, nf, use, smem, sh, st);
-    else launch_batch<512>(precision, fd, order, nf, use, smem, sh, st);
-    return cudaGetLastError();
+    return precision == 1 ? launch_batch_prec<1>(fd, order, nf, pl, st) : launch_batch_prec<0>(fd, order, nf, pl, st);
 }
 
 cudaError_t prepare_inc_init_batch(int precision, int max_n) {
     const size_t ismem = align16((size_t)2 * max_n) + align16((size_t)8 * max_n);
     if (ismem <= 48 * 1024) return cudaSuccess;
-    return precision == 1 ? set_smem(k_inc_init_batch<kInitThreads, 1>, ismem)
-                          : set_smem(k_inc_init_batch<kInitThreads, 0>, ismem);
+    return precision == 1 ? prepare_init_prec<1>(ismem) : prepare_init_prec<0>(ismem);
 }
 
 cudaError_t launch_inc_init_batch(int precision, int max_n, const BatchFeeder *fd, const int *order,
-                                  const int *cta_off, int nf, int ctas, cudaStream_t st) {
+                                  const int *cta_off, int nf, int cta0, int ctas, cudaStream_t st) {
     if (nf <= 0 || ctas <= 0) return cudaSuccess;
     const size_t ismem = align16((size_t)2 * max_n) + align16((size_t)8 * max_n);
     k_inc_zero_batch<<<nf, 256, 0, st>>>(fd, order, nf);
-    if (precision == 1) k_inc_init_batch<kInitThreads, 1><<<ctas, kInitThreads, ismem, st>>>(fd, order, cta_off, nf);
-    else k_inc_init_batch<kInitThreads, 0><<<ctas, kInitThreads, ismem, st>>>(fd, order, cta_off, nf);
+    if (precision == 1) launch_init_prec<1>(fd, order, cta_off, nf, cta0, ctas, ismem, st);
+    else launch_init_prec<0>(fd, order, cta_off, nf, cta0, ctas, ismem, st);
     return cudaGetLastError();
 }
+
+#endif
 
 }  // namespace okr

@@ -151,11 +151,12 @@ __global__ void k_export(Topo T, State S, double *super_vred, int *super_of, dou
 // one cluster per feeder (verify = 1: every merge also re-evaluates every candidate and counts
 // mismatches of the carried scores in C->inc_mismatch).
 //
-// Launch shape of that CTA: threads (256, 384 or 512), warps that evaluate the
+// Launch shape of each CTA: threads (256, 384 or 512), warps that evaluate the
 // merge beside the changed-set scan (cw, 1 .. threads/32 - 1), work entries in
 // shared memory (se, 1 .. 256; the rest in device memory) and where the
-// selection records live (rec: -1 automatic, 0 device memory, 1 shared memory,
-// 2 shared memory with the largest MICE per super-node; batches take 0 or 1).
+// selection records live (rec: -1 automatic; a forced placement is one CTA's:
+// 0 device memory, 1 shared memory, 2 shared memory with the largest MICE per
+// super-node, single feeders only).
 // Every shape gives the same results.
 struct IncShape {
     int threads, cw, se, rec;
@@ -190,20 +191,25 @@ struct IncPlan {
 bool inc_plan(int n, const IncShape &raw, bool records_iters, IncPlan *out);
 cudaError_t launch_search_inc(int precision, Topo T, State S, Search X, Inc I, Ctrl *C, int verify, const IncPlan &pl,
                               cudaStream_t st);
-// Many feeders: one CTA each, in the order given (prepare_search_inc_batch with
-// the same precision, shape and at least the same largest feeder first: it
-// sets the kernel's shared-memory attribute, which a stream capture must not
-// see).
-cudaError_t prepare_search_inc_batch(int precision, int max_n, IncShape sh);
-cudaError_t launch_search_inc_batch(int precision, int max_n, const BatchFeeder *fd, const int *order, int nf,
-                                    IncShape sh, cudaStream_t st);
+// Many feeders, in the order given (largest first): `count` of them by clusters
+// of `cs` CTAs (inc_batch_clusters, from their buses and merges), the others by
+// one CTA each, in launches that may run side by side.  inc_batch_plan: the plan
+// of one launch, false when the shape's record placement does not fit.
+// prepare_search_inc_batch sets the kernels' shared-memory attribute, which a
+// stream capture must not see.
+bool inc_batch_plan(int max_n, int cs, const IncShape &raw, IncPlan *out);
+void inc_batch_clusters(int precision, int nf, const int *n, const int *merges, int num_sms, const IncShape &raw, int *count,
+                        int *cs);
+cudaError_t prepare_search_inc_batch(int precision, const IncPlan &pl);
+cudaError_t launch_search_inc_batch(int precision, const BatchFeeder *fd, const int *order, int nf, const IncPlan &pl,
+                                    cudaStream_t st);
 // The batch's first evaluation on many CTAs, before launch_search_inc_batch
 // (which then takes it as done): cta_off[i] = the first CTA of order[i]
-// (inc_init_batch_ctas(n) each), ctas = their total; it first zeroes the
+// (inc_init_batch_ctas(n) each), cta0 = cta_off[0], ctas = their total; it first zeroes the
 // feeders' carried sums.  prepare_inc_init_batch sets the kernel's
 // shared-memory attribute (before any stream capture).
 cudaError_t prepare_inc_init_batch(int precision, int max_n);
 cudaError_t launch_inc_init_batch(int precision, int max_n, const BatchFeeder *fd, const int *order,
-                                  const int *cta_off, int nf, int ctas, cudaStream_t st);
+                                  const int *cta_off, int nf, int cta0, int ctas, cudaStream_t st);
 
 }  // namespace okr

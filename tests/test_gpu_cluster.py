@@ -43,3 +43,26 @@ def test_cluster_and_one_cta_give_the_same_run(ctx, n, scen, target, precision):
         for k, v in runs[0][0].items():
             assert np.array_equal(v, dec[k]), k
         assert np.array_equal(runs[0][1], sup) and np.array_equal(runs[0][2], vred) and runs[0][3] == counts
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("sizes", [(700, 520, 90), (640, 499, 500, 501, 30, 9) + (40,) * 40,
+                                   (700, 260) + (60,) * 150])
+def test_batches_searched_by_clusters_and_single_ctas_give_the_single_runs(ctx, sizes, precision):
+    """Clusters of eight where SMs are left, of two for a long chain among many
+    (152 feeders on 152 SMs); the other feeders by one CTA each, beside them: every feeder's result is its single run's, bit for bit."""
+    import paper_2510_19608_gb300 as K
+    feeders = [fg.make_feeder(n, 40 + 7 * i, phase_mode=(0.7, 0.1, 0.2)) for i, n in enumerate(sizes)]
+    p = K.default_params(margin=0.005, target_reduction=0.3, precision=precision)
+    items, parts, _ = ctx.reduce_batch(feeders, p)
+    plan = ctx.batch_plan(feeders, p)
+    again, parts2, _ = plan.run()
+    plan.close()
+    assert again == items and all(np.array_equal(a, b) for a, b in zip(parts, parts2))
+    for i in sorted(set([0, 1, 2, 3, 4, 5, len(sizes) - 1]) & set(range(len(sizes)))):
+        ctx.reduce(feeders[i], p)
+        s = ctx.summary()
+        assert items[i]["status"] == 0
+        assert [items[i][k] for k in ("n_iter", "stop_reason", "n_kept", "candidates", "smice", "max_error")] == \
+            [s[k] for k in ("n_iter", "stop_reason", "n_kept", "candidates", "smice", "max_error")]
+        assert np.array_equal(parts[i], ctx.assignment())
