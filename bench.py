@@ -36,17 +36,17 @@ FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 FLOPS_PER_ITEM = 40
 # DRAM bytes of one search launch on this workload from the ncu capture in
 # profiles/, valid only for the kernel source it was taken on (None otherwise)
-NCU_TRAFFIC = {"bytes": 1166336 + 768, "source": "paper_2510_19608_gb300/csrc/okr_incr.cu",
-               "sha256_prefix": "56d4cc024db929ed", "summary": "profiles/k_search_inc_feeder1000.md"}
+NCU_TRAFFIC = {"bytes": 1131264 + 4352, "source": "paper_2510_19608_gb300/csrc/okr_incr.cu",
+               "sha256_prefix": "c75d19b8ab76bc9e", "summary": "profiles/k_search_inc_feeder1000.md"}
 L2_FLUSH_BYTES = 256 << 20  # > 129 MB L2
 
 # Latency floor of one merge of the incremental search.  One merge is a chain
 # of phases, each of which needs the previous one's result: selection, the
-# merge's own FP64 evaluation (beside the changed-set scan), the rebuilt
-# candidates, the terms that change.  The floor takes, per phase, its longest
+# merge's own FP64 evaluation (beside it the changed and the rebuilt
+# candidates), the terms that change.  The floor takes, per phase, its longest
 # chain of dependent steps at the latencies measured on a GB300 (one-off
 # clock64 probes, one CTA of 512 threads), with unlimited parallelism inside a
-# phase.  Cycles:
+# phase and no cost for what the cluster's CTAs tell each other.  Cycles:
 PRIM_CYCLES = {"l2": 290,        # dependent L2 load (ld.global.cg, 8 MB footprint)
                "l1": 47,         # dependent load through L1 / shared memory, data the CTA wrote
                "bar": 48,        # __syncthreads of 512 threads arriving together
@@ -56,12 +56,11 @@ PRIM_CYCLES = {"l2": 290,        # dependent L2 load (ld.global.cg, 8 MB footpri
 MERGE_CHAIN = {
     # two block reductions over the selection records, then the winner's candidate
     "select": lambda c: 2 * (c["l1"] + c["bar"]) + c["l2"],
-    # position -> lca -> path impedance -> 3-term complex product (6 dependent
-    # DFMAs) -> magnitude -> barrier
-    "merge_eval": lambda c: c["l1"] + 2 * c["l2"] + 6 * c["dfma"] + c["dsqrt_add"] + c["bar"],
-    # a rebuilt pair: label -> parent's cluster -> lca -> child offsets -> child
-    # search -> subtree size (six dependent L2 loads), then a barrier
-    "rebuild": lambda c: 6 * c["l2"] + c["bar"],
+    # the longer of: position -> lca -> path impedance -> 3-term complex product
+    # (6 dependent DFMAs) -> magnitude -> barrier; a rebuilt pair: label ->
+    # parent's cluster -> lca -> child offsets -> child search -> subtree size
+    # (six dependent L2 loads), then a barrier
+    "merge": lambda c: max(c["l1"] + 2 * c["l2"] + 6 * c["dfma"] + c["dsqrt_add"] + c["bar"], 6 * c["l2"] + c["bar"]),
     # offsets scan (two barriers), entry lookup (four shared loads), state, lca
     # and path-impedance loads, one FP32 term (about 40 dependent operations),
     # the sums' shared update, a barrier, the carried sum's load, a barrier
@@ -259,7 +258,7 @@ def run_reference(args, rank, world):
 def batch_line(K, ctx, reps=3):
     """Many-feeder workload: 256 seeded feeders, n ~ U[200, 2000], targets in
     {50, 70, 90} %, margin 0.005, reduced by okr_reduce_batch: the incremental
-    engine (one CTA per feeder) and the sweep engine (one persistent launch,
+    engine (one CTA per feeder, clusters for the longest) and the sweep engine (one persistent launch,
     autotuned teams), each with FP32 terms (FP64 rescoring and merges) and in
     plain FP64.  Inputs (about 1 GB of device buffers) exceed L2, so no flush
     is needed between repetitions."""
@@ -412,8 +411,8 @@ def sweeps_line(K, ctx):
 
 
 def search_roofline(K, ctx, dfeed, run, search_ms: float, merges: int) -> dict:
-    """Roofline block of the incremental search kernel (one CTA runs a
-    feeder's whole search, a chain of dependent merges): its per-merge time
+    """Roofline block of the incremental search kernel (one cluster of CTAs runs
+    a feeder's whole search, a chain of dependent merges): its per-merge time
     against the latency floor of a merge, and, beside it, its counted FP32
     arithmetic against the FP32 ALU peak.  search_ms: the kernel's CUDA-event
     time per launch; items are counted by the kernel in one profiled run."""
@@ -437,10 +436,10 @@ def search_roofline(K, ctx, dfeed, run, search_ms: float, merges: int) -> dict:
                     "frac": achieved_flops / FP32_PEAK_TFLOPS,
                     "peak_source": "derived FP32 ALU rate: 152 SMs x 128 lanes x 2 flop x 2.07 GHz"},
             # incremental engine's phase timer (CTA 0): selection = block summaries and pass A (11) + pass B (0);
-            # changed set = the winner's record (12) + the scan beside the merge's evaluation (1)
+            # merge = the winner's record (12) + the merge's evaluation, the changed and the rebuilt candidates (1)
             "phase_us_per_merge": {k: round(1e3 * v / max(merges, 1), 3) for k, v in (
-                ("select", ps["phase_ms"][11] + ps["phase_ms"][0]), ("changed_set", ps["phase_ms"][12] + ps["phase_ms"][1]),
-                ("merge_and_rebuild", ps["phase_ms"][2]), ("terms", ps["phase_ms"][3]))},
+                ("select", ps["phase_ms"][11] + ps["phase_ms"][0]), ("merge", ps["phase_ms"][12] + ps["phase_ms"][1]),
+                ("terms", ps["phase_ms"][3]))},
             "rechecks": ps["rechecks"], "recheck_candidates": ps["recheck_cands"],
             "shape": {k: ps[k] for k in ("inc_threads", "inc_eval_warps", "inc_shared_entries", "inc_records")}}
 
@@ -616,15 +615,15 @@ def run_ours(args, rank, world, local):
     e2e = {"value": cand_per_step / e2e_s, "unit": "candidates/s", "h2d_bytes_per_step": int(h2d),
            "d2h_bytes_per_step": int(d2h), "time_to_optimal_s": e2e_s}
 
-    # ---- roofline of the dominant kernel: the search kernel (one CTA runs the
-    # whole search), timed with CUDA events around its launch on the library
+    # ---- roofline of the dominant kernel: the search kernel (one cluster of CTAs
+    # runs the whole search), timed with CUDA events around its launch on the library
     # stream; its (candidate, phase-node, scenario) items are counted by the
     # kernel in one profiled step
     search_ms = summ_last["search_ms"]
     roofline = search_roofline(K, ctx, dfeed, run, search_ms, summ["n_iter"])
     roofline["traffic"] = _ncu_traffic()
     roofline["share_of_step"] = search_ms / (ms / args.steps)
-    roofline["note"] = ("one CTA runs the whole search, a chain of dependent merges: its time is latency, not "
+    roofline["note"] = ("one cluster of CTAs runs the whole search, a chain of dependent merges: its time is latency, not "
                         "arithmetic or memory traffic; frac = latency floor / measured time per merge")
     # output Y_Kron of the chosen network (Sec. II-B), formed once per feeder
     yk, _ = ctx.kron()
@@ -648,7 +647,7 @@ def run_ours(args, rank, world, local):
                 "config": _workload_config(f, run) | {
                     "engine": "incremental: every candidate's score carried across merges as an exact fixed-point "
                               "sum of its terms; only the terms whose inputs the last merge changed are evaluated "
-                              "again; one CTA",
+                              "again; one cluster of eight CTAs",
                     "precision": "FP32 terms with carried rigorous bounds, FP64 rescoring of the candidates the bound "
                                  "cannot separate, FP64 merges",
                     "value_counts": "every candidate of every iteration gets its exact score and feasibility; the "

@@ -106,7 +106,8 @@ typedef struct okr_params {
                                      the last merge changed are evaluated again (exact: a carried
                                      score is a fixed-point sum of its terms; precision 0 carries FP64
                                      terms, precision 1 FP32 terms with a carried error bound and an
-                                     FP64 rescoring where the bound cannot decide); one CTA per feeder.
+                                     FP64 rescoring where the bound cannot decide); one CTA or one cluster
+                                     of CTAs per feeder.
                                      Needs objective 0 and scorer_topk 0 (else OKR_EINVAL);
                                      record_iters records scores but not scorer features;
                                    OKR_ENGINE_VERIFY (3): as 2, and after every merge every candidate
@@ -154,9 +155,11 @@ typedef struct okr_summary {
     double phase_ms[16];        /* profile mode: time of CTA 0 per step of an iteration.  Sweep engine:
                                    selection, FP64 recheck, merge, candidate setup, barrier, merge
                                    bookkeeping, list update, offsets, compaction, chunk map, barrier,
-                                   sweep.  Incremental engine: selection, changed set, merge with the
-                                   rebuilt candidates beside it, the terms that change (before and
-                                   after the merge, one pass, with the write-back) */
+                                   sweep.  Incremental engine: selection (0 and 11), the merge (1: its
+                                   evaluation, and beside it the last merge's write-back, the changed
+                                   and the rebuilt candidates and the bookkeeping; 12: the winner's
+                                   record), the terms that change (3: before and after the merge, one
+                                   pass); 2 is 0 */
     double kron_ms;             /* device time of the last okr_kron since the reduction (0 if none) */
     int32_t scorer_fallbacks;   /* learned pruning: iterations re-evaluated exhaustively because the
                                    scorer's k candidates were all infeasible */
@@ -175,9 +178,10 @@ typedef struct okr_summary {
 } okr_summary;
 
 /* Launch shape of the incremental engine: each CTA of a feeder's search (one,
- * or the CTAs of a cluster; a forced record placement runs one).  Every shape gives the same results; only the time differs.  Set per
- * context (okr_set_inc_shape), used by the later okr_reduce* and
- * okr_reduce_batch calls on it.  A field of 0 takes its default. */
+ * or the CTAs of a cluster; a forced record placement runs one, and in a batch
+ * a thread count other than the clusters' too).  Every shape gives the same
+ * results; only the time differs.  Set per context (okr_set_inc_shape), used by
+ * the later okr_reduce* and okr_reduce_batch calls on it.  A field of 0 takes its default. */
 typedef struct okr_inc_shape {
     int32_t threads;            /* threads of a CTA: 256, 384 or 512 (0 = 384 for one CTA, 256 for a
                                    cluster's) */

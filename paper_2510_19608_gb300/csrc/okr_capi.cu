@@ -544,7 +544,7 @@ okr_status run_search(okr_ctx *ctx, const okr_params *p) {
     return OKR_OK;
 }
 
-// Initial state, then one CTA runs the whole search with carried scores
+// Initial state, then one CTA or one cluster runs the whole search with carried scores
 // (okr_incr.cu); then the export.
 okr_status run_search_inc(okr_ctx *ctx, const okr_params *p) {
     cudaStream_t st = ctx->stream;

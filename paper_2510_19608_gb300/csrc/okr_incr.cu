@@ -60,7 +60,7 @@
 // The write-back waits for the next merge's step 2, whose evaluation reads the
 // not yet written values through the overlay, so no barrier is needed for it.
 // (Rebuilding in a step of its own, between barriers, with the write-back after
-// the terms took 14.0 us a merge on 1,000 buses, a cluster, FP32 terms; 9.9 now.)
+// the terms took 14.0 us a merge on 1,000 buses, a cluster, FP32 terms; 9.8 now.)
 #include "okr_internal.cuh"
 #include "okr_kernels.cuh"
 
@@ -2595,9 +2595,10 @@ bool inc_smem(int n, bool maxm, const IncShape &sh, int *rec_mode, size_t *bytes
 // slot pairs, the FP64 evaluation of the merge, the changed terms and the
 // records (which then always fit shared memory, the carried sums and candidates
 // up to about 4,200 buses), and pays three cluster barriers a merge and L2 in
-// place of L1 latency.  Search ms, one CTA of 384 threads / eight of 256:
-//   FP64 terms:  40 buses 0.50 / 0.47, 101 1.21 / 1.12, 333 (3 scenarios) 5.4 / 3.2, 1,000 9.5 / 6.0, 3,100 59.2 / 33.0
-//   FP32 terms:  40 buses 0.54 / 0.54, 101 1.32 / 1.31, 333 (3 scenarios) 3.8 / 2.9, 1,000 6.7 / 4.9, 3,100 44.9 / 27.4
+// place of L1 latency.  us a merge, one CTA of 384 threads / eight of 256 (one
+// scenario; 400 buses two):
+//   FP64 terms:  60 buses 13.4 / 12.3, 100 12.5 / 11.6, 400 16.3 / 11.7, 600 15.3 / 11.2, 1,500 17.7 / 11.5
+//   FP32 terms:  60 buses 12.0 / 11.5, 100 11.1 / 10.6, 400 13.2 / 10.9, 600 12.2 / 9.8, 1,500 13.8 / 9.8
 // A forced record placement asks for one CTA's memory, and recorded iterations
 // are compacted by one CTA.
 bool inc_plan(int n, const IncShape &raw, bool records_iters, IncPlan *out) {
@@ -2613,7 +2614,7 @@ bool inc_plan(int n, const IncShape &raw, bool records_iters, IncPlan *out) {
     const bool own = b + sums_bytes(np) <= kIncSmemMax;
     out->mode = own ? 2 + 4 : 2;
     out->bytes = own ? b + sums_bytes(np) : b;
-    // fewer warps meet at the cluster's barriers (384 threads: 1,000 buses 5.2 ms, 3,100 buses 26.6 ms)
+    // fewer warps meet at the cluster's barriers (384 threads, FP32 terms: 100 buses 11.3 us, 1,500 10.2)
     if (raw.threads == 0) {
         IncShape sh = raw;
         sh.threads = 256;
@@ -2783,7 +2784,7 @@ bool inc_batch_plan(int max_n, int cs, const IncShape &raw, IncPlan *out) {
 // scenario: 600 buses 12.2 / 9.8 us, 1,500 13.8 / 9.8).  Otherwise the feeders
 // whose chain alone outlasts an even share of the work by a quarter take two (a
 // merge on two CTAs costs 1.7 of the SM time of one, on four 2.7: more would take
-// from the others what the longest chains gain).  256 feeders of 60 .. 1,600
+// from the others what the longest chains gain).  256 feeders of 200 .. 2,000
 // buses, FP32: 30.1 ms of search, 32.8 with one CTA each; 48 feeders of 60 .. 400
 // with eight for the 14 largest 4.8 ms, with one CTA each 4.6.
 void inc_batch_clusters(int precision, int nf, const int *n, const int *merges, int num_sms, const IncShape &raw, int *count,

@@ -148,8 +148,8 @@ int search_blocks_per_sm();     // CTAs of the search kernel that fit one SM (0 
 __global__ void k_export(Topo T, State S, double *super_vred, int *super_of, double *vhat_out);
 
 // okr_incr.cu -- the search with scores carried across iterations: one CTA or
-// one cluster per feeder (verify = 1: every merge also re-evaluates every candidate and counts
-// mismatches of the carried scores in C->inc_mismatch).
+// one cluster per feeder (verify = 1: every merge also re-evaluates every
+// candidate and counts mismatches of the carried scores in C->inc_mismatch).
 //
 // Launch shape of each CTA: threads (256, 384 or 512), warps that evaluate the
 // merge beside the changed-set scan (cw, 1 .. threads/32 - 1), work entries in
@@ -205,8 +205,8 @@ cudaError_t launch_search_inc_batch(int precision, const BatchFeeder *fd, const 
                                     cudaStream_t st);
 // The batch's first evaluation on many CTAs, before launch_search_inc_batch
 // (which then takes it as done): cta_off[i] = the first CTA of order[i]
-// (inc_init_batch_ctas(n) each), cta0 = cta_off[0], ctas = their total; it first zeroes the
-// feeders' carried sums.  prepare_inc_init_batch sets the kernel's
+// (inc_init_batch_ctas(n) each), cta0 = cta_off[0], ctas = their total; it
+// first zeroes the feeders' carried sums.  prepare_inc_init_batch sets the kernel's
 // shared-memory attribute (before any stream capture).
 cudaError_t prepare_inc_init_batch(int precision, int max_n);
 cudaError_t launch_inc_init_batch(int precision, int max_n, const BatchFeeder *fd, const int *order,
