@@ -103,23 +103,6 @@ __device__ __forceinline__ u128 to_fx(double d) {
     return (b >> 63) ? (u128)0 - v : v;
 }
 
-// The same truncation for a float, with integer operations only (FP64
-// instructions are scarce on this GPU): equal to to_fx((double)f).
-__device__ __forceinline__ u128 to_fx32(float f) {
-    const unsigned b = __float_as_uint(f);
-    int e = (int)((b >> 23) & 0xff);
-    if (e == 0xff) return 0;
-    unsigned m = b & 0x7fffffu;
-    if (e == 0) e = 1;
-    else m |= 1u << 23;
-    // f = m * 2^(e - 150), so f * 2^100 = m * 2^(e - 50)
-    const int sh = e - 150 + kFxShift;
-    u128 v;
-    if (sh >= 0) v = sh >= 128 ? (u128)0 : ((u128)m << sh);
-    else v = sh <= -32 ? (u128)0 : (u128)(m >> (-sh));
-    return (b >> 31) ? (u128)0 - v : v;
-}
-
 __device__ __forceinline__ double fx_to_d(u128 v) {
     const bool neg = (v & kSignBit) != 0;
     const u128 a = neg ? (u128)0 - v : v;
@@ -363,7 +346,7 @@ __device__ __forceinline__ u128 limb_sum(const int (*x)[kTile + 1], int i) {
 __device__ __forceinline__ void limb_add(int (*x)[kTile + 1], int i, int k, int piece) {
     if (piece != 0 && k < kLimbs) atomicAdd(&x[k][i], piece);
 }
-// Adds sgn * to_fx32(f) to sum i: lane p of the scenario's four adds piece p
+// Adds sgn * to_fx((double)f) to sum i: lane p of the scenario's four adds piece p
 // (a 24-bit mantissa at any shift lies in three limbs); p = 3 adds `extra` to
 // the lowest limb.
 __device__ __forceinline__ void add_fx32(int (*x)[kTile + 1], int i, float f, int sgn, int p, int extra) {
