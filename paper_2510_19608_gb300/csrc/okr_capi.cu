@@ -317,7 +317,8 @@ int *host_pf_iters(okr_ctx *ctx) { return host_err(ctx) + 1; }
 // The host waits for the topology's check of the tree (the later kernels index
 // through its renumbering); with check_lines it also waits for the lines and
 // reads the tree's statistics, else a singular line is reported with the
-// caller's last read of the error flag (the load flow skips its work then).
+// caller's last read of the error flag (the load flow, which does not read the
+// inverses, runs all the same).
 okr_status build_topology(okr_ctx *ctx, int n, int L, const double *vslack, bool check_lines = true) {
     cudaStream_t st = ctx->stream;
     CK(join_side(ctx));                     // (a failed call may have left side work unjoined)

@@ -527,7 +527,9 @@ __device__ __forceinline__ unsigned pf_ld_acquire(const unsigned *p) {
 }
 
 // Grid barrier on a monotonic counter; bounded by max_spins polls: returns
-// false (and sets err = 6) when the wait gives up or another CTA already gave up.
+// false (and sets err = 6, where no other error stands) when the wait gives up or
+// another CTA already gave up.  count[1] says that one has: err cannot, since the
+// line inverses beside the load flow may have named a singular line in it.
 __device__ bool pf_grid_sync(unsigned *count, int *err, unsigned nblocks, unsigned &epoch, long long max_spins) {
     __shared__ int s_ok;
     __syncthreads();
@@ -540,9 +542,12 @@ __device__ bool pf_grid_sync(unsigned *count, int *err, unsigned nblocks, unsign
         long long spins = 0;
         // one L2 round trip per poll; another CTA's give-up is looked for every 64 polls
         while (pf_ld_acquire(count) < target) {
-            if (++spins > max_spins || ((spins & 63) == 0 && *(volatile int *)err == 6)) { ok = 0; break; }
+            if (++spins > max_spins || ((spins & 63) == 0 && *(volatile unsigned *)(count + 1) != 0)) { ok = 0; break; }
         }
-        if (!ok) atomicCAS(err, 0, 6);
+        if (!ok) {
+            atomicExch(count + 1, 1u);
+            atomicCAS(err, 0, 6);
+        }
         __threadfence();
         s_ok = ok;
     }
@@ -560,8 +565,8 @@ __global__ void __launch_bounds__(256) k_power_flow(int n, int L, Topo T, const 
     const int gt = blockIdx.x * nt + tid, gs = (int)G * nt;
     const size_t N3 = (size_t)3 * n;
     const size_t tot = (size_t)L * N3;
-    // an earlier setup step failed (every CTA reads the same flag: no writer runs)
-    if (*reinterpret_cast<volatile const int *>(err) != 0) return;
+    // (no CTA looks at err before the barriers: the line inverses, which run beside
+    // this kernel, may be setting it, and a CTA that left would be waited for)
     const int maxd = T.maxd[0];
     const double tol2 = tol * tol;                  // the test is max |dV|^2 < tol^2
     unsigned epoch = 0;
@@ -830,8 +835,8 @@ __device__ void dev_power_flow_smem(int n, int l, const Topo &T, const double *_
 __global__ void __launch_bounds__(kPfThreads) k_power_flow_cta(int n, Topo T, const double *__restrict__ s_in, double tol,
                                                                int max_iter, int *iters, int *err) {
     extern __shared__ double2 pfc_sm[];
-    // an earlier setup step failed
-    if (*reinterpret_cast<volatile const int *>(err) != 0) return;
+    // (err is not looked at: the line inverses beside this kernel may be setting it,
+    // and threads that saw it and left would leave the tree half loaded)
     dev_power_flow_smem(n, blockIdx.x, T, s_in, tol, max_iter, iters, err, pfc_sm);
 }
 
