@@ -360,12 +360,14 @@ __global__ void k_lca_fill(int n, const int *__restrict__ parent, const int *__r
     dev_lca_fill(n, parent, sz, depth, st, lca, (size_t)blockIdx.x * blockDim.x + threadIdx.x, (size_t)gridDim.x * blockDim.x);
 }
 
-// Line impedances in preorder (a grid stride over the 9 n entries).
+// Line impedances in preorder (a grid stride over the 9 n entries).  z_in may be
+// the caller's own array, of which nothing but a double's alignment is asked: two
+// 8-byte loads an entry.
 __device__ void dev_line_copy(int n, Topo T, const double *__restrict__ z_in, int first, int stride) {
     for (int e = first; e < 9 * n; e += stride) {
         const int v = e / 9, q = e - 9 * v, i = T.orig[v];
-        const double2 *z = reinterpret_cast<const double2 *>(z_in) + (size_t)i * 9 + q;
-        T.zl[e] = v == 0 ? make_double2(0.0, 0.0) : *z;
+        const double *z = z_in + 2 * ((size_t)i * 9 + q);
+        T.zl[e] = v == 0 ? make_double2(0.0, 0.0) : make_double2(z[0], z[1]);
     }
 }
 

@@ -4,6 +4,9 @@ A singular line: its inverse is formed beside the load flow and names it in the
 setup's error flag while the load flow runs.  The call returns the singular line
 at once (no CTA of the load flow waits for one that left), whatever the size, and
 leaves the context as it was.
+
+A device array of doubles at an odd multiple of 8 bytes is a double's array like
+any other for the entry point that reads the caller's memory.
 """
 import time
 
@@ -48,3 +51,29 @@ def test_a_singular_line_beside_the_load_flow_is_reported_at_once(ctx, n, scen):
                 assert rep == 0 or dt < STALL_S, dt
     v, i, sweeps = ctx.power_flow(f)
     assert np.array_equal(v, want[0]) and np.array_equal(i, want[1]) and sweeps == want[2]
+
+
+@pytest.mark.parametrize("n,scen", [(5, 1), (256, 2), (300, 3)])
+def test_static_load_flow_reads_arrays_at_any_double_s_address(n, scen):
+    import torch
+    import paper_2510_19608_gb300 as K
+    f = fg.make_feeder(n, 21, phase_mode=(0.5, 0.2, 0.3), n_scen=scen)
+    par, ph = torch.from_numpy(f.parent).cuda(), torch.from_numpy(f.phases).cuda()
+    runs = []
+    for shift in (0, 1):                    # doubles from a 16-byte boundary
+        z = torch.zeros(f.z_line.size + 2, dtype=torch.float64, device="cuda")
+        s = torch.zeros(f.s_load.size + 2, dtype=torch.float64, device="cuda")
+        z[shift:shift + f.z_line.size] = torch.from_numpy(f.z_line.reshape(-1)).cuda()
+        s[shift:shift + f.s_load.size] = torch.from_numpy(f.s_load.reshape(-1)).cuda()
+        v = torch.full((scen * n * 6 + 2,), float("nan"), dtype=torch.float64, device="cuda")
+        i = torch.full((scen * n * 6 + 2,), float("nan"), dtype=torch.float64, device="cuda")
+        assert z.data_ptr() % 16 == 0 and v.data_ptr() % 16 == 0
+        at = 8 * shift
+        df = K.device_feeder(n, scen, par.data_ptr(), ph.data_ptr(), z.data_ptr() + at, s.data_ptr() + at, f.v_slack)
+        torch.cuda.synchronize()
+        sw = K.power_flow_static(df, v.data_ptr() + at, i.data_ptr() + at, torch.cuda.current_stream().cuda_stream)
+        k = scen * n * 6
+        runs.append((sw, v[shift:shift + k].cpu().numpy(), i[shift:shift + k].cpu().numpy()))
+    assert runs[0][0] == runs[1][0]
+    assert np.isfinite(runs[0][1]).all()
+    assert np.array_equal(runs[0][1], runs[1][1]) and np.array_equal(runs[0][2], runs[1][2])
