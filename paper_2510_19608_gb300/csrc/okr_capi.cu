@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
+#include <cstdint>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -2081,9 +2082,11 @@ okr_status mlp_upload(okr_ctx *ctx, const float *x, const float *t, long long N)
 // The features a forward pass reads, and room for its predictions.  Each feature
 // is read once, so where the GPU reads host memory through the host's page
 // tables the kernel takes them from there (168 MB: 0.88 ms, the copy alone 1.06
-// to 1.09, and the products run beside it); elsewhere they are copied.
+// to 1.09, and the products run beside it); elsewhere they are copied.  So are
+// features that do not lie at a float's address (a slice of a packed buffer),
+// which a copy takes and a load does not.
 okr_status mlp_features(okr_ctx *ctx, const float *x, long long N, const float **xd) {
-    if (!ctx->reads_host) {
+    if (!ctx->reads_host || reinterpret_cast<uintptr_t>(x) % sizeof(float) != 0) {
         *xd = nullptr;
         const okr_status s = mlp_upload(ctx, x, nullptr, N);
         *xd = ctx->mlp_x;
