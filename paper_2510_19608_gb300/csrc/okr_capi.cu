@@ -2230,7 +2230,8 @@ okr_status okr_scorer_predict_tc(okr_ctx *ctx, const float *x, int64_t n, float 
     int herr = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(y, yd, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    const cudaError_t w = cudaStreamSynchronize(ctx->stream);   // (after a failed step too: a kernel may be reading x)
+    if (e == cudaSuccess) e = w;
     if (e != cudaSuccess) out = fail(ctx, OKR_ECUDA, "tensor-core inference: %s", cudaGetErrorString(e));
     else if (herr) out = fail(ctx, OKR_ETIMEOUT, "tensor-core inference: a wait for the products gave up");
     return out;
@@ -2245,9 +2246,11 @@ okr_status okr_scorer_predict(okr_ctx *ctx, const float *x, int64_t n, float *y)
     okr_status s = mlp_features(ctx, x, n, &xd);
     if (s != OKR_OK) return s;
     float *yd = ctx->mlp_t;                     // the targets' buffer holds the predictions
-    CK(mlp_forward(ctx->mb, xd, (int)n, yd, ctx->num_sms, ctx->stream));
-    CK(cudaMemcpyAsync(y, yd, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
+    cudaError_t e = mlp_forward(ctx->mb, xd, (int)n, yd, ctx->num_sms, ctx->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(y, yd, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost, ctx->stream);
+    const cudaError_t w = cudaStreamSynchronize(ctx->stream);   // (after a failed step too: a kernel may be reading x)
+    CK(e);
+    CK(w);
     return OKR_OK;
 }
 
