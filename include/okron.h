@@ -415,7 +415,9 @@ okr_status okr_scorer_gradient(okr_ctx *ctx, const float *x, const float *t, int
  * mean squared error over each pass (may be NULL). */
 okr_status okr_scorer_train(okr_ctx *ctx, const float *x, const float *t, int64_t n, int32_t batch, int32_t epochs,
                             float lr, double *epoch_loss);
-/* Predictions y (HOST [n]) for x (HOST [n][n_features]). */
+/* Predictions y (HOST [n]) for x (HOST [n][n_features]).  x is read until the
+ * call returns, by the GPU in place where it shares the host's page tables: all
+ * n x n_features floats must be there. */
 okr_status okr_scorer_predict(okr_ctx *ctx, const float *x, int64_t n, float *y);
 /* The same network on the tensor cores (tcgen05, 128 samples per product):
  * the features and the hidden activations enter each product as bfloat16

@@ -238,6 +238,7 @@ class Context:
         self._check(lib().okr_create(C.byref(self._h), int(device), C.c_void_p(stream) if stream else None))
         self.n_bus = 0
         self.n_scen = 0
+        self.n_features = 0
 
     def close(self):
         if self._h:
@@ -437,6 +438,7 @@ class Context:
     def scorer_init(self, n_features: int, theta=None):
         th = None if theta is None else np.ascontiguousarray(theta, dtype=np.float32)
         self._check(lib().okr_scorer_init(self._h, int(n_features), _ptr(th) if th is not None else None))
+        self.n_features = int(n_features)
 
     def scorer_params(self) -> np.ndarray:
         k = C.c_int32()
@@ -461,8 +463,16 @@ class Context:
                                            float(lr), _ptr(el)))
         return el[:epochs]
 
-    def scorer_predict(self, x) -> np.ndarray:
+    def _features(self, x) -> np.ndarray:
+        """The features of an inference call, which the GPU may read in place: an
+        array that ends before the last sample's is refused here."""
         x = np.ascontiguousarray(x, dtype=np.float32)
+        if x.size < x.shape[0] * self.n_features:
+            raise ValueError(f"{x.shape[0]} samples of {self.n_features} features, got {x.size} values")
+        return x
+
+    def scorer_predict(self, x) -> np.ndarray:
+        x = self._features(x)
         y = np.zeros(x.shape[0], np.float32)
         self._check(lib().okr_scorer_predict(self._h, _ptr(x), int(x.shape[0]), _ptr(y)))
         return y
@@ -470,7 +480,7 @@ class Context:
     def scorer_predict_tc(self, x) -> np.ndarray:
         """okr_scorer_predict_tc: the same network on the tensor cores (bfloat16
         layer inputs, FP32 accumulation)."""
-        x = np.ascontiguousarray(x, dtype=np.float32)
+        x = self._features(x)
         y = np.zeros(x.shape[0], np.float32)
         self._check(lib().okr_scorer_predict_tc(self._h, _ptr(x), int(x.shape[0]), _ptr(y)))
         return y

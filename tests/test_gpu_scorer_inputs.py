@@ -1,6 +1,7 @@
 """Scorer inference on what a caller may hand over: features in host memory at
 any address give the same predictions, whether the kernels read them in place or
-from a copy; and a call that returns an error has finished with them."""
+from a copy; a call that returns an error has finished with them; and an array
+that ends before the last sample's features is refused before the GPU reads it."""
 import ctypes as C
 
 import numpy as np
@@ -67,3 +68,14 @@ def test_a_failed_call_reads_the_features_no_longer(which):
             pass
         assert st.query()
         assert np.array_equal(getattr(ctx, which)(x), y)
+
+
+def test_too_few_features_are_refused(ctx):
+    theta, x = _problem(14, 64, 5)
+    ctx.scorer_init(14, theta)
+    y = ctx.scorer_predict(x)
+    for bad in (x[:, :13], x.reshape(-1), x[:, :0]):
+        for f in (ctx.scorer_predict, ctx.scorer_predict_tc):
+            with pytest.raises(ValueError):
+                f(bad)
+    assert np.array_equal(ctx.scorer_predict(x), y)
