@@ -1269,7 +1269,8 @@ __global__ void __launch_bounds__(1024) k_eval_reduced(Topo T, const int *__rest
 cudaError_t launch_eval_reduced(Topo T, const int *sup, const int *moff, const int *mem, double2 *W, double2 *V,
                                 double *vred, double *err, cudaStream_t st) {
     const size_t smem = T.n <= kPfCta ? pf_cta_bytes(T.n) : 0;
-    if (smem > 48 * 1024) {
+    // (the limit without asking is 48 KB less the kernel's static arrays)
+    if (smem > 0) {
         const cudaError_t e = cudaFuncSetAttribute(k_eval_reduced, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)pf_cta_bytes(kPfCta));
         if (e != cudaSuccess) return e;
