@@ -858,7 +858,7 @@ cudaError_t launch_power_flow(int n, int L, Topo T, const double *s_in, double t
     const size_t smem = n <= kPfShared ? sizeof(double2) * (size_t)n + tree_bytes(n) : 0;
     unsigned *bar = reinterpret_cast<unsigned *>(red + 3 * L);
     cudaError_t e = cudaMemsetAsync(red, 0, sizeof(double) * (3 * L + 1), st);
-    if (e == cudaSuccess && smem > 48 * 1024)
+    if (e == cudaSuccess && smem > 0)       // (without asking: 48 KB less the static arrays)
         e = cudaFuncSetAttribute(k_power_flow, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(sizeof(double2) * kPfShared + tree_bytes(kPfShared)));
     if (e != cudaSuccess) return e;

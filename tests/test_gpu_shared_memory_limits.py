@@ -37,3 +37,14 @@ vhat, _ = O.operating_points(f)
 err, w = ctx.evaluate(f, np.arange({n}, dtype=np.int32))
 assert err.max() <= 1e-10 and np.abs(w - vhat).max() <= 1e-10
 """)
+
+
+# (a slice and the tree: 16 n + about 10 n bytes)
+@pytest.mark.parametrize("n", [1888, 1889, 1890, 1891])
+def test_load_flow(n):
+    _run(f"""
+f = feeder({n}, 2)
+vhat, _ = O.operating_points(f)
+v, i, _ = ctx.power_flow(f)
+assert np.abs(v - vhat).max() <= 1e-10
+""")
