@@ -1384,8 +1384,6 @@ static okr_status batch_fill(okr_ctx *ctx, BatchRun &R, const okr_feeder *feeder
     // attributes the launches need, set before any stream capture
     CK(prepare_batch_setup());
     for (int g = 2; g < 4; ++g) {
-        int max_n = 2;
-        for (int f : R.ord[g]) max_n = std::max(max_n, R.nbus[f]);
         if (!R.ord[g].empty()) {
             // the largest by clusters, the others by one CTA each beside them
             std::vector<int> nb, mg;
@@ -1401,7 +1399,7 @@ static okr_status batch_fill(okr_ctx *ctx, BatchRun &R, const okr_feeder *feeder
                 return fail(ctx, OKR_EINTERNAL, "batch: no launch plan");
             if (k > 0) CK(prepare_search_inc_batch(g - 2, R.plan[g - 2][0]));
             if (k < (int)nb.size()) CK(prepare_search_inc_batch(g - 2, R.plan[g - 2][1]));
-            CK(prepare_inc_init_batch(g - 2, max_n));
+            CK(prepare_inc_init_batch(g - 2));
         }
     }
     return OKR_OK;

@@ -2532,6 +2532,14 @@ template <typename K>
 cudaError_t set_smem(K kern, size_t bytes) {
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
+// The first evaluation's, at every size: without asking a launch gets 48 KB less
+// the kernel's 17 KB of static arrays.  Always the same limit: it is the process's,
+// and one set for a smaller feeder would hold for a larger one's launch on another
+// thread.
+template <typename K>
+cudaError_t set_init_smem(K kern) {
+    return set_smem(kern, kIncSmemMax);
+}
 
 }  // namespace
 
@@ -2542,7 +2550,7 @@ template <int PREC> cudaError_t launch_one_prec(Topo T, State S, Search X, Inc I
 template <int PREC> cudaError_t prepare_batch_prec(const IncPlan &pl);
 template <int PREC> cudaError_t launch_batch_prec(const BatchFeeder *fd, const int *order, int nf, const IncPlan &pl, cudaStream_t st);
 template <int PREC> int batch_clusters_prec(const IncPlan &pl);          // clusters of the plan resident at once
-template <int PREC> cudaError_t prepare_init_prec(size_t ismem);
+template <int PREC> cudaError_t prepare_init_prec();
 template <int PREC> void launch_init_prec(const BatchFeeder *fd, const int *order, const int *cta_off, int nf, int cta0, int ctas,
                                           size_t ismem, cudaStream_t st);
 
@@ -2648,7 +2656,7 @@ cudaError_t launch_one(Topo T, State S, Search X, Inc I, Ctrl *C, int verify, co
     const size_t ismem = align16((size_t)2 * T.n) + align16((size_t)8 * T.n);
     cudaError_t e = cudaMemsetAsync(I.acc, 0, reinterpret_cast<const char *>(I.vmay + 2 * (size_t)T.n) -
                                                   reinterpret_cast<const char *>(I.acc), st);
-    if (e == cudaSuccess && ismem > 48 * 1024) e = set_smem(k_inc_init<kInitThreads, PREC>, ismem);
+    if (e == cudaSuccess) e = set_init_smem(k_inc_init<kInitThreads, PREC>);
     if (e == cudaSuccess) k_inc_init<kInitThreads, PREC><<<ginit, kInitThreads, ismem, st>>>(T, S, X, I, C);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -2708,8 +2716,8 @@ int batch_clusters_prec(const IncPlan &pl) {
     return e == cudaSuccess ? count : 0;
 }
 template <int PREC>
-cudaError_t prepare_init_prec(size_t ismem) {
-    return set_smem(k_inc_init_batch<kInitThreads, PREC>, ismem);
+cudaError_t prepare_init_prec() {
+    return set_init_smem(k_inc_init_batch<kInitThreads, PREC>);
 }
 template <int PREC>
 void launch_init_prec(const BatchFeeder *fd, const int *order, const int *cta_off, int nf, int cta0, int ctas, size_t ismem,
@@ -2723,7 +2731,7 @@ template cudaError_t launch_one_prec<0>(Topo, State, Search, Inc, Ctrl *, int, c
 template cudaError_t prepare_batch_prec<0>(const IncPlan &);
 template cudaError_t launch_batch_prec<0>(const BatchFeeder *, const int *, int, const IncPlan &, cudaStream_t);
 template int batch_clusters_prec<0>(const IncPlan &);
-template cudaError_t prepare_init_prec<0>(size_t);
+template cudaError_t prepare_init_prec<0>();
 template void launch_init_prec<0>(const BatchFeeder *, const int *, const int *, int, int, int, size_t, cudaStream_t);
 
 #else
@@ -2732,7 +2740,7 @@ extern template cudaError_t launch_one_prec<0>(Topo, State, Search, Inc, Ctrl *,
 extern template cudaError_t prepare_batch_prec<0>(const IncPlan &);
 extern template cudaError_t launch_batch_prec<0>(const BatchFeeder *, const int *, int, const IncPlan &, cudaStream_t);
 extern template int batch_clusters_prec<0>(const IncPlan &);
-extern template cudaError_t prepare_init_prec<0>(size_t);
+extern template cudaError_t prepare_init_prec<0>();
 extern template void launch_init_prec<0>(const BatchFeeder *, const int *, const int *, int, int, int, size_t, cudaStream_t);
 
 cudaError_t launch_search_inc(int precision, Topo T, State S, Search X, Inc I, Ctrl *C, int verify, const IncPlan &pl,
@@ -2800,10 +2808,8 @@ cudaError_t launch_search_inc_batch(int precision, const BatchFeeder *fd, const 
     return precision == 1 ? launch_batch_prec<1>(fd, order, nf, pl, st) : launch_batch_prec<0>(fd, order, nf, pl, st);
 }
 
-cudaError_t prepare_inc_init_batch(int precision, int max_n) {
-    const size_t ismem = align16((size_t)2 * max_n) + align16((size_t)8 * max_n);
-    if (ismem <= 48 * 1024) return cudaSuccess;
-    return precision == 1 ? prepare_init_prec<1>(ismem) : prepare_init_prec<0>(ismem);
+cudaError_t prepare_inc_init_batch(int precision) {
+    return precision == 1 ? prepare_init_prec<1>() : prepare_init_prec<0>();
 }
 
 cudaError_t launch_inc_init_batch(int precision, int max_n, const BatchFeeder *fd, const int *order,

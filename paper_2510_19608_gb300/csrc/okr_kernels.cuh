@@ -208,7 +208,7 @@ cudaError_t launch_search_inc_batch(int precision, const BatchFeeder *fd, const 
 // (inc_init_batch_ctas(n) each), cta0 = cta_off[0], ctas = their total; it
 // first zeroes the feeders' carried sums.  prepare_inc_init_batch sets the kernel's
 // shared-memory attribute (before any stream capture).
-cudaError_t prepare_inc_init_batch(int precision, int max_n);
+cudaError_t prepare_inc_init_batch(int precision);
 cudaError_t launch_inc_init_batch(int precision, int max_n, const BatchFeeder *fd, const int *order,
                                   const int *cta_off, int nf, int cta0, int ctas, cudaStream_t st);
 
