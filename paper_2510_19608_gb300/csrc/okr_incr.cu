@@ -2528,17 +2528,14 @@ constexpr int kInitThreads = 384;           // CTAs of the first evaluation
 constexpr int kClusterMin = 32;             // buses from which a cluster searches (inc_plan)
 constexpr int kBatchCluster = 500;          // ... one of a batch's feeders (inc_batch_clusters)
 
+// Before every launch, whatever its size: without asking a launch gets 48 KB less
+// the kernel's 17 to 21 KB of static arrays.  Always the same limit: it is the
+// process's, and one set for a smaller feeder would hold for a larger one's launch
+// on another thread (fifteen threads with feeders of 4 to 1,200 buses: 8 of 30,000
+// calls refused).
 template <typename K>
-cudaError_t set_smem(K kern, size_t bytes) {
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-// The first evaluation's, at every size: without asking a launch gets 48 KB less
-// the kernel's 17 KB of static arrays.  Always the same limit: it is the process's,
-// and one set for a smaller feeder would hold for a larger one's launch on another
-// thread.
-template <typename K>
-cudaError_t set_init_smem(K kern) {
-    return set_smem(kern, kIncSmemMax);
+cudaError_t set_smem(K kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kIncSmemMax);
 }
 
 }  // namespace
@@ -2634,7 +2631,7 @@ cudaLaunchConfig_t search_config(int ctas, int threads, int cs, size_t bytes, cu
 
 template <int NT, int PREC, int CS>
 cudaError_t launch_cs(Topo T, State S, Search X, Inc I, Ctrl *C, int verify, const IncPlan &pl, cudaStream_t st) {
-    const cudaError_t e = set_smem(k_search_inc<NT, PREC, CS>, pl.bytes);
+    const cudaError_t e = set_smem(k_search_inc<NT, PREC, CS>);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute at[1];
     const cudaLaunchConfig_t cfg = search_config(CS, NT, CS, pl.bytes, st, at);
@@ -2656,7 +2653,7 @@ cudaError_t launch_one(Topo T, State S, Search X, Inc I, Ctrl *C, int verify, co
     const size_t ismem = align16((size_t)2 * T.n) + align16((size_t)8 * T.n);
     cudaError_t e = cudaMemsetAsync(I.acc, 0, reinterpret_cast<const char *>(I.vmay + 2 * (size_t)T.n) -
                                                   reinterpret_cast<const char *>(I.acc), st);
-    if (e == cudaSuccess) e = set_init_smem(k_inc_init<kInitThreads, PREC>);
+    if (e == cudaSuccess) e = set_smem(k_inc_init<kInitThreads, PREC>);
     if (e == cudaSuccess) k_inc_init<kInitThreads, PREC><<<ginit, kInitThreads, ismem, st>>>(T, S, X, I, C);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -2692,7 +2689,7 @@ cudaError_t launch_one_prec(Topo T, State S, Search X, Inc I, Ctrl *C, int verif
 template <int PREC>
 cudaError_t prepare_batch_prec(const IncPlan &pl) {
     return batch_kernels<PREC>(pl.cs, pl.sh.threads, [&](auto nt, auto c) {
-        return set_smem(k_search_inc_batch<decltype(nt)::value, PREC, decltype(c)::value>, pl.bytes);
+        return set_smem(k_search_inc_batch<decltype(nt)::value, PREC, decltype(c)::value>);
     });
 }
 template <int PREC>
@@ -2709,7 +2706,7 @@ int batch_clusters_prec(const IncPlan &pl) {
         const auto kern = k_search_inc_batch<decltype(nt)::value, PREC, cs>;
         cudaLaunchAttribute at[1];
         const cudaLaunchConfig_t cfg = search_config(cs, decltype(nt)::value, cs, pl.bytes, nullptr, at);
-        const cudaError_t e1 = set_smem(kern, pl.bytes);
+        const cudaError_t e1 = set_smem(kern);
         return e1 != cudaSuccess ? e1 : cudaOccupancyMaxActiveClusters(&count, kern, &cfg);
     });
     if (e != cudaSuccess) cudaGetLastError();
@@ -2717,7 +2714,7 @@ int batch_clusters_prec(const IncPlan &pl) {
 }
 template <int PREC>
 cudaError_t prepare_init_prec() {
-    return set_init_smem(k_inc_init_batch<kInitThreads, PREC>);
+    return set_smem(k_inc_init_batch<kInitThreads, PREC>);
 }
 template <int PREC>
 void launch_init_prec(const BatchFeeder *fd, const int *order, const int *cta_off, int nf, int cta0, int ctas, size_t ismem,
