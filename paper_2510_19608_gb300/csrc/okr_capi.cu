@@ -139,6 +139,8 @@ okr_status fail(okr_ctx *c, okr_status s, const char *fmt, ...) {
     vsnprintf(buf, sizeof buf, fmt, ap);
     va_end(ap);
     if (c) c->err = buf;
+    // the runtime keeps a failed call's error for the thread's next check of a launch
+    if (s == OKR_ECUDA || s == OKR_ENOMEM) cudaGetLastError();
     return s;
 }
 
