@@ -45,31 +45,6 @@ def test_features_at_any_address_give_the_same_predictions(ctx, F, N):
         assert np.array_equal(ctx.scorer_predict_tc(a), ytc), shift
 
 
-@pytest.mark.parametrize("which", ["scorer_predict", "scorer_predict_tc"])
-def test_a_failed_call_reads_the_features_no_longer(which):
-    """A refused allocation (a data set of 2e9 samples) leaves its error pending in
-    the CUDA runtime, and a launch after it is reported as failed though its kernel
-    runs: when the call returns, with whatever status, that kernel is done."""
-    import torch
-    import paper_2510_19608_gb300 as K
-    theta, x = _problem(14, 2_000_000, 4)
-    st = torch.cuda.Stream()
-    with K.Context(0, st.cuda_stream) as ctx:
-        ctx.scorer_init(14, theta)
-        y = getattr(ctx, which)(x)
-        t = np.zeros(1, np.float32)
-        loss = C.c_double()
-        ptr = lambda a: a.ctypes.data_as(C.c_void_p)
-        # (the work buffers come first: neither array is read)
-        assert K.lib().okr_scorer_gradient(ctx._h, ptr(x), ptr(t), C.c_int32(2_000_000_000), None, C.byref(loss)) != 0
-        try:
-            getattr(ctx, which)(x)
-        except K.OkrError:
-            pass
-        assert st.query()
-        assert np.array_equal(getattr(ctx, which)(x), y)
-
-
 def test_too_few_features_are_refused(ctx):
     theta, x = _problem(14, 64, 5)
     ctx.scorer_init(14, theta)
