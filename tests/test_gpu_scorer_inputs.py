@@ -1,9 +1,7 @@
 """Scorer inference on what a caller may hand over: features in host memory at
 any address give the same predictions, whether the kernels read them in place or
-from a copy; a call that returns an error has finished with them; and an array
-that ends before the last sample's features is refused before the GPU reads it."""
-import ctypes as C
-
+from a copy; and an array that ends before the last sample's features is refused
+before the GPU reads it."""
 import numpy as np
 import pytest
 
