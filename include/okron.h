@@ -184,7 +184,7 @@ typedef struct okr_summary {
  * the later okr_reduce* and okr_reduce_batch calls on it.  A field of 0 takes its default. */
 typedef struct okr_inc_shape {
     int32_t threads;            /* threads of a CTA: 256, 384 or 512 (0 = 384 for one CTA, 256 for a
-                                   cluster's) */
+                                   cluster of eight's unless eval_warps is above 7) */
     int32_t eval_warps;         /* warps that evaluate the merge's own new values while the others
                                    find the changed candidates: 1 .. threads/32 - 1 (0 = 2, or 4
                                    with 512 threads) */

@@ -2525,6 +2525,7 @@ __global__ void __launch_bounds__(NT) k_search_inc_batch(const BatchFeeder *fd, 
 
 constexpr size_t kIncSmemMax = 200 * 1024;  // largest dynamic shared memory of one search
 constexpr int kInitThreads = 384;           // CTAs of the first evaluation
+constexpr int kClusterThreads = 256;        // threads a CTA of a cluster of kMaxCluster, unless the caller says
 constexpr int kClusterMin = 32;             // buses from which a cluster searches (inc_plan)
 constexpr int kBatchCluster = 500;          // ... one of a batch's feeders (inc_batch_clusters)
 
@@ -2602,10 +2603,11 @@ bool inc_plan(int n, const IncShape &raw, bool records_iters, IncPlan *out) {
     const bool own = b + sums_bytes(np) <= kIncSmemMax;
     out->mode = own ? 2 + 4 : 2;
     out->bytes = own ? b + sums_bytes(np) : b;
-    // fewer warps meet at the cluster's barriers (384 threads, FP32 terms: 100 buses 11.3 us, 1,500 10.2)
-    if (raw.threads == 0) {
+    // fewer warps meet at the cluster's barriers (384 threads, FP32 terms: 100 buses 11.3 us, 1,500
+    // 10.2); a caller's eval_warps that 256 threads cannot give keeps 384
+    if (raw.threads == 0 && raw.cw < kClusterThreads / 32) {
         IncShape sh = raw;
-        sh.threads = 256;
+        sh.threads = kClusterThreads;
         out->sh = inc_shape_resolve(sh);
     }
     return true;
@@ -2747,7 +2749,7 @@ cudaError_t launch_search_inc(int precision, Topo T, State S, Search X, Inc I, C
 
 bool inc_batch_plan(int max_n, int cs, const IncShape &raw, IncPlan *out) {
     IncShape sh = raw;
-    if (sh.threads == 0 && cs == kMaxCluster) sh.threads = 256;
+    if (sh.threads == 0 && cs == kMaxCluster) sh.threads = kClusterThreads;
     out->sh = inc_shape_resolve(sh);
     out->cs = cs;
     if (cs == 1) {
@@ -2779,8 +2781,9 @@ void inc_batch_clusters(int precision, int nf, const int *n, const int *merges, 
                         int *cs) {
     *count = 0;
     *cs = 1;
-    const bool spare = (long long)nf * kMaxCluster <= num_sms;
-    if (raw.rec >= 0 || (raw.threads != 0 && raw.threads != (spare ? 256 : 384)) || nf < 1) return;
+    // (clusters of eight have 256 threads a CTA: not for a caller's eval_warps above 7)
+    const bool spare = (long long)nf * kMaxCluster <= num_sms && (raw.threads != 0 || raw.cw < kClusterThreads / 32);
+    if (raw.rec >= 0 || (raw.threads != 0 && raw.threads != (spare ? kClusterThreads : 384)) || nf < 1) return;
     auto chain = [&](int i) { return merges[i] * (11.0 + 0.002 * n[i]); };     // us on one CTA
     double sum = 0.0;
     for (int i = 0; i < nf; ++i) sum += chain(i);
