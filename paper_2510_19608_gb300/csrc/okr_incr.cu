@@ -327,12 +327,14 @@ __device__ int slot_geometry(const Topo &T, const State &S, const View &V, int n
 // 2^(kLimbBits i - 100)): a term is added limb by limb by the four lanes of its
 // scenario, each with one 32-bit add that returns nothing, and the entry's
 // 128-bit sum is put together once, modulo 2^128 -- the same integer as adding
-// 128-bit terms, in any order.  An entry takes at most 2 states x 4 scenarios x
-// 13,900 positions, 111,200 adds below 2^14 in size, which 31 bits hold.  (The
+// 128-bit terms, in any order.  An entry takes at most 2 states x kMaxScen scenarios
+// x n positions, a limb one add of at most 2^14 + 2 in size each: 31 bits hold
+// kLimbMaxBus buses (16,382), and kIncSmemMax admits fewer (asserted there).  (The
 // 128-bit adds these replace, a 64-bit shared add that returns the old value,
 // then the carry's, cost about 500 cycles of each round's chain, and the
 // 128-bit shifts and shuffles before them as much.)
 constexpr int kLimbBits = 14, kLimbs = 10, kTile = 192;
+constexpr int kLimbMaxBus = (int)(INT_MAX / (2 * kMaxScen * ((1 << kLimbBits) + 2)));
 struct EvalSmem {
     int d[kLimbs][kTile + 1], b[kLimbs][kTile + 1];     // (+ 1: the limbs of an entry in different banks)
     int n1[kTile], n2[kTile];
@@ -2524,6 +2526,12 @@ __global__ void __launch_bounds__(NT) k_search_inc_batch(const BatchFeeder *fd, 
 }
 
 constexpr size_t kIncSmemMax = 200 * 1024;  // largest dynamic shared memory of one search
+// no feeder that fits (fewest entries in shared memory, one CTA or a cluster) overflows the sums' limbs
+constexpr size_t least_bytes(int n, int cs) {
+    return base_bytes(n, 1, cs) + (cs > 1 ? align16(rec_maxm_bytes(own_pairs(n, 0, cs))) : 0);
+}
+static_assert(least_bytes(kLimbMaxBus + 1, 1) > kIncSmemMax && least_bytes(kLimbMaxBus + 1, 2) > kIncSmemMax &&
+              least_bytes(kLimbMaxBus + 1, kMaxCluster) > kIncSmemMax, "limb_sum: more buses than 31 bits hold");
 constexpr int kInitThreads = 384;           // CTAs of the first evaluation
 constexpr int kClusterThreads = 256;        // threads a CTA of a cluster of kMaxCluster, unless the caller says
 constexpr int kClusterMin = 32;             // buses from which a cluster searches (inc_plan)
