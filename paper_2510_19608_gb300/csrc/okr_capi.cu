@@ -1415,7 +1415,7 @@ static okr_status batch_enqueue(okr_ctx *ctx, BatchRun &R, cudaStream_t st, bool
     if (!captured) CK(join_side(ctx));          // (the setup forks onto the side stream)
     CK(cudaMemcpyAsync(R.base, R.hb, R.staged, cudaMemcpyHostToDevice, st));
     CK(cudaEventRecordWithFlags(R.ev[0], st, evf));
-    CK(launch_batch_setup(nf, R.maxL, R.max_nn, R.bs_d, kPfTol, kPfMaxIter, ctx->num_sms, st, ctx->side, R.ev_fork,
+    CK(launch_batch_setup(nf, R.maxL, R.max_nn, R.tot_n, R.bs_d, kPfTol, kPfMaxIter, ctx->num_sms, st, ctx->side, R.ev_fork,
                           R.ev_join));
     CK(cudaEventRecordWithFlags(R.ev[1], st, evf));
     R.ctas = 0;

@@ -57,7 +57,7 @@ cudaError_t prepare_batch_setup();
 // the line inverses, path impedances and LCA tables run on `side` (forked from st after the per-feeder prep by
 // ev_fork, joined back into st by ev_join before the call returns), the load
 // flows on st.
-cudaError_t launch_batch_setup(int nf, int max_L, long long max_nn, const BatchSetup *bs, double tol, int max_iter,
+cudaError_t launch_batch_setup(int nf, int max_L, long long max_nn, long long tot_n, const BatchSetup *bs, double tol, int max_iter,
                                int num_sms, cudaStream_t st, cudaStream_t side, cudaEvent_t ev_fork,
                                cudaEvent_t ev_join);
 

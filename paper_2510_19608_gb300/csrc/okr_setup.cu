@@ -75,6 +75,41 @@ __device__ bool inv3_lanes(const double2 *a, unsigned m, int j, double2 (&w)[3],
     return ok;
 }
 
+// The same by one thread, operation for operation: half the FP64 instructions (a
+// group's idle lanes and repeated magnitudes cost as much as its columns), a chain
+// three times as long.
+__device__ bool inv3_thread(const double2 *a, unsigned m, double2 *out) {
+    int idx[3], k = 0;
+    for (int p = 0; p < 3; ++p)
+        if (m >> p & 1u) idx[k++] = p;
+    double2 w[3][6];
+    for (int i = 0; i < k; ++i)
+        for (int j = 0; j < 2 * k; ++j)
+            w[i][j] = (j < k) ? a[idx[i] * 3 + idx[j]] : make_double2(j - k == i ? 1.0 : 0.0, 0.0);
+    for (int q = 0; q < 9; ++q) out[q] = make_double2(0.0, 0.0);
+    for (int c = 0; c < k; ++c) {
+        int piv = c;
+        double best = cmag(w[c][c]);
+        for (int i = c + 1; i < k; ++i) {
+            const double v = cmag(w[i][c]);
+            if (v > best) { best = v; piv = i; }
+        }
+        if (best == 0.0) return false;
+        if (piv != c)
+            for (int j = 0; j < 2 * k; ++j) { const double2 t = w[c][j]; w[c][j] = w[piv][j]; w[piv][j] = t; }
+        const double2 d = w[c][c];
+        for (int j = 0; j < 2 * k; ++j) w[c][j] = cdiv(w[c][j], d);
+        for (int i = 0; i < k; ++i) {
+            if (i == c) continue;
+            const double2 f = w[i][c];
+            for (int j = 0; j < 2 * k; ++j) w[i][j] = csub(w[i][j], cmul(f, w[c][j]));
+        }
+    }
+    for (int i = 0; i < k; ++i)
+        for (int j = 0; j < k; ++j) out[idx[i] * 3 + idx[j]] = w[i][k + j];
+    return true;
+}
+
 __device__ __forceinline__ void block_barrier() { __syncthreads(); }
 
 // out[i] = in[0] + ... + in[i - 1] for i <= n (one CTA, blockDim.x a multiple
@@ -394,6 +429,15 @@ __device__ void dev_line_inverses(int n, Topo T, int *err, int first, int stride
             for (int i = 0; i < 3; ++i)
                 if (i < k) y[idx[i] * 3 + cj] = w[i];
         }
+    }
+}
+
+// The same, one thread per line (for batches, whose lines fill the FP64 units).
+__device__ void dev_line_inverses_wide(int n, Topo T, int *err, int first, int stride) {
+    for (int v = first; v < n; v += stride) {
+        double2 y[9];
+        if (!inv3_thread(T.zl + (size_t)v * 9, v > 0 ? T.ph[v] : 0u, y)) atomicExch(err, 2);
+        for (int q = 0; q < 9; ++q) T.yl[(size_t)v * 9 + q] = y[q];
     }
 }
 
@@ -733,22 +777,27 @@ __global__ void __launch_bounds__(256) k_power_flow(int n, int L, Topo T, const 
 }
 
 // The load flow of one scenario by one CTA with everything it touches in a sweep
-// but the loads and the line impedances in shared memory (voltages, currents and
-// the tree): the same sweep, operation for operation, as k_power_flow, with block
+// but the loads and the line impedances in shared memory (voltages, VS, currents
+// and the tree): the same sweep, operation for operation, as k_power_flow, with block
 // barriers in place of grid barriers.  For small feeders, whose grid barriers and
 // trips to L2 were the time (40 buses: 145 us), and for batches, whose many CTAs
 // spread the FP64 work.
 constexpr int kPfCta = 1920;        // buses whose load flow fits one CTA's shared memory
 constexpr int kPfSmall = 256;       // buses up to which a single feeder takes one CTA per scenario
 constexpr int kPfThreads = 512;
-__host__ __device__ constexpr size_t pf_cta_bytes(int n) { return sizeof(double2) * 6 * (size_t)n + tree_bytes(n); }
+__host__ __device__ constexpr size_t pf_cta_bytes(int n, bool vs = true) {
+    return sizeof(double2) * (vs ? 6 : 3) * (size_t)n + tree_bytes(n);
+}
+// (VS false: the voltages stay in device memory, each read and written by one thread
+// but the slack's, which no sweep writes)
+template <bool VS>
 __device__ void dev_power_flow_smem(int n, int l, const Topo &T, const double *__restrict__ s_in, double tol,
                                     int max_iter, int *iters, int *err, double2 *sm) {
     __shared__ double s_mx[32];
     __shared__ int s_ok;
     const int tid = threadIdx.x, nt = blockDim.x, maxd = T.maxd[0];
-    double2 *V = sm, *W = sm + 3 * (size_t)n;
-    const TreeSm tr = load_tree(T, n, maxd, sm + 6 * (size_t)n);
+    double2 *W = sm, *V = VS ? sm + 3 * (size_t)n : T.vhat + (size_t)l * 3 * n;
+    const TreeSm tr = load_tree(T, n, maxd, sm + (VS ? 6 : 3) * (size_t)n);
     for (int e = tid; e < 3 * n; e += nt) {
         const int p = e / n, v = e - p * n;
         V[e] = (T.ph[v] >> p & 1u) ? T.vslack[p] : make_double2(0.0, 0.0);
@@ -827,7 +876,7 @@ __device__ void dev_power_flow_smem(int n, int l, const Topo &T, const double *_
         __syncthreads();
         if (s_ok) { conv = true; break; }
     }
-    for (int e = tid; e < 3 * n; e += nt) T.vhat[(size_t)l * 3 * n + e] = V[e];
+    for (int e = tid; VS && e < 3 * n; e += nt) T.vhat[(size_t)l * 3 * n + e] = V[e];
     if (tid == 0) {
         iters[l] = conv ? it : -1;
         if (!conv) atomicCAS(err, 0, 3);
@@ -839,7 +888,7 @@ __global__ void __launch_bounds__(kPfThreads) k_power_flow_cta(int n, Topo T, co
     extern __shared__ double2 pfc_sm[];
     // (err is not looked at: the line inverses beside this kernel may be setting it,
     // and threads that saw it and left would leave the tree half loaded)
-    dev_power_flow_smem(n, blockIdx.x, T, s_in, tol, max_iter, iters, err, pfc_sm);
+    dev_power_flow_smem<true>(n, blockIdx.x, T, s_in, tol, max_iter, iters, err, pfc_sm);
 }
 
 // One CTA per scenario on small feeders; otherwise the cooperative load flow
@@ -1057,13 +1106,19 @@ __global__ void __launch_bounds__(1024) k_batch_prep(const BatchSetup *bs) {
     dev_line_copy(b.n, b.T, b.z_in, threadIdx.x, blockDim.x);
 }
 
-// Line inverses (blockIdx.x = 9) and path impedances, entry blockIdx.x of the
+// Line inverses (blockIdx.x >= 9) and path impedances, entry blockIdx.x of the
 // matrices; blockIdx.y = feeder.  Beside the load flows, which read neither.
+// WIDE: one thread per line, for batches whose lines fill the FP64 units that the
+// load flows want too (launch_batch_setup); otherwise eight lanes per line, for the
+// chains' latency.  A kernel each: both in one took the registers of both.
+template <bool WIDE>
 __global__ void __launch_bounds__(256) k_batch_lines(const BatchSetup *bs) {
     const BatchSetup &b = bs[blockIdx.y];
     if (*(volatile int *)b.err == 1) return;
-    if (blockIdx.x >= 9) dev_line_inverses(b.n, b.T, b.err, (blockIdx.x - 9) * blockDim.x + threadIdx.x, (gridDim.x - 9) * blockDim.x);
-    else dev_path_impedance(b.n, b.T, blockIdx.x, nullptr);
+    const int first = (blockIdx.x - 9) * blockDim.x + threadIdx.x, stride = (gridDim.x - 9) * blockDim.x;
+    if (blockIdx.x < 9) dev_path_impedance(b.n, b.T, blockIdx.x, nullptr);
+    else if (WIDE) dev_line_inverses_wide(b.n, b.T, b.err, first, stride);
+    else dev_line_inverses(b.n, b.T, b.err, first, stride);
 }
 
 // LCA tables: blockIdx.y = feeder.
@@ -1075,13 +1130,14 @@ __global__ void k_batch_lca(const BatchSetup *bs) {
 }
 
 // Load flow: blockIdx.y = feeder, blockIdx.x = scenario.
+template <bool VS>
 __global__ void __launch_bounds__(kPfThreads) k_batch_pf(const BatchSetup *bs, double tol, int max_iter) {
     extern __shared__ double2 pfb_sm[];
     __shared__ BatchSetup b;
     if (threadIdx.x == 0) b = bs[blockIdx.y];
     __syncthreads();
     if ((int)blockIdx.x >= b.L || *(volatile int *)b.err == 1) return;
-    if (b.n <= kPfCta) dev_power_flow_smem(b.n, blockIdx.x, b.T, b.s_in, tol, max_iter, b.pf_iters, b.err, pfb_sm);
+    if (b.n <= kPfCta) dev_power_flow_smem<VS>(b.n, blockIdx.x, b.T, b.s_in, tol, max_iter, b.pf_iters, b.err, pfb_sm);
     else dev_power_flow_cta(b.n, blockIdx.x, b.T, b.s_in, tol, max_iter, b.J, b.pf_iters, b.err);
 }
 
@@ -1107,18 +1163,15 @@ __global__ void __launch_bounds__(1024) k_batch_finish(const BatchSetup *bs) {
     for (int i = threadIdx.x; i < b.n / 32 + 2; i += blockDim.x) b.bmax[i] = 0.0;
 }
 
-// Dynamic shared memory of a batch's load flows (its largest feeder; larger than
-// kPfCta run in device memory).
-static size_t batch_pf_smem(long long max_nn) {
-    int n = 1;
-    while (n < kPfCta && (long long)n * n < max_nn) ++n;
-    return pf_cta_bytes(n);
-}
+constexpr size_t kPfHalfSm = 112 * 1024;    // shared memory of a CTA of which an SM holds two
 cudaError_t prepare_batch_setup() {
-    return cudaFuncSetAttribute(k_batch_pf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pf_cta_bytes(kPfCta));
+    const cudaError_t e = cudaFuncSetAttribute(k_batch_pf<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)pf_cta_bytes(kPfCta));
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(k_batch_pf<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       (int)pf_cta_bytes(kPfCta, false));
 }
 
-cudaError_t launch_batch_setup(int nf, int max_L, long long max_nn, const BatchSetup *bs, double tol, int max_iter,
+cudaError_t launch_batch_setup(int nf, int max_L, long long max_nn, long long tot_n, const BatchSetup *bs, double tol, int max_iter,
                                int num_sms, cudaStream_t st, cudaStream_t side, cudaEvent_t ev_fork,
                                cudaEvent_t ev_join) {
     if (nf <= 0) return cudaSuccess;
@@ -1131,11 +1184,27 @@ cudaError_t launch_batch_setup(int nf, int max_L, long long max_nn, const BatchS
     long long bx = (max_nn + 255) / 256;
     if (bx > num_sms * 2) bx = num_sms * 2;
     if (bx < 1) bx = 1;
-    k_batch_lines<<<dim3(9 + 8, nf), 256, 0, side>>>(bs);
+    // (one thread per line from 15,000 lines on, and 128 a feeder: fewer would be a
+    // warp or two a feeder; the setup of 300 feeders of 900 buses, one scenario, 2.19 ->
+    // 1.94 ms, of 16 such 0.87 either way, of 600 of 60 0.40 / 0.42)
+    if (tot_n > 15000 && tot_n >= 128LL * nf) k_batch_lines<true><<<dim3(9 + 8, nf), 256, 0, side>>>(bs);
+    else k_batch_lines<false><<<dim3(9 + 8, nf), 256, 0, side>>>(bs);
     k_batch_lca<<<dim3((unsigned)bx, nf), 256, 0, side>>>(bs);
     e = cudaEventRecord(ev_join, side);
     if (e != cudaSuccess) return e;
-    k_batch_pf<<<dim3(max_L, nf), kPfThreads, batch_pf_smem(max_nn), st>>>(bs, tol, max_iter);
+    // every CTA has the shared memory of the largest feeder (larger than kPfCta: of
+    // kPfCta, and they run in device memory).  Where that lets one CTA run on an SM
+    // and there are more than two rounds of them, the voltages stay in device memory
+    // and two run: one feeder of 1,900 buses beside 2,000 of 40, four scenarios, setup
+    // 3.80 -> 3.09 ms; 600 of 1,280, one scenario, 6.33 -> 6.12; with two rounds it
+    // gains nothing (300 of 1,900: 5.33 / 5.57), with one it loses (16 of 1,280: 0.74 / 1.16).
+    int n = 1;
+    while (n < kPfCta && (long long)n * n < max_nn) ++n;
+    const size_t smem = pf_cta_bytes(n);
+    if (smem > kPfHalfSm && (long long)nf * max_L > 2 * num_sms)
+        k_batch_pf<false><<<dim3(max_L, nf), kPfThreads, pf_cta_bytes(n, false), st>>>(bs, tol, max_iter);
+    else
+        k_batch_pf<true><<<dim3(max_L, nf), kPfThreads, smem, st>>>(bs, tol, max_iter);
     e = cudaStreamWaitEvent(st, ev_join, 0);            // (the injections read the line inverses)
     if (e != cudaSuccess) return e;
     k_batch_finish<<<nf, 1024, 0, st>>>(bs);
