@@ -1569,8 +1569,12 @@ static okr_status reduce_batch_impl(okr_ctx *ctx, int32_t nf, const okr_feeder *
     s = batch_fill(ctx, R, feeders);
     if (s != OKR_OK) return s;
     s = batch_enqueue(ctx, R, ctx->stream, super_of != nullptr, false);
+    // (after a refused launch too: the side stream's searches and the copy out of the
+    // pinned block would meet the next call's buffers)
+    if (s != OKR_OK) cudaStreamSynchronize(ctx->side);
+    const cudaError_t w = cudaStreamSynchronize(ctx->stream);
     if (s != OKR_OK) return s;
-    CK(cudaStreamSynchronize(ctx->stream));
+    CK(w);
     return batch_finish(ctx, R, items, super_of, stats);
 }
 
