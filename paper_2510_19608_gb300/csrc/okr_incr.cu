@@ -44,9 +44,9 @@
 // applied in FP64.
 //
 // Execution.  One cluster of eight CTAs (inc_plan; in a batch one CTA, or a
-// cluster for the longest searches, inc_batch_clusters) runs a feeder's whole search; its steps are separated by block or cluster barriers
-// only (no grid barrier, no device-side wait).  The chain of dependent merges
-// bounds it: neither a pipe nor memory is busy, so what counts is the number of
+// cluster for the longest searches, inc_batch_clusters) runs a feeder's whole
+// search; its steps are separated by block or cluster barriers only (no grid
+// barrier, no device-side wait).  The chain of dependent merges bounds it: neither a pipe nor memory is busy, so what counts is the number of
 // dependent steps per merge and the latency of each.  A term is evaluated by a
 // group of lanes, one per (scenario, phase).  Each merge takes three steps:
 //   1. selection over the records (in a cluster two exchanges of minima);
@@ -2535,7 +2535,8 @@ static_assert(least_bytes(kLimbMaxBus + 1, 1) > kIncSmemMax && least_bytes(kLimb
 constexpr int kInitThreads = 384;           // CTAs of the first evaluation
 constexpr int kClusterThreads = 256;        // threads a CTA of a cluster of kMaxCluster, unless the caller says
 constexpr int kClusterMin = 32;             // buses from which a cluster searches (inc_plan)
-constexpr int kBatchCluster = 500;          // ... one of a batch's feeders (inc_batch_clusters)
+constexpr int kBatchCluster = 500;          // ... one of a batch's feeders (inc_batch_clusters; below it eight CTAs
+                                            // were slower in the one batch tried, two have not been measured)
 
 // Before every launch, whatever its size: without asking a launch gets 48 KB less
 // the kernel's 17 to 21 KB of static arrays.  Always the same limit: it is the
@@ -2590,9 +2591,9 @@ bool inc_smem(int n, bool maxm, const IncShape &sh, int *rec_mode, size_t *bytes
 
 // One CTA or a cluster of kMaxCluster.  A cluster shares out the scan over the
 // slot pairs, the FP64 evaluation of the merge, the changed terms and the
-// records (which then always fit shared memory, the carried sums and candidates
-// up to about 4,200 buses), and pays three cluster barriers a merge and L2 in
-// place of L1 latency.  us a merge, one CTA of 384 threads / eight of 256 (one
+// records (in shared memory up to 9,792 buses, above which one CTA searches; the
+// carried sums and candidates too up to 4,404), and pays three cluster barriers a
+// merge and L2 in place of L1 latency.  us a merge, one CTA of 384 threads / eight of 256 (one
 // scenario; 400 buses two):
 //   FP64 terms:  60 buses 13.4 / 12.3, 100 12.5 / 11.6, 400 16.3 / 11.7, 600 15.3 / 11.2, 1,500 17.7 / 11.5
 //   FP32 terms:  60 buses 12.0 / 11.5, 100 11.1 / 10.6, 400 13.2 / 10.9, 600 12.2 / 9.8, 1,500 13.8 / 9.8
@@ -2792,7 +2793,9 @@ void inc_batch_clusters(int precision, int nf, const int *n, const int *merges, 
     // (clusters of eight have 256 threads a CTA: not for a caller's eval_warps above 7)
     const bool spare = (long long)nf * kMaxCluster <= num_sms && (raw.threads != 0 || raw.cw < kClusterThreads / 32);
     if (raw.rec >= 0 || (raw.threads != 0 && raw.threads != (spare ? kClusterThreads : 384)) || nf < 1) return;
-    auto chain = [&](int i) { return merges[i] * (11.0 + 0.002 * n[i]); };     // us on one CTA
+    // us on one CTA, FP32 terms (compared with the other feeders of the launch, which
+    // have the same precision: FP64 terms cost a tenth to a quarter more on each)
+    auto chain = [&](int i) { return merges[i] * (11.0 + 0.002 * n[i]); };
     double sum = 0.0;
     for (int i = 0; i < nf; ++i) sum += chain(i);
     int k = 0, max_n = 2;

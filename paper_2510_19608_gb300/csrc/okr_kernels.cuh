@@ -50,15 +50,16 @@ struct BatchSetup {
     double *dec_maxerr, *mrank, *bmax;
     int *arrive;
 };
-// prepare_batch_setup sets the load flow's shared-memory attribute (before any
+// prepare_batch_setup sets the load flows' shared-memory attributes (before any
 // stream capture).
 cudaError_t prepare_batch_setup();
 // Setup of many feeders in five launches (CTA per feeder, per feeder x scenario):
-// the line inverses, path impedances and LCA tables run on `side` (forked from st after the per-feeder prep by
-// ev_fork, joined back into st by ev_join before the call returns), the load
-// flows on st.
-cudaError_t launch_batch_setup(int nf, int max_L, long long max_nn, long long tot_n, const BatchSetup *bs, double tol, int max_iter,
-                               int num_sms, cudaStream_t st, cudaStream_t side, cudaEvent_t ev_fork,
+// the line inverses, path impedances and LCA tables run on `side` (forked from st
+// after the per-feeder prep by ev_fork, joined back into st by ev_join before the
+// call returns), the load flows on st.  max_nn: the largest feeder's buses squared;
+// tot_n: the buses of all.
+cudaError_t launch_batch_setup(int nf, int max_L, long long max_nn, long long tot_n, const BatchSetup *bs, double tol,
+                               int max_iter, int num_sms, cudaStream_t st, cudaStream_t side, cudaEvent_t ev_fork,
                                cudaEvent_t ev_join);
 
 // The reduced network of a caller assignment (one CTA per scenario).

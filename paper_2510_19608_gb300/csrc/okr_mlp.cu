@@ -140,7 +140,8 @@ __device__ __forceinline__ void tile_store(float *out, int tx, int ty, const flo
 // tx units tx, tx + 32, tx + 64, tx + 96 (16 sums a thread; five shared loads,
 // 32 bytes a thread, feed 16 multiply-adds: the loads' 128 bytes a cycle and SM
 // bound it).  For few samples: 4,096 of a training step are 128 CTAs, 25 us
-// forward and back (195 us in two kernels before).  TRAIN: the whole pass forward and back through the activations,
+// forward and back (195 us in two kernels before).  TRAIN: the whole pass forward and back through
+// the activations,
 //   dy = scale (y - t); d3 = dy w4 [h3 > 0]; d2 = (d3 W3^T) [h2 > 0];
 //   d1 = (d2 W2^T) [h1 > 0],
 // with h1, h2, h3, d1, d2, d3 [N][H] and dy [N] written for the weight
@@ -396,9 +397,9 @@ struct WJob {
 // 32 x 16 (2 x 4 each: one 8-byte and one 16-byte shared load feed eight
 // multiply-adds; 2 x 2 outputs were bound by the shared loads, 77 us against 33
 // for 4,096 samples, of which the chains of 2,048 samples at 12 instructions
-// each are 12 us and the staging and waits the rest), the segment's rows of A and D pass through a four-stage
-// cp.async pipeline.  The last CTA of a segment sums the squared errors into
-// loss[seg].
+// each are 12 us and the staging and waits the rest), the segment's rows of A and D
+// pass through a three-stage cp.async pipeline.  The last CTA of a segment sums the
+// squared errors into loss[seg].
 constexpr int kWThreads = 64, kWK = 32, kWC = 16;
 __global__ void __launch_bounds__(kWThreads) k_mlp_wgrad(WJob j0, WJob j1, WJob j2, WJob j3, const float *__restrict__ y,
                                                          const float *__restrict__ t, int N, int P, float *part,

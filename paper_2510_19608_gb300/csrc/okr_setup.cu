@@ -1090,8 +1090,8 @@ __device__ void dev_power_flow_cta(int n, int l, const Topo &T, const double *__
     }
 }
 
-// Per feeder, one CTA: validation and renumbering, children, sparse table,
-// line inverses, path impedances.
+// Per feeder, one CTA: validation and renumbering, children, sparse table, line
+// impedances in preorder.
 __global__ void __launch_bounds__(1024) k_batch_prep(const BatchSetup *bs) {
     __shared__ BatchSetup b;
     if (threadIdx.x == 0) b = bs[blockIdx.x];
@@ -1171,8 +1171,8 @@ cudaError_t prepare_batch_setup() {
                                                        (int)pf_cta_bytes(kPfCta, false));
 }
 
-cudaError_t launch_batch_setup(int nf, int max_L, long long max_nn, long long tot_n, const BatchSetup *bs, double tol, int max_iter,
-                               int num_sms, cudaStream_t st, cudaStream_t side, cudaEvent_t ev_fork,
+cudaError_t launch_batch_setup(int nf, int max_L, long long max_nn, long long tot_n, const BatchSetup *bs, double tol,
+                               int max_iter, int num_sms, cudaStream_t st, cudaStream_t side, cudaEvent_t ev_fork,
                                cudaEvent_t ev_join) {
     if (nf <= 0) return cudaSuccess;
     k_batch_prep<<<nf, 1024, 0, st>>>(bs);
