@@ -36,8 +36,8 @@ FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 FLOPS_PER_ITEM = 40
 # DRAM bytes of one search launch on this workload from the ncu capture in
 # profiles/, valid only for the kernel source it was taken on (None otherwise)
-NCU_TRAFFIC = {"bytes": 1129216 + 4864, "source": "paper_2510_19608_gb300/csrc/okr_incr.cu",
-               "sha256_prefix": "9e45052b307a77f7", "summary": "profiles/k_search_inc_feeder1000.md"}
+NCU_TRAFFIC = {"bytes": 1131008 + 4352, "source": "paper_2510_19608_gb300/csrc/okr_incr.cu",
+               "sha256_prefix": "7e1afdd002ed541f", "summary": "profiles/k_search_inc_feeder1000.md"}
 L2_FLUSH_BYTES = 256 << 20  # > 129 MB L2
 
 # Latency floor of one merge of the incremental search.  One merge is a chain

@@ -1199,9 +1199,9 @@ cudaError_t launch_batch_setup(int nf, int max_L, long long max_nn, long long to
     if (e != cudaSuccess) return e;
     // every CTA has the shared memory of the largest feeder (larger than kPfCta: of
     // kPfCta, and they run in device memory).  Where that lets one CTA run on an SM
-    // and there are more than two rounds of them, the voltages stay in device memory
+    // and there are more than two waves of them, the voltages stay in device memory
     // and two run: one feeder of 1,900 buses beside 2,000 of 40, four scenarios, setup
-    // 3.80 -> 3.09 ms; 600 of 1,280, one scenario, 6.33 -> 6.12; with two rounds it
+    // 3.80 -> 3.09 ms; 600 of 1,280, one scenario, 6.33 -> 6.12; with two waves it
     // gains nothing (300 of 1,900: 5.33 / 5.57), with one it loses (16 of 1,280: 0.74 / 1.16).
     int n = 1;
     while (n < kPfCta && (long long)n * n < max_nn) ++n;
