@@ -2,7 +2,7 @@
 
 Line inverses: eight lanes per line up to 15,000 lines in the batch or 128 a feeder,
 one thread per line above.  Load flows: the voltages in device memory when the
-largest feeder leaves room for one CTA on an SM and there are more than two rounds of
+largest feeder leaves room for one CTA on an SM and there are more than two waves of
 them; in device memory altogether above 1,920 buses.
 """
 import numpy as np
